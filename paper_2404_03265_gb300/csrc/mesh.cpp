@@ -407,6 +407,10 @@ std::string finalize_mesh(Mesh& m, int k) {
       lm.slot_leaf[slot] = m.nslot[ln];
       if (m.nhang[ln] < 0 && m.nminlev[ln] == l) lm.slot_flags[slot] |= 16;  // home level of a leaf DoF
     }
+    for (uint64_t c : t.lev[l]) {
+      const int64_t i = int64_t(c >> 32), j = int64_t(c & 0xffffffffu);
+      lm.slot_flags[lslot[l][gkey(i * k, j * k)]] |= 32;
+    }
     auto lfind = [&](int64_t gx, int64_t gy) -> int32_t {
       if (gx < 0 || gy < 0 || gx > gnx || gy > gny) return -1;
       auto it = lslot[l].find(gkey(gx, gy));

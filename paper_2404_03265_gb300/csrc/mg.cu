@@ -142,6 +142,27 @@ __global__ void k_copy_in(int64_t nsl, int ncomp, DevHome home, const double* __
   }
 }
 
+// One block per level brick: every level slot is written, so the level defects
+// need no separate clearing.
+template <typename T>
+__global__ void k_level_defects(const LevBrick* __restrict__ bricks, const int32_t* __restrict__ home_leaf, int ncomp,
+                                int64_t nsl, const double* __restrict__ r, T* d, T* x0,
+                                const uint8_t* __restrict__ lcm, int fixbits) {
+  pdl_trigger();
+  const LevBrick b = bricks[blockIdx.x];
+  for (int i = threadIdx.x; i < 900; i += blockDim.x) {
+    const int32_t s = b.base + i;
+    const int32_t leaf = home_leaf[b.off + s];
+    const uint8_t cm = leaf >= 0 ? lcm[leaf] : uint8_t(0);
+    for (int c = 0; c < ncomp; ++c) {
+      const int bit = (fixbits == 4) ? 4 : (1 << c);
+      const int64_t o = int64_t(ncomp) * b.off + c * int64_t(b.n) + s;
+      d[o] = (leaf >= 0 && !(cm & bit)) ? T(r[c * nsl + leaf]) : T(0);
+      if (b.off == 0) x0[o] = T(0);
+    }
+  }
+}
+
 template <typename T>
 __global__ void k_copy_out(int64_t nsl, int ncomp, DevHome home, const T* __restrict__ x,
                            const double* __restrict__ r, double* z, const uint8_t* __restrict__ lcm,
@@ -569,6 +590,15 @@ cudaError_t mg_copy_in(int64_t ns_leaf, int ncomp, DevHome home, const double* r
   return cudaGetLastError();
 }
 template <typename T>
+cudaError_t mg_level_defects(int32_t nbricks, const LevBrick* bricks, const int32_t* home_leaf, int ncomp,
+                             int64_t ns_leaf, const double* r, T* d, T* x0, const uint8_t* leaf_cmask, int fixbits,
+                             cudaStream_t s) {
+  if (nbricks > 0)
+    k_level_defects<T><<<unsigned(nbricks), TPB, 0, s>>>(bricks, home_leaf, ncomp, ns_leaf, r, d, x0, leaf_cmask,
+                                                         fixbits);
+  return cudaGetLastError();
+}
+template <typename T>
 cudaError_t mg_copy_out(int64_t ns_leaf, int ncomp, DevHome home, const T* x, const double* r, double* z,
                         const uint8_t* leaf_cmask, const uint8_t* leaf_flags, int fixbits, cudaStream_t s, bool pdl) {
   if (ns_leaf > 0)
@@ -688,6 +718,8 @@ cudaError_t copy64(int64_t n, double* dst, const double* src, cudaStream_t s) {
   template cudaError_t mg_prolong<T>(int32_t, int, int64_t, int64_t, const int32_t*, const int32_t*,           \
                                      const float*, const T*, T*, const uint8_t*, int, cudaStream_t, bool);     \
   template cudaError_t mg_copy_in<T>(int64_t, int, DevHome, const double*, T*, const uint8_t*, int, cudaStream_t); \
+  template cudaError_t mg_level_defects<T>(int32_t, const LevBrick*, const int32_t*, int, int64_t, const double*, T*, \
+                                           T*, const uint8_t*, int, cudaStream_t);                              \
   template cudaError_t mg_copy_out<T>(int64_t, int, DevHome, const T*, const double*, double*, const uint8_t*,     \
                                       const uint8_t*, int, cudaStream_t, bool);                                    \
   template cudaError_t mg_chebyshev_first_res<T>(int64_t, T*, T*, T*, const T*, const T*, const T*, T, T*,        \

@@ -6,6 +6,8 @@
 
 #include <cstdint>
 
+#include "smooth.cuh"
+
 namespace pff {
 
 // Level-mesh device tables (one per refinement level).
@@ -20,6 +22,14 @@ struct DevLevel {
   const int32_t* R_ptr = nullptr;  // restriction rows (level-1 slots) -> this level's slots
   const int32_t* R_col = nullptr;
   const float* R_val = nullptr;
+  const SmoothTile* tiles = nullptr;  // Q1, level >= 1: tiles of the fused smoothers (smooth.cuh)
+  int32_t ntiles = 0;
+};
+
+// A brick of the concatenated level storage (900 slots): its level's slot offset
+// and slot count, and the brick's first slot on its level.
+struct LevBrick {
+  int32_t off, n, base;
 };
 
 // Home level of each leaf slot: a free leaf node's defect enters, and its
@@ -61,6 +71,13 @@ cudaError_t mg_prolong(int32_t nf, int ncomp, int64_t nf_stride, int64_t nc_stri
 template <typename T>
 cudaError_t mg_copy_in(int64_t ns_leaf, int ncomp, DevHome home, const double* r, T* d, const uint8_t* leaf_cmask,
                        int fixbits, cudaStream_t s);
+// level_defects: d on every level slot, the leaf r on home-level nodes whose
+// component is free and 0 elsewhere, and x0 = 0 on level 0 (the first of the bricks'
+// levels).  home_leaf: per level slot (concatenated) its leaf slot or -1.
+template <typename T>
+cudaError_t mg_level_defects(int32_t nbricks, const LevBrick* bricks, const int32_t* home_leaf, int ncomp,
+                             int64_t ns_leaf, const double* r, T* d, T* x0, const uint8_t* leaf_cmask, int fixbits,
+                             cudaStream_t s);
 template <typename T>
 cudaError_t mg_copy_out(int64_t ns_leaf, int ncomp, DevHome home, const T* x, const double* r, double* z,
                         const uint8_t* leaf_cmask, const uint8_t* leaf_flags, int fixbits, cudaStream_t s,

@@ -552,9 +552,17 @@ cudaError_t vcycle_t(pff_mg& mg, int b, const double* r, double* z, cudaStream_t
     c.af = float(T(ca)); c.bf = float(T(cb)); c.ad = double(T(ca)); c.bd = double(T(cb));
     return c;
   };
-  VC(cudaMemsetAsync(d, 0, nc * N * sizeof(T), s));
-  VC(cudaMemsetAsync(x, 0, nc * N * sizeof(T), s));
-  VC(mg_copy_in<T>(nsleaf, nc, D.home, r, d, pb.cmask, B.fixbits, s));
+  // One launch per level and direction (smooth.cu): FP32, Q1, the default cell loop.
+  // FP64 stays on the sweeps (its time is the FP64 rate, and the tiles' halo cells
+  // would add to it); a forced strip height asks for the sweeps.
+  const bool tiles = sizeof(T) == 4 && M.k == 1 && fuse && pb.sweep_sh == 0 && mg.degree == 3;
+  if (tiles) {
+    VC(mg_level_defects<T>(D.n_lev_bricks, D.lev_bricks, D.home_leaf, nc, nsleaf, r, d, rr, pb.cmask, B.fixbits, s));
+  } else {
+    VC(cudaMemsetAsync(d, 0, nc * N * sizeof(T), s));
+    VC(cudaMemsetAsync(x, 0, nc * N * sizeof(T), s));
+    VC(mg_copy_in<T>(nsleaf, nc, D.home, r, d, pb.cmask, B.fixbits, s));
+  }
   // Chebyshev on level l over [a, bb], `degree` applications of D^-1: solve A v = rhs
   // from v = 0 into out (buffers yp, y, t).  The three iterates (current,
   // previous, next) rotate roles each step; the start is chosen so that the last
@@ -602,6 +610,54 @@ cudaError_t vcycle_t(pff_mg& mg, int b, const double* r, double* z, cudaStream_t
     }
     return cudaSuccess;
   };
+  if constexpr (sizeof(T) == 4) {
+    if (tiles) {
+      auto args = [&](int l) {
+        const DevLevel& lv = D.levels[l].lv;
+        const DevLevel& lc = D.levels[l - 1].lv;
+        const int64_t o = nc * lv.off, oc = nc * lc.off;
+        ApplyArgs k;
+        std::memset(&k, 0, sizeof(k));
+        for (int q = 0; q <= M.Lf && q < kMaxLevels; ++q) { k.hx[q] = M.tree.hx(q); k.hy[q] = M.tree.hy(q); }
+        fill_material(pb.prm, k, pb.has_ecell);
+        fill_cell_constants(k, M.Lf + 1);
+        SmoothArgs a;
+        std::memset(&a, 0, sizeof(a));
+        a.tiles = lv.tiles; a.ntiles = lv.ntiles;
+        a.n = lv.n_slots; a.nc = lc.n_slots;
+        a.flags = lv.flags; a.cmask = mg.cmask + lv.off; a.cmask_c = mg.cmask + lc.off;
+        a.lin = mg.lin32 + 4 * lv.off;
+        a.ecell = pb.has_ecell ? pb.lev_ecell32 + lv.off : nullptr;
+        a.dinv = dinv + o; a.d = d + o; a.dc = d + oc;
+        a.m = k.mf; a.g = k.gf[l];
+        const double lam = B.lam[l];
+        if (lam > 0) {
+          const double lo = mg.lo * lam, hi = mg.hi * lam;
+          const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo), sigma = theta / delta;
+          const double r0 = 1.0 / sigma, r1 = 1.0 / (2.0 * sigma - r0), r2 = 1.0 / (2.0 * sigma - r1);
+          a.c0 = float(1.0 / theta);
+          a.a1 = float(r1 * r0); a.b1 = float(2.0 * r1 / delta);
+          a.a2 = float(r2 * r1); a.b2 = float(2.0 * r2 / delta);
+        }
+        return a;
+      };
+      for (int l = nl - 1; l >= 1; --l) {
+        SmoothArgs a = args(l);
+        a.xout = x + nc * D.levels[l].lv.off;
+        VC(launch_smooth_down(a, block_op(b), s));
+      }
+      if (mg.coarse_mode == 1) VC(cheb_ab(0, d, rr, B.c0_a, B.c0_b, B.c0_deg, false));
+      else VC(mg_coarse<T>(B.n_coarse, B.coarse_idx, B.coarse_inv, d, rr, B.coarse_tmp, s, true));
+      for (int l = 1; l < nl; ++l) {
+        SmoothArgs a = args(l);
+        a.x = x + nc * D.levels[l].lv.off;
+        a.xc = rr + nc * D.levels[l - 1].lv.off;
+        a.xout = rr + nc * D.levels[l].lv.off;
+        VC(launch_smooth_up(a, block_op(b), s));
+      }
+      return mg_copy_out<T>(nsleaf, nc, D.home, rr, r, z, pb.cmask, pb.mesh->dev.slot_flags, B.fixbits, s, true);
+    }
+  }
   // smoothing on level l >= 1: degree mg.degree on [lo, hi] * lambda_max
   auto smooths = [&](int l) { return l >= 1 && B.lam[l] > 0 && mg.degree >= 1; };
   auto cheb = [&](int l, const T* rhs, T* out, bool first_done) -> cudaError_t {

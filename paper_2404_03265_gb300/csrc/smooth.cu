@@ -1,0 +1,441 @@
+// Fused level smoothers of the FP32 Q1 V-cycle (Sec. 3.2 of Kolditz & Wick,
+// arXiv 2404.03265): a whole smoothing of one level, with its transfer, in one launch.
+//
+// Down: Chebyshev degree 3 from zero on A x = d, the residual d - A x and its
+// restriction into the coarser level.  Up: prolongation of the coarse correction and
+// Chebyshev degree 3 on the new residual.  Each does three level applies; a block
+// takes a tile of 15 x 15 nodes and evaluates the cells around it that the three
+// applies need (halo 4 down, 3 up), so nothing is exchanged between blocks.
+//
+// Why: level meshes of a crack mesh hold 10^2..10^5 nodes; a launch per apply is a
+// chain of ~100 dependent launches of 4-6 us, each a few serial L2 round trips and
+// cell rows, with most of the chip idle.  One tile per block needs one round trip
+// per level and direction, and the halo's extra cells (1.8x down, 1.5x up) cost
+// idle issue slots.  Measured (u block, 1.04M-DoF crack mesh, 13 levels): 101 launches
+// and 482 us before, 29 launches and 172 us with the tiles.
+//
+// Arithmetic: every cell, nodal sum, smoother step and transfer row is the
+// expression and order of sweep_q1_kernel, k_restrict and k_prolong (the transfer
+// weights 1, 1/2, 1/4 are exact), so the results are the same bits; cells evaluated
+// by two tiles give the same values in both.
+//
+// Layout in a block: thread t holds the cell pair (i, j), (i, j + CW / 2) as the two
+// members of every packed operation, with the pair's Gauss-point coefficients in
+// registers for all three applies, and up to NPT window nodes (their defect, inverse
+// diagonal and iterates) in registers.  Iterates go through shared memory node by
+// node, cell contributions as four corner arrays.
+#include "smooth.cuh"
+
+#include "cheb.cuh"
+#include "pdl.cuh"
+#include "q1_pair.cuh"
+
+namespace pff {
+
+namespace {
+
+constexpr int TN = kSmoothTile;
+constexpr int TPB = 256;
+constexpr int NB = 30;   // node slots per brick side
+
+using P = float2;
+
+// components of a block's node value: UU two (u_x, u_y), PP one
+template <int OP> struct Comp;
+template <> struct Comp<OP_UU> { static constexpr int NC = 2; using V = float2; };
+template <> struct Comp<OP_PP> { static constexpr int NC = 1; using V = float; };
+
+__device__ __forceinline__ float& comp(float2& v, int c) { return c ? v.y : v.x; }
+__device__ __forceinline__ float comp(const float2& v, int c) { return c ? v.y : v.x; }
+__device__ __forceinline__ float& comp(float& v, int) { return v; }
+__device__ __forceinline__ float comp(const float& v, int) { return v; }
+
+// component c of window nodes a, b as a pair
+template <typename V>
+__device__ __forceinline__ P two(const V* s, int a, int b, int c) {
+  return make_float2(comp(s[a], c), comp(s[b], c));
+}
+
+// The x-independent Gauss-point factors of a cell pair: UU g(phi~), PP the mass coefficient.
+// sv: window node values, UU phi~ in .x; PP (u_x, u_y).
+template <int OP, int NW, typename V>
+__device__ __forceinline__ void cell_coef(const V* sv, int a, int b, const MatConst<float>& m,
+                                          const LevGeom<float>& g, P ec, P q[2][2]) {
+  const P omk = pbc(m.omk);
+  auto init = [&](PField<P>& f, int c, P& b0) {
+    b0 = two(sv, a, b, c);
+    const P t0 = two(sv, a + NW, b + NW, c);
+    f.init(b0, psub(two(sv, a + 1, b + 1, c), b0), t0, psub(two(sv, a + NW + 1, b + NW + 1, c), t0));
+  };
+  if constexpr (OP == OP_UU) {
+    PField<P> f;
+    P b0, v[2][2];
+    init(f, 0, b0);
+    f.values(b0, v);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) q[i][j] = pfma(omk, pmul(v[i][j], v[i][j]), pbc(m.kap));
+  } else {
+    const P ihx = pbc(g.ihx), ihy = pbc(g.ihy), pp = pbc(m.p);
+    const P oc2ml = pmul(omk, pmul(pbc(m.c2ml), ec)), ocl = pmul(omk, pmul(pbc(m.cl), ec)),
+            ocm = pmul(omk, pmul(pbc(m.cm), ec));
+    PField<P> fx, fy;
+    P b0, e11[2], e22[2], uyx[2], uxy[2];
+    init(fx, 0, b0);
+    init(fy, 1, b0);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      e11[i] = pmul(fx.dxi[i], ihx);
+      uyx[i] = pmul(fy.dxi[i], ihx);
+      e22[i] = pmul(fy.deta[i], ihy);
+      uxy[i] = pmul(fx.deta[i], ihy);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const P ge12 = padd(uxy[i], uyx[j]);
+        const P q11 = pfma(oc2ml, e11[j], pfma(ocl, e22[i], pp));
+        const P q22 = pfma(ocl, e11[j], pfma(oc2ml, e22[i], pp));
+        const P q12 = pmul(ocm, ge12);
+        q[i][j] = pfma(q11, e11[j],
+                       pfma(q22, e22[i], pfma(q12, ge12, pfma(pp, padd(e11[j], e22[i]), pbc(m.gcl)))));
+      }
+  }
+}
+
+// Cell contributions r[component][corner] of a cell pair (corners 0 (0,0), 1 (1,0), 2 (0,1), 3 (1,1)).
+template <int OP, int NW, typename V>
+__device__ __forceinline__ void cell_apply(const V* xs, int a, int b, const MatConst<float>& m,
+                                           const LevGeom<float>& g, P ec, const P q[2][2],
+                                           P r[Comp<OP>::NC][4]) {
+  const P zero = pbc(0.f);
+#pragma unroll
+  for (int c = 0; c < Comp<OP>::NC; ++c)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r[c][k] = zero;
+  auto init = [&](PField<P>& f, int c, P& b0) {
+    b0 = two(xs, a, b, c);
+    const P t0 = two(xs, a + NW, b + NW, c);
+    f.init(b0, psub(two(xs, a + 1, b + 1, c), b0), t0, psub(two(xs, a + NW + 1, b + NW + 1, c), t0));
+  };
+  if constexpr (OP == OP_UU) {
+    const P ihx = pbc(g.ihx), ihy = pbc(g.ihy);
+    const P c2ml = pmul(pbc(m.c2ml), ec), cl = pmul(pbc(m.cl), ec), cm = pmul(pbc(m.cm), ec);
+    PField<P> fx, fy;
+    P b0, ax[2], dy[2], bxy[2], cyx[2], S11[2][2], S12[2][2], S22[2][2];
+    init(fx, 0, b0);
+    init(fy, 1, b0);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      ax[i] = pmul(fx.dxi[i], ihx);
+      cyx[i] = pmul(fy.dxi[i], ihx);
+      dy[i] = pmul(fy.deta[i], ihy);
+      bxy[i] = pmul(fx.deta[i], ihy);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const P bc = padd(bxy[i], cyx[j]);
+        S11[i][j] = pmul(q[i][j], pfma(c2ml, ax[j], pmul(cl, dy[i])));
+        S22[i][j] = pmul(q[i][j], pfma(cl, ax[j], pmul(c2ml, dy[i])));
+        S12[i][j] = pmul(q[i][j], pmul(cm, bc));
+      }
+    const P wx = pbc(g.wx), wy = pbc(g.wy), nwx = pbc(-g.wx), nwy = pbc(-g.wy);
+    ptest_grad(padd(S11[0][0], S11[1][0]), padd(S11[0][1], S11[1][1]), padd(S12[0][0], S12[0][1]),
+               padd(S12[1][0], S12[1][1]), wx, wy, nwx, nwy, r[0]);
+    ptest_grad(padd(S12[0][0], S12[1][0]), padd(S12[0][1], S12[1][1]), padd(S22[0][0], S22[0][1]),
+               padd(S22[1][0], S22[1][1]), wx, wy, nwx, nwy, r[1]);
+  } else {
+    PField<P> f;
+    P b0, v[2][2], fv[2][2];
+    init(f, 0, b0);
+    f.values(b0, v);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) fv[i][j] = pmul(q[i][j], v[i][j]);
+    ptest_value(fv, pbc(g.jxw), r[0]);
+    ptest_grad(f.dxi[0], f.dxi[1], f.deta[0], f.deta[1], pbc(g.wpx), pbc(g.wpy), pbc(-g.wpx), pbc(-g.wpy), r[0]);
+  }
+}
+
+// HW: halo of the window (4 down, 3 up).  Window nodes and cells are numbered from
+// the window's corner; cell (i, j) has its lower-left node at node (i, j).
+template <int OP, bool DOWN>
+struct SmoothSmem {
+  static constexpr int HW = DOWN ? 4 : 3;
+  static constexpr int NW = TN + 2 * HW;   // window nodes per side
+  static constexpr int CW = NW - 1;        // window cells per side
+  static constexpr int NPT = (NW * NW + TPB - 1) / TPB;
+  static_assert(CW % 2 == 0 && CW * (CW / 2) <= TPB, "one cell pair per thread");
+  using V = typename Comp<OP>::V;
+  union {
+    struct {
+      float2 lin[NW * NW];   // UU phi~ in .x, PP u_x, u_y
+      float e[NW * NW];      // modulus of the cell whose lower-left node this is
+    };
+    V con[4][CW * CW];       // cell contributions by corner
+  };
+  V xs[NW * NW];
+  int32_t tile[20];
+  uint8_t cell[NW * NW];     // bit0 the node exists, bit5 the cell whose lower-left node this is exists
+};
+
+template <int OP, bool DOWN>
+__global__ void __launch_bounds__(TPB, 2) smooth_kernel(const __grid_constant__ SmoothArgs a) {
+  using S = SmoothSmem<OP, DOWN>;
+  using V = typename Comp<OP>::V;
+  constexpr int NC = Comp<OP>::NC, HW = S::HW, NW = S::NW, CW = S::CW, NPT = S::NPT, HC = CW / 2;
+  __shared__ S sm;
+  pdl_trigger();
+  const int tid = threadIdx.x;
+  if (tid < 20) sm.tile[tid] = __ldg(reinterpret_cast<const int32_t*>(a.tiles + blockIdx.x) + tid);
+  __syncthreads();
+  const int pos = sm.tile[18];
+  const int n0 = TN * (pos & 1) - HW, r0 = TN * ((pos >> 1) & 1) - HW;   // brick position of window node 0
+  constexpr int fix0 = OP == OP_UU ? 1 : 4;
+  // ---- tables and set-up data, which no kernel of the chain writes: window nodes,
+  // the cells' factors
+  int32_t slot[NPT];
+  uint32_t cm[NPT];
+  V di[NPT];
+#pragma unroll
+  for (int k = 0; k < NPT; ++k) {
+    const int w = tid + TPB * k;
+    slot[k] = -1;
+    cm[k] = 0;
+    di[k] = V();
+    if (w < NW * NW) {
+      const int n = n0 + w % NW, r = r0 + w / NW;
+      const int dx = n < 0 ? 0 : (n >= NB ? 2 : 1), dy = r < 0 ? 0 : (r >= NB ? 2 : 1);
+      const int32_t base = sm.tile[3 * dy + dx];
+      uint8_t f = 0;
+      if (base >= 0) {
+        const int32_t s = base + (n - NB * (dx - 1)) + NB * (r - NB * (dy - 1));
+        f = __ldg(a.flags + s);
+        if (f & 1) slot[k] = s;
+      }
+      float2 li = make_float2(0.f, 0.f);
+      float e = 1.f;
+      const int32_t s = slot[k];
+      if (s >= 0) {
+        cm[k] = __ldg(a.cmask + s);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) comp(di[k], c) = __ldg(a.dinv + c * int64_t(a.n) + s);
+        if constexpr (OP == OP_UU) {
+          li.x = __ldg(a.lin + 3 * int64_t(a.n) + s);
+        } else {
+          li.x = __ldg(a.lin + s);
+          li.y = __ldg(a.lin + int64_t(a.n) + s);
+        }
+        if (a.ecell != nullptr && (f & 32)) e = __ldg(a.ecell + s);
+      }
+      sm.lin[w] = li;
+      sm.e[w] = e;
+      sm.cell[w] = f & 33;
+    }
+  }
+  __syncthreads();
+  const int ci = tid % CW, cj = tid / CW;
+  const bool has = cj < HC;
+  const int nA = ci + NW * (has ? cj : 0), nB = nA + NW * HC;   // lower-left nodes of the pair
+  const bool actA = has && (sm.cell[nA] & 32), actB = has && (sm.cell[nB] & 32);
+  P q[2][2], ec = pbc(1.f);
+  if (actA || actB) {
+    if (a.ecell != nullptr) ec = make_float2(sm.e[nA], sm.e[nB]);
+    cell_coef<OP, NW>(sm.lin, nA, nB, a.m, a.g, ec, q);
+  }
+  // ---- from here on what the preceding kernel wrote
+  pdl_wait();
+  V dv[NPT], xv[NPT];   // defect (then residual), iterate
+#pragma unroll
+  for (int k = 0; k < NPT; ++k) {
+    const int w = tid + TPB * k;
+    dv[k] = V();
+    xv[k] = V();
+    const int32_t s = slot[k];
+    if (s >= 0) {
+#pragma unroll
+      for (int c = 0; c < NC; ++c) comp(dv[k], c) = a.d[c * int64_t(a.n) + s];
+      if constexpr (!DOWN) {
+        // x + P xc: coarse nodes in ascending (y, x), zero weights left out
+        const int n = n0 + w % NW, r = r0 + w / NW;
+        const int cx = (n >> 1) + TN * ((pos >> 2) & 1), cy = (r >> 1) + TN * ((pos >> 3) & 1);
+        const int nx = n & 1, ny = r & 1;
+        const float wt = (nx ? 0.5f : 1.f) * (ny ? 0.5f : 1.f);
+        V acc;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) comp(acc, c) = a.x[c * int64_t(a.n) + s];
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            if ((b && !ny) || (e && !nx)) continue;
+            const int gx = cx + e, gy = cy + b;
+            const int dx = gx < 0 ? 0 : (gx >= NB ? 2 : 1), dy = gy < 0 ? 0 : (gy >= NB ? 2 : 1);
+            const int32_t cs = sm.tile[9 + 3 * dy + dx] + (gx - NB * (dx - 1)) + NB * (gy - NB * (dy - 1));
+#pragma unroll
+            for (int c = 0; c < NC; ++c) comp(acc, c) += wt * a.xc[c * int64_t(a.nc) + cs];
+          }
+#pragma unroll
+        for (int c = 0; c < NC; ++c) comp(xv[k], c) = (cm[k] & (fix0 << c)) ? 0.f : comp(acc, c);
+      } else {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) comp(xv[k], c) = cheb_first_of(a.c0, comp(di[k], c), comp(dv[k], c));
+      }
+    }
+    if (w < NW * NW) sm.xs[w] = xv[k];
+  }
+  // Down: the restriction's row of this thread.  P^T of the residual goes onto the
+  // coarse nodes at the tile's even positions; thread t takes position (t % 8, t / 8).
+  // Rows are summed in ascending storage slot: bricks by (row, column), nodes by
+  // (row, column) in each; absent nodes add zero.
+  int32_t cs = -1, rw = 0;
+  uint32_t cmc = 0;
+  V dcv = V();
+  if constexpr (DOWN) {
+    constexpr int TC = (TN + 1) / 2;
+    const int wx = HW + 2 * (tid % TC) + (pos & 1), wy = HW + 2 * (tid / TC) + ((pos >> 1) & 1);   // even brick positions
+    if (tid < TC * TC && wx < HW + TN && wy < HW + TN && (sm.cell[wx + NW * wy] & 1)) {
+      rw = wx + NW * wy;
+      const int n = n0 + wx, r = r0 + wy;
+      cs = sm.tile[9 + 4] + (n >> 1) + TN * ((pos >> 2) & 1) + NB * ((r >> 1) + TN * ((pos >> 3) & 1));
+      cmc = __ldg(a.cmask_c + cs);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) comp(dcv, c) = a.dc[c * int64_t(a.nc) + cs];
+    }
+  }
+  __syncthreads();   // sm.lin and sm.e are no longer read: sm.con takes their place
+  V pv[NPT], xf[NPT];   // previous iterate; up: the prolonged x
+#pragma unroll
+  for (int k = 0; k < NPT; ++k) { pv[k] = V(); xf[k] = xv[k]; }
+#pragma unroll
+  for (int step = 0; step < 3; ++step) {
+    const int R = HW - 1 - step;   // nodes within R of the tile are updated from cells within R + 1
+    {
+      const int lo = HW - R - 1, hi = HW + TN + R - 1;   // window cells per direction
+      const bool cx = ci >= lo && ci <= hi;
+      const bool inA = has && cx && cj >= lo && cj <= hi, inB = has && cx && cj + HC >= lo && cj + HC <= hi;
+      if (inA || inB) {
+        P r[NC][4];
+        if ((inA && actA) || (inB && actB)) {
+          cell_apply<OP, NW>(sm.xs, nA, nB, a.m, a.g, ec, q, r);
+        } else {
+#pragma unroll
+          for (int c = 0; c < NC; ++c)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) r[c][e] = pbc(0.f);
+        }
+        const int iA = ci + CW * cj, iB = iA + CW * HC;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          V vA, vB;
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            comp(vA, c) = actA ? r[c][e].x : 0.f;
+            comp(vB, c) = actB ? r[c][e].y : 0.f;
+          }
+          sm.con[e][iA] = vA;
+          sm.con[e][iB] = vB;
+        }
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NPT; ++k) {
+      const int w = tid + TPB * k;
+      const int wx = w % NW, wy = w / NW;
+      if (w < NW * NW && wx >= HW - R && wx < HW + TN + R && wy >= HW - R && wy < HW + TN + R) {
+        const int i = wx + CW * wy;   // the cell above right of the node
+        const V c2 = sm.con[2][i - CW], c3 = sm.con[3][i - CW - 1], c1 = sm.con[1][i - 1], c0 = sm.con[0][i];
+        V out;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          const float y = ((comp(c2, c) + comp(c3, c)) + comp(c1, c)) + comp(c0, c);
+          const float ye = (slot[k] < 0 || (cm[k] & (fix0 << c))) ? 0.f : y;
+          const float dk = comp(dv[k], c), dik = comp(di[k], c), xk = comp(xv[k], c);
+          float o;
+          if (DOWN ? step == 2 : step == 0) {
+            const float rk = dk - ye;
+            if (DOWN) {
+              o = rk;   // the residual to restrict
+            } else {
+              comp(dv[k], c) = rk;
+              o = cheb_first_of(a.c0, dik, rk);
+              comp(pv[k], c) = 0.f;
+              comp(xv[k], c) = o;
+            }
+          } else {
+            const bool second = DOWN ? step == 1 : step == 2;
+            o = cheb_next(xk, comp(pv[k], c), dik, dk, ye, second ? a.a2 : a.a1, second ? a.b2 : a.b1);
+            comp(pv[k], c) = xk;
+            comp(xv[k], c) = o;
+          }
+          comp(out, c) = o;
+        }
+        if (DOWN || step < 2) sm.xs[w] = out;
+        if (step == (DOWN ? 1 : 2)) {
+          // the tile's own nodes
+          if (slot[k] >= 0 && wx >= HW && wx < HW + TN && wy >= HW && wy < HW + TN) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+              a.xout[c * int64_t(a.n) + slot[k]] = DOWN ? comp(out, c) : comp(xf[k], c) + comp(out, c);
+          }
+        }
+      }
+    }
+    if (DOWN || step < 2) __syncthreads();
+  }
+  if constexpr (DOWN) {
+    if (cs >= 0) {
+      const int w = rw;
+      const bool crossx = n0 + rw % NW == 0, crossy = r0 + rw / NW == 0;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        float v[3][3];
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+#pragma unroll
+          for (int e = 0; e < 3; ++e)
+            v[b][e] = ((b == 1 ? 1.f : 0.5f) * (e == 1 ? 1.f : 0.5f)) * comp(sm.xs[w + (e - 1) + NW * (b - 1)], c);
+        float acc = comp(dcv, c);
+        acc += v[0][0];
+        if (crossx && !crossy) {   // the left brick's column first
+          acc += v[1][0];
+          acc += v[2][0];
+          acc += v[0][1];
+          acc += v[0][2];
+        } else {
+          acc += v[0][1];
+          acc += v[0][2];
+          acc += v[1][0];
+          if (crossx) acc += v[2][0];
+        }
+        acc += v[1][1];
+        acc += v[1][2];
+        if (!crossx) acc += v[2][0];
+        acc += v[2][1];
+        acc += v[2][2];
+        a.dc[c * int64_t(a.nc) + cs] = (cmc & (fix0 << c)) ? 0.f : acc;
+      }
+    }
+  }
+}
+
+template <bool DOWN>
+cudaError_t launch_smooth(const SmoothArgs& a, int op, cudaStream_t s) {
+  if (a.ntiles <= 0) return cudaSuccess;
+  if (op == OP_UU) return launch_ex(true, &smooth_kernel<OP_UU, DOWN>, unsigned(a.ntiles), TPB, 0, s, a);
+  if (op == OP_PP) return launch_ex(true, &smooth_kernel<OP_PP, DOWN>, unsigned(a.ntiles), TPB, 0, s, a);
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+cudaError_t launch_smooth_down(const SmoothArgs& a, int op, cudaStream_t s) { return launch_smooth<true>(a, op, s); }
+cudaError_t launch_smooth_up(const SmoothArgs& a, int op, cudaStream_t s) { return launch_smooth<false>(a, op, s); }
+
+}  // namespace pff

@@ -1,0 +1,51 @@
+// Fused level smoothers of the FP32 Q1 V-cycle (smooth.cu).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "kernels.cuh"
+
+namespace pff {
+
+// A tile of kSmoothTile x kSmoothTile node positions of a level brick (four tiles
+// per brick; only tiles that hold a node are listed).  Node (n, r) of the window
+// around the tile lies in one of the brick's 3x3 neighbours; the coarser level's
+// nodes under the window lie in the 3x3 neighbours of the parent brick.
+constexpr int kSmoothTile = 15;
+struct SmoothTile {
+  int32_t fb[9];   // storage bases of the brick's 3x3 neighbours on this level (-1 absent)
+  int32_t cb[9];   // the same of the parent brick (bx / 2, by / 2) on the next coarser level
+  int32_t pos;     // tile column | tile row << 1 | (bx & 1) << 2 | (by & 1) << 3
+  int32_t pad;
+};
+
+// One level and block of the V-cycle.  Vectors: ncomp blocks of n (coarse: nc) floats.
+struct SmoothArgs {
+  const SmoothTile* tiles;
+  int32_t ntiles;
+  int32_t n, nc;           // slots of this level, of the next coarser one
+  const uint8_t* flags;    // level slot flags: bit0 node, bit5 the cell whose lower-left node this is exists
+  const uint8_t* cmask;
+  const uint8_t* cmask_c;
+  const float* lin;        // 4 blocks of n
+  const float* ecell;      // per-cell modulus at cell slots, or nullptr
+  const float* dinv;
+  const float* d;          // level defect
+  float* dc;               // down: coarse defect, the restricted residual is added
+  const float* x;          // up: the pre-smoothed iterate
+  const float* xc;         // up: the coarse correction
+  float* xout;             // down: the pre-smoothed iterate; up: the level's result
+  MatConst<float> m;
+  LevGeom<float> g;
+  float c0, a1, b1, a2, b2;   // Chebyshev steps: c0 D^-1, then (a, b) of cheb_next twice; all 0: no smoothing
+};
+
+// Down: x = p(D^-1 A) D^-1 d (Chebyshev degree 3 from zero), then dc += P^T (d - A x).
+// Up: x += P xc, then x += p(D^-1 A) D^-1 (d - A x).
+// op: OP_UU or OP_PP.  Launched programmatically dependent on the preceding kernel.
+cudaError_t launch_smooth_down(const SmoothArgs& a, int op, cudaStream_t s);
+cudaError_t launch_smooth_up(const SmoothArgs& a, int op, cudaStream_t s);
+
+}  // namespace pff

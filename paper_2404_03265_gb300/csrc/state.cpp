@@ -2,6 +2,7 @@
 #include "state.h"
 
 #include <cstring>
+#include <unordered_map>
 
 namespace pff {
 
@@ -20,6 +21,38 @@ static DevLayout upload_layout(DevAllocs& mem, const Layout& L) {
   d.units = mem.upload(units);
   d.cellmask = mem.upload(L.cellmask);
   return d;
+}
+
+// Tiles of the fused smoothers: every quarter of a brick of level mesh lm that holds
+// a node, with the storage bases around the brick and around its parent brick (bx / 2,
+// by / 2) of the next coarser level.
+static std::vector<SmoothTile> smooth_tiles(const LevelMesh& lm, const LevelMesh& coarse) {
+  const int NB = lm.lay.NB;
+  std::unordered_map<uint64_t, int32_t> parent;
+  for (size_t b = 0; b < coarse.lay.bricks.size(); ++b)
+    parent[cell_key(coarse.lay.bricks[b].bx, coarse.lay.bricks[b].by)] = int32_t(b);
+  std::vector<SmoothTile> out;
+  for (size_t b = 0; b < lm.lay.bricks.size(); ++b) {
+    const BrickDesc& d = lm.lay.bricks[b];
+    const auto it = parent.find(cell_key(d.bx >> 1, d.by >> 1));
+    for (int q = 0; q < 4; ++q) {
+      const int x0 = kSmoothTile * (q & 1), y0 = kSmoothTile * (q >> 1);
+      bool any = false;
+      for (int j = y0; j < y0 + kSmoothTile && !any; ++j)
+        for (int i = x0; i < x0 + kSmoothTile && !any; ++i)
+          any = lm.slot_X[b * size_t(NB) * NB + i + size_t(NB) * j] >= 0;
+      if (!any) continue;
+      SmoothTile t;
+      for (int e = 0; e < 9; ++e) {
+        t.fb[e] = d.nbr_base[e];
+        t.cb[e] = it == parent.end() ? -1 : coarse.lay.bricks[it->second].nbr_base[e];
+      }
+      t.pos = q | (d.bx & 1) << 2 | (d.by & 1) << 3;
+      t.pad = 0;
+      out.push_back(t);
+    }
+  }
+  return out;
 }
 
 std::string upload_mesh(pff_mesh& pm) {
@@ -60,6 +93,11 @@ std::string upload_mesh(pff_mesh& pm) {
     L.lv.n_slots = int32_t(lm.lay.n_slots);
     L.lv.off = off;
     off += lm.lay.n_slots;
+    if (M.k == 1 && l > 0) {
+      const std::vector<SmoothTile> tiles = smooth_tiles(lm, M.levels[l - 1]);
+      L.lv.tiles = D.mem.upload(tiles);
+      L.lv.ntiles = int32_t(tiles.size());
+    }
     L.lv.flags = D.mem.upload(lm.slot_flags);
     L.lv.slot_leaf = D.mem.upload(lm.slot_leaf);
     std::vector<float> pv(lm.P_val.begin(), lm.P_val.end()), rv(lm.R_val.begin(), lm.R_val.end());
@@ -84,6 +122,20 @@ std::string upload_mesh(pff_mesh& pm) {
     L.cell_child = D.mem.upload(lm.cell_child);
   }
   D.lev_total = off;
+  if (M.k == 1) {
+    std::vector<LevBrick> lb;
+    std::vector<int32_t> home(size_t(off), -1);
+    for (size_t l = 0; l < M.levels.size(); ++l) {
+      const LevelMesh& lm = M.levels[l];
+      const DevLevel& lv = D.levels[l].lv;
+      for (size_t b = 0; b < lm.lay.bricks.size(); ++b)
+        lb.push_back({int32_t(lv.off), lv.n_slots, int32_t(b) * lm.lay.NB * lm.lay.NB});
+      for (size_t i = 0; i < lm.copy_leaf.size(); ++i) home[size_t(lv.off) + lm.copy_level[i]] = lm.copy_leaf[i];
+    }
+    D.lev_bricks = D.mem.upload(lb);
+    D.n_lev_bricks = int32_t(lb.size());
+    D.home_leaf = D.mem.upload(home);
+  }
   {
     // each free leaf node is on the copy list of exactly one level (its home)
     std::vector<int32_t> hoff(size_t(M.lay.n_slots), 0), hslot(size_t(M.lay.n_slots), -1),

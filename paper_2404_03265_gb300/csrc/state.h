@@ -72,6 +72,11 @@ struct DevMesh {
   };
   std::vector<Level> levels;
   int64_t lev_total = 0;     // sum of level slot counts
+  // Q1: the bricks of all levels in storage order, and per level slot its leaf slot
+  // when this is the node's home level (else -1)
+  LevBrick* lev_bricks = nullptr;
+  int32_t n_lev_bricks = 0;
+  int32_t* home_leaf = nullptr;
   DevHome home;              // per leaf slot: its home level (copy in and out of the V-cycle)
   void release() {
     mem.release();
