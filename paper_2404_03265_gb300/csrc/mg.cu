@@ -143,21 +143,40 @@ __global__ void k_copy_in(int64_t nsl, int ncomp, DevHome home, const double* __
 }
 
 // One block per level brick: every level slot is written, so the level defects
-// need no separate clearing.
+// need no separate clearing.  The loads of a thread's slots are issued together.
+constexpr int LD_SLOTS = 900;                            // slots per brick
+constexpr int LD_N = (LD_SLOTS + TPB - 1) / TPB;
 template <typename T>
-__global__ void k_level_defects(const LevBrick* __restrict__ bricks, const int32_t* __restrict__ home_leaf, int ncomp,
-                                int64_t nsl, const double* __restrict__ r, T* d, T* x0,
-                                const uint8_t* __restrict__ lcm, int fixbits) {
+__global__ void __launch_bounds__(TPB) k_level_defects(const LevBrick* __restrict__ bricks,
+                                                       const int32_t* __restrict__ home_leaf, int ncomp, int64_t nsl,
+                                                       const double* __restrict__ r, T* d, T* x0,
+                                                       const uint8_t* __restrict__ lcm, int fixbits) {
   pdl_trigger();
   const LevBrick b = bricks[blockIdx.x];
-  for (int i = threadIdx.x; i < 900; i += blockDim.x) {
-    const int32_t s = b.base + i;
-    const int32_t leaf = home_leaf[b.off + s];
-    const uint8_t cm = leaf >= 0 ? lcm[leaf] : uint8_t(0);
-    for (int c = 0; c < ncomp; ++c) {
+  int32_t leaf[LD_N];
+#pragma unroll
+  for (int k = 0; k < LD_N; ++k) {
+    const int i = threadIdx.x + TPB * k;
+    leaf[k] = i < LD_SLOTS ? home_leaf[b.off + b.base + i] : -1;
+  }
+  double v[LD_N][2];
+  uint8_t cm[LD_N];
+#pragma unroll
+  for (int k = 0; k < LD_N; ++k) {
+    cm[k] = leaf[k] >= 0 ? lcm[leaf[k]] : uint8_t(0);
+    v[k][0] = leaf[k] >= 0 ? r[leaf[k]] : 0.0;
+    v[k][1] = leaf[k] >= 0 && ncomp > 1 ? r[nsl + leaf[k]] : 0.0;
+  }
+#pragma unroll
+  for (int k = 0; k < LD_N; ++k) {
+    const int i = threadIdx.x + TPB * k;
+    if (i >= LD_SLOTS) break;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      if (c >= ncomp) break;
       const int bit = (fixbits == 4) ? 4 : (1 << c);
-      const int64_t o = int64_t(ncomp) * b.off + c * int64_t(b.n) + s;
-      d[o] = (leaf >= 0 && !(cm & bit)) ? T(r[c * nsl + leaf]) : T(0);
+      const int64_t o = int64_t(ncomp) * b.off + c * int64_t(b.n) + b.base + i;
+      d[o] = (cm[k] & bit) ? T(0) : T(v[k][c]);
       if (b.off == 0) x0[o] = T(0);
     }
   }
@@ -168,12 +187,14 @@ __global__ void k_copy_out(int64_t nsl, int ncomp, DevHome home, const T* __rest
                            const double* __restrict__ r, double* z, const uint8_t* __restrict__ lcm,
                            const uint8_t* __restrict__ lflags, int fixbits) {
   pdl_trigger();
-  pdl_wait();
+  bool waited = false;   // the tables of the first slot are read before the wait
   GRID_STRIDE(s, nsl) {
-    const uint8_t cm = lcm[s];
-    const bool node = (lflags[s] & 1) && !(lflags[s] & 4);
+    const uint8_t cm = lcm[s], lf = lflags[s];
     const int32_t b = home.slot[s];
-    const int64_t base = b >= 0 ? int64_t(ncomp) * home.off[s] + b : 0, nl = b >= 0 ? home.nsl[s] : 0;
+    const int64_t off = home.off[s], nl = home.nsl[s];
+    const bool node = (lf & 1) && !(lf & 4);
+    const int64_t base = b >= 0 ? int64_t(ncomp) * off + b : 0;
+    if (!waited) { pdl_wait(); waited = true; }
     for (int c = 0; c < ncomp; ++c) {
       const int bit = (fixbits == 4) ? 4 : (1 << c);
       double v = 0.0;
@@ -182,6 +203,7 @@ __global__ void k_copy_out(int64_t nsl, int ncomp, DevHome home, const T* __rest
       z[c * nsl + s] = v;
     }
   }
+  if (!waited) pdl_wait();
 }
 
 template <typename T>
@@ -211,14 +233,6 @@ __global__ void k_cheb_step_add(int64_t n, T* xadd, const T* __restrict__ x, con
   GRID_STRIDE(i, n) {
     xadd[i] += cheb_next(x[i], xprev[i], dinv[i], d[i], ax[i], a, b);
   }
-}
-
-// Dense FP64 coarse solve: tmp = d[idx] (to FP64), x[idx] = Ainv tmp; one block per row group.
-template <typename T>
-__global__ void k_coarse_gather(int32_t n, const int32_t* idx, const T* d, double* tmp) {
-  pdl_trigger();
-  pdl_wait();
-  GRID_STRIDE(i, n) tmp[i] = double(d[idx[i]]);
 }
 
 // Blocked Gauss-Jordan inversion in place, panels of GJB pivots.  With P the
@@ -371,18 +385,37 @@ __global__ void __launch_bounds__(TPB) k_gj_update(int32_t n, int32_t k0, int32_
   }
 }
 
+// Dense FP64 coarse solve x[idx] = Ainv d[idx], d taken to FP64: one warp per row,
+// lanes stride the columns, fixed-order warp reduction.  The first CP columns of a
+// lane (all of them on a 16 x 16 coarse mesh) and their indices are read before the wait.
 template <typename T>
-__global__ void k_coarse_matvec(int32_t n, const int32_t* idx, const double* __restrict__ A,
-                                const double* __restrict__ tmp, T* x) {
-  pdl_trigger();
-  pdl_wait();
-  // one warp per row, lanes stride the columns, fixed-order warp reduction
+__global__ void k_coarse_matvec(int32_t n, const int32_t* __restrict__ idx, const double* __restrict__ A, const T* d,
+                                T* x) {
+  constexpr int CP = 16;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  const int row = warp < n ? warp : n - 1;
+  double a[CP];
+  int32_t ix[CP];
+#pragma unroll
+  for (int q = 0; q < CP; ++q) {
+    const int j = lane + 32 * q;
+    a[q] = j < n ? A[int64_t(row) * n + j] : 0.0;
+    ix[q] = j < n ? idx[j] : 0;
+  }
+  const int32_t out = idx[row];
+  pdl_wait();
+  pdl_trigger();
   if (warp >= n) return;
+  T t[CP];
+#pragma unroll
+  for (int q = 0; q < CP; ++q) t[q] = d[ix[q]];
   double acc = 0.0;
-  for (int j = lane; j < n; j += 32) acc += A[int64_t(warp) * n + j] * tmp[j];
+#pragma unroll
+  for (int q = 0; q < CP; ++q)
+    if (lane + 32 * q < n) acc += a[q] * double(t[q]);
+  for (int j = lane + 32 * CP; j < n; j += 32) acc += A[int64_t(row) * n + j] * double(d[idx[j]]);
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if (lane == 0) x[idx[warp]] = T(acc);
+  if (lane == 0) x[out] = T(acc);
 }
 
 __global__ void k_inject_lin(int32_t nsl, const int32_t* __restrict__ sl, const double* __restrict__ lin,
@@ -639,14 +672,11 @@ cudaError_t mg_spd_invert(int32_t n, double* A, double* scr, int32_t* bad, cudaS
 }
 
 template <typename T>
-cudaError_t mg_coarse(int32_t n, const int32_t* idx, const double* Ainv, const T* d, T* x, double* tmp,
-                      cudaStream_t s, bool pdl) {
+cudaError_t mg_coarse(int32_t n, const int32_t* idx, const double* Ainv, const T* d, T* x, cudaStream_t s, bool pdl) {
   if (n <= 0) return cudaSuccess;
-  cudaError_t e = launch_ex(pdl, &k_coarse_gather<T>, blocks_for(n), TPB, 0, s, n, idx, d, tmp);
-  if (e != cudaSuccess) return e;
   const int warps_per_block = TPB / 32;
   return launch_ex(pdl, &k_coarse_matvec<T>, unsigned((n + warps_per_block - 1) / warps_per_block), TPB, 0, s, n, idx,
-                   Ainv, static_cast<const double*>(tmp), x);
+                   Ainv, d, x);
 }
 
 cudaError_t mg_inject_lin(int32_t ns_l, const int32_t* slot_leaf, const double* lin64, int64_t ns_leaf,
@@ -726,7 +756,7 @@ cudaError_t copy64(int64_t n, double* dst, const double* src, cudaStream_t s) {
                                                  cudaStream_t, bool);                                              \
   template cudaError_t mg_chebyshev_step_add<T>(int64_t, T*, const T*, const T*, const T*, const T*, const T*, T, \
                                                 T, cudaStream_t, bool);                                            \
-  template cudaError_t mg_coarse<T>(int32_t, const int32_t*, const double*, const T*, T*, double*, cudaStream_t, bool);
+  template cudaError_t mg_coarse<T>(int32_t, const int32_t*, const double*, const T*, T*, cudaStream_t, bool);
 INST(float)
 INST(double)
 #undef INST

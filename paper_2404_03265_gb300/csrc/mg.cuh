@@ -23,7 +23,7 @@ struct DevLevel {
   const int32_t* R_col = nullptr;
   const float* R_val = nullptr;
   const SmoothTile* tiles = nullptr;  // Q1, level >= 1: tiles of the fused smoothers (smooth.cuh)
-  int32_t ntiles = 0;
+  int32_t ntiles = 0, tile = 0;       // their number and nodes per side
 };
 
 // A brick of the concatenated level storage (900 slots): its level's slot offset
@@ -102,8 +102,8 @@ cudaError_t mg_spd_invert(int32_t n, double* A, double* scr, int32_t* bad, cudaS
 
 // coarse solve x[idx] = Ainv (d[idx]) (dense FP64 inverse over the interior entries)
 template <typename T>
-cudaError_t mg_coarse(int32_t n, const int32_t* idx, const double* Ainv, const T* d, T* x, double* tmp,
-                      cudaStream_t s, bool pdl = false);
+cudaError_t mg_coarse(int32_t n, const int32_t* idx, const double* Ainv, const T* d, T* x, cudaStream_t s,
+                      bool pdl = false);
 
 // ---- set-up kernels
 // level lin (4 blocks of ns_l, double and float) from leaf lin64 (4 blocks of ns_leaf)

@@ -171,9 +171,10 @@ std::string mg_alloc(pff_mg& mg) {
 // Per Newton step: level linearisation, level constraint masks, inverse
 // diagonals, eigenvalue estimates and the coarse inverse of both blocks.
 void mg_release_graphs(pff_mg& mg) {
-  for (auto& g : mg.vc_exec)
-    if (g) { cudaGraphExecDestroy(g); g = nullptr; }
-  if (mg.vc_both) { cudaGraphExecDestroy(mg.vc_both); mg.vc_both = nullptr; }
+  for (int g = 0; g < 3; ++g) {
+    if (mg.vc_exec[g]) { cudaGraphExecDestroy(mg.vc_exec[g]); mg.vc_exec[g] = nullptr; }
+    if (mg.vc_graph[g]) { cudaGraphDestroy(mg.vc_graph[g]); mg.vc_graph[g] = nullptr; }
+  }
 }
 
 void mg_release_setup_graph(pff_mg& mg) {
@@ -478,7 +479,6 @@ std::string mg_setup(pff_mg& mg, cudaStream_t s) {
         const int32_t cap = std::max(nI, 1);
         B.coarse_idx = mg.mem.alloc<int32_t>(cap);
         B.coarse_inv = mg.mem.alloc<double>(int64_t(cap) * cap);
-        B.coarse_tmp = mg.mem.alloc<double>(cap);
         B.coarse_rc = mg.mem.alloc<double>(mg_spd_scratch(cap));
         if (!mg.mem.err.empty()) return mg.mem.err;
         B.coarse_cap = cap;
@@ -524,6 +524,24 @@ std::string mg_setup(pff_mg& mg, cudaStream_t s) {
 
 namespace {
 
+// While a V-cycle graph is captured: the node of the kernel just launched on s, which
+// takes nargs arguments, r at position r_arg and z at z_arg (-1: not)
+cudaError_t note_node(pff_mg& mg, int b, int which, int nargs, int r_arg, int z_arg, cudaStream_t s) {
+  if (!mg.vc_note[b]) return cudaSuccess;
+  cudaStreamCaptureStatus st;
+  const cudaGraphNode_t* dep = nullptr;
+  size_t n = 0;
+  const cudaError_t e = cudaStreamGetCaptureInfo(s, &st, nullptr, nullptr, &dep, nullptr, &n);
+  if (e != cudaSuccess) return e;
+  if (st != cudaStreamCaptureStatusActive || n != 1) return cudaErrorUnknown;
+  pff_mg::VcIo& io = *mg.vc_note[b];
+  io.node[which] = dep[0];
+  io.arg[which].resize(size_t(nargs));
+  io.r_arg[which] = r_arg;
+  if (which == 1) io.z_arg = z_arg;
+  return cudaSuccess;
+}
+
 template <typename T>
 cudaError_t vcycle_t(pff_mg& mg, int b, const double* r, double* z, cudaStream_t s) {
   pff_problem& pb = *mg.pb;
@@ -558,10 +576,12 @@ cudaError_t vcycle_t(pff_mg& mg, int b, const double* r, double* z, cudaStream_t
   const bool tiles = sizeof(T) == 4 && M.k == 1 && fuse && pb.sweep_sh == 0 && mg.degree == 3;
   if (tiles) {
     VC(mg_level_defects<T>(D.n_lev_bricks, D.lev_bricks, D.home_leaf, nc, nsleaf, r, d, rr, pb.cmask, B.fixbits, s));
+    VC(note_node(mg, b, 0, 9, 4, -1, s));
   } else {
     VC(cudaMemsetAsync(d, 0, nc * N * sizeof(T), s));
     VC(cudaMemsetAsync(x, 0, nc * N * sizeof(T), s));
     VC(mg_copy_in<T>(nsleaf, nc, D.home, r, d, pb.cmask, B.fixbits, s));
+    VC(note_node(mg, b, 0, 7, 3, -1, s));
   }
   // Chebyshev on level l over [a, bb], `degree` applications of D^-1: solve A v = rhs
   // from v = 0 into out (buffers yp, y, t).  The three iterates (current,
@@ -623,7 +643,7 @@ cudaError_t vcycle_t(pff_mg& mg, int b, const double* r, double* z, cudaStream_t
         fill_cell_constants(k, M.Lf + 1);
         SmoothArgs a;
         std::memset(&a, 0, sizeof(a));
-        a.tiles = lv.tiles; a.ntiles = lv.ntiles;
+        a.tiles = lv.tiles; a.ntiles = lv.ntiles; a.tile = lv.tile;
         a.n = lv.n_slots; a.nc = lc.n_slots;
         a.flags = lv.flags; a.cmask = mg.cmask + lv.off; a.cmask_c = mg.cmask + lc.off;
         a.lin = mg.lin32 + 4 * lv.off;
@@ -647,15 +667,19 @@ cudaError_t vcycle_t(pff_mg& mg, int b, const double* r, double* z, cudaStream_t
         VC(launch_smooth_down(a, block_op(b), s));
       }
       if (mg.coarse_mode == 1) VC(cheb_ab(0, d, rr, B.c0_a, B.c0_b, B.c0_deg, false));
-      else VC(mg_coarse<T>(B.n_coarse, B.coarse_idx, B.coarse_inv, d, rr, B.coarse_tmp, s, true));
+      else VC(mg_coarse<T>(B.n_coarse, B.coarse_idx, B.coarse_inv, d, rr, s, true));
       for (int l = 1; l < nl; ++l) {
         SmoothArgs a = args(l);
         a.x = x + nc * D.levels[l].lv.off;
         a.xc = rr + nc * D.levels[l - 1].lv.off;
         a.xout = rr + nc * D.levels[l].lv.off;
-        VC(launch_smooth_up(a, block_op(b), s));
+        // the first one is dependent in this way only behind k_coarse_matvec: without a
+        // coarse launch down(1) itself precedes it, and the Chebyshev coarse solver's
+        // kernels let it start before they wait
+        VC(launch_smooth_up(a, block_op(b), s, l > 1 || (mg.coarse_mode == 0 && B.n_coarse > 0)));
       }
-      return mg_copy_out<T>(nsleaf, nc, D.home, rr, r, z, pb.cmask, pb.mesh->dev.slot_flags, B.fixbits, s, true);
+      VC(mg_copy_out<T>(nsleaf, nc, D.home, rr, r, z, pb.cmask, pb.mesh->dev.slot_flags, B.fixbits, s, true));
+      return note_node(mg, b, 1, 9, 4, 5, s);
     }
   }
   // smoothing on level l >= 1: degree mg.degree on [lo, hi] * lambda_max
@@ -687,7 +711,7 @@ cudaError_t vcycle_t(pff_mg& mg, int b, const double* r, double* z, cudaStream_t
   }
   // coarse
   if (mg.coarse_mode == 1) VC(cheb_ab(0, d, x, B.c0_a, B.c0_b, B.c0_deg, false));
-  else VC(mg_coarse<T>(B.n_coarse, B.coarse_idx, B.coarse_inv, d, x, B.coarse_tmp, s, true));
+  else VC(mg_coarse<T>(B.n_coarse, B.coarse_idx, B.coarse_inv, d, x, s, true));
   // Post-smoothing on level l of the defect d - A x, from zero, added to x: the
   // first step applies A to x and forms the defect, the last adds instead of
   // storing.  The level defect d is free once the first step has read it.
@@ -757,6 +781,7 @@ cudaError_t vcycle_t(pff_mg& mg, int b, const double* r, double* z, cudaStream_t
     VC(cheb_post(l));
   }
   VC(mg_copy_out<T>(nsleaf, nc, D.home, x, r, z, pb.cmask, pb.mesh->dev.slot_flags, B.fixbits, s, true));
+  VC(note_node(mg, b, 1, 9, 4, 5, s));
 #undef VC
   return cudaSuccess;
 }
@@ -768,82 +793,106 @@ static cudaError_t vcycle_direct(pff_mg& mg, int block, const double* r, double*
   return vcycle_t<float>(mg, block, r, z, s);
 }
 
-// Capture the V-cycle of one block, reading vc_in and writing vc_out at the
-// block's offset; false if the graph could not be made (the direct path is used).
-static bool vcycle_capture(pff_mg& mg, int block) {
-  const int64_t n = mg.pb->mesh->m.lay.n_slots;
-  const int64_t off = block == 0 ? 0 : 2 * n;
-  if (!mg.cap_stream && cudaStreamCreateWithFlags(&mg.cap_stream, cudaStreamNonBlocking) != cudaSuccess) return false;
-  if (cudaStreamBeginCapture(mg.cap_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return false;
-  const cudaError_t e = vcycle_direct(mg, block, mg.vc_in + off, mg.vc_out + off, mg.cap_stream);
-  cudaGraph_t g = nullptr;
-  const cudaError_t e2 = cudaStreamEndCapture(mg.cap_stream, &g);
-  bool ok = e == cudaSuccess && e2 == cudaSuccess && g != nullptr;
-  if (ok) ok = cudaGraphInstantiate(&mg.vc_exec[block], g, 0) == cudaSuccess;
-  if (g) cudaGraphDestroy(g);
-  if (!ok) {
-    mg.vc_exec[block] = nullptr;
-    cudaGetLastError();   // clear a capture error; the direct path follows
-  }
-  return ok;
-}
-
-cudaError_t mg_vcycle(pff_mg& mg, int block, const double* r, double* z, cudaStream_t s) {
-  if (mg.graphs_ok && mg.vc_in && mg.vc_out) {
-    if (!mg.vc_exec[block] && !vcycle_capture(mg, block)) mg.graphs_ok = false;
-    if (mg.vc_exec[block]) {
-      const int64_t n = mg.pb->mesh->m.lay.n_slots;
-      const int64_t off = block == 0 ? 0 : 2 * n;
-      const size_t bytes = size_t(block == 0 ? 2 * n : n) * sizeof(double);
-      cudaError_t e = cudaMemcpyAsync(mg.vc_in + off, r, bytes, cudaMemcpyDeviceToDevice, s);
-      if (e == cudaSuccess) e = cudaGraphLaunch(mg.vc_exec[block], s);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(z, mg.vc_out + off, bytes, cudaMemcpyDeviceToDevice, s);
-      return e;
-    }
-  }
-  return vcycle_direct(mg, block, r, z, s);
-}
-
-// Capture both blocks' V-cycles as one graph.  They share no buffer (each block
-// has its own level vectors, inverse diagonals and coarse data; the staging
-// vectors are split at 2 n_slots), so the phi block runs on a second branch
-// forked from and joined back into the capture stream.
-static bool precond_capture(pff_mg& mg) {
+// Capture graph g: block g, or both for g = 2.  The blocks share no buffer (each has
+// its own level vectors, inverse diagonals and coarse data; the staging vectors are
+// split at 2 n_slots), so the phi block runs on a second branch forked from and joined
+// back into the capture stream.  False if the graph could not be made (the direct path
+// is used).
+static bool vcycle_capture(pff_mg& mg, int g) {
   const int64_t n = mg.pb->mesh->m.lay.n_slots;
   if (!mg.cap_stream && cudaStreamCreateWithFlags(&mg.cap_stream, cudaStreamNonBlocking) != cudaSuccess) return false;
   if (!mg.cap_stream2 && cudaStreamCreateWithFlags(&mg.cap_stream2, cudaStreamNonBlocking) != cudaSuccess) return false;
   if (!mg.ev_fork && cudaEventCreateWithFlags(&mg.ev_fork, cudaEventDisableTiming) != cudaSuccess) return false;
   if (!mg.ev_join && cudaEventCreateWithFlags(&mg.ev_join, cudaEventDisableTiming) != cudaSuccess) return false;
   if (cudaStreamBeginCapture(mg.cap_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return false;
-  cudaError_t e = cudaEventRecord(mg.ev_fork, mg.cap_stream);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(mg.cap_stream2, mg.ev_fork, 0);
-  if (e == cudaSuccess) e = vcycle_direct(mg, 1, mg.vc_in + 2 * n, mg.vc_out + 2 * n, mg.cap_stream2);
-  if (e == cudaSuccess) e = vcycle_direct(mg, 0, mg.vc_in, mg.vc_out, mg.cap_stream);
-  if (e == cudaSuccess) e = cudaEventRecord(mg.ev_join, mg.cap_stream2);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(mg.cap_stream, mg.ev_join, 0);
-  cudaGraph_t g = nullptr;
-  const cudaError_t e2 = cudaStreamEndCapture(mg.cap_stream, &g);
-  bool ok = e == cudaSuccess && e2 == cudaSuccess && g != nullptr;
-  if (ok) ok = cudaGraphInstantiate(&mg.vc_both, g, 0) == cudaSuccess;
-  if (g) cudaGraphDestroy(g);
-  if (!ok) {
-    mg.vc_both = nullptr;
-    cudaGetLastError();
+  for (int b = 0; b < 2; ++b) {
+    mg.vc_io[g][b] = pff_mg::VcIo();
+    mg.vc_note[b] = &mg.vc_io[g][b];
   }
-  return ok;
+  cudaError_t e = cudaSuccess;
+  if (g < 2) {
+    const int64_t off = g == 0 ? 0 : 2 * n;
+    e = vcycle_direct(mg, g, mg.vc_in + off, mg.vc_out + off, mg.cap_stream);
+  } else {
+    e = cudaEventRecord(mg.ev_fork, mg.cap_stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(mg.cap_stream2, mg.ev_fork, 0);
+    if (e == cudaSuccess) e = vcycle_direct(mg, 1, mg.vc_in + 2 * n, mg.vc_out + 2 * n, mg.cap_stream2);
+    if (e == cudaSuccess) e = vcycle_direct(mg, 0, mg.vc_in, mg.vc_out, mg.cap_stream);
+    if (e == cudaSuccess) e = cudaEventRecord(mg.ev_join, mg.cap_stream2);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(mg.cap_stream, mg.ev_join, 0);
+  }
+  mg.vc_note[0] = mg.vc_note[1] = nullptr;
+  cudaGraph_t gr = nullptr;
+  const cudaError_t e2 = cudaStreamEndCapture(mg.cap_stream, &gr);
+  bool ok = e == cudaSuccess && e2 == cudaSuccess && gr != nullptr;
+  for (int b = 0; b < 2 && ok; ++b) {
+    if (g < 2 && b != g) continue;
+    pff_mg::VcIo& io = mg.vc_io[g][b];
+    for (int w = 0; w < 2 && ok; ++w) {
+      ok = io.node[w] && cudaGraphKernelNodeGetParams(io.node[w], &io.prm[w]) == cudaSuccess;
+      if (ok) std::copy_n(io.prm[w].kernelParams, io.arg[w].size(), io.arg[w].begin());
+    }
+  }
+  if (ok) ok = cudaGraphInstantiate(&mg.vc_exec[g], gr, 0) == cudaSuccess;
+  if (!ok) {
+    if (gr) cudaGraphDestroy(gr);
+    mg.vc_exec[g] = nullptr;
+    cudaGetLastError();   // clear a capture error; the direct path follows
+    return false;
+  }
+  mg.vc_graph[g] = gr;
+  return true;
+}
+
+// r and z of block b in graph g's next launch
+static cudaError_t vcycle_bind(pff_mg& mg, int g, int b, const double* r, double* z) {
+  pff_mg::VcIo& io = mg.vc_io[g][b];
+  for (int w = 0; w < 2; ++w) {
+    io.arg[w][io.r_arg[w]] = &r;
+    if (w == 1) io.arg[w][io.z_arg] = &z;
+    io.prm[w].kernelParams = io.arg[w].data();
+    const cudaError_t e = cudaGraphExecKernelNodeSetParams(mg.vc_exec[g], io.node[w], &io.prm[w]);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// One replay of graph g; blocks of the call: b0 .. b1
+static cudaError_t vcycle_replay(pff_mg& mg, int g, const double* r, double* z, cudaStream_t s) {
+  const int64_t n = mg.pb->mesh->m.lay.n_slots;
+  const int b0 = g == 2 ? 0 : g, b1 = g == 2 ? 1 : g;
+  const int64_t off = b0 == 0 ? 0 : 2 * n, len = (b0 == 0 ? 2 * n : 0) + (b1 == 1 ? n : 0);
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  const bool capturing = cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaSuccess;
+  if (capturing) {
+    cudaGetLastError();
+    const size_t bytes = size_t(len) * sizeof(double);
+    for (int b = b0; b <= b1 && e == cudaSuccess; ++b)
+      e = vcycle_bind(mg, g, b, mg.vc_in + (b == 0 ? 0 : 2 * n), mg.vc_out + (b == 0 ? 0 : 2 * n));
+    if (e == cudaSuccess) e = cudaMemcpyAsync(mg.vc_in + off, r, bytes, cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess) e = cudaGraphLaunch(mg.vc_exec[g], s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(z, mg.vc_out + off, bytes, cudaMemcpyDeviceToDevice, s);
+    return e;
+  }
+  for (int b = b0; b <= b1 && e == cudaSuccess; ++b)
+    e = vcycle_bind(mg, g, b, r + (b == b0 ? 0 : 2 * n), z + (b == b0 ? 0 : 2 * n));
+  return e == cudaSuccess ? cudaGraphLaunch(mg.vc_exec[g], s) : e;
+}
+
+cudaError_t mg_vcycle(pff_mg& mg, int block, const double* r, double* z, cudaStream_t s) {
+  if (mg.graphs_ok && mg.vc_in && mg.vc_out) {
+    if (!mg.vc_exec[block] && !vcycle_capture(mg, block)) mg.graphs_ok = false;
+    if (mg.vc_exec[block]) return vcycle_replay(mg, block, r, z, s);
+  }
+  return vcycle_direct(mg, block, r, z, s);
 }
 
 cudaError_t mg_precond(pff_mg& mg, const double* v, double* z, cudaStream_t s) {
   const int64_t n = mg.pb->mesh->m.lay.n_slots;
   if (mg.graphs_ok && mg.vc_in && mg.vc_out) {
-    if (!mg.vc_both && !precond_capture(mg)) mg.graphs_ok = false;
-    if (mg.vc_both) {
-      const size_t bytes = size_t(3 * n) * sizeof(double);
-      cudaError_t e = cudaMemcpyAsync(mg.vc_in, v, bytes, cudaMemcpyDeviceToDevice, s);
-      if (e == cudaSuccess) e = cudaGraphLaunch(mg.vc_both, s);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(z, mg.vc_out, bytes, cudaMemcpyDeviceToDevice, s);
-      return e;
-    }
+    if (!mg.vc_exec[2] && !vcycle_capture(mg, 2)) mg.graphs_ok = false;
+    if (mg.vc_exec[2]) return vcycle_replay(mg, 2, v, z, s);
   }
   cudaError_t e = vcycle_direct(mg, 0, v, z, s);
   if (e == cudaSuccess) e = vcycle_direct(mg, 1, v + 2 * n, z + 2 * n, s);

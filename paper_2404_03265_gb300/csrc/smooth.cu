@@ -34,8 +34,6 @@ namespace pff {
 
 namespace {
 
-constexpr int TN = kSmoothTile;
-constexpr int TPB = 256;
 constexpr int NB = 30;   // node slots per brick side
 
 using P = float2;
@@ -162,15 +160,19 @@ __device__ __forceinline__ void cell_apply(const V* xs, int a, int b, const MatC
   }
 }
 
-// HW: halo of the window (4 down, 3 up).  Window nodes and cells are numbered from
-// the window's corner; cell (i, j) has its lower-left node at node (i, j).
-template <int OP, bool DOWN>
+// TN: nodes per tile side; HW: halo of the window (4 down, 3 up).  Window nodes and
+// cells are numbered from the window's corner; cell (i, j) has its lower-left node at
+// node (i, j).
+template <int OP, bool DOWN, int TN>
 struct SmoothSmem {
   static constexpr int HW = DOWN ? 4 : 3;
-  static constexpr int NW = TN + 2 * HW;   // window nodes per side
-  static constexpr int CW = NW - 1;        // window cells per side
+  static constexpr int NW = TN + 2 * HW;     // window nodes per side
+  static constexpr int CW = NW - 1;          // window cells per side
+  static constexpr int HC = (CW + 1) / 2;    // cell rows of a pair's first member
+  static constexpr int CN = NW / 2 + 2;      // up: coarse nodes under the window, per side
+  static constexpr int TPB = (CW * HC + 31) / 32 * 32;
   static constexpr int NPT = (NW * NW + TPB - 1) / TPB;
-  static_assert(CW % 2 == 0 && CW * (CW / 2) <= TPB, "one cell pair per thread");
+  static_assert(CN * CN <= TPB && ((TN + 1) / 2) * ((TN + 1) / 2) <= TPB, "one thread per coarse node");
   using V = typename Comp<OP>::V;
   union {
     struct {
@@ -180,117 +182,157 @@ struct SmoothSmem {
     V con[4][CW * CW];       // cell contributions by corner
   };
   V xs[NW * NW];
+  V xc[DOWN ? 1 : CN * CN];
   int32_t tile[20];
   uint8_t cell[NW * NW];     // bit0 the node exists, bit5 the cell whose lower-left node this is exists
 };
 
-template <int OP, bool DOWN>
-__global__ void __launch_bounds__(TPB, 2) smooth_kernel(const __grid_constant__ SmoothArgs a) {
-  using S = SmoothSmem<OP, DOWN>;
+template <int OP, bool DOWN, int TN>
+__global__ void __launch_bounds__(SmoothSmem<OP, DOWN, TN>::TPB, 768 / SmoothSmem<OP, DOWN, TN>::TPB)
+smooth_kernel(const __grid_constant__ SmoothArgs a) {
+  using S = SmoothSmem<OP, DOWN, TN>;
   using V = typename Comp<OP>::V;
-  constexpr int NC = Comp<OP>::NC, HW = S::HW, NW = S::NW, CW = S::CW, NPT = S::NPT, HC = CW / 2;
+  constexpr int NC = Comp<OP>::NC, HW = S::HW, NW = S::NW, CW = S::CW, NPT = S::NPT, HC = S::HC, TPB = S::TPB;
+  constexpr int HB = NB / 2;   // coarse nodes per brick side
   __shared__ S sm;
-  pdl_trigger();
   const int tid = threadIdx.x;
   if (tid < 20) sm.tile[tid] = __ldg(reinterpret_cast<const int32_t*>(a.tiles + blockIdx.x) + tid);
   __syncthreads();
   const int pos = sm.tile[18];
-  const int n0 = TN * (pos & 1) - HW, r0 = TN * ((pos >> 1) & 1) - HW;   // brick position of window node 0
+  const int n0 = TN * (pos & 7) - HW, r0 = TN * ((pos >> 3) & 7) - HW;   // brick position of window node 0
+  const int ox = HB * ((pos >> 6) & 1), oy = HB * ((pos >> 7) & 1);      // the brick's corner in its parent brick
   constexpr int fix0 = OP == OP_UU ? 1 : 4;
   // ---- tables and set-up data, which no kernel of the chain writes: window nodes,
-  // the cells' factors
+  // the cells' factors.  All loads of a thread's nodes are issued together (a position
+  // without a brick reads slot 0 and is masked), so a tile pays one round trip.
   int32_t slot[NPT];
   uint32_t cm[NPT];
   V di[NPT];
+  {
+    uint8_t f[NPT];
+    float2 li[NPT];
+    float e[NPT];
 #pragma unroll
-  for (int k = 0; k < NPT; ++k) {
-    const int w = tid + TPB * k;
-    slot[k] = -1;
-    cm[k] = 0;
-    di[k] = V();
-    if (w < NW * NW) {
+    for (int k = 0; k < NPT; ++k) {
+      const int w = tid + TPB * k;
       const int n = n0 + w % NW, r = r0 + w / NW;
       const int dx = n < 0 ? 0 : (n >= NB ? 2 : 1), dy = r < 0 ? 0 : (r >= NB ? 2 : 1);
-      const int32_t base = sm.tile[3 * dy + dx];
-      uint8_t f = 0;
-      if (base >= 0) {
-        const int32_t s = base + (n - NB * (dx - 1)) + NB * (r - NB * (dy - 1));
-        f = __ldg(a.flags + s);
-        if (f & 1) slot[k] = s;
-      }
-      float2 li = make_float2(0.f, 0.f);
-      float e = 1.f;
-      const int32_t s = slot[k];
-      if (s >= 0) {
-        cm[k] = __ldg(a.cmask + s);
+      const int32_t base = w < NW * NW ? sm.tile[3 * dy + dx] : -1;
+      const int32_t s = base < 0 ? 0 : base + (n - NB * (dx - 1)) + NB * (r - NB * (dy - 1));
+      f[k] = __ldg(a.flags + s);
+      cm[k] = __ldg(a.cmask + s);
 #pragma unroll
-        for (int c = 0; c < NC; ++c) comp(di[k], c) = __ldg(a.dinv + c * int64_t(a.n) + s);
-        if constexpr (OP == OP_UU) {
-          li.x = __ldg(a.lin + 3 * int64_t(a.n) + s);
-        } else {
-          li.x = __ldg(a.lin + s);
-          li.y = __ldg(a.lin + int64_t(a.n) + s);
-        }
-        if (a.ecell != nullptr && (f & 32)) e = __ldg(a.ecell + s);
+      for (int c = 0; c < NC; ++c) comp(di[k], c) = __ldg(a.dinv + c * int64_t(a.n) + s);
+      li[k] = make_float2(0.f, 0.f);
+      if constexpr (OP == OP_UU) {
+        li[k].x = __ldg(a.lin + 3 * int64_t(a.n) + s);
+      } else {
+        li[k].x = __ldg(a.lin + s);
+        li[k].y = __ldg(a.lin + int64_t(a.n) + s);
       }
-      sm.lin[w] = li;
-      sm.e[w] = e;
-      sm.cell[w] = f & 33;
+      e[k] = a.ecell != nullptr ? __ldg(a.ecell + s) : 1.f;
+      slot[k] = base < 0 ? -1 : s;
+    }
+#pragma unroll
+    for (int k = 0; k < NPT; ++k) {
+      const int w = tid + TPB * k;
+      if (slot[k] < 0 || !(f[k] & 1)) {
+        slot[k] = -1;
+        f[k] = 0;
+        cm[k] = 0;
+        di[k] = V();
+        li[k] = make_float2(0.f, 0.f);
+      }
+      if (w < NW * NW) {
+        sm.lin[w] = li[k];
+        sm.e[w] = (f[k] & 32) ? e[k] : 1.f;
+        sm.cell[w] = f[k] & 33;
+      }
     }
   }
   __syncthreads();
   const int ci = tid % CW, cj = tid / CW;
   const bool has = cj < HC;
-  const int nA = ci + NW * (has ? cj : 0), nB = nA + NW * HC;   // lower-left nodes of the pair
-  const bool actA = has && (sm.cell[nA] & 32), actB = has && (sm.cell[nB] & 32);
+  const int nA = ci + NW * (has ? cj : 0), nB = has && cj + HC < CW ? nA + NW * HC : nA;   // lower-left nodes of the pair
+  const bool hasB = has && cj + HC < CW;
+  const bool actA = has && (sm.cell[nA] & 32), actB = hasB && (sm.cell[nB] & 32);
   P q[2][2], ec = pbc(1.f);
   if (actA || actB) {
     if (a.ecell != nullptr) ec = make_float2(sm.e[nA], sm.e[nB]);
     cell_coef<OP, NW>(sm.lin, nA, nB, a.m, a.g, ec, q);
   }
-  // ---- from here on what the preceding kernel wrote
-  pdl_wait();
-  V dv[NPT], xv[NPT];   // defect (then residual), iterate
+  // ---- level vectors.  The next launch may start once every block is past its wait
+  // (the trigger follows it), so a block that runs knows that the launch before the
+  // preceding one has completed.  Up: the defect and the pre-smoothed iterate are
+  // older than that and are read before the wait, the coarse correction after it.
+  V dv[NPT], xv[NPT], xl[NPT];   // defect (then residual), iterate; up: the pre-smoothed iterate
+  auto level_loads = [&]() {
 #pragma unroll
-  for (int k = 0; k < NPT; ++k) {
-    const int w = tid + TPB * k;
-    dv[k] = V();
-    xv[k] = V();
-    const int32_t s = slot[k];
-    if (s >= 0) {
+    for (int k = 0; k < NPT; ++k) {
+      const int32_t s = slot[k] < 0 ? 0 : slot[k];
 #pragma unroll
       for (int c = 0; c < NC; ++c) comp(dv[k], c) = a.d[c * int64_t(a.n) + s];
       if constexpr (!DOWN) {
-        // x + P xc: coarse nodes in ascending (y, x), zero weights left out
-        const int n = n0 + w % NW, r = r0 + w / NW;
-        const int cx = (n >> 1) + TN * ((pos >> 2) & 1), cy = (r >> 1) + TN * ((pos >> 3) & 1);
-        const int nx = n & 1, ny = r & 1;
-        const float wt = (nx ? 0.5f : 1.f) * (ny ? 0.5f : 1.f);
-        V acc;
 #pragma unroll
-        for (int c = 0; c < NC; ++c) comp(acc, c) = a.x[c * int64_t(a.n) + s];
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            if ((b && !ny) || (e && !nx)) continue;
-            const int gx = cx + e, gy = cy + b;
-            const int dx = gx < 0 ? 0 : (gx >= NB ? 2 : 1), dy = gy < 0 ? 0 : (gy >= NB ? 2 : 1);
-            const int32_t cs = sm.tile[9 + 3 * dy + dx] + (gx - NB * (dx - 1)) + NB * (gy - NB * (dy - 1));
-#pragma unroll
-            for (int c = 0; c < NC; ++c) comp(acc, c) += wt * a.xc[c * int64_t(a.nc) + cs];
-          }
-#pragma unroll
-        for (int c = 0; c < NC; ++c) comp(xv[k], c) = (cm[k] & (fix0 << c)) ? 0.f : comp(acc, c);
-      } else {
-#pragma unroll
-        for (int c = 0; c < NC; ++c) comp(xv[k], c) = cheb_first_of(a.c0, comp(di[k], c), comp(dv[k], c));
+        for (int c = 0; c < NC; ++c) comp(xl[k], c) = a.x[c * int64_t(a.n) + s];
       }
     }
-    if (w < NW * NW) sm.xs[w] = xv[k];
+  };
+  if constexpr (!DOWN) level_loads();
+  pdl_wait();
+  pdl_trigger();
+  if constexpr (DOWN) level_loads();
+  {
+    if constexpr (!DOWN) {
+      // the coarse nodes under the window (those without a brick are parents of no window node)
+      constexpr int CN = S::CN;
+      if (tid < CN * CN) {
+        const int gx = (n0 >> 1) + ox + tid % CN, gy = (r0 >> 1) + oy + tid / CN;
+        const int dx = gx < 0 ? 0 : (gx >= NB ? 2 : 1), dy = gy < 0 ? 0 : (gy >= NB ? 2 : 1);
+        const int32_t base = sm.tile[9 + 3 * dy + dx];
+        const int32_t cs = base < 0 ? 0 : base + (gx - NB * (dx - 1)) + NB * (gy - NB * (dy - 1));
+        V v;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) comp(v, c) = a.xc[c * int64_t(a.nc) + cs];
+        sm.xc[tid] = v;
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int k = 0; k < NPT; ++k) {
+      const int w = tid + TPB * k;
+      const bool node = slot[k] >= 0;
+      if (!node) dv[k] = V();
+      if constexpr (DOWN) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) comp(xv[k], c) = cheb_first_of(a.c0, comp(di[k], c), comp(dv[k], c));
+      } else {
+        // x + P xc: the row's coarse nodes in ascending (y, x), zero weights left out
+        constexpr int CN = S::CN;
+        xv[k] = V();
+        if (node) {
+          const int n = n0 + w % NW, r = r0 + w / NW;
+          const int q = (n >> 1) - (n0 >> 1) + CN * ((r >> 1) - (r0 >> 1));
+          const bool nx = n & 1, ny = r & 1;
+          const float wt = (nx ? 0.5f : 1.f) * (ny ? 0.5f : 1.f);
+          const int qx = nx ? q + 1 : q, qy = ny ? q + CN : q;
+          const V p0 = sm.xc[q], p1 = sm.xc[qx], p2 = sm.xc[qy], p3 = sm.xc[qx + qy - q];
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            float acc = comp(xl[k], c);
+            acc += wt * comp(p0, c);
+            if (nx) acc += wt * comp(p1, c);
+            if (ny) acc += wt * comp(p2, c);
+            if (nx && ny) acc += wt * comp(p3, c);
+            comp(xv[k], c) = (cm[k] & (fix0 << c)) ? 0.f : acc;
+          }
+        }
+      }
+      if (w < NW * NW) sm.xs[w] = xv[k];
+    }
   }
   // Down: the restriction's row of this thread.  P^T of the residual goes onto the
-  // coarse nodes at the tile's even positions; thread t takes position (t % 8, t / 8).
+  // coarse nodes at the tile's even positions, one per thread.
   // Rows are summed in ascending storage slot: bricks by (row, column), nodes by
   // (row, column) in each; absent nodes add zero.
   int32_t cs = -1, rw = 0;
@@ -298,11 +340,11 @@ __global__ void __launch_bounds__(TPB, 2) smooth_kernel(const __grid_constant__ 
   V dcv = V();
   if constexpr (DOWN) {
     constexpr int TC = (TN + 1) / 2;
-    const int wx = HW + 2 * (tid % TC) + (pos & 1), wy = HW + 2 * (tid / TC) + ((pos >> 1) & 1);   // even brick positions
+    const int wx = HW + 2 * (tid % TC) + (n0 + HW) % 2, wy = HW + 2 * (tid / TC) + (r0 + HW) % 2;   // even brick positions
     if (tid < TC * TC && wx < HW + TN && wy < HW + TN && (sm.cell[wx + NW * wy] & 1)) {
       rw = wx + NW * wy;
       const int n = n0 + wx, r = r0 + wy;
-      cs = sm.tile[9 + 4] + (n >> 1) + TN * ((pos >> 2) & 1) + NB * ((r >> 1) + TN * ((pos >> 3) & 1));
+      cs = sm.tile[9 + 4] + (n >> 1) + ox + NB * ((r >> 1) + oy);
       cmc = __ldg(a.cmask_c + cs);
 #pragma unroll
       for (int c = 0; c < NC; ++c) comp(dcv, c) = a.dc[c * int64_t(a.nc) + cs];
@@ -318,7 +360,7 @@ __global__ void __launch_bounds__(TPB, 2) smooth_kernel(const __grid_constant__ 
     {
       const int lo = HW - R - 1, hi = HW + TN + R - 1;   // window cells per direction
       const bool cx = ci >= lo && ci <= hi;
-      const bool inA = has && cx && cj >= lo && cj <= hi, inB = has && cx && cj + HC >= lo && cj + HC <= hi;
+      const bool inA = has && cx && cj >= lo && cj <= hi, inB = hasB && cx && cj + HC >= lo && cj + HC <= hi;
       if (inA || inB) {
         P r[NC][4];
         if ((inA && actA) || (inB && actB)) {
@@ -339,7 +381,7 @@ __global__ void __launch_bounds__(TPB, 2) smooth_kernel(const __grid_constant__ 
             comp(vB, c) = actB ? r[c][e].y : 0.f;
           }
           sm.con[e][iA] = vA;
-          sm.con[e][iB] = vB;
+          if (hasB) sm.con[e][iB] = vB;
         }
       }
     }
@@ -425,17 +467,32 @@ __global__ void __launch_bounds__(TPB, 2) smooth_kernel(const __grid_constant__ 
   }
 }
 
-template <bool DOWN>
-cudaError_t launch_smooth(const SmoothArgs& a, int op, cudaStream_t s) {
-  if (a.ntiles <= 0) return cudaSuccess;
-  if (op == OP_UU) return launch_ex(true, &smooth_kernel<OP_UU, DOWN>, unsigned(a.ntiles), TPB, 0, s, a);
-  if (op == OP_PP) return launch_ex(true, &smooth_kernel<OP_PP, DOWN>, unsigned(a.ntiles), TPB, 0, s, a);
+template <bool DOWN, int TN>
+cudaError_t launch_tile(const SmoothArgs& a, int op, cudaStream_t s, bool pdl) {
+  constexpr unsigned tpb = SmoothSmem<OP_UU, DOWN, TN>::TPB;
+  if (op == OP_UU) return launch_ex(pdl, &smooth_kernel<OP_UU, DOWN, TN>, unsigned(a.ntiles), tpb, 0, s, a);
+  if (op == OP_PP) return launch_ex(pdl, &smooth_kernel<OP_PP, DOWN, TN>, unsigned(a.ntiles), tpb, 0, s, a);
   return cudaErrorInvalidValue;
+}
+
+template <bool DOWN>
+cudaError_t launch_smooth(const SmoothArgs& a, int op, cudaStream_t s, bool pdl) {
+  if (a.ntiles <= 0) return cudaSuccess;
+  switch (a.tile) {
+    case 6: return launch_tile<DOWN, 6>(a, op, s, pdl);
+    case 10: return launch_tile<DOWN, 10>(a, op, s, pdl);
+    case 15: return launch_tile<DOWN, 15>(a, op, s, pdl);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 }  // namespace
 
-cudaError_t launch_smooth_down(const SmoothArgs& a, int op, cudaStream_t s) { return launch_smooth<true>(a, op, s); }
-cudaError_t launch_smooth_up(const SmoothArgs& a, int op, cudaStream_t s) { return launch_smooth<false>(a, op, s); }
+cudaError_t launch_smooth_down(const SmoothArgs& a, int op, cudaStream_t s) {
+  return launch_smooth<true>(a, op, s, true);
+}
+cudaError_t launch_smooth_up(const SmoothArgs& a, int op, cudaStream_t s, bool pdl) {
+  return launch_smooth<false>(a, op, s, pdl);
+}
 
 }  // namespace pff

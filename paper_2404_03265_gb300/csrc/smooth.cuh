@@ -9,22 +9,21 @@
 
 namespace pff {
 
-// A tile of kSmoothTile x kSmoothTile node positions of a level brick (four tiles
-// per brick; only tiles that hold a node are listed).  Node (n, r) of the window
-// around the tile lies in one of the brick's 3x3 neighbours; the coarser level's
-// nodes under the window lie in the 3x3 neighbours of the parent brick.
-constexpr int kSmoothTile = 15;
+// A tile of node positions of a level brick: tile x tile nodes, tile in {6, 10, 15}
+// (25, 9 or 4 tiles per brick; only tiles that hold a node are listed).  Node (n, r)
+// of the window around the tile lies in one of the brick's 3x3 neighbours; the coarser
+// level's nodes under the window lie in the 3x3 neighbours of the parent brick.
 struct SmoothTile {
   int32_t fb[9];   // storage bases of the brick's 3x3 neighbours on this level (-1 absent)
   int32_t cb[9];   // the same of the parent brick (bx / 2, by / 2) on the next coarser level
-  int32_t pos;     // tile column | tile row << 1 | (bx & 1) << 2 | (by & 1) << 3
+  int32_t pos;     // tile column | tile row << 3 | (bx & 1) << 6 | (by & 1) << 7
   int32_t pad;
 };
 
 // One level and block of the V-cycle.  Vectors: ncomp blocks of n (coarse: nc) floats.
 struct SmoothArgs {
   const SmoothTile* tiles;
-  int32_t ntiles;
+  int32_t ntiles, tile;    // tiles, and nodes per tile side
   int32_t n, nc;           // slots of this level, of the next coarser one
   const uint8_t* flags;    // level slot flags: bit0 node, bit5 the cell whose lower-left node this is exists
   const uint8_t* cmask;
@@ -44,8 +43,11 @@ struct SmoothArgs {
 
 // Down: x = p(D^-1 A) D^-1 d (Chebyshev degree 3 from zero), then dc += P^T (d - A x).
 // Up: x += P xc, then x += p(D^-1 A) D^-1 (d - A x).
-// op: OP_UU or OP_PP.  Launched programmatically dependent on the preceding kernel.
+// op: OP_UU or OP_PP.  Launched programmatically dependent on the preceding kernel of
+// the stream (up: when pdl is set).  Up reads d and x before it waits for that kernel,
+// so with pdl that kernel must let it start (pdl_trigger) only after the one that
+// wrote d and x has completed.
 cudaError_t launch_smooth_down(const SmoothArgs& a, int op, cudaStream_t s);
-cudaError_t launch_smooth_up(const SmoothArgs& a, int op, cudaStream_t s);
+cudaError_t launch_smooth_up(const SmoothArgs& a, int op, cudaStream_t s, bool pdl);
 
 }  // namespace pff

