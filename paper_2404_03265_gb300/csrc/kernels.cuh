@@ -58,6 +58,20 @@ struct DevLayout {
   const uint32_t* cellmask = nullptr;
 };
 
+// The Q1 leaf mesh as compact lists (leaf_cells.cu): its cells in brick order, and per
+// node slot the cells around it.
+struct LeafCells {
+  int32_t ncells = 0;
+  const int4* corner = nullptr;     // per cell its nodes (0,0), (1,0), (0,1), (1,1): slot, or -2 - hanging entry
+  const uint8_t* level = nullptr;
+  const int32_t* slot = nullptr;    // cell slot (per-cell data)
+  // per node slot the cells (own, left, below, below-left; -1 none) whose contributions it
+  // sums; x = -2 - i: entry i of the fix-up list instead
+  const int4* node = nullptr;
+  const int4* part = nullptr;       // the same per partial sum of the fix-up list
+  void* out = nullptr;              // 12 blocks of ncells: the cells' contributions (3 * corner + component)
+};
+
 // Material constants of the cell kernels (level independent), precomputed on
 // the host in the kernel's precision (no double arithmetic in FP32 kernels).
 template <typename T>
@@ -107,6 +121,7 @@ struct ChebEpi {
 
 struct ApplyArgs {
   DevLayout lay;
+  LeafCells lc;           // Q1 leaf
   const DevHanging* hang;
   const uint8_t* cmask;   // per slot: bit0/bit1 u_x/u_y fixed, bit2 phi fixed
   const void* lin;        // 4 blocks of n_slots T: u_x, u_y, phi, phi_tilde (hanging entries resolved)
@@ -169,6 +184,15 @@ template <typename T>
 cudaError_t launch_apply(const ApplyArgs& a, int op, cudaStream_t s);
 template <typename T>
 cudaError_t launch_fixup(const FixupArgs& a, cudaStream_t s);
+
+// A Q1 leaf operator with its fix-up in two passes over a.lc (leaf_cells.cu): any but
+// OP_VJP in FP64, OP_FULL and OP_FULL_T in FP32; no level operators.
+template <typename T>
+cudaError_t launch_leaf_cells(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);
+template <>
+cudaError_t launch_leaf_cells<double>(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);
+template <>
+cudaError_t launch_leaf_cells<float>(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);
 
 // state conversion: lin64/lin32 blocks (u_x, u_y, phi, phi_t), hanging entries from parents;
 // u is the displacement in block layout (u_x block, u_y block)

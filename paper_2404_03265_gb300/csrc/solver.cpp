@@ -33,6 +33,8 @@ cudaError_t leaf_op(pff_problem& pb, int kop, int mode, const double* lin, const
   ApplyArgs a;
   std::memset(&a, 0, sizeof(a));
   a.lay = D.leaf;
+  a.lc = D.cells;
+  a.lc.out = pb.cell_buf;
   a.hang = D.hang;
   a.cmask = cmask;
   a.lin = lin;
@@ -53,9 +55,7 @@ cudaError_t leaf_op(pff_problem& pb, int kop, int mode, const double* lin, const
   FixupArgs f;
   f.n = D.nfix; f.n_slots = M.lay.n_slots; f.slot = D.fix_slot; f.ptr = D.fix_ptr; f.part = D.fix_part;
   f.w = D.fix_w; f.cmask = cmask; f.xu = xu; f.xp = xp; f.yu = yu; f.yp = yp; f.ibuf = a.ibuf; f.mode = mode;
-  RET(launch_apply<double>(a, kop, s));
-  if (kop == OP_VJP) return cudaSuccess;  // per-cell outputs only
-  return launch_fixup<double>(f, s);
+  return launch_leaf<double>(a, f, kop, s);
 }
 
 std::string ensure_workspace(pff_problem& pb, int restart) {

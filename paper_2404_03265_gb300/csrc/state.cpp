@@ -1,6 +1,7 @@
 // Device uploads and operator dispatch behind the C-ABI.
 #include "state.h"
 
+#include <algorithm>
 #include <cstring>
 #include <unordered_map>
 
@@ -56,6 +57,91 @@ static std::vector<SmoothTile> smooth_tiles(const LevelMesh& lm, const LevelMesh
   return out;
 }
 
+// Tables of the two-pass leaf operators (Q1)
+static LeafCells upload_leaf_cells(DevAllocs& mem, const Mesh& M) {
+  const int NB = M.lay.NB;
+  const size_t ns = size_t(M.lay.n_slots);
+  // cells in the order of their slots (brick by brick, and so level by level), each
+  // level filled up to an even number with a repeated cell that no node refers to
+  std::vector<int32_t> cells(M.cell_slot), at(ns, -1), slot;
+  std::sort(cells.begin(), cells.end());
+  auto level_of = [&](int32_t s) { return M.lay.bricks[size_t(s) / (size_t(NB) * NB)].level; };
+  for (size_t q = 0; q < cells.size(); ++q) {
+    at[cells[q]] = int32_t(slot.size());
+    slot.push_back(cells[q]);
+    if ((q + 1 == cells.size() || level_of(cells[q + 1]) != level_of(cells[q])) && slot.size() % 2)
+      slot.push_back(cells[q]);
+  }
+  const size_t nc = slot.size();
+  std::vector<int4> corner(nc), node(ns, make_int4(-1, -1, -1, -1)), part(size_t(M.n_partials));
+  std::vector<uint8_t> level(nc);
+  const int W = M.lay.W;
+  for (size_t q = 0; q < nc; ++q) {
+    const int32_t s = slot[q];
+    const BrickDesc& d = M.lay.bricks[size_t(s) / (size_t(NB) * NB)];
+    const int n = s % (NB * NB) % NB, r = s % (NB * NB) / NB;
+    int32_t code[4];
+    for (int e = 0; e < 4; ++e) {
+      const int i = n + (e & 1), j = r + (e >> 1);   // brick position, 0..NB
+      code[e] = d.irr >= 0 ? M.lay.win[size_t(d.irr) * W * W + (i + 1) + size_t(W) * (j + 1)]
+                           : d.nbr_base[(j < NB ? 3 : 6) + (i < NB ? 1 : 2)] + i % NB + NB * (j % NB);
+    }
+    corner[q] = make_int4(code[0], code[1], code[2], code[3]);
+    level[q] = uint8_t(d.level);
+  }
+  for (size_t b = 0; b < M.lay.bricks.size(); ++b) {
+    const BrickDesc& d = M.lay.bricks[b];
+    auto cell_at = [&](int n, int r) -> int32_t {   // the leaf cell of this level at brick position (n, r) >= -1
+      const int32_t base = d.nbr_base[(r < 0 ? 0 : 3) + (n < 0 ? 0 : 1)];
+      return base < 0 ? -1 : at[size_t(base) + (n < 0 ? n + NB : n) + size_t(NB) * (r < 0 ? r + NB : r)];
+    };
+    for (int r = 0; r < NB; ++r)
+      for (int n = 0; n < NB; ++n) {
+        const size_t o = size_t(n) + size_t(NB) * r, s = b * size_t(NB) * NB + o;
+        const int4 k = make_int4(cell_at(n, r), cell_at(n - 1, r), cell_at(n, r - 1), cell_at(n - 1, r - 1));
+        const int32_t p = d.irr >= 0 ? M.lay.own_part[size_t(d.irr) * NB * NB + o] : -1;
+        if (p >= 0) part[p] = k;
+        if (M.slot_node[s] >= 0) node[s] = k;
+      }
+  }
+  for (size_t i = 0; i < M.fix_slot.size(); ++i) node[M.fix_slot[i]] = make_int4(-2 - int32_t(i), -1, -1, -1);
+  LeafCells L;
+  L.ncells = int32_t(nc);
+  L.corner = mem.upload(corner);
+  L.level = mem.upload(level);
+  L.slot = mem.upload(slot);
+  L.node = mem.upload(node);
+  L.part = mem.upload(part);
+  return L;
+}
+
+// A leaf operator and its fix-up: Q1 in two passes over the cell and node lists where
+// that is the faster path (leaf_cells.cu), else the cell loop and the fix-up kernel.
+//  - FP64: always two passes (bound by the FP64 rate, and they evaluate only cells that
+//    exist): Jacobian 992 -> 741 us on 4.1M DoFs, 633 -> 204 us on the 1.04M-DoF crack
+//    mesh, 45 -> 22 us on 4.3k DoFs.  A forced strip height asks for the sweep's Jacobian.
+//  - FP32: two passes up to kTwoPassCells, while the 48 bytes of contributions per cell
+//    stay small beside L2: 13.1 -> 11.1 us on 65k DoFs, 30.7 -> 19.6 us on the crack mesh,
+//    26.6 -> 22.0 us at 0.53M cells, but 31.1 -> 34.0 us at 0.77M and 37.9 -> 61 us at
+//    1.36M (the sweep writes no contributions to memory).
+constexpr int32_t kTwoPassCells = 650000;
+static bool use_two_passes(const ApplyArgs& a, int op, bool f64) {
+  if (a.fe_degree != 1 || op == OP_VJP || a.lc.out == nullptr) return false;
+  const bool jacobian = op == OP_FULL || op == OP_FULL_T;
+  if (a.sweep_sh != 0 && jacobian) return false;
+  return f64 || (jacobian && a.lc.ncells <= kTwoPassCells);
+}
+
+template <typename T>
+cudaError_t launch_leaf(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s) {
+  if (use_two_passes(a, op, sizeof(T) == 8)) return launch_leaf_cells<T>(a, f, op, s);
+  const cudaError_t e = launch_apply<T>(a, op, s);
+  if (e != cudaSuccess || op == OP_VJP) return e;   // OP_VJP: per-cell outputs only
+  return launch_fixup<T>(f, s);
+}
+template cudaError_t launch_leaf<float>(const ApplyArgs&, const FixupArgs&, int, cudaStream_t);
+template cudaError_t launch_leaf<double>(const ApplyArgs&, const FixupArgs&, int, cudaStream_t);
+
 std::string upload_mesh(pff_mesh& pm) {
   DevMesh& D = pm.dev;
   int dev = 0;
@@ -67,6 +153,7 @@ std::string upload_mesh(pff_mesh& pm) {
   }
   const Mesh& M = pm.m;
   D.leaf = upload_layout(D.mem, M.lay);
+  if (M.k == 1) D.cells = upload_leaf_cells(D.mem, M);
   std::vector<DevHanging> hh(M.hang.size());
   for (size_t h = 0; h < M.hang.size(); ++h) {
     hh[h].slot = M.hang[h].slot;
@@ -180,17 +267,19 @@ std::string upload_mesh(pff_mesh& pm) {
 std::string alloc_problem(pff_problem& pb) {
   const Mesh& M = pb.mesh->m;
   const int64_t ns = M.lay.n_slots;
-  pb.lin64 = pb.bufs.alloc<double>(4 * ns);
-  pb.lin32 = pb.bufs.alloc<float>(4 * ns);
-  pb.cmask = pb.bufs.alloc<uint8_t>(ns);
-  pb.cmask_dir = pb.bufs.alloc<uint8_t>(ns);
-  pb.ibuf64 = pb.bufs.alloc<double>(3 * M.n_partials);
-  pb.ibuf32 = pb.bufs.alloc<float>(3 * M.n_partials);
   const int64_t nh = int64_t(M.hang.size());
-  pb.hlin64 = pb.bufs.alloc<double>(4 * nh);
-  pb.hlin32 = pb.bufs.alloc<float>(4 * nh);
-  pb.hx64 = pb.bufs.alloc<double>(3 * nh);
-  pb.hx32 = pb.bufs.alloc<float>(3 * nh);
+  pb.bufs.reserve(pb.lin64, 4 * ns);
+  pb.bufs.reserve(pb.lin32, 4 * ns);
+  pb.bufs.reserve(pb.cmask, ns);
+  pb.bufs.reserve(pb.cmask_dir, ns);
+  pb.bufs.reserve(pb.ibuf64, 3 * M.n_partials);
+  pb.bufs.reserve(pb.ibuf32, 3 * M.n_partials);
+  pb.bufs.reserve(pb.hlin64, 4 * nh);
+  pb.bufs.reserve(pb.hlin32, 4 * nh);
+  pb.bufs.reserve(pb.hx64, 3 * nh);
+  pb.bufs.reserve(pb.hx32, 3 * nh);
+  if (M.k == 1) pb.bufs.reserve(pb.cell_buf, 12 * size_t(pb.mesh->dev.cells.ncells));
+  pb.bufs.commit();
   if (!pb.bufs.err.empty()) {
     std::string err = pb.bufs.err;
     pb.bufs.release();
@@ -230,6 +319,8 @@ cudaError_t leaf_apply(pff_problem& pb, int precision, int op, const void* xu, c
   ApplyArgs a;
   std::memset(&a, 0, sizeof(a));
   a.lay = D.leaf;
+  a.lc = D.cells;
+  a.lc.out = pb.cell_buf;
   a.hang = D.hang;
   a.cmask = pb.cmask;
   a.lin = precision == PFF_F64 ? static_cast<const void*>(pb.lin64) : static_cast<const void*>(pb.lin32);
@@ -254,15 +345,7 @@ cudaError_t leaf_apply(pff_problem& pb, int precision, int op, const void* xu, c
   FixupArgs f;
   f.n = D.nfix; f.n_slots = M.lay.n_slots; f.slot = D.fix_slot; f.ptr = D.fix_ptr; f.part = D.fix_part; f.w = D.fix_w;
   f.cmask = pb.cmask; f.xu = xu; f.xp = xp; f.yu = yu; f.yp = yp; f.ibuf = a.ibuf; f.mode = a.mode;
-  cudaError_t e;
-  if (precision == PFF_F64) {
-    e = launch_apply<double>(a, kop, s);
-    if (e == cudaSuccess) e = launch_fixup<double>(f, s);
-  } else {
-    e = launch_apply<float>(a, kop, s);
-    if (e == cudaSuccess) e = launch_fixup<float>(f, s);
-  }
-  return e;
+  return precision == PFF_F64 ? launch_leaf<double>(a, f, kop, s) : launch_leaf<float>(a, f, kop, s);
 }
 
 }  // namespace pff

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -29,6 +30,26 @@ struct DevAllocs {
     ptrs.push_back(p);
     return static_cast<T*>(p);
   }
+  // Several blocks out of one allocation: reserve(n) each pointer, then commit() once.
+  struct Part {
+    void** p;
+    size_t off;
+  };
+  std::vector<Part> parts;
+  size_t part_bytes = 0;
+  template <typename T>
+  void reserve(T*& p, size_t n) {
+    p = nullptr;
+    parts.push_back({reinterpret_cast<void**>(&p), part_bytes});
+    part_bytes += (std::max<size_t>(n, 1) * sizeof(T) + 255) / 256 * 256;
+  }
+  void commit() {
+    unsigned char* base = parts.empty() ? nullptr : alloc<unsigned char>(part_bytes);
+    for (const Part& q : parts)
+      if (base) *q.p = base + q.off;
+    parts.clear();
+    part_bytes = 0;
+  }
   template <typename T>
   T* upload(const std::vector<T>& v) {
     T* p = alloc<T>(v.size());
@@ -49,6 +70,7 @@ struct DevMesh {
   bool uploaded = false;
   int device = -1;
   DevLayout leaf;
+  LeafCells cells;             // Q1 (its contribution buffer belongs to each problem)
   DevHanging* hang = nullptr;
   int32_t nhang = 0;
   int32_t nfix = 0;
@@ -156,6 +178,7 @@ struct pff_problem {
   float* hlin32 = nullptr;
   double* hx64 = nullptr;    // per hanging node: the input resolved from its parents, 3 blocks of n_hang
   float* hx32 = nullptr;
+  double* cell_buf = nullptr;  // Q1: 12 doubles per leaf cell, the contributions of the two-pass operators
   bool has_state = false;
   // per-cell modulus E_K (cell-slot layout; levels concatenated like level vectors)
   bool has_ecell = false;
@@ -266,6 +289,9 @@ void fill_material(const pff_params& prm, ApplyArgs& a, bool unit_E = false);
 // the current device (noalloc.cu).
 cudaError_t noalloc_prepare();
 void leaf_modulus(const pff_problem& pb, int precision, ApplyArgs& a);
+// a leaf operator with its fix-up, by the faster path (state.cpp)
+template <typename T>
+cudaError_t launch_leaf(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);
 cudaError_t leaf_apply(pff_problem& pb, int precision, int op, const void* xu, const void* xp, void* yu,
                        void* yp, cudaStream_t s);
 cudaError_t launch_leaf_cmask(int64_t n, const uint8_t* slot_flags, const uint8_t* active, uint8_t* cmask,
