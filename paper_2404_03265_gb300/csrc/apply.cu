@@ -28,6 +28,7 @@
 #include "cheb.cuh"
 #include "pdl.cuh"
 #include "q1_cell.cuh"
+#include "q2_jac.cuh"
 
 #include <cmath>
 #include <mutex>
@@ -862,7 +863,12 @@ cudaError_t launch_apply(const ApplyArgs& a, int op, cudaStream_t s) {
   if (a.lay.nbricks <= 0) return cudaSuccess;
   // the fused Chebyshev store exists in the level block operators only
   if (a.ch.mode != CHEB_OFF && op != OP_UU && op != OP_PP) return cudaErrorInvalidValue;
-  if (a.fe_degree == 2) return launch_apply_q2<T>(a, op, s);
+  if (a.fe_degree == 2) {
+    ApplyArgs b = a;
+    const uintptr_t al = reinterpret_cast<uintptr_t>(a.yu) | reinterpret_cast<uintptr_t>(a.yp);
+    b.pair_store = al % (2 * sizeof(T)) == 0 && a.n_slots % 2 == 0;
+    return launch_apply_q2<T>(b, op, s);
+  }
   if (a.fe_degree != 1) return cudaErrorInvalidValue;
   switch (op) {
     case OP_FULL: return launch_sweep<T, OP_FULL>(a, s);

@@ -17,11 +17,13 @@
 //      that take the same contractions travel as pairs (u_x with u_y of the
 //      input and of the linearisation, the input dphi with phi), one paired
 //      FP32 instruction for both, and the shared tiles interleave each pair;
-//   3. the cells' nodal contributions are added into a shared tile in four
-//      colour phases (cells of equal (i, j) parity share no node), so every
-//      nodal sum has a fixed order;
-//   4. the owned nodes are written (constraint rows, partial sums, holes), or
-//      for the level block operators the fused Chebyshev step of ChebEpi.
+//   3. the cells write their contributions to shared memory, one column per cell, and a
+//      thread sums them for the four owned nodes (2i, 2j) .. (2i + 1, 2j + 1): the cells
+//      around a node in the order (even column, even row), (odd, even), (even, odd),
+//      (odd, odd), so every nodal sum has a fixed order;
+//   4. the owned nodes are written (constraint rows, partial sums, holes; pairs of
+//      unconstrained nodes of regular bricks as one 8-byte store in FP32), or for the
+//      level block operators the fused Chebyshev step of ChebEpi.
 
 constexpr int Q2NB = 30;          // owned node slots per side
 constexpr int Q2W = 33;           // window nodes per side (-2..30)
@@ -51,8 +53,7 @@ struct Q2Smem {
   using P = typename VT<T>::T2;
   static constexpr int NBUF = sizeof(T) == 4 ? 2 : 1;
   P f[NBUF][Q2NP][Q2WW];    // node fields of the window, as pairs (q2_pair, q2_half)
-  P yu[Q2WW];               // nodal sums, u_x and u_y
-  T yp[Q2WW];               // nodal sums, phi
+  T con[27][Q2T];           // contributions of the window's cells: 3 * (local node) + component
   uint32_t cmw[NBUF][Q2WW]; // prefetch: the aligned word holding each node's constraint byte
   int32_t nb[NBUF][9];      // storage bases of the 3x3 neighbour bricks
   uint8_t cmsh[NBUF][Q2WW]; // prefetch: byte position of the constraint byte in its word
@@ -318,36 +319,53 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
   const int ci = tid % Q2C, cj = tid / Q2C;          // window cell (cell ci - 1, cj - 1)
   const int cbase = 2 * ci + Q2W * 2 * cj;            // window node (0, 0) of the cell
   const int G = int(gridDim.x);
+  // this thread's window nodes: neighbour brick (index into nbr_base) << 16 | slot in it
+  constexpr int NWN = (Q2WW + Q2T - 1) / Q2T;
+  int32_t wpos[NWN];
+#pragma unroll
+  for (int e = 0; e < NWN; ++e) {
+    const int w = tid + Q2T * e, n = w % Q2W - 2, r = w / Q2W - 2;
+    const int dx = n < 0 ? 0 : (n >= Q2NB ? 2 : 1), dy = r < 0 ? 0 : (r >= Q2NB ? 2 : 1);
+    wpos[e] = (3 * dy + dx) << 16 | ((n - (dx - 1) * Q2NB) + Q2NB * (r - (dy - 1) * Q2NB));
+  }
   // window of regular brick bn into buffer bu: cp.async of every used field and of
   // the word holding each node's constraint byte; committed as one group
   auto prefetch = [&](int bn, int bu) {
     const BrickDesc* bdn = a.lay.bricks + bn;
-    int32_t nbv[9];
+    if (tid < 9) sm.nb[bu][tid] = __ldg(bdn->nbr_base + tid);
+    int32_t code[NWN];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) nbv[i] = __ldg(bdn->nbr_base + i);
-    if (tid < 9) sm.nb[bu][tid] = nbv[tid];
-    for (int w = tid; w < Q2WW; w += Q2T) {
-      const int32_t code = q2_slot(nbv, w % Q2W - 2, w / Q2W - 2);
+    for (int e = 0; e < NWN; ++e)
+      code[e] = tid + Q2T * e < Q2WW ? __ldg(bdn->nbr_base + (wpos[e] >> 16)) + (wpos[e] & 0xffff) : 0;
+#pragma unroll
+    for (int e = 0; e < NWN; ++e) {
+      const int w = tid + Q2T * e;
+      if (w >= Q2WW) break;
 #pragma unroll
       for (int f = 0; f < NF; ++f)
-        if (field_used<OP>(f)) cp_one(&q2_field<T>(sm.f[bu], f, w), field_ptr<T>(a, f) + code);
-      cp_async4(&sm.cmw[bu][w], a.cmask + (code & ~3));
-      sm.cmsh[bu][w] = uint8_t(code & 3);
+        if (field_used<OP>(f)) cp_one(&q2_field<T>(sm.f[bu], f, w), field_ptr<T>(a, f) + code[e]);
+      cp_async4(&sm.cmw[bu][w], a.cmask + (code[e] & ~3));
+      sm.cmsh[bu][w] = uint8_t(code[e] & 3);
     }
     cp_async_commit();
   };
-  auto regular = [&](int bn) { return __ldg(&a.lay.bricks[bn].irr) < 0; };
   int cur = 0;
   bool pending = false;   // buffer cur holds a prefetch of brick b not yet waited for
-  if (NBUF == 2 && int(blockIdx.x) < a.lay.nbricks && regular(blockIdx.x)) {
+  // irregular-table index and level of the current and the next brick: read one brick
+  // ahead, so that no block waits for them
+  auto desc = [&](int bn) -> int2 {
+    if (bn >= a.lay.nbricks) return make_int2(0, 0);
+    return make_int2(__ldg(&a.lay.bricks[bn].irr), __ldg(&a.lay.bricks[bn].level));
+  };
+  int2 dc = desc(blockIdx.x), dn = desc(blockIdx.x + G);
+  if (NBUF == 2 && int(blockIdx.x) < a.lay.nbricks && dc.x < 0) {
     prefetch(blockIdx.x, 0);
     pending = true;
   }
 #pragma unroll 1
   for (int b = blockIdx.x; b < a.lay.nbricks; b += G) {
     const BrickDesc* bd = a.lay.bricks + b;
-    const int irr = __ldg(&bd->irr);
-    const int level = __ldg(&bd->level);
+    const int irr = dc.x, level = dc.y;
     P (*fb)[Q2WW] = sm.f[cur];
     const int32_t* nbc = sm.nb[cur];
     __syncthreads();   // the previous brick's tiles are no longer read
@@ -362,7 +380,6 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
           if (cmw & 2) q2_field<T>(fb, F_XV, w) = T(0);
           if (cmw & 4) q2_field<T>(fb, F_XP, w) = T(0);
         }
-        if (!isVjp) { sm.yu[w] = pbc(T(0)); sm.yp[w] = T(0); }
       }
     } else {
       if (tid < 9) sm.nb[cur][tid] = __ldg(bd->nbr_base + tid);
@@ -403,13 +420,13 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
         for (int f = 0; f < NF; ++f)
           if (field_used<OP>(f)) q2_field<T>(fb, f, w) = v[f];
         sm.cm[w] = cmw;
-        if (!isVjp) { sm.yu[w] = pbc(T(0)); sm.yp[w] = T(0); }
       }
     }
     __syncthreads();
     // the next brick's window streams in while this one computes
     bool next_pending = false;
-    if (NBUF == 2 && b + G < a.lay.nbricks && regular(b + G)) {
+    const int2 dnn = desc(b + 2 * G);
+    if (NBUF == 2 && b + G < a.lay.nbricks && dn.x < 0) {
       prefetch(b + G, cur ^ 1);
       next_pending = true;
     }
@@ -423,7 +440,12 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
     if (a.ecell != nullptr && act) ec = ldg(reinterpret_cast<const T*>(a.ecell) + q2_slot(nbc, 2 * ci - 2, 2 * cj - 2));
     P ru[9];
     T rp[9], cell[3];
-    if (act) q2_cell<T, OP>(fb, cbase, mc, geom<T>(a, level), tb, ec, ru, rp, cell);
+    if (act) {
+      if constexpr (OP == OP_FULL || OP == OP_FULL_T || OP == OP_RESID)
+        q2_jac<T, OP>([&](int k, int i, int j) { return fb[k][cbase + i + Q2W * j]; }, mc, geom<T>(a, level), ec, ru, rp);
+      else
+        q2_cell<T, OP>(fb, cbase, mc, geom<T>(a, level), tb, ec, ru, rp, cell);
+    }
     if constexpr (isVjp) {
       // the brick owns the cells whose lower-left node it owns (cells 0..14)
       if (act && ci >= 1 && cj >= 1) {
@@ -433,38 +455,84 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
         for (int q = 0; q < 3; ++q) co[q * a.n_slots + s] = cell[q];
       }
     } else {
-      // 3. colour phases: cells of one (i, j) parity add their 9 x 3 contributions
-#pragma unroll 1
-      for (int ph = 0; ph < 4; ++ph) {
-        if (act && (ci & 1) == (ph & 1) && (cj & 1) == (ph >> 1)) {
+      // 3. contributions to shared memory, then the owned nodes' sums
+      if (!act) {
 #pragma unroll
-          for (int bb = 0; bb < 3; ++bb)
-#pragma unroll
-            for (int aa = 0; aa < 3; ++aa) {
-              const int w = cbase + aa + Q2W * bb;
-              sm.yu[w] = padd(sm.yu[w], ru[aa + 3 * bb]);
-              sm.yp[w] += rp[aa + 3 * bb];
-            }
-        }
-        __syncthreads();
+        for (int e = 0; e < 9; ++e) { ru[e] = pbc(T(0)); rp[e] = T(0); }
       }
-      // 4. owned nodes (level block operators: or the fused Chebyshev store)
+      constexpr bool outU = OP != OP_PP && OP != OP_PP_DIAG && OP != OP_MASS && OP != OP_TCV && OP != OP_PHIT_VJP;
+      constexpr bool outP = OP != OP_UU && OP != OP_UU_DIAG;
+#pragma unroll
+      for (int e = 0; e < 9; ++e) {
+        if (outU) { sm.con[3 * e][tid] = ru[e].x; sm.con[3 * e + 1][tid] = ru[e].y; }
+        if (outP) sm.con[3 * e + 2][tid] = rp[e];
+      }
+      __syncthreads();
       const int own_base = nbc[4];
-      for (int o = tid; o < Q2NB * Q2NB; o += Q2T) {
-        const int oi = o % Q2NB, oj = o / Q2NB;
-        const int w = (oi + 2) + Q2W * (oj + 2);
-        if constexpr (OP == OP_UU || OP == OP_PP) {
-          if (a.ch.mode != CHEB_OFF) {
-            const int act_s = irr >= 0 ? int(__ldg(a.lay.own_act + irr * (Q2NB * Q2NB) + o)) : int(kActFinal);
-            ChebOps<T, OP> co;
-            cheb_load<T, OP>(a, own_base + o, co);
-            cheb_store<T, OP>(a, own_base + o, act_s, sm.cm[w], sm.yu[w].x, sm.yu[w].y, sm.yp[w], co);
-            continue;
+      if (tid < 225) {
+        const int i = tid % 15, j = tid / 15;
+        const int own = (i + 1) + Q2C * (j + 1);   // the window cell above right of node (2i, 2j)
+        const bool ox = (i + 1) & 1, oy = (j + 1) & 1;   // its column, row is odd: its neighbour's comes first
+#pragma unroll
+        for (int py = 0; py < 2; ++py) {
+          T y[2][3];
+#pragma unroll
+          for (int px = 0; px < 2; ++px) {
+            // per direction the even cell (first) and the odd one: offset from own, local node
+            const int cx0 = px || !ox ? 0 : -1, ax0 = px ? 1 : (ox ? 2 : 0), cx1 = ox ? 0 : -1, ax1 = ox ? 0 : 2;
+            const int cy0 = py || !oy ? 0 : -Q2C, ay0 = py ? 1 : (oy ? 2 : 0), cy1 = oy ? 0 : -Q2C, ay1 = oy ? 0 : 2;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+              y[px][q] = T(0);
+              if (!(q < 2 ? outU : outP)) continue;
+              T v = sm.con[3 * (ax0 + 3 * ay0) + q][own + cx0 + cy0];
+              if (!px) v += sm.con[3 * (ax1 + 3 * ay0) + q][own + cx1 + cy0];
+              if (!py) {
+                v += sm.con[3 * (ax0 + 3 * ay1) + q][own + cx0 + cy1];
+                if (!px) v += sm.con[3 * (ax1 + 3 * ay1) + q][own + cx1 + cy1];
+              }
+              y[px][q] = v;
+            }
+          }
+          // 4. owned nodes (level block operators: or the fused Chebyshev store)
+          const int oi = 2 * i, oj = 2 * j + py, o = oi + Q2NB * oj;
+          const int w = (oi + 2) + Q2W * (oj + 2);
+          const uint8_t cm0 = sm.cm[w], cm1 = sm.cm[w + 1];
+          bool done = false;
+          if constexpr (OP == OP_UU || OP == OP_PP) {
+            if (a.ch.mode != CHEB_OFF) {
+#pragma unroll
+              for (int px = 0; px < 2; ++px) {
+                const int act_s = irr >= 0 ? int(__ldg(a.lay.own_act + irr * (Q2NB * Q2NB) + o + px)) : int(kActFinal);
+                ChebOps<T, OP> co;
+                cheb_load<T, OP>(a, own_base + o + px, co);
+                cheb_store<T, OP>(a, own_base + o + px, act_s, px ? cm1 : cm0, y[px][0], y[px][1], y[px][2], co);
+              }
+              done = true;
+            }
+          }
+          if (!done && irr < 0 && (cm0 | cm1) == 0) {
+            T* yu = reinterpret_cast<T*>(a.yu) + own_base + o;
+            T* yp = reinterpret_cast<T*>(a.yp) + own_base + o;
+            if (a.pair_store) {   // even slots of 8-byte (FP64: 16-byte) aligned vectors
+              if (outU) {
+                *reinterpret_cast<P*>(yu) = P{y[0][0], y[1][0]};
+                *reinterpret_cast<P*>(yu + a.n_slots) = P{y[0][1], y[1][1]};
+              }
+              if (outP) *reinterpret_cast<P*>(yp) = P{y[0][2], y[1][2]};
+            } else {
+              if (outU) { yu[0] = y[0][0]; yu[1] = y[1][0]; yu[a.n_slots] = y[0][1]; yu[a.n_slots + 1] = y[1][1]; }
+              if (outP) { yp[0] = y[0][2]; yp[1] = y[1][2]; }
+            }
+          } else if (!done) {
+            write_node<T, OP>(a, irr, own_base, oi, oj, cm0, y[0][0], y[0][1], y[0][2]);
+            write_node<T, OP>(a, irr, own_base, oi + 1, oj, cm1, y[1][0], y[1][1], y[1][2]);
           }
         }
-        write_node<T, OP>(a, irr, own_base, oi, oj, sm.cm[w], sm.yu[w].x, sm.yu[w].y, sm.yp[w]);
       }
     }
+    dc = dn;
+    dn = dnn;
     if (NBUF == 2) cur ^= 1;
     pending = next_pending;
   }

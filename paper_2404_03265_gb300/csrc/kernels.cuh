@@ -58,18 +58,20 @@ struct DevLayout {
   const uint32_t* cellmask = nullptr;
 };
 
-// The Q1 leaf mesh as compact lists (leaf_cells.cu): its cells in brick order, and per
-// node slot the cells around it.
+// The leaf mesh as compact lists (leaf_cells.cu, leaf_cells_q2.cu): its cells in brick
+// order, and per node slot the cells around it.
 struct LeafCells {
   int32_t ncells = 0;
-  const int4* corner = nullptr;     // per cell its nodes (0,0), (1,0), (0,1), (1,1): slot, or -2 - hanging entry
+  const int4* corner = nullptr;     // Q1: per cell its nodes (0,0), (1,0), (0,1), (1,1): slot, or -2 - hanging entry
+  const int32_t* nodes9 = nullptr;  // Q2: 9 blocks of ncells, the same for node a + 3 b
   const uint8_t* level = nullptr;
   const int32_t* slot = nullptr;    // cell slot (per-cell data)
   // per node slot the cells (own, left, below, below-left; -1 none) whose contributions it
   // sums; x = -2 - i: entry i of the fix-up list instead
   const int4* node = nullptr;
   const int4* part = nullptr;       // the same per partial sum of the fix-up list
-  void* out = nullptr;              // 12 blocks of ncells: the cells' contributions (3 * corner + component)
+  const uint8_t* part_pos = nullptr;   // Q2: parity of the partial's brick position, column | row << 1
+  void* out = nullptr;              // 12 (Q2: 27) blocks of ncells: the contributions (3 * node + component)
 };
 
 // Material constants of the cell kernels (level independent), precomputed on
@@ -121,7 +123,7 @@ struct ChebEpi {
 
 struct ApplyArgs {
   DevLayout lay;
-  LeafCells lc;           // Q1 leaf
+  LeafCells lc;           // leaf operators
   const DevHanging* hang;
   const uint8_t* cmask;   // per slot: bit0/bit1 u_x/u_y fixed, bit2 phi fixed
   const void* lin;        // 4 blocks of n_slots T: u_x, u_y, phi, phi_tilde (hanging entries resolved)
@@ -149,6 +151,7 @@ struct ApplyArgs {
   int mode;
   int fe_degree;
   int sweep_sh;           // Q1 strip half-height: 0 = by mesh size, else 15, 5 or 1 (schedules of DevLayout::units)
+  int pair_store;         // Q2: the output vectors allow stores of two neighbouring slots (set by launch_apply)
   int pdl_in;             // Q1: launched dependent on the preceding kernel, which wrote x (pdl.cuh)
   ChebEpi ch;             // level applies: fused Chebyshev store (mode CHEB_OFF: plain y = A x)
 };
@@ -193,6 +196,9 @@ template <>
 cudaError_t launch_leaf_cells<double>(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);
 template <>
 cudaError_t launch_leaf_cells<float>(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);
+
+// The same for Q2 in FP64 (leaf_cells_q2.cu): OP_FULL, OP_FULL_T, OP_RESID.
+cudaError_t launch_leaf_cells_q2(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);
 
 // state conversion: lin64/lin32 blocks (u_x, u_y, phi, phi_t), hanging entries from parents;
 // u is the displacement in block layout (u_x block, u_y block)

@@ -57,7 +57,7 @@ static std::vector<SmoothTile> smooth_tiles(const LevelMesh& lm, const LevelMesh
   return out;
 }
 
-// Tables of the two-pass leaf operators (Q1)
+// Tables of the two-pass leaf operators
 static LeafCells upload_leaf_cells(DevAllocs& mem, const Mesh& M) {
   const int NB = M.lay.NB;
   const size_t ns = size_t(M.lay.n_slots);
@@ -73,41 +73,55 @@ static LeafCells upload_leaf_cells(DevAllocs& mem, const Mesh& M) {
       slot.push_back(cells[q]);
   }
   const size_t nc = slot.size();
-  std::vector<int4> corner(nc), node(ns, make_int4(-1, -1, -1, -1)), part(size_t(M.n_partials));
-  std::vector<uint8_t> level(nc);
-  const int W = M.lay.W;
+  const int k = M.k, W = M.lay.W;
+  std::vector<int4> corner(k == 1 ? nc : 0), node(ns, make_int4(-1, -1, -1, -1)), part(size_t(M.n_partials));
+  std::vector<int32_t> nodes9(k == 2 ? 9 * nc : 0);
+  std::vector<uint8_t> level(nc), part_pos(size_t(M.n_partials), 0);
   for (size_t q = 0; q < nc; ++q) {
     const int32_t s = slot[q];
     const BrickDesc& d = M.lay.bricks[size_t(s) / (size_t(NB) * NB)];
     const int n = s % (NB * NB) % NB, r = s % (NB * NB) / NB;
-    int32_t code[4];
-    for (int e = 0; e < 4; ++e) {
-      const int i = n + (e & 1), j = r + (e >> 1);   // brick position, 0..NB
-      code[e] = d.irr >= 0 ? M.lay.win[size_t(d.irr) * W * W + (i + 1) + size_t(W) * (j + 1)]
-                           : d.nbr_base[(j < NB ? 3 : 6) + (i < NB ? 1 : 2)] + i % NB + NB * (j % NB);
-    }
-    corner[q] = make_int4(code[0], code[1], code[2], code[3]);
+    int32_t code[9];
+    for (int b = 0; b <= k; ++b)
+      for (int a = 0; a <= k; ++a) {
+        const int i = n + a, j = r + b;   // brick position, 0..NB
+        code[a + (k + 1) * b] = d.irr >= 0 ? M.lay.win[size_t(d.irr) * W * W + (i + k) + size_t(W) * (j + k)]
+                                           : d.nbr_base[(j < NB ? 3 : 6) + (i < NB ? 1 : 2)] + i % NB + NB * (j % NB);
+      }
+    if (k == 1) corner[q] = make_int4(code[0], code[1], code[2], code[3]);
+    else
+      for (int e = 0; e < 9; ++e) nodes9[size_t(e) * nc + q] = code[e];
     level[q] = uint8_t(d.level);
   }
   for (size_t b = 0; b < M.lay.bricks.size(); ++b) {
     const BrickDesc& d = M.lay.bricks[b];
-    auto cell_at = [&](int n, int r) -> int32_t {   // the leaf cell of this level at brick position (n, r) >= -1
+    auto cell_at = [&](int n, int r) -> int32_t {   // the leaf cell of this level with lower-left node (n, r) >= -k
       const int32_t base = d.nbr_base[(r < 0 ? 0 : 3) + (n < 0 ? 0 : 1)];
       return base < 0 ? -1 : at[size_t(base) + (n < 0 ? n + NB : n) + size_t(NB) * (r < 0 ? r + NB : r)];
     };
     for (int r = 0; r < NB; ++r)
       for (int n = 0; n < NB; ++n) {
         const size_t o = size_t(n) + size_t(NB) * r, s = b * size_t(NB) * NB + o;
-        const int4 k = make_int4(cell_at(n, r), cell_at(n - 1, r), cell_at(n, r - 1), cell_at(n - 1, r - 1));
+        const int px = n % k, py = r % k, n0 = n - px, r0 = r - py;   // inside a Q2 cell: no left (lower) neighbour
+        const int4 q = make_int4(cell_at(n0, r0), px ? -1 : cell_at(n0 - k, r0), py ? -1 : cell_at(n0, r0 - k),
+                                 px || py ? -1 : cell_at(n0 - k, r0 - k));
         const int32_t p = d.irr >= 0 ? M.lay.own_part[size_t(d.irr) * NB * NB + o] : -1;
-        if (p >= 0) part[p] = k;
-        if (M.slot_node[s] >= 0) node[s] = k;
+        if (p >= 0) {
+          part[p] = q;
+          part_pos[p] = uint8_t(px | py << 1);
+        }
+        if (M.slot_node[s] >= 0) node[s] = q;
       }
   }
   for (size_t i = 0; i < M.fix_slot.size(); ++i) node[M.fix_slot[i]] = make_int4(-2 - int32_t(i), -1, -1, -1);
   LeafCells L;
   L.ncells = int32_t(nc);
-  L.corner = mem.upload(corner);
+  if (k == 1) {
+    L.corner = mem.upload(corner);
+  } else {
+    L.nodes9 = mem.upload(nodes9);
+    L.part_pos = mem.upload(part_pos);
+  }
   L.level = mem.upload(level);
   L.slot = mem.upload(slot);
   L.node = mem.upload(node);
@@ -126,15 +140,17 @@ static LeafCells upload_leaf_cells(DevAllocs& mem, const Mesh& M) {
 //    1.36M (the sweep writes no contributions to memory).
 constexpr int32_t kTwoPassCells = 650000;
 static bool use_two_passes(const ApplyArgs& a, int op, bool f64) {
-  if (a.fe_degree != 1 || op == OP_VJP || a.lc.out == nullptr) return false;
+  if (op == OP_VJP || a.lc.out == nullptr) return false;
   const bool jacobian = op == OP_FULL || op == OP_FULL_T;
+  if (a.fe_degree == 2) return f64 && (jacobian || op == OP_RESID);
   if (a.sweep_sh != 0 && jacobian) return false;
   return f64 || (jacobian && a.lc.ncells <= kTwoPassCells);
 }
 
 template <typename T>
 cudaError_t launch_leaf(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s) {
-  if (use_two_passes(a, op, sizeof(T) == 8)) return launch_leaf_cells<T>(a, f, op, s);
+  if (use_two_passes(a, op, sizeof(T) == 8))
+    return a.fe_degree == 1 ? launch_leaf_cells<T>(a, f, op, s) : launch_leaf_cells_q2(a, f, op, s);
   const cudaError_t e = launch_apply<T>(a, op, s);
   if (e != cudaSuccess || op == OP_VJP) return e;   // OP_VJP: per-cell outputs only
   return launch_fixup<T>(f, s);
@@ -153,7 +169,7 @@ std::string upload_mesh(pff_mesh& pm) {
   }
   const Mesh& M = pm.m;
   D.leaf = upload_layout(D.mem, M.lay);
-  if (M.k == 1) D.cells = upload_leaf_cells(D.mem, M);
+  D.cells = upload_leaf_cells(D.mem, M);
   std::vector<DevHanging> hh(M.hang.size());
   for (size_t h = 0; h < M.hang.size(); ++h) {
     hh[h].slot = M.hang[h].slot;
@@ -278,7 +294,7 @@ std::string alloc_problem(pff_problem& pb) {
   pb.bufs.reserve(pb.hlin32, 4 * nh);
   pb.bufs.reserve(pb.hx64, 3 * nh);
   pb.bufs.reserve(pb.hx32, 3 * nh);
-  if (M.k == 1) pb.bufs.reserve(pb.cell_buf, 12 * size_t(pb.mesh->dev.cells.ncells));
+  pb.bufs.reserve(pb.cell_buf, (M.k == 1 ? 12 : 27) * size_t(pb.mesh->dev.cells.ncells));
   pb.bufs.commit();
   if (!pb.bufs.err.empty()) {
     std::string err = pb.bufs.err;

@@ -70,7 +70,7 @@ struct DevMesh {
   bool uploaded = false;
   int device = -1;
   DevLayout leaf;
-  LeafCells cells;             // Q1 (its contribution buffer belongs to each problem)
+  LeafCells cells;             // (the contribution buffer belongs to each problem)
   DevHanging* hang = nullptr;
   int32_t nhang = 0;
   int32_t nfix = 0;
@@ -178,7 +178,7 @@ struct pff_problem {
   float* hlin32 = nullptr;
   double* hx64 = nullptr;    // per hanging node: the input resolved from its parents, 3 blocks of n_hang
   float* hx32 = nullptr;
-  double* cell_buf = nullptr;  // Q1: 12 doubles per leaf cell, the contributions of the two-pass operators
+  double* cell_buf = nullptr;  // 12 (Q2: 27) doubles per leaf cell, the contributions of the two-pass operators
   bool has_state = false;
   // per-cell modulus E_K (cell-slot layout; levels concatenated like level vectors)
   bool has_ecell = false;
