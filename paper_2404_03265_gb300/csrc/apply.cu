@@ -83,48 +83,6 @@ __device__ __forceinline__ const T* field_ptr(const ApplyArgs& a, int f) {
   }
 }
 
-// Final write of owned node (n, c) of an irregular brick: storage action,
-// partial sum, constraint rows.
-template <typename T, int OP>
-__device__ __forceinline__ void write_node(const ApplyArgs& a, int irr, int own_base, int n, int c, uint8_t cm,
-                                           T y0, T y1, T y2) {
-  constexpr bool outU = (OP != OP_PP && OP != OP_PP_DIAG && OP != OP_MASS && OP != OP_TCV && OP != OP_PHIT_VJP);
-  constexpr bool outP = (OP != OP_UU && OP != OP_UU_DIAG);
-  constexpr bool isDiag = (OP == OP_UU_DIAG || OP == OP_PP_DIAG);
-  T* yu = reinterpret_cast<T*>(a.yu);
-  T* yv = yu + a.n_slots;
-  T* yp = reinterpret_cast<T*>(a.yp);
-  const int o = n + NB * c;
-  int act_s = kActFinal, part = -1;
-  if (irr >= 0) {
-    act_s = __ldg(a.lay.own_act + irr * (NB * NB) + o);
-    part = __ldg(a.lay.own_part + irr * (NB * NB) + o);
-  }
-  const int slot = own_base + o;
-  if (part >= 0) {
-    T* ib = reinterpret_cast<T*>(a.ibuf) + 3 * int64_t(part);
-    ib[0] = y0; ib[1] = y1; ib[2] = y2;
-  }
-  if (act_s == kActFinal) {
-    if (isDiag) {
-      if (cm & 1) y0 = T(0);
-      if (cm & 2) y1 = T(0);
-      if (cm & 4) y2 = T(0);
-    } else if (cm) {
-      const bool ident = (a.mode & MODE_IDENTITY) != 0;
-      const T* xu = reinterpret_cast<const T*>(a.xu);
-      if (cm & 1) y0 = ident ? ldg(xu + slot) : T(0);
-      if (cm & 2) y1 = ident ? ldg(xu + a.n_slots + slot) : T(0);
-      if (cm & 4) y2 = ident ? ldg(reinterpret_cast<const T*>(a.xp) + slot) : T(0);
-    }
-    if (outU) { yu[slot] = y0; yv[slot] = y1; }
-    if (outP) yp[slot] = y2;
-  } else if (act_s == kActZero) {
-    if (outU) { yu[slot] = T(0); yv[slot] = T(0); }
-    if (outP) yp[slot] = T(0);
-  }
-}
-
 // ---- column sweep (the Q1 cell loop) ---------------------------------------
 //
 // One warp takes a strip of 2 SH owned node rows r0 .. r0 + 2 SH - 1 of a brick.
@@ -184,6 +142,13 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
 template <typename T>
 __device__ __forceinline__ void cp_one(T* dst, const T* src) {
   if constexpr (sizeof(T) == 4) cp_async4(dst, src); else cp_async8(dst, src);
+}
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+}
+template <typename T>   // two neighbours, aligned to their size
+__device__ __forceinline__ void cp_two(T* dst, const T* src) {
+  if constexpr (sizeof(T) == 4) cp_async8(dst, src); else cp_async16(dst, src);
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int K>
@@ -760,11 +725,28 @@ void fill_q2(Q2Tab<T>& t) {
   }
 }
 
+template <typename T>
+void fill_q2_mat(Q2Mat<T>& c, const ApplyArgs& a) {
+  const double yx = a.hy[0] / a.hx[0], xy = a.hx[0] / a.hy[0], c2 = 2.0 * a.mu + a.lam, ok = 1.0 - a.kappa;
+  c.al = T(c2 * yx); c.alt = T(c2 * xy); c.be = T(a.lam); c.ga = T(a.mu * xy); c.gat = T(a.mu * yx); c.de = T(a.mu);
+  c.oal = T(ok * c2 * yx); c.oalt = T(ok * c2 * xy); c.obe = T(ok * a.lam);
+  c.oga = T(ok * a.mu * xy); c.ogat = T(ok * a.mu * yx); c.ode = T(ok * a.mu);
+  const double w[3] = {25.0 / 324.0, 40.0 / 324.0, 64.0 / 324.0};
+  for (int i = 0; i < 3; ++i) {
+    c.omkw[i] = T(w[i] * ok); c.kapw[i] = T(w[i] * a.kappa);
+    c.gxxw[i] = T(w[i] * a.gc_times_l * yx); c.gyyw[i] = T(w[i] * a.gc_times_l * xy);
+  }
+}
+
 void fill_cell_constants(ApplyArgs& a, int nlevels) {
   fill_mat(a.mf, a);
   fill_mat(a.md, a);
   fill_q2(a.q2f);
   fill_q2(a.q2d);
+  if (nlevels > 0) {
+    fill_q2_mat(a.q2mf, a);
+    fill_q2_mat(a.q2md, a);
+  }
   for (int l = 0; l < nlevels && l < kMaxLevels; ++l) {
     fill_geom(a.gf[l], a, a.hx[l], a.hy[l]);
     fill_geom(a.gd[l], a, a.hx[l], a.hy[l]);
@@ -867,6 +849,9 @@ cudaError_t launch_apply(const ApplyArgs& a, int op, cudaStream_t s) {
     ApplyArgs b = a;
     const uintptr_t al = reinterpret_cast<uintptr_t>(a.yu) | reinterpret_cast<uintptr_t>(a.yp);
     b.pair_store = al % (2 * sizeof(T)) == 0 && a.n_slots % 2 == 0;
+    const uintptr_t in = reinterpret_cast<uintptr_t>(a.xu) | reinterpret_cast<uintptr_t>(a.xp) |
+                         reinterpret_cast<uintptr_t>(a.lin);
+    b.wide = in % 16 == 0;   // (a block of n_slots values is a multiple of 16 bytes)
     return launch_apply_q2<T>(b, op, s);
   }
   if (a.fe_degree != 1) return cudaErrorInvalidValue;

@@ -9,14 +9,14 @@
 // A brick owns 30 x 30 node slots = 15 x 15 Q2 cells; its window holds the
 // 33 x 33 nodes -2..30 and the 16 x 16 cells -1..14 (all cells touching an
 // owned node).  A block of 256 threads takes one brick at a time:
-//   1. the window's node fields go to shared memory (hanging values from their
-//      parents, fixed input components masked, absent nodes zero);
+//   1. the window's node fields go to shared memory, one plane per field (hanging values
+//      from their parents, fixed input components masked, absent nodes zero);
 //   2. each thread evaluates one cell, sum-factorised: per Gauss row eta_q2 the
 //      3x3 nodal values collapse to three column values, then to the row's
 //      three Gauss points; the test runs the same two steps backwards.  Fields
 //      that take the same contractions travel as pairs (u_x with u_y of the
 //      input and of the linearisation, the input dphi with phi), one paired
-//      FP32 instruction for both, and the shared tiles interleave each pair;
+//      FP32 instruction for both;
 //   3. the cells write their contributions to shared memory, one column per cell, and a
 //      thread sums them for the four owned nodes (2i, 2j) .. (2i + 1, 2j + 1): the cells
 //      around a node in the order (even column, even row), (odd, even), (even, odd),
@@ -24,6 +24,11 @@
 //   4. the owned nodes are written (constraint rows, partial sums, holes; pairs of
 //      unconstrained nodes of regular bricks as one 8-byte store in FP32), or for the
 //      level block operators the fused Chebyshev step of ChebEpi.
+
+// Measured (Jacobian FP32, 16.4M DoFs): 212 us with single-value copies, colour phases and
+// plain contractions; 176 us in this form, with half the error against 64 bits.  16 warps
+// an SM wait in turn for the window, the barriers and the stores of irregular bricks
+// (issue slots 36% busy); the vectors and the linearisation take 32 us at the copy rate.
 
 constexpr int Q2NB = 30;          // owned node slots per side
 constexpr int Q2W = 33;           // window nodes per side (-2..30)
@@ -45,25 +50,60 @@ __device__ __forceinline__ constexpr bool q2_pair_used(int k) {
        : k == 2 ? field_used<OP>(F_XP) || field_used<OP>(F_LP) : field_used<OP>(F_LT);
 }
 
+// A plane holds the rows -2..30 of columns 0..29 (the brick's own block and, around it in
+// the same row order, the last two rows of the brick below and the first row of the one
+// above, 32 values), then columns -2, -1, then column 30.  So a regular brick arrives as
+// 16-byte copies of contiguous storage but for the two side halos: 248 + 66 copies per
+// field instead of 1,089 single values.
+constexpr int Q2ROWS = 992;                          // 33 rows of 30, and 2 values past the last
+constexpr int Q2LEFT = Q2ROWS, Q2RIGHT = Q2LEFT + 2 * Q2W;
+constexpr int Q2PL = Q2RIGHT + Q2W + 1;
+// plane offset of window node (wx, wy), wx, wy = 0..32
+__device__ __forceinline__ int q2_at(int wx, int wy) {
+  return wx < 2 ? Q2LEFT + 2 * wy + wx : wx == Q2W - 1 ? Q2RIGHT + wy : wx - 2 + Q2NB * wy;
+}
+
 // FP32 keeps two window buffers: while a block computes one brick, the window
-// of its next brick, when regular, streams into the other with cp.async.  FP64
-// (twice the bytes per field) keeps one and gathers each brick in turn.
+// of its next brick streams into the other with cp.async.  FP64 (twice the bytes
+// per field) keeps one and gathers each brick in turn.
 template <typename T>
 struct Q2Smem {
   using P = typename VT<T>::T2;
   static constexpr int NBUF = sizeof(T) == 4 ? 2 : 1;
-  P f[NBUF][Q2NP][Q2WW];    // node fields of the window, as pairs (q2_pair, q2_half)
-  T con[27][Q2T];           // contributions of the window's cells: 3 * (local node) + component
-  uint32_t cmw[NBUF][Q2WW]; // prefetch: the aligned word holding each node's constraint byte
-  int32_t nb[NBUF][9];      // storage bases of the 3x3 neighbour bricks
-  uint8_t cmsh[NBUF][Q2WW]; // prefetch: byte position of the constraint byte in its word
-  uint8_t cm[Q2WW];         // constraint-mask byte of each window node of the current brick
+  alignas(16) T f[NBUF][NF][Q2PL];   // node fields of the window
+  P conu[9][Q2T];           // contributions of the window's cells by local node: u_x and u_y
+  T conp[9][Q2T];           // phi
+  // constraint-mask bytes: the plane layout's rows, then the aligned words that hold
+  // columns -2, -1 and column 30 of each window row
+  alignas(16) uint8_t cm[NBUF][Q2ROWS + 4 * 2 * Q2W];
+  alignas(16) int32_t own[NBUF][Q2NB * Q2NB];   // irregular bricks: DevLayout::own of the owned slots
+  int32_t nb[3][9];         // storage bases of the 3x3 neighbour bricks of three bricks in turn
 };
 
-template <typename T>
-__device__ __forceinline__ T& q2_field(typename VT<T>::T2 (*fb)[Q2WW], int f, int w) {
-  return half_of<T>(fb[q2_pair(f)][w], q2_half(f));
-}
+// Nodes (a, b) of window cell (ci, cj): value pair k (q2_pair) of the fields OP reads.
+template <typename T, int OP>
+struct Q2Node {
+  using P = typename VT<T>::T2;
+  const T* pl;
+  int o[3], st[3];   // per column a: plane offset of its node (a, 0), and the row stride
+  __device__ __forceinline__ void at(int ci, int cj) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int wx = 2 * ci + a;
+      o[a] = q2_at(wx, 2 * cj);
+      st[a] = wx < 2 ? 2 : wx == Q2W - 1 ? 1 : Q2NB;
+    }
+  }
+  template <int F>
+  __device__ __forceinline__ T field(int e) const {
+    if constexpr (field_used<OP>(F)) return pl[F * Q2PL + e]; else return T(0);
+  }
+  __device__ __forceinline__ P operator()(int k, int a, int b) const {
+    const int e = o[a] + b * st[a];
+    return k == 0 ? P{field<F_XU>(e), field<F_XV>(e)} : k == 1 ? P{field<F_LU>(e), field<F_LV>(e)}
+         : k == 2 ? P{field<F_XP>(e), field<F_LP>(e)} : P{field<F_LT>(e), T(0)};
+  }
+};
 
 // Storage slot of node (n, r) (brick-relative, -2..30) of a brick whose
 // neighbour bases are nb; the caller guarantees the neighbour exists.
@@ -162,11 +202,10 @@ __device__ __forceinline__ void q2_point(const Q2Point<T>& q, const MatConst<T>&
   (void)se;
 }
 
-// One Q2 cell: node (a, b) of the cell (a along x, b along y) is window node
-// base + a + Q2W * b.  Contributions to node A = a + 3 b: ru[A] (components u_x,
+// One Q2 cell, its node (a, b) (a along x, b along y) read by ld.  Contributions to node A = a + 3 b: ru[A] (components u_x,
 // u_y) and rp[A] (phi).  cell[]: per-cell values (OP_VJP).
 template <typename T, int OP>
-__device__ __forceinline__ void q2_cell(const typename VT<T>::T2 (*fb)[Q2WW], int base, const MatConst<T>& m,
+__device__ __forceinline__ void q2_cell(const Q2Node<T, OP>& ld, const MatConst<T>& m,
                                         const LevGeom<T>& g, const Q2Tab<T>& tb, T ec, typename VT<T>::T2 ru[9],
                                         T rp[9], T cell[3]) {
   using N = Needs<OP>;
@@ -185,10 +224,9 @@ __device__ __forceinline__ void q2_cell(const typename VT<T>::T2 (*fb)[Q2WW], in
 #pragma unroll
     for (int k = 0; k < Q2NP; ++k) {
       if (!q2_pair_used<OP>(k)) continue;
-      const P* fl = fb[k] + base;
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        const P v0 = fl[a], v1 = fl[a + Q2W], v2 = fl[a + 2 * Q2W];
+        const P v0 = ld(k, a, 0), v1 = ld(k, a, 1), v2 = ld(k, a, 2);
         V[k][a] = pfma(pbc(tb.L[2][q2]), v2, pfma(pbc(tb.L[1][q2]), v1, pmul(pbc(tb.L[0][q2]), v0)));
         if (k < Q2NP - 1)
           E[k][a] = pfma(pbc(tb.D[2][q2]), v2, pfma(pbc(tb.D[1][q2]), v1, pmul(pbc(tb.D[0][q2]), v0)));
@@ -305,6 +343,10 @@ template <typename T> __device__ __forceinline__ const Q2Tab<T>& q2tab(const App
 template <> __device__ __forceinline__ const Q2Tab<float>& q2tab<float>(const ApplyArgs& a) { return a.q2f; }
 template <> __device__ __forceinline__ const Q2Tab<double>& q2tab<double>(const ApplyArgs& a) { return a.q2d; }
 
+template <typename T> __device__ __forceinline__ const Q2Mat<T>& q2mat(const ApplyArgs& a);
+template <> __device__ __forceinline__ const Q2Mat<float>& q2mat<float>(const ApplyArgs& a) { return a.q2mf; }
+template <> __device__ __forceinline__ const Q2Mat<double>& q2mat<double>(const ApplyArgs& a) { return a.q2md; }
+
 template <typename T, int OP>
 __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(const __grid_constant__ ApplyArgs a) {
   using P = typename VT<T>::T2;
@@ -317,40 +359,111 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
   const MatConst<T>& mc = matc<T>(a);
   const Q2Tab<T>& tb = q2tab<T>(a);
   const int ci = tid % Q2C, cj = tid / Q2C;          // window cell (cell ci - 1, cj - 1)
-  const int cbase = 2 * ci + Q2W * 2 * cj;            // window node (0, 0) of the cell
+  Q2Node<T, OP> node;
+  node.at(ci, cj);
   const int G = int(gridDim.x);
-  // this thread's window nodes: neighbour brick (index into nbr_base) << 16 | slot in it
-  constexpr int NWN = (Q2WW + Q2T - 1) / Q2T;
-  int32_t wpos[NWN];
+  constexpr int NWN = (Q2WW + Q2T - 1) / Q2T;   // window nodes per thread
+  // Constraint byte of window node (wx, wy) (plane layout of Q2Smem::cm)
+  auto cm_at = [&](const uint8_t* cm, int wx, int wy) -> uint32_t {
+    if (wx >= 2 && wx < Q2W - 1) return cm[wx - 2 + Q2NB * wy];
+    const int r = wy < 2 ? Q2NB - 2 + wy : wy == Q2W - 1 ? 0 : wy - 2;   // brick row of the node's storage
+    const int byte = wx < 2 ? (Q2NB * r + Q2NB - 2) % 4 + wx : Q2NB * r % 4;
+    return cm[Q2ROWS + 4 * ((wx < 2 ? 0 : Q2W) + wy) + byte];
+  };
+  // Window of the brick with neighbour bases nb and irregular-table index irn into buffer
+  // bu as one group of cp.async; hanging nodes are resolved from their parents, absent
+  // ones are zero
+  auto prefetch = [&](const int32_t* nb, int irn, int bu) {
+    if (irn < 0 && a.wide) {
+      constexpr int E = 16 / int(sizeof(T));
+      const int32_t below = nb[1], own = nb[4], above = nb[7];
+      auto src_of = [&](int v) {
+        return v < 2 * Q2NB ? below + Q2NB * (Q2NB - 2) + v
+               : v < 2 * Q2NB + Q2NB * Q2NB ? own + v - 2 * Q2NB : above + v - 2 * Q2NB - Q2NB * Q2NB;
+      };
+      for (int t = tid; t < Q2ROWS / E; t += Q2T) {
+        const int32_t src = src_of(t * E);
 #pragma unroll
-  for (int e = 0; e < NWN; ++e) {
-    const int w = tid + Q2T * e, n = w % Q2W - 2, r = w / Q2W - 2;
-    const int dx = n < 0 ? 0 : (n >= Q2NB ? 2 : 1), dy = r < 0 ? 0 : (r >= Q2NB ? 2 : 1);
-    wpos[e] = (3 * dy + dx) << 16 | ((n - (dx - 1) * Q2NB) + Q2NB * (r - (dy - 1) * Q2NB));
-  }
-  // window of regular brick bn into buffer bu: cp.async of every used field and of
-  // the word holding each node's constraint byte; committed as one group
-  auto prefetch = [&](int bn, int bu) {
-    const BrickDesc* bdn = a.lay.bricks + bn;
-    if (tid < 9) sm.nb[bu][tid] = __ldg(bdn->nbr_base + tid);
+        for (int f = 0; f < NF; ++f)
+          if (field_used<OP>(f)) cp_async16(&sm.f[bu][f][t * E], field_ptr<T>(a, f) + src);
+      }
+      if (tid < Q2ROWS / 4) cp_async4(&sm.cm[bu][4 * tid], a.cmask + src_of(4 * tid));
+      // side halos: the fields f = group mod 3, one window row of one side per thread
+      const int group = tid / (2 * Q2W), h = tid % (2 * Q2W), wy = h % Q2W, side = h / Q2W;
+      const int dy = wy < 2 ? 0 : wy == Q2W - 1 ? 2 : 1, r = wy < 2 ? Q2NB - 2 + wy : wy == Q2W - 1 ? 0 : wy - 2;
+      const int32_t src = nb[3 * dy + 2 * side] + Q2NB * r + (side ? 0 : Q2NB - 2);
+      if (group < 3) {
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+          if (field_used<OP>(f) && f % 3 == group) {
+            const T* p = field_ptr<T>(a, f) + src;
+            if (side) cp_one(&sm.f[bu][f][Q2RIGHT + wy], p);
+            else cp_two(&sm.f[bu][f][Q2LEFT + 2 * wy], p);
+          }
+        if (group == 2) cp_async4(&sm.cm[bu][Q2ROWS + 4 * h], a.cmask + (src & ~3));
+      }
+      cp_async_commit();
+      return;
+    }
+    if (irn >= 0 && tid < Q2NB * Q2NB / 4)
+      cp_async16(&sm.own[bu][4 * tid], a.lay.own + int64_t(irn) * (Q2NB * Q2NB) + 4 * tid);
     int32_t code[NWN];
 #pragma unroll
+    for (int e = 0; e < NWN; ++e) {
+      const int w = tid + Q2T * e;
+      code[e] = kAbsent;
+      if (w < Q2WW)
+        code[e] = irn < 0 ? q2_slot(nb, w % Q2W - 2, w / Q2W - 2) : __ldg(a.lay.win + int64_t(irn) * Q2WW + w);
+    }
+#pragma unroll
     for (int e = 0; e < NWN; ++e)
-      code[e] = tid + Q2T * e < Q2WW ? __ldg(bdn->nbr_base + (wpos[e] >> 16)) + (wpos[e] & 0xffff) : 0;
+      if (code[e] >= 0) {
+        const int at = q2_at((tid + Q2T * e) % Q2W, (tid + Q2T * e) / Q2W);
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+          if (field_used<OP>(f)) cp_one(&sm.f[bu][f][at], field_ptr<T>(a, f) + code[e]);
+      }
+    uint8_t cm[NWN];
+#pragma unroll
+    for (int e = 0; e < NWN; ++e) cm[e] = code[e] >= 0 ? __ldg(a.cmask + code[e]) : uint8_t(0);
 #pragma unroll
     for (int e = 0; e < NWN; ++e) {
       const int w = tid + Q2T * e;
       if (w >= Q2WW) break;
+      const int wx = w % Q2W, wy = w / Q2W;
+      if (wx >= 2 && wx < Q2W - 1) {
+        sm.cm[bu][wx - 2 + Q2NB * wy] = cm[e];
+      } else {
+        const int r = wy < 2 ? Q2NB - 2 + wy : wy == Q2W - 1 ? 0 : wy - 2;
+        const int byte = wx < 2 ? (Q2NB * r + Q2NB - 2) % 4 + wx : Q2NB * r % 4;
+        sm.cm[bu][Q2ROWS + 4 * ((wx < 2 ? 0 : Q2W) + wy) + byte] = cm[e];
+      }
+      if (code[e] >= 0) continue;
+      const int at = q2_at(wx, wy);
+      T v[NF];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) v[f] = T(0);
+      if (code[e] != kAbsent) {
+        const DevHanging& h = a.hang[-2 - code[e]];
+#pragma unroll
+        for (int f = F_LU; f < NF; ++f)
+          if (field_used<OP>(f)) v[f] = ldg(field_ptr<T>(a, f) + h.slot);
+        for (int p = 0; p < 3; ++p) {
+          const int ps = h.parent[p];
+          const T wgt = T(h.weight[p]);
+          const uint8_t pc = mask ? __ldg(a.cmask + ps) : uint8_t(0);
+#pragma unroll
+          for (int f = F_XU; f <= F_XP; ++f)
+            if (field_used<OP>(f) && !(pc & (1 << f))) v[f] += wgt * ldg(field_ptr<T>(a, f) + ps);
+        }
+      }
 #pragma unroll
       for (int f = 0; f < NF; ++f)
-        if (field_used<OP>(f)) cp_one(&q2_field<T>(sm.f[bu], f, w), field_ptr<T>(a, f) + code[e]);
-      cp_async4(&sm.cmw[bu][w], a.cmask + (code[e] & ~3));
-      sm.cmsh[bu][w] = uint8_t(code[e] & 3);
+        if (field_used<OP>(f)) sm.f[bu][f][at] = v[f];
     }
     cp_async_commit();
   };
   int cur = 0;
-  bool pending = false;   // buffer cur holds a prefetch of brick b not yet waited for
   // irregular-table index and level of the current and the next brick: read one brick
   // ahead, so that no block waits for them
   auto desc = [&](int bn) -> int2 {
@@ -358,78 +471,45 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
     return make_int2(__ldg(&a.lay.bricks[bn].irr), __ldg(&a.lay.bricks[bn].level));
   };
   int2 dc = desc(blockIdx.x), dn = desc(blockIdx.x + G);
-  if (NBUF == 2 && int(blockIdx.x) < a.lay.nbricks && dc.x < 0) {
-    prefetch(blockIdx.x, 0);
-    pending = true;
+  // neighbour bases: of brick number i of this block in sm.nb[i % 3], two bricks ahead
+  auto base_of = [&](int bn) { return tid < 9 && bn < a.lay.nbricks ? __ldg(a.lay.bricks[bn].nbr_base + tid) : 0; };
+  if (tid < 9) {
+    sm.nb[0][tid] = base_of(blockIdx.x);
+    sm.nb[1][tid] = base_of(blockIdx.x + G);
   }
+  __syncthreads();
+  if (NBUF == 2 && int(blockIdx.x) < a.lay.nbricks) prefetch(sm.nb[0], dc.x, 0);
+  int turn = 0;
 #pragma unroll 1
   for (int b = blockIdx.x; b < a.lay.nbricks; b += G) {
-    const BrickDesc* bd = a.lay.bricks + b;
     const int irr = dc.x, level = dc.y;
-    P (*fb)[Q2WW] = sm.f[cur];
-    const int32_t* nbc = sm.nb[cur];
+    node.pl = &sm.f[cur][0][0];
+    const int32_t* nbc = sm.nb[turn];
     __syncthreads();   // the previous brick's tiles are no longer read
-    if (pending) {
-      // 1a. the prefetched window: constraint bytes, masked input components, a zero output tile
-      cp_async_wait<0>();
-      for (int w = tid; w < Q2WW; w += Q2T) {
-        const uint8_t cmw = uint8_t((sm.cmw[cur][w] >> (8 * sm.cmsh[cur][w])) & 0xffu);
-        sm.cm[w] = cmw;
-        if (mask && cmw) {
-          if (cmw & 1) q2_field<T>(fb, F_XU, w) = T(0);
-          if (cmw & 2) q2_field<T>(fb, F_XV, w) = T(0);
-          if (cmw & 4) q2_field<T>(fb, F_XP, w) = T(0);
+    if (NBUF == 1) prefetch(nbc, irr, 0);
+    // 1. the window: masked input components
+    cp_async_wait<0>();
+    const uint8_t* cmw = sm.cm[cur];
+    if (mask) {
+      __syncthreads();   // the constraint bytes come from other threads
+#pragma unroll
+      for (int e = 0; e < NWN; ++e) {
+        const int w = tid + Q2T * e;
+        if (w >= Q2WW) break;
+        const uint32_t cm = cm_at(cmw, w % Q2W, w / Q2W);
+        if (cm) {
+          const int at = q2_at(w % Q2W, w / Q2W);
+          if (cm & 1) sm.f[cur][F_XU][at] = T(0);
+          if (cm & 2) sm.f[cur][F_XV][at] = T(0);
+          if (cm & 4) sm.f[cur][F_XP][at] = T(0);
         }
-      }
-    } else {
-      if (tid < 9) sm.nb[cur][tid] = __ldg(bd->nbr_base + tid);
-      __syncthreads();
-      // 1b. window node fields (and a zero output tile)
-      for (int w = tid; w < Q2WW; w += Q2T) {
-        const int wx = w % Q2W, wy = w / Q2W;
-        const int32_t code = irr < 0 ? q2_slot(nbc, wx - 2, wy - 2) : __ldg(a.lay.win + int64_t(irr) * Q2WW + w);
-        T v[NF];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) v[f] = T(0);
-        uint8_t cmw = 0;
-        if (code >= 0) {
-          cmw = __ldg(a.cmask + code);
-#pragma unroll
-          for (int f = 0; f < NF; ++f)
-            if (field_used<OP>(f)) v[f] = ldg(field_ptr<T>(a, f) + code);
-          if (mask && cmw) {
-            if (cmw & 1) v[F_XU] = T(0);
-            if (cmw & 2) v[F_XV] = T(0);
-            if (cmw & 4) v[F_XP] = T(0);
-          }
-        } else if (code != kAbsent) {
-          const DevHanging& h = a.hang[-2 - code];
-#pragma unroll
-          for (int f = F_LU; f < NF; ++f)
-            if (field_used<OP>(f)) v[f] = ldg(field_ptr<T>(a, f) + h.slot);
-          for (int p = 0; p < 3; ++p) {
-            const int ps = h.parent[p];
-            const T wgt = T(h.weight[p]);
-            const uint8_t pc = mask ? __ldg(a.cmask + ps) : uint8_t(0);
-#pragma unroll
-            for (int f = F_XU; f <= F_XP; ++f)
-              if (field_used<OP>(f) && !(pc & (1 << f))) v[f] += wgt * ldg(field_ptr<T>(a, f) + ps);
-          }
-        }
-#pragma unroll
-        for (int f = 0; f < NF; ++f)
-          if (field_used<OP>(f)) q2_field<T>(fb, f, w) = v[f];
-        sm.cm[w] = cmw;
       }
     }
     __syncthreads();
     // the next brick's window streams in while this one computes
-    bool next_pending = false;
     const int2 dnn = desc(b + 2 * G);
-    if (NBUF == 2 && b + G < a.lay.nbricks && dn.x < 0) {
-      prefetch(b + G, cur ^ 1);
-      next_pending = true;
-    }
+    const int32_t nb2 = base_of(b + 2 * G);
+    if (NBUF == 2 && b + G < a.lay.nbricks) prefetch(sm.nb[(turn + 1) % 3], dn.x, cur ^ 1);
     // 2. one cell per thread
     bool act = true;
     if (irr >= 0) {
@@ -442,9 +522,10 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
     T rp[9], cell[3];
     if (act) {
       if constexpr (OP == OP_FULL || OP == OP_FULL_T || OP == OP_RESID)
-        q2_jac<T, OP>([&](int k, int i, int j) { return fb[k][cbase + i + Q2W * j]; }, mc, geom<T>(a, level), ec, ru, rp);
+        if (a.ecell == nullptr) q2_jac<T, OP, false>(node, q2mat<T>(a), Q2Own<T>(mc, geom<T>(a, level), T(1)), ru, rp);
+        else q2_jac<T, OP, true>(node, q2mat<T>(a), Q2Own<T>(mc, geom<T>(a, level), ec), ru, rp);
       else
-        q2_cell<T, OP>(fb, cbase, mc, geom<T>(a, level), tb, ec, ru, rp, cell);
+        q2_cell<T, OP>(node, mc, geom<T>(a, level), tb, ec, ru, rp, cell);
     }
     if constexpr (isVjp) {
       // the brick owns the cells whose lower-left node it owns (cells 0..14)
@@ -464,8 +545,8 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
       constexpr bool outP = OP != OP_UU && OP != OP_UU_DIAG;
 #pragma unroll
       for (int e = 0; e < 9; ++e) {
-        if (outU) { sm.con[3 * e][tid] = ru[e].x; sm.con[3 * e + 1][tid] = ru[e].y; }
-        if (outP) sm.con[3 * e + 2][tid] = rp[e];
+        if (outU) sm.conu[e][tid] = ru[e];
+        if (outP) sm.conp[e][tid] = rp[e];
       }
       __syncthreads();
       const int own_base = nbc[4];
@@ -481,29 +562,32 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
             // per direction the even cell (first) and the odd one: offset from own, local node
             const int cx0 = px || !ox ? 0 : -1, ax0 = px ? 1 : (ox ? 2 : 0), cx1 = ox ? 0 : -1, ax1 = ox ? 0 : 2;
             const int cy0 = py || !oy ? 0 : -Q2C, ay0 = py ? 1 : (oy ? 2 : 0), cy1 = oy ? 0 : -Q2C, ay1 = oy ? 0 : 2;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-              y[px][q] = T(0);
-              if (!(q < 2 ? outU : outP)) continue;
-              T v = sm.con[3 * (ax0 + 3 * ay0) + q][own + cx0 + cy0];
-              if (!px) v += sm.con[3 * (ax1 + 3 * ay0) + q][own + cx1 + cy0];
+            auto sum = [&](auto (*con)[Q2T]) {
+              auto v = con[ax0 + 3 * ay0][own + cx0 + cy0];
+              if (!px) v = padd(v, con[ax1 + 3 * ay0][own + cx1 + cy0]);
               if (!py) {
-                v += sm.con[3 * (ax0 + 3 * ay1) + q][own + cx0 + cy1];
-                if (!px) v += sm.con[3 * (ax1 + 3 * ay1) + q][own + cx1 + cy1];
+                v = padd(v, con[ax0 + 3 * ay1][own + cx0 + cy1]);
+                if (!px) v = padd(v, con[ax1 + 3 * ay1][own + cx1 + cy1]);
               }
-              y[px][q] = v;
-            }
+              return v;
+            };
+            const P yu = outU ? sum(sm.conu) : P{T(0), T(0)};
+            y[px][0] = yu.x;
+            y[px][1] = yu.y;
+            y[px][2] = outP ? sum(sm.conp) : T(0);
           }
           // 4. owned nodes (level block operators: or the fused Chebyshev store)
           const int oi = 2 * i, oj = 2 * j + py, o = oi + Q2NB * oj;
-          const int w = (oi + 2) + Q2W * (oj + 2);
-          const uint8_t cm0 = sm.cm[w], cm1 = sm.cm[w + 1];
+          const uint8_t cm0 = cmw[oi + Q2NB * (oj + 2)], cm1 = cmw[oi + 1 + Q2NB * (oj + 2)];
+          // storage actions and partial sums of irregular bricks
+          const uint32_t w0 = irr >= 0 ? uint32_t(sm.own[cur][o]) : uint32_t(kActFinal) << 30,
+                         w1 = irr >= 0 ? uint32_t(sm.own[cur][o + 1]) : uint32_t(kActFinal) << 30;
           bool done = false;
           if constexpr (OP == OP_UU || OP == OP_PP) {
             if (a.ch.mode != CHEB_OFF) {
 #pragma unroll
               for (int px = 0; px < 2; ++px) {
-                const int act_s = irr >= 0 ? int(__ldg(a.lay.own_act + irr * (Q2NB * Q2NB) + o + px)) : int(kActFinal);
+                const int act_s = int((px ? w1 : w0) >> 30);
                 ChebOps<T, OP> co;
                 cheb_load<T, OP>(a, own_base + o + px, co);
                 cheb_store<T, OP>(a, own_base + o + px, act_s, px ? cm1 : cm0, y[px][0], y[px][1], y[px][2], co);
@@ -525,16 +609,18 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
               if (outP) { yp[0] = y[0][2]; yp[1] = y[1][2]; }
             }
           } else if (!done) {
-            write_node<T, OP>(a, irr, own_base, oi, oj, cm0, y[0][0], y[0][1], y[0][2]);
-            write_node<T, OP>(a, irr, own_base, oi + 1, oj, cm1, y[1][0], y[1][1], y[1][2]);
+            store_owned<T, OP>(a, own_base + o, int(w0 >> 30), int(w0 & 0x3fffffffu) - 1, cm0, y[0][0], y[0][1], y[0][2]);
+            store_owned<T, OP>(a, own_base + o + 1, int(w1 >> 30), int(w1 & 0x3fffffffu) - 1, cm1, y[1][0], y[1][1],
+                               y[1][2]);
           }
         }
       }
     }
     dc = dn;
     dn = dnn;
+    if (tid < 9) sm.nb[(turn + 2) % 3][tid] = nb2;
+    turn = (turn + 1) % 3;
     if (NBUF == 2) cur ^= 1;
-    pending = next_pending;
   }
   cp_async_wait<0>();
 }

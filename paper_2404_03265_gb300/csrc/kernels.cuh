@@ -102,6 +102,16 @@ struct Q2Tab {
   T w[3];
 };
 
+// Q2 Jacobian and residual on reference derivatives (q2_jac.cuh): elastic constants times
+// the cell's aspect ratio, which is that of the coarse cells on every level, and weighted
+// coefficients by class of Gauss point (0 corner, 1 edge, 2 centre).
+template <typename T>
+struct Q2Mat {
+  T al, alt, be, ga, gat, de;            // c2ml hy/hx, c2ml hx/hy, cl, cm hx/hy, cm hy/hx, cm
+  T oal, oalt, obe, oga, ogat, ode;      // the same times 1 - kappa
+  T omkw[3], kapw[3], gxxw[3], gyyw[3];  // weight times 1 - kappa, kappa, G_c l hy/hx, G_c l hx/hy
+};
+
 // Chebyshev step fused into the store of a level apply (OP_UU, OP_PP): instead
 // of y = A x the sweep writes, per level entry i (component blocks of n_slots):
 //   CHEB_STEP       out[i]  = x + a (x - prev) + b dinv (rhs - A x)
@@ -148,10 +158,13 @@ struct ApplyArgs {
   LevGeom<double> gd[kMaxLevels];
   Q2Tab<float> q2f;
   Q2Tab<double> q2d;
+  Q2Mat<float> q2mf;
+  Q2Mat<double> q2md;
   int mode;
   int fe_degree;
   int sweep_sh;           // Q1 strip half-height: 0 = by mesh size, else 15, 5 or 1 (schedules of DevLayout::units)
   int pair_store;         // Q2: the output vectors allow stores of two neighbouring slots (set by launch_apply)
+  int wide;               // Q2: the input vectors allow 16-byte copies of whole bricks (set by launch_apply)
   int pdl_in;             // Q1: launched dependent on the preceding kernel, which wrote x (pdl.cuh)
   ChebEpi ch;             // level applies: fused Chebyshev store (mode CHEB_OFF: plain y = A x)
 };

@@ -36,6 +36,7 @@ struct CellArgs {
   int64_t n;   // slots
   int mode;
   MatConst<double> m;
+  Q2Mat<double> k;
   LevGeom<double> g[kMaxLevels];
 };
 struct NodeArgs {
@@ -59,8 +60,11 @@ struct NodeArgs {
 // A block takes 32 cells: warp w evaluates their Gauss row w, so a cell's work is spread
 // over three warps (a third of the serial chain of a thread per cell, and units fine
 // enough to balance over the SMs); the rows' contributions meet in shared memory.
-template <int OP>
-__global__ void __launch_bounds__(96) q2_cell_kernel(const __grid_constant__ CellArgs a) {
+// Measured on the 267k-DoF band mesh (22k cells), operator apply: brick kernel 141 us, one
+// thread per cell 97 us, this split 72 us (85 us when the compiler aims at 80 registers
+// and more resident blocks: the FP64 pipe wants independent instructions, not warps).
+template <int OP, bool MOD>
+__global__ void __launch_bounds__(96, 5) q2_cell_kernel(const __grid_constant__ CellArgs a) {
   constexpr bool X = OP != OP_RESID;   // the operator reads an input
   __shared__ double xs[X ? 27 : 1][32];
   __shared__ double red[3][27][32];
@@ -105,7 +109,7 @@ __global__ void __launch_bounds__(96) q2_cell_kernel(const __grid_constant__ Cel
       slot[e] = h.slot;   // the resolved linearisation
     }
   }
-  const double ec = a.ecell != nullptr ? a.ecell[cs] : 1.0;
+  const double ec = MOD ? a.ecell[cs] : 1.0;
   if (X) __syncthreads();
   auto ld = [&](int k, int i, int j) -> double2 {
     const int e = i + 3 * j;
@@ -116,7 +120,7 @@ __global__ void __launch_bounds__(96) q2_cell_kernel(const __grid_constant__ Cel
     return make_double2(a.lin[3 * a.n + s], 0.0);
   };
   {
-    const Q2Const<double> k(a.m, a.g[lev], ec);
+    const Q2Own<double> own(a.m, a.g[lev], ec);
     double2 ru[9];
     double rp[9];
 #pragma unroll
@@ -124,9 +128,9 @@ __global__ void __launch_bounds__(96) q2_cell_kernel(const __grid_constant__ Cel
       ru[e] = make_double2(0.0, 0.0);
       rp[e] = 0.0;
     }
-    if (row == 0) q2_jac_row<double, OP, 0>(ld, k, ru, rp);
-    else if (row == 1) q2_jac_row<double, OP, 1>(ld, k, ru, rp);
-    else q2_jac_row<double, OP, 2>(ld, k, ru, rp);
+    if (row == 0) q2_jac_row<double, OP, MOD>(RowAt<double, 0>(), ld, a.k, own, ru, rp);
+    else if (row == 1) q2_jac_row<double, OP, MOD>(RowAt<double, 1>(), ld, a.k, own, ru, rp);
+    else q2_jac_row<double, OP, MOD>(RowAt<double, 2>(), ld, a.k, own, ru, rp);
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
       red[row][3 * e + 0][lane] = ru[e].x;
@@ -209,6 +213,7 @@ cudaError_t launch_op(const ApplyArgs& a, const FixupArgs& f, cudaStream_t s) {
   c.n = a.n_slots;
   c.mode = a.mode;
   c.m = a.md;
+  c.k = a.q2md;
   for (int l = 0; l < kMaxLevels; ++l) c.g[l] = a.gd[l];
   c.out = static_cast<double*>(a.lc.out);
   NodeArgs n;
@@ -227,7 +232,7 @@ cudaError_t launch_op(const ApplyArgs& a, const FixupArgs& f, cudaStream_t s) {
   // it reads or writes a vector); under a capture that may not be a kernel
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   const bool pdl = cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
-  const cudaError_t e = launch_ex(pdl, &q2_cell_kernel<OP>, unsigned((a.lc.ncells + 31) / 32), 96u, 0, s, c);
+  const cudaError_t e = launch_ex(pdl, a.ecell ? &q2_cell_kernel<OP, true> : &q2_cell_kernel<OP, false>, unsigned((a.lc.ncells + 31) / 32), 96u, 0, s, c);
   if (e != cudaSuccess) return e;
   return launch_ex(true, &q2_node_kernel, unsigned((a.n_slots + NODE_TPB - 1) / NODE_TPB), unsigned(NODE_TPB), 0, s, n);
 }

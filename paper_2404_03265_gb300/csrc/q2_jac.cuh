@@ -55,70 +55,108 @@ __device__ __forceinline__ void q2_test_deriv(const P f[3], P r[3]) {
   r[1] = pmul(bc<P>(T(-2)), h);
   r[2] = padd(h, t);
 }
-// value and derivative along eta of a column (v0, v1, v2) on Gauss row Q
-template <int Q, typename P>
-__device__ __forceinline__ void q2_row(P v0, P v1, P v2, P& V, P& E) {
-  using T = typename Elem<P>::T;
-  if constexpr (Q == 1) {
-    V = v1;
-    E = psub(v2, v0);
-  } else {
-    P d, c;
-    q2_even_odd(v0, v1, v2, d, c);
-    V = pfma(bc<P>(T((Q - 1) * kQ2S)), d, pfma(bc<P>(T(0.3)), c, v1));
-    E = pfma(bc<P>(T(4.0 * (Q - 1) * kQ2S)), c, d);
-  }
-}
-template <int Q, typename P>
-__device__ __forceinline__ P q2_row_value(P v0, P v1, P v2) {
-  using T = typename Elem<P>::T;
-  if constexpr (Q == 1) return v1;
-  constexpr double t = (Q - 1) * kQ2S;
-  return pfma(bc<P>(T(2 * t * t + t)), v2, pfma(bc<P>(T(1 - 4 * t * t)), v1, pmul(bc<P>(T(2 * t * t - t)), v0)));
-}
-// r[a + 3 b] += l_b(row) V[a] + l_b'(row) E[a]
-template <int Q, typename P>
-__device__ __forceinline__ void q2_scatter(const P V[3], const P E[3], P r[9]) {
-  using T = typename Elem<P>::T;
-  constexpr double t = (Q - 1) * kQ2S;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
+// A Gauss row eta = t.  RowAt<T, Q>: known when compiled (the middle row costs next to
+// nothing); RowVar: at run time, so that a loop over the rows keeps only one of them in
+// registers.
+template <typename T, int Q>
+struct RowAt {
+  static constexpr double t = (Q - 1) * kQ2S;
+  // value and derivative along eta of a column (v0, v1, v2)
+  template <typename P>
+  __device__ __forceinline__ void column(P v0, P v1, P v2, P& V, P& E) const {
     if constexpr (Q == 1) {
-      r[a] = psub(r[a], E[a]);
-      r[a + 3] = padd(r[a + 3], V[a]);
-      r[a + 6] = padd(r[a + 6], E[a]);
+      V = v1;
+      E = psub(v2, v0);
     } else {
-      r[a] = pfma(bc<P>(T(2 * t * t - t)), V[a], pfma(bc<P>(T(4 * t - 1)), E[a], r[a]));
-      r[a + 3] = pfma(bc<P>(T(1 - 4 * t * t)), V[a], pfma(bc<P>(T(-8 * t)), E[a], r[a + 3]));
-      r[a + 6] = pfma(bc<P>(T(2 * t * t + t)), V[a], pfma(bc<P>(T(4 * t + 1)), E[a], r[a + 6]));
+      P d, c;
+      q2_even_odd(v0, v1, v2, d, c);
+      V = pfma(bc<P>(T(t)), d, pfma(bc<P>(T(0.3)), c, v1));
+      E = pfma(bc<P>(T(4.0 * t)), c, d);
     }
   }
-}
+  template <typename P>
+  __device__ __forceinline__ P value(P v0, P v1, P v2) const {
+    if constexpr (Q == 1) return v1;
+    else return pfma(bc<P>(T(2 * t * t + t)), v2, pfma(bc<P>(T(1 - 4 * t * t)), v1, pmul(bc<P>(T(2 * t * t - t)), v0)));
+  }
+  // r[a + 3 b] += l_b(t) V[a] + l_b'(t) E[a]
+  template <typename P>
+  __device__ __forceinline__ void scatter(const P V[3], const P E[3], P r[9]) const {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      if constexpr (Q == 1) {
+        r[a] = psub(r[a], E[a]);
+        r[a + 3] = padd(r[a + 3], V[a]);
+        r[a + 6] = padd(r[a + 6], E[a]);
+      } else {
+        r[a] = pfma(bc<P>(T(2 * t * t - t)), V[a], pfma(bc<P>(T(4 * t - 1)), E[a], r[a]));
+        r[a + 3] = pfma(bc<P>(T(1 - 4 * t * t)), V[a], pfma(bc<P>(T(-8 * t)), E[a], r[a + 3]));
+        r[a + 6] = pfma(bc<P>(T(2 * t * t + t)), V[a], pfma(bc<P>(T(4 * t + 1)), E[a], r[a + 6]));
+      }
+    }
+  }
+  __device__ __forceinline__ int weight_class(int i) const { return (i == 1) + (Q == 1); }
+  __device__ __forceinline__ T weight(int i) const {
+    constexpr double w1[3] = {5.0 / 18.0, 8.0 / 18.0, 5.0 / 18.0};
+    return T(w1[i] * w1[Q]);
+  }
+};
 
-// Per-cell constants: elastic ones times the reference-to-physical factors and the cell's area
 template <typename T>
-struct Q2Const {
-  T al, alt, be, ga, gat, de;          // c2ml hy/hx, c2ml hx/hy, cl, cm hx/hy, cm hy/hx, cm
-  T oal, oalt, obe, oga, ogat, ode;    // the same times 1 - kappa
-  T px, py, gcl, gxx, gyy, omk, kap;
-  __device__ __forceinline__ Q2Const(const MatConst<T>& m, const LevGeom<T>& g, T ec) {
-    const T area = T(4) * g.jxw, kx = g.ihx * g.ihx * area, ky = g.ihy * g.ihy * area, kxy = g.ihx * g.ihy * area;
-    const T c2 = m.c2ml * ec, l = m.cl * ec, mu = m.cm * ec;
-    al = c2 * kx; alt = c2 * ky; be = l * kxy; ga = mu * ky; gat = mu * kx; de = mu * kxy;
-    oal = m.omk * al; oalt = m.omk * alt; obe = m.omk * be; oga = m.omk * ga; ogat = m.omk * gat; ode = m.omk * de;
-    px = m.p * g.ihx * area; py = m.p * g.ihy * area;
-    gcl = m.gcl * area; gxx = m.gcL * kx; gyy = m.gcL * ky;
-    omk = m.omk; kap = m.kap;
+struct RowVar {
+  T t;
+  bool mid;
+  __device__ __forceinline__ explicit RowVar(int q) : t(T(kQ2S) * T(q - 1)), mid(q == 1) {}
+  template <typename P>
+  __device__ __forceinline__ void column(P v0, P v1, P v2, P& V, P& E) const {
+    P d, c;
+    q2_even_odd(v0, v1, v2, d, c);
+    V = pfma(bc<P>(t), d, pfma(bc<P>(mid ? T(0) : T(0.3)), c, v1));
+    E = pfma(bc<P>(T(4) * t), c, d);
+  }
+  template <typename P>
+  __device__ __forceinline__ P value(P v0, P v1, P v2) const {
+    const T h = mid ? T(0) : T(0.3);
+    return pfma(bc<P>(h + t), v2, pfma(bc<P>(T(1) - T(2) * h), v1, pmul(bc<P>(h - t), v0)));
+  }
+  template <typename P>
+  __device__ __forceinline__ void scatter(const P V[3], const P E[3], P r[9]) const {
+    const T h = mid ? T(0) : T(0.3);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      r[a] = pfma(bc<P>(h - t), V[a], pfma(bc<P>(T(4) * t - T(1)), E[a], r[a]));
+      r[a + 3] = pfma(bc<P>(T(1) - T(2) * h), V[a], pfma(bc<P>(T(-8) * t), E[a], r[a + 3]));
+      r[a + 6] = pfma(bc<P>(h + t), V[a], pfma(bc<P>(T(4) * t + T(1)), E[a], r[a + 6]));
+    }
+  }
+  __device__ __forceinline__ int weight_class(int i) const { return (i == 1) + (mid ? 1 : 0); }
+  __device__ __forceinline__ T weight(int i) const {
+    return (i == 1 ? T(8.0 / 18.0) : T(5.0 / 18.0)) * (mid ? T(8.0 / 18.0) : T(5.0 / 18.0));
+  }
+};
+
+// The cell's own constants beside Q2Mat (kernels.cuh): p hy, p hx, G_c/l times the area, modulus
+template <typename T>
+struct Q2Own {
+  T px, py, gcl, ec;
+  __device__ __forceinline__ Q2Own(const MatConst<T>& m, const LevGeom<T>& g, T e) {
+    const T area = T(4) * g.jxw;   // hx hy
+    px = m.p * (g.ihx * area);
+    py = m.p * (g.ihy * area);
+    gcl = m.gcl * area;
+    ec = e;
   }
 };
 
 // One Gauss row: ld(k, a, b) is field pair k at the cell's node (a, b): 0 the input
 // (u_x, u_y), 1 the linearisation's (u_x, u_y), 2 (input dphi, phi), 3 (phi_tilde, -).
-template <typename T, int OP, int Q, class Load>
-__device__ __forceinline__ void q2_jac_row(const Load& ld, const Q2Const<T>& k, typename VT<T>::T2 ru[9], T rp[9]) {
+// MOD: the cell has a modulus of its own (o.ec; the constants are those of unit E).
+template <typename T, int OP, bool MOD, class Row, class Load>
+__device__ __forceinline__ void q2_jac_row(const Row& row, const Load& ld, const Q2Mat<T>& k, const Q2Own<T>& o,
+                                           typename VT<T>::T2 ru[9], T rp[9]) {
   using P = typename VT<T>::T2;
   constexpr bool RES = OP == OP_RESID;
-  constexpr double sgn = RES ? -1.0 : 1.0;   // R = -A
+  // (the residual is R = -A)
   // ---- fields at the row's three points: reference derivatives and values
   P xdx[3], xdy[3], ldx[3], ldy[3], val[3];   // (u_x, u_y) of input and linearisation; (dphi, phi)
   T pdx[3], pdy[3], pt[3];                    // gradient of dphi (residual: of phi), phi_tilde
@@ -126,14 +164,14 @@ __device__ __forceinline__ void q2_jac_row(const Load& ld, const Q2Const<T>& k, 
     P V[3], E[3], d, c;
     if constexpr (!RES) {
 #pragma unroll
-      for (int a = 0; a < 3; ++a) q2_row<Q>(ld(0, a, 0), ld(0, a, 1), ld(0, a, 2), V[a], E[a]);
+      for (int a = 0; a < 3; ++a) row.column(ld(0, a, 0), ld(0, a, 1), ld(0, a, 2), V[a], E[a]);
       q2_even_odd(V[0], V[1], V[2], d, c);
       q2_derivs(d, c, xdx);
       q2_even_odd(E[0], E[1], E[2], d, c);
       q2_values(E[1], d, c, xdy);
     }
 #pragma unroll
-    for (int a = 0; a < 3; ++a) q2_row<Q>(ld(1, a, 0), ld(1, a, 1), ld(1, a, 2), V[a], E[a]);
+    for (int a = 0; a < 3; ++a) row.column(ld(1, a, 0), ld(1, a, 1), ld(1, a, 2), V[a], E[a]);
     q2_even_odd(V[0], V[1], V[2], d, c);
     q2_derivs(d, c, ldx);
     q2_even_odd(E[0], E[1], E[2], d, c);
@@ -141,7 +179,7 @@ __device__ __forceinline__ void q2_jac_row(const Load& ld, const Q2Const<T>& k, 
     T Es[3], Vs[3], ds, cs;
     if constexpr (RES) {
 #pragma unroll
-      for (int a = 0; a < 3; ++a) q2_row<Q>(ld(2, a, 0).y, ld(2, a, 1).y, ld(2, a, 2).y, Vs[a], Es[a]);
+      for (int a = 0; a < 3; ++a) row.column(ld(2, a, 0).y, ld(2, a, 1).y, ld(2, a, 2).y, Vs[a], Es[a]);
       T v[3];
       q2_even_odd(Vs[0], Vs[1], Vs[2], ds, cs);
       q2_values(Vs[1], ds, cs, v);
@@ -152,9 +190,9 @@ __device__ __forceinline__ void q2_jac_row(const Load& ld, const Q2Const<T>& k, 
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         const P v0 = ld(2, a, 0), v1 = ld(2, a, 1), v2 = ld(2, a, 2);
-        V[a] = q2_row_value<Q>(v0, v1, v2);
+        V[a] = row.value(v0, v1, v2);
         T unused;
-        q2_row<Q>(v0.x, v1.x, v2.x, unused, Es[a]);
+        row.column(v0.x, v1.x, v2.x, unused, Es[a]);
       }
       q2_even_odd(V[0], V[1], V[2], d, c);
       q2_values(V[1], d, c, val);
@@ -163,7 +201,7 @@ __device__ __forceinline__ void q2_jac_row(const Load& ld, const Q2Const<T>& k, 
     q2_even_odd(Es[0], Es[1], Es[2], ds, cs);
     q2_values(Es[1], ds, cs, pdy);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) Vs[a] = q2_row_value<Q>(ld(3, a, 0).x, ld(3, a, 1).x, ld(3, a, 2).x);
+    for (int a = 0; a < 3; ++a) Vs[a] = row.value(ld(3, a, 0).x, ld(3, a, 1).x, ld(3, a, 2).x);
     q2_even_odd(Vs[0], Vs[1], Vs[2], ds, cs);
     q2_values(Vs[1], ds, cs, pt);
   }
@@ -172,27 +210,37 @@ __device__ __forceinline__ void q2_jac_row(const Load& ld, const Q2Const<T>& k, 
   T f0[3], gx[3], gy[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    constexpr double w1[3] = {5.0 / 18.0, 8.0 / 18.0, 5.0 / 18.0};
-    const T W = T(sgn * w1[i] * w1[Q]);
+    const T W = RES ? -row.weight(i) : row.weight(i);
     const T a = ldx[i].x, b = ldy[i].x, c = ldx[i].y, d = ldy[i].y;   // u_x,xi u_x,eta u_y,xi u_y,eta
-    const T g = pfma(pmul(W, k.omk), pmul(pt[i], pt[i]), pmul(W, k.kap));
-    const T q11 = RES ? pfma(k.oal, a, pmul(k.obe, d)) : pfma(k.oal, a, pfma(k.obe, d, k.px));
-    const T q22 = RES ? pfma(k.obe, a, pmul(k.oalt, d)) : pfma(k.obe, a, pfma(k.oalt, d, k.py));
-    const T t1 = pfma(k.oga, b, pmul(k.ode, c)), t2 = pfma(k.ode, b, pmul(k.ogat, c));
+    const int wi = row.weight_class(i);   // corner, edge, centre
+    T g = pfma(k.omkw[wi], pmul(pt[i], pt[i]), k.kapw[wi]);   // signed weight times g(phi~)
+    if (RES) g = -g;
+    T q11 = pfma(k.oal, a, pmul(k.obe, d)), q22 = pfma(k.obe, a, pmul(k.oalt, d));
+    T t1 = pfma(k.oga, b, pmul(k.ode, c)), t2 = pfma(k.ode, b, pmul(k.ogat, c));
+    if constexpr (MOD) {
+      g = pmul(g, o.ec);
+      t1 = pmul(t1, o.ec);
+      t2 = pmul(t2, o.ec);
+      q11 = RES ? pmul(q11, o.ec) : pfma(o.ec, q11, o.px);
+      q22 = RES ? pmul(q22, o.ec) : pfma(o.ec, q22, o.py);
+    } else if constexpr (!RES) {
+      q11 = padd(q11, o.px);
+      q22 = padd(q22, o.py);
+    }
     // (1 - kappa) sigma(u):e(u), in the Jacobian with p div u once
     const T se = pfma(q11, a, pfma(q22, d, pfma(t1, b, pmul(t2, c))));
     const T ph = val[i].y;
     if constexpr (RES) {
       const T pp = pmul(W, pmul(pt[i], pt[i]));
-      Fx[i].x = pfma(g, pfma(k.al, a, pmul(k.be, d)), pmul(k.px, pp));
+      Fx[i].x = pfma(g, pfma(k.al, a, pmul(k.be, d)), pmul(o.px, pp));
       Fy[i].x = pmul(g, pfma(k.ga, b, pmul(k.de, c)));
       Fx[i].y = pmul(g, pfma(k.de, b, pmul(k.gat, c)));
-      Fy[i].y = pfma(g, pfma(k.be, a, pmul(k.alt, d)), pmul(k.py, pp));
-      const T dv = pfma(k.px, a, pmul(k.py, d));
-      f0[i] = pmul(W, pfma(ph, pfma(T(2), dv, se), pmul(k.gcl, psub(ph, T(1)))));
+      Fy[i].y = pfma(g, pfma(k.be, a, pmul(k.alt, d)), pmul(o.py, pp));
+      const T dv = pfma(o.px, a, pmul(o.py, d));
+      f0[i] = pmul(W, pfma(ph, pfma(T(2), dv, se), pmul(o.gcl, psub(ph, T(1)))));
     } else {
       const T A = xdx[i].x, B = xdy[i].x, C = xdx[i].y, D = xdy[i].y, xp = val[i].x;
-      const T m = pfma(k.px, a, pfma(k.py, d, padd(se, k.gcl)));
+      const T m = pfma(o.px, a, pfma(o.py, d, padd(se, o.gcl)));
       Fx[i].x = pmul(g, pfma(k.al, A, pmul(k.be, D)));
       Fy[i].x = pmul(g, pfma(k.ga, B, pmul(k.de, C)));
       Fx[i].y = pmul(g, pfma(k.de, B, pmul(k.gat, C)));
@@ -209,15 +257,15 @@ __device__ __forceinline__ void q2_jac_row(const Load& ld, const Q2Const<T>& k, 
         f0[i] = pmul(W, pmul(m, xp));
       }
     }
-    gx[i] = pmul(pmul(W, k.gxx), pdx[i]);
-    gy[i] = pmul(pmul(W, k.gyy), pdy[i]);
+    gx[i] = pmul(RES ? -k.gxxw[wi] : k.gxxw[wi], pdx[i]);
+    gy[i] = pmul(RES ? -k.gyyw[wi] : k.gyyw[wi], pdy[i]);
   }
   // ---- tests
   {
     P V[3], E[3];
     q2_test_deriv(Fx, V);
     q2_test_value(Fy, E);
-    q2_scatter<Q>(V, E, ru);
+    row.scatter(V, E, ru);
   }
   {
     T V[3], E[3], V0[3];
@@ -226,25 +274,23 @@ __device__ __forceinline__ void q2_jac_row(const Load& ld, const Q2Const<T>& k, 
 #pragma unroll
     for (int a = 0; a < 3; ++a) V[a] = padd(V[a], V0[a]);
     q2_test_value(gy, E);
-    q2_scatter<Q>(V, E, rp);
+    row.scatter(V, E, rp);
   }
 }
 
 // Contributions of one cell to its node a + 3 b: ru (u_x, u_y), rp (phi).  OP: OP_FULL,
-// OP_FULL_T or OP_RESID.  ec: the cell's modulus (m then holds unit-E constants), or 1.
-template <typename T, int OP, class Load>
-__device__ __forceinline__ void q2_jac(const Load& ld, const MatConst<T>& m, const LevGeom<T>& g, T ec,
+// OP_FULL_T or OP_RESID.
+template <typename T, int OP, bool MOD, class Load>
+__device__ __forceinline__ void q2_jac(const Load& ld, const Q2Mat<T>& k, const Q2Own<T>& o,
                                        typename VT<T>::T2 ru[9], T rp[9]) {
   using P = typename VT<T>::T2;
-  const Q2Const<T> k(m, g, ec);
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     ru[i] = P{T(0), T(0)};
     rp[i] = T(0);
   }
-  q2_jac_row<T, OP, 0>(ld, k, ru, rp);
-  q2_jac_row<T, OP, 1>(ld, k, ru, rp);
-  q2_jac_row<T, OP, 2>(ld, k, ru, rp);
+#pragma unroll 1
+  for (int q = 0; q < 3; ++q) q2_jac_row<T, OP, MOD>(RowVar<T>(q), ld, k, o, ru, rp);
 }
 
 }  // namespace pff
