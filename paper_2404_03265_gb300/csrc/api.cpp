@@ -241,7 +241,8 @@ extern "C" void pff_problem_destroy(pff_problem* pb) {
   if (!pb) return;
   for (auto& e : pb->gm_ev)
     if (e) cudaEventDestroy(e);
-  pb->ws.mem.release();
+  if (pb->gm_read) cudaEventDestroy(pb->gm_read);
+  release_workspace(pb->ws);
   pb->bufs.release();
   delete pb;
 }

@@ -7,6 +7,7 @@
 #include <cstdint>
 
 #include "kernels.cuh"
+#include "pdl.cuh"
 #include "solve.cuh"
 
 namespace pff {
@@ -187,18 +188,26 @@ __device__ __forceinline__ int64_t basis_row(int64_t i, int64_t ldb) {
   return (i / kBasisBlock) * ldb + (i % kBasisBlock);
 }
 
-// partial[b * k + j] = sum over this block's rows of V_j . w.  The basis vectors
-// go in chunks of MD_J (the last one of k mod MD_J, its own instantiation, so no
-// multiply is spent on padding); a thread visits its rows i = t, t + S, t + 2 S,
-// ... (S = the grid's thread count) in that order, as a plain grid-stride dot
-// does, but issues the loads of MD_R consecutive visits (w and the chunk's basis
-// entries each) together.  It keeps one sum per vector of the chunk, and the
-// block reduces them in one shared-memory tree (fixed order).
+// One Gram-Schmidt stage of an Arnoldi step in one launch (the stages were eight: each is
+// an FP64-bound pass over the basis, and on small meshes a launch and its gap cost more
+// than the pass).  Rows are visited as a plain grid-stride dot does: i = t, t + S, t + 2 S,
+// ... (S = the grid's thread count), the loads of MD_R visits issued together.
+//   GS_GATHER  w[i] = z[map[i]]
+//   GS_AXPY    w[i] -= sum_j h[j] V_j[i] (the sum in the order j = 0, 1, ...)
+// then out[j] = V_j . w, j < k, or with NORM out[0] = w . w.  A block's partial sums of a
+// vector come from one shared-memory tree over its threads; the last block to finish adds
+// the blocks' partials in a fixed order, so the sums do not depend on which block that is.
+// The basis vectors go in chunks of MD_J (the last one in its own instantiation, so no
+// multiply is spent on padding).
 constexpr int MD_J = 8;
 constexpr int MD_R = 4;
+constexpr int MAX_BASIS = 512;
+enum GsStage : int { GS_GATHER = 0, GS_AXPY = 1 };
+
+// w is written by the same thread earlier in the kernel: plain loads
 template <int JN>
-__device__ __forceinline__ void md_chunk(int64_t n, const double* __restrict__ Vc, int64_t ldb,
-                                         const double* __restrict__ w, double (&sh)[MD_J][TPB]) {
+__device__ __forceinline__ void md_chunk(int64_t n, const double* __restrict__ Vc, int64_t ldb, const double* w,
+                                         double (&sh)[MD_J][TPB]) {
   const int64_t S = int64_t(gridDim.x) * TPB;
   double acc[JN];
 #pragma unroll
@@ -225,52 +234,128 @@ __device__ __forceinline__ void md_chunk(int64_t n, const double* __restrict__ V
   for (int q = 0; q < JN; ++q) sh[q][threadIdx.x] = acc[q];
 }
 
-__global__ void k_multidot_partial(int64_t n, int k, const double* __restrict__ V, int64_t ldb,
-                                   const double* __restrict__ w, double* partial) {
+template <int STAGE, bool NORM>
+__global__ void __launch_bounds__(TPB) k_gram_schmidt(int64_t n, int k, const double* __restrict__ V, int64_t ldb,
+                                                      const double* __restrict__ z, const int32_t* __restrict__ map,
+                                                      const double* __restrict__ h, double* w, double* partial,
+                                                      unsigned* count, double* out) {
   __shared__ double sh[MD_J][TPB];
-  for (int j0 = 0; j0 < k; j0 += MD_J) {
-    const int jn = k - j0 < MD_J ? k - j0 : MD_J;
-    const double* Vc = V + int64_t(j0) * kBasisBlock;
-    switch (jn) {
-      case 1: md_chunk<1>(n, Vc, ldb, w, sh); break;
-      case 2: md_chunk<2>(n, Vc, ldb, w, sh); break;
-      case 3: md_chunk<3>(n, Vc, ldb, w, sh); break;
-      case 4: md_chunk<4>(n, Vc, ldb, w, sh); break;
-      case 5: md_chunk<5>(n, Vc, ldb, w, sh); break;
-      case 6: md_chunk<6>(n, Vc, ldb, w, sh); break;
-      case 7: md_chunk<7>(n, Vc, ldb, w, sh); break;
-      default: md_chunk<8>(n, Vc, ldb, w, sh); break;
+  __shared__ double hs[STAGE == GS_AXPY ? MAX_BASIS : 1];
+  __shared__ bool last;
+  pdl_wait();
+  pdl_trigger();
+  const int tid = threadIdx.x;
+  const int64_t S = int64_t(gridDim.x) * TPB;
+  double nrm = 0.0;
+  if (STAGE == GS_AXPY) {
+    for (int j = tid; j < k; j += TPB) hs[j] = h[j];
+    __syncthreads();
+  }
+  for (int64_t i0 = int64_t(blockIdx.x) * TPB + tid; i0 < n; i0 += MD_R * S) {
+    double v[MD_R];
+    if (STAGE == GS_GATHER) {
+      int32_t at[MD_R];
+#pragma unroll
+      for (int e = 0; e < MD_R; ++e) at[e] = i0 + e * S < n ? map[i0 + e * S] : 0;
+#pragma unroll
+      for (int e = 0; e < MD_R; ++e) v[e] = z[at[e]];
+    } else {
+      double acc[MD_R];
+      int64_t bi[MD_R];
+#pragma unroll
+      for (int e = 0; e < MD_R; ++e) {
+        const int64_t i = i0 + e * S < n ? i0 + e * S : i0;
+        acc[e] = 0.0;
+        v[e] = w[i];
+        bi[e] = basis_row(i, ldb);
+      }
+      int j = 0;
+      for (; j + 4 <= k; j += 4) {
+        double x[4][MD_R];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int e = 0; e < MD_R; ++e) x[q][e] = V[bi[e] + (j + q) * kBasisBlock];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int e = 0; e < MD_R; ++e) acc[e] += hs[j + q] * x[q][e];
+      }
+      for (; j < k; ++j)
+#pragma unroll
+        for (int e = 0; e < MD_R; ++e) acc[e] += hs[j] * V[bi[e] + j * kBasisBlock];
+#pragma unroll
+      for (int e = 0; e < MD_R; ++e) v[e] -= acc[e];
+    }
+#pragma unroll
+    for (int e = 0; e < MD_R; ++e)
+      if (i0 + e * S < n) {
+        w[i0 + e * S] = v[e];
+        if (NORM) nrm += v[e] * v[e];
+      }
+  }
+  // block partials: partial[j * gridDim.x + block]
+  const int nj = NORM ? 1 : k;
+  for (int j0 = 0; j0 < nj; j0 += MD_J) {
+    const int jn = nj - j0 < MD_J ? nj - j0 : MD_J;
+    if (NORM) {
+      sh[0][tid] = nrm;
+    } else {
+      const double* Vc = V + int64_t(j0) * kBasisBlock;
+      switch (jn) {
+        case 1: md_chunk<1>(n, Vc, ldb, w, sh); break;
+        case 2: md_chunk<2>(n, Vc, ldb, w, sh); break;
+        case 3: md_chunk<3>(n, Vc, ldb, w, sh); break;
+        case 4: md_chunk<4>(n, Vc, ldb, w, sh); break;
+        case 5: md_chunk<5>(n, Vc, ldb, w, sh); break;
+        case 6: md_chunk<6>(n, Vc, ldb, w, sh); break;
+        case 7: md_chunk<7>(n, Vc, ldb, w, sh); break;
+        default: md_chunk<8>(n, Vc, ldb, w, sh); break;
+      }
     }
     __syncthreads();
     for (int o = TPB / 2; o > 0; o >>= 1) {
-      if (threadIdx.x < o) {
-        for (int q = 0; q < jn; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + o];
+      if (tid < o) {
+        for (int q = 0; q < jn; ++q) sh[q][tid] += sh[q][tid + o];
       }
       __syncthreads();
     }
-    if (threadIdx.x < jn) partial[int64_t(blockIdx.x) * k + j0 + threadIdx.x] = sh[threadIdx.x][0];
+    if (tid < jn) partial[int64_t(j0 + tid) * gridDim.x + blockIdx.x] = sh[tid][0];
     __syncthreads();
+  }
+  // the last block adds the blocks' partials: a warp per vector, fixed order
+  __threadfence();
+  if (tid == 0) last = atomicAdd(count, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (tid == 0) *count = 0u;   // for the next launch
+  const int lane = tid & 31;
+  for (int j = tid >> 5; j < nj; j += TPB / 32) {
+    double acc = 0.0;
+    for (unsigned b = lane; b < gridDim.x; b += 32) acc += __ldcg(partial + int64_t(j) * gridDim.x + b);
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if (lane == 0) out[j] = acc;
   }
 }
 
-__global__ void k_multidot_final(int nb, int k, const double* __restrict__ partial, double* out) {
+// partial[b] of one vector, added by k_vector_final (plain sums)
+__global__ void k_vector_final(int nb, const double* __restrict__ partial, double* out) {
   __shared__ double sh[TPB];
-  const int j = blockIdx.x;
   double acc = 0.0;
-  for (int b = threadIdx.x; b < nb; b += TPB) acc += partial[int64_t(b) * k + j];
+  for (int b = threadIdx.x; b < nb; b += TPB) acc += partial[b];
   sh[threadIdx.x] = acc;
   __syncthreads();
   for (int o = TPB / 2; o > 0; o >>= 1) {
     if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
     __syncthreads();
   }
-  if (threadIdx.x == 0) out[j] = sh[0];
+  if (threadIdx.x == 0) out[0] = sh[0];
 }
 
 // w[map(i)] += sign * sum_j h_j V_j[i] (the sum in the order j = 0, 1, ...; loads
 // of four basis entries are issued together; h staged in shared memory; map(i) = i
 // without a map)
-constexpr int MAX_BASIS = 512;
 __global__ void k_multi_axpy(int64_t n, int k, const double* __restrict__ V, int64_t ldb, const double* __restrict__ h,
                              double sign, double* w, const int32_t* __restrict__ map) {
   __shared__ double hs[MAX_BASIS];
@@ -294,19 +379,15 @@ __global__ void k_multi_axpy(int64_t n, int k, const double* __restrict__ V, int
   }
 }
 
-// basis vector j = a x, also written to vc[map(i)] (map(i) = i without a map; x may
-// be vc when there is no map)
-__global__ void k_store_basis(int64_t n, double* V, int64_t ldb, int j, const double* x, double a, double* vc,
-                              const int32_t* __restrict__ map) {
+// basis vector j = a x, also written to vc[map[i]]; a = 1 / sqrt(nn[0]) when nn is given
+__global__ void k_store_basis(int64_t n, double* V, int64_t ldb, int j, const double* __restrict__ x, double a,
+                              const double* nn, double* vc, const int32_t* __restrict__ map) {
+  if (nn) a = __ddiv_rn(1.0, __dsqrt_rn(nn[0]));
   GRID_STRIDE(i, n) {
     const double v = a * x[i];
     V[basis_row(i, ldb) + int64_t(j) * kBasisBlock] = v;
-    vc[map ? int64_t(map[i]) : i] = v;
+    vc[map[i]] = v;
   }
-}
-
-__global__ void k_gather(int64_t n, const int32_t* __restrict__ map, const double* __restrict__ x, double* out) {
-  GRID_STRIDE(i, n) out[i] = x[map[i]];
 }
 
 __global__ void k_sum_partial(int64_t n, const double* __restrict__ a, double* part) {
@@ -400,12 +481,32 @@ cudaError_t axpby(int64_t n, double* out, const double* x, double a, const doubl
 
 int reduction_partials() { return RED_BLOCKS; }
 
-cudaError_t multidot(int64_t n, int k, const double* V, int64_t ldb, const double* w, double* partial, double* out,
-                     cudaStream_t s) {
-  if (k <= 0) return cudaSuccess;
-  k_multidot_partial<<<RED_BLOCKS, TPB, 0, s>>>(n, k, V, ldb, w, partial);
-  k_multidot_final<<<k, TPB, 0, s>>>(RED_BLOCKS, k, partial, out);
-  return cudaGetLastError();
+// blocks of a Gram-Schmidt stage: a fixed function of the rows (so are its sums)
+static unsigned gs_blocks(int64_t n) {
+  const int64_t b = (n + TPB - 1) / TPB;
+  return unsigned(b < 1 ? 1 : b < RED_BLOCKS ? b : RED_BLOCKS);
+}
+
+cudaError_t gs_gather_dot(int64_t n, int k, const double* V, int64_t ldb, const double* z, const int32_t* map,
+                          double* w, double* partial, unsigned* count, double* out, cudaStream_t s) {
+  const double* none = nullptr;
+  if (k > 0)
+    return launch_ex(true, &k_gram_schmidt<GS_GATHER, false>, gs_blocks(n), unsigned(TPB), 0, s, n, k, V, ldb, z, map,
+                     none, w, partial, count, out);
+  return launch_ex(true, &k_gram_schmidt<GS_GATHER, true>, gs_blocks(n), unsigned(TPB), 0, s, n, 0, V, ldb, z, map,
+                   none, w, partial, count, out);
+}
+
+cudaError_t gs_axpy_dot(int64_t n, int k, const double* V, int64_t ldb, const double* h, double* w, bool norm,
+                        double* partial, unsigned* count, double* out, cudaStream_t s) {
+  if (k <= 0 || k > MAX_BASIS) return cudaErrorInvalidValue;
+  const double* none = nullptr;
+  const int32_t* nomap = nullptr;
+  if (norm)
+    return launch_ex(true, &k_gram_schmidt<GS_AXPY, true>, gs_blocks(n), unsigned(TPB), 0, s, n, k, V, ldb, none,
+                     nomap, h, w, partial, count, out);
+  return launch_ex(true, &k_gram_schmidt<GS_AXPY, false>, gs_blocks(n), unsigned(TPB), 0, s, n, k, V, ldb, none, nomap,
+                   h, w, partial, count, out);
 }
 
 cudaError_t multi_axpy(int64_t n, int k, const double* V, int64_t ldb, const double* h, double sign, double* w,
@@ -415,14 +516,9 @@ cudaError_t multi_axpy(int64_t n, int k, const double* V, int64_t ldb, const dou
   return cudaGetLastError();
 }
 
-cudaError_t store_basis(int64_t n, double* V, int64_t ldb, int j, const double* x, double a, double* vc,
-                        cudaStream_t s, const int32_t* map) {
-  if (n > 0) k_store_basis<<<blocks_for(n), TPB, 0, s>>>(n, V, ldb, j, x, a, vc, map);
-  return cudaGetLastError();
-}
-
-cudaError_t gather(int64_t n, const int32_t* map, const double* x, double* out, cudaStream_t s) {
-  if (n > 0) k_gather<<<blocks_for(n), TPB, 0, s>>>(n, map, x, out);
+cudaError_t store_basis(int64_t n, double* V, int64_t ldb, int j, const double* x, double a, const double* nn,
+                        double* vc, const int32_t* map, cudaStream_t s) {
+  if (n > 0) k_store_basis<<<blocks_for(n), TPB, 0, s>>>(n, V, ldb, j, x, a, nn, vc, map);
   return cudaGetLastError();
 }
 
@@ -433,7 +529,7 @@ cudaError_t extrapolate_phi(int64_t n, const double* p1, const double* p2, doubl
 
 cudaError_t vsum(int64_t n, const double* a, double* partial, double* out, cudaStream_t s) {
   k_sum_partial<<<RED_BLOCKS, TPB, 0, s>>>(n, a, partial);
-  k_multidot_final<<<1, TPB, 0, s>>>(RED_BLOCKS, 1, partial, out);
+  k_vector_final<<<1, TPB, 0, s>>>(RED_BLOCKS, partial, out);
   return cudaGetLastError();
 }
 

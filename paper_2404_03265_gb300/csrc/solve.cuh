@@ -45,17 +45,20 @@ int reduction_partials();
 // so the rows of one block of all vectors are adjacent in memory.
 constexpr int64_t kBasisBlock = 2048;
 inline int64_t basis_blocks(int64_t n) { return (n + kBasisBlock - 1) / kBasisBlock; }
-// out[j] = V_j . w, j < k
-cudaError_t multidot(int64_t n, int k, const double* V, int64_t ldb, const double* w, double* partial, double* out,
-                     cudaStream_t s);
+// Gram-Schmidt stages, one launch each (partial: reduction_partials() doubles per vector,
+// count: one unsigned that is 0 between launches):
+//   gs_gather_dot: w[i] = z[map[i]], out[j] = V_j . w, j < k (k = 0: out[0] = w . w)
+//   gs_axpy_dot: w -= sum_j h[j] V_j, out[j] = V_j . w, j < k (norm: out[0] = w . w)
+cudaError_t gs_gather_dot(int64_t n, int k, const double* V, int64_t ldb, const double* z, const int32_t* map,
+                          double* w, double* partial, unsigned* count, double* out, cudaStream_t s);
+cudaError_t gs_axpy_dot(int64_t n, int k, const double* V, int64_t ldb, const double* h, double* w, bool norm,
+                        double* partial, unsigned* count, double* out, cudaStream_t s);
 // w[map[i]] += sign * sum_j h[j] V_j[i]  (h on the device; map[i] = i when map is null)
 cudaError_t multi_axpy(int64_t n, int k, const double* V, int64_t ldb, const double* h, double sign, double* w,
                        cudaStream_t s, const int32_t* map = nullptr);
-// V_j = a x, and vc[map[i]] = a x[i] (map[i] = i when map is null; x may then be vc)
-cudaError_t store_basis(int64_t n, double* V, int64_t ldb, int j, const double* x, double a, double* vc,
-                        cudaStream_t s, const int32_t* map = nullptr);
-// out[i] = x[map[i]], i < n
-cudaError_t gather(int64_t n, const int32_t* map, const double* x, double* out, cudaStream_t s);
+// V_j = a x, and vc[map[i]] = a x[i]; with nn (device) a = 1 / sqrt(nn[0]) instead
+cudaError_t store_basis(int64_t n, double* V, int64_t ldb, int j, const double* x, double a, const double* nn,
+                        double* vc, const int32_t* map, cudaStream_t s);
 cudaError_t vsum(int64_t n, const double* a, double* partial, double* out, cudaStream_t s);
 // phi_tilde = clip(2 phi^(n-1) - phi^(n-2), 0, 1) per slot
 cudaError_t extrapolate_phi(int64_t n, const double* p1, const double* p2, double* out, cudaStream_t s);

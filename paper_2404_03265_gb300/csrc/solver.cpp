@@ -58,12 +58,17 @@ cudaError_t leaf_op(pff_problem& pb, int kop, int mode, const double* lin, const
   return launch_leaf<double>(a, f, kop, s);
 }
 
+void release_workspace(SolverWS& W) {
+  W.mem.release();
+  if (W.host) cudaFreeHost(W.host);
+  W = SolverWS();
+}
+
 std::string ensure_workspace(pff_problem& pb, int restart) {
   SolverWS& W = pb.ws;
   const int64_t n = pb.mesh->m.lay.n_slots;
   if (W.ready && W.restart >= restart) return "";
-  W.mem.release();
-  W = SolverWS();
+  release_workspace(W);
   W.restart = restart;
   const int64_t n3 = 3 * n;
   {
@@ -97,20 +102,28 @@ std::string ensure_workspace(pff_problem& pb, int restart) {
   W.hh = W.mem.alloc<double>(2 * (restart + 1) + 1);
   W.scal = W.mem.alloc<double>(8);
   W.bad = W.mem.alloc<int>(1);
+  W.count = W.mem.alloc<unsigned>(1);
   W.x32 = W.mem.alloc<float>(n3);
   W.y32 = W.mem.alloc<float>(n3);
   if (!W.mem.err.empty()) return W.mem.err;
-  if (cudaMemset(W.vc, 0, n3 * sizeof(double)) != cudaSuccess) return "workspace: cudaMemset failed";
+  if (cudaMallocHost(reinterpret_cast<void**>(&W.host), (3 * size_t(restart + 1) + 8) * sizeof(double)) != cudaSuccess) {
+    W.host = nullptr;
+    return "workspace: cudaMallocHost failed";
+  }
+  if (cudaMemset(W.vc, 0, n3 * sizeof(double)) != cudaSuccess ||
+      cudaMemset(W.count, 0, sizeof(unsigned)) != cudaSuccess)
+    return "workspace: cudaMemset failed";
   W.ready = true;
   return "";
 }
 
 static cudaError_t norm2(pff_problem& pb, int64_t n, const double* a, double* out_host, cudaStream_t s) {
   SolverWS& W = pb.ws;
+  double* h = W.host + 3 * (W.restart + 1) + 4;
   RET(dot64(n, a, a, W.partial, W.scal, s));
-  RET(cudaMemcpyAsync(out_host, W.scal, sizeof(double), cudaMemcpyDeviceToHost, s));
+  RET(cudaMemcpyAsync(h, W.scal, sizeof(double), cudaMemcpyDeviceToHost, s));
   RET(cudaStreamSynchronize(s));
-  *out_host = std::sqrt(*out_host);
+  *out_host = std::sqrt(*h);
   return cudaSuccess;
 }
 
@@ -136,14 +149,25 @@ cudaError_t gmres_solve(pff_problem& pb, pff_mg& mg, int transpose, const double
   };
   for (auto& e : pb.gm_ev)
     if (!e) RET(cudaEventCreate(&e));
-  cudaEvent_t* ev = pb.gm_ev;
+  if (!pb.gm_read) RET(cudaEventCreateWithFlags(&pb.gm_read, cudaEventDisableTiming));
   RET(cudaMemsetAsync(x, 0, n3 * sizeof(double), s));
   const int64_t ldb = int64_t(restart + 1) * kBasisBlock;   // row-block stride of the basis
   const int64_t nc = W.nc;
-  RET(precond(mg, b, W.w, s));
-  RET(gather(nc, W.map, W.w, W.wc, s));
+  const size_t nhh = 2 * size_t(restart + 1) + 1;
+  double* const hh = W.host;             // pinned: one step's coefficients (both passes) and |w|^2,
+  double* const yh = W.host + nhh;       // the solution's coefficients,
+  double* const bh = yh + restart + 1;   // a squared norm
+  // w = map-rows of P^-1 v, its norm to the host
+  auto start = [&](const double* v, double& beta) -> cudaError_t {
+    RET(precond(mg, v, W.w, s));
+    RET(gs_gather_dot(nc, 0, W.V, ldb, W.w, W.map, W.wc, W.partial, W.count, W.scal, s));
+    RET(cudaMemcpyAsync(bh, W.scal, sizeof(double), cudaMemcpyDeviceToHost, s));
+    RET(cudaStreamSynchronize(s));
+    beta = std::sqrt(*bh);
+    return cudaSuccess;
+  };
   double beta = 0.0;
-  RET(norm2(pb, nc, W.wc, &beta, s));
+  RET(start(b, beta));
   res = GmresResult();
   res.initial = beta;
   if (!(beta > 0.0)) {
@@ -153,38 +177,49 @@ cudaError_t gmres_solve(pff_problem& pb, pff_mg& mg, int transpose, const double
   }
   const double target = rtol * beta;
   int it = 0;
-  std::vector<double> H(size_t(restart + 1) * restart), cs(restart), sn(restart), g(restart + 1),
-      hh(2 * (restart + 1) + 1);
+  std::vector<double> H(size_t(restart + 1) * restart), cs(restart), sn(restart), g(restart + 1);
   double* h1d = W.hh;                     // first pass coefficients
   double* h2d = W.hh + (restart + 1);     // second pass
   double* nwd = W.hh + 2 * (restart + 1); // |w|^2
+  // basis vector j (from W.wc, scaled by a or by 1 / sqrt(|w|^2) on the device) and A V_j
+  // into W.tmp; events of step j in set j % 2
+  auto next = [&](int j, double a, const double* nn) -> cudaError_t {
+    cudaEvent_t* ev = pb.gm_ev + 4 * (j % 2);
+    RET(store_basis(nc, W.V, ldb, j, W.wc, a, nn, W.vc, W.map, s));
+    RET(cudaEventRecord(ev[0], s));
+    RET(A(W.vc, W.tmp));
+    return cudaEventRecord(ev[1], s);
+  };
   while (it < maxiter) {
     std::fill(H.begin(), H.end(), 0.0);
     std::fill(g.begin(), g.end(), 0.0);
     g[0] = beta;
-    RET(store_basis(nc, W.V, ldb, 0, W.wc, 1.0 / beta, W.vc, s, W.map));
+    RET(next(0, 1.0 / beta, nullptr));
     int jd = 0;
     bool conv = false;
     for (int j = 0; j < restart; ++j) {
-      // W.vc holds V_j in slot layout
-      RET(cudaEventRecord(ev[0], s));
-      RET(A(W.vc, W.tmp));
-      RET(cudaEventRecord(ev[1], s));
+      // W.vc holds V_j in slot layout, W.tmp = A V_j
+      cudaEvent_t* ev = pb.gm_ev + 4 * (j % 2);
       RET(precond(mg, W.tmp, W.w, s));
       RET(cudaEventRecord(ev[2], s));
       // classical Gram-Schmidt, twice, on the node rows; the coefficients stay on
       // the device until one copy brings both passes and |w|^2 to the host
-      RET(gather(nc, W.map, W.w, W.wc, s));
-      RET(multidot(nc, j + 1, W.V, ldb, W.wc, W.partial, h1d, s));
-      RET(multi_axpy(nc, j + 1, W.V, ldb, h1d, -1.0, W.wc, s));
-      RET(multidot(nc, j + 1, W.V, ldb, W.wc, W.partial, h2d, s));
-      RET(multi_axpy(nc, j + 1, W.V, ldb, h2d, -1.0, W.wc, s));
-      RET(dot64(nc, W.wc, W.wc, W.partial, nwd, s));
+      RET(gs_gather_dot(nc, j + 1, W.V, ldb, W.w, W.map, W.wc, W.partial, W.count, h1d, s));
+      RET(gs_axpy_dot(nc, j + 1, W.V, ldb, h1d, W.wc, false, W.partial, W.count, h2d, s));
+      RET(gs_axpy_dot(nc, j + 1, W.V, ldb, h2d, W.wc, true, W.partial, W.count, nwd, s));
       RET(cudaEventRecord(ev[3], s));
-      RET(cudaMemcpyAsync(hh.data(), W.hh, hh.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
-      RET(cudaStreamSynchronize(s));
-      const double* h = hh.data();
-      const double* h2 = hh.data() + (restart + 1);
+      RET(cudaMemcpyAsync(hh, W.hh, nhh * sizeof(double), cudaMemcpyDeviceToHost, s));
+      RET(cudaEventRecord(pb.gm_read, s));
+      // The next basis vector and its apply are launched before the host has seen this
+      // step's coefficients, unless the residual's last reduction says that this step
+      // converges: the host's turn then costs the device nothing.  A step that converges
+      // all the same leaves one apply unused (no result depends on it).
+      const double red = j > 0 ? std::fabs(g[j]) / std::fabs(g[j - 1]) : 1.0;
+      const bool ahead = j + 1 < restart && it + 1 < maxiter && !(std::fabs(g[j]) * red <= target);
+      if (ahead) RET(next(j + 1, 0.0, nwd));
+      RET(cudaEventSynchronize(pb.gm_read));
+      const double* h = hh;
+      const double* h2 = hh + (restart + 1);
       const double hn = std::sqrt(hh[2 * (restart + 1)]);
       float ms[3] = {0.f, 0.f, 0.f};
       for (int q = 0; q < 3; ++q) RET(cudaEventElapsedTime(&ms[q], ev[q], ev[q + 1]));
@@ -213,17 +248,16 @@ cudaError_t gmres_solve(pff_problem& pb, pff_mg& mg, int transpose, const double
         conv = std::fabs(g[j + 1]) <= target || hn == 0.0;
         break;
       }
-      RET(store_basis(nc, W.V, ldb, j + 1, W.wc, 1.0 / hn, W.vc, s, W.map));
+      if (!ahead && j + 1 < restart) RET(next(j + 1, 1.0 / hn, nullptr));
     }
     // y = H^-1 g (upper triangular), x += V y
-    std::vector<double> y(jd, 0.0);
     for (int i = jd - 1; i >= 0; --i) {
       double t = g[i];
-      for (int k = i + 1; k < jd; ++k) t -= H[size_t(i) * restart + k] * y[k];
-      y[i] = t / H[size_t(i) * restart + i];
+      for (int k = i + 1; k < jd; ++k) t -= H[size_t(i) * restart + k] * yh[k];
+      yh[i] = t / H[size_t(i) * restart + i];
     }
     if (jd > 0) {
-      RET(cudaMemcpyAsync(W.h, y.data(), jd * sizeof(double), cudaMemcpyHostToDevice, s));
+      RET(cudaMemcpyAsync(W.h, yh, jd * sizeof(double), cudaMemcpyHostToDevice, s));
       RET(multi_axpy(nc, jd, W.V, ldb, W.h, 1.0, x, s, W.map));
     }
     res.iterations = it;
@@ -233,9 +267,7 @@ cudaError_t gmres_solve(pff_problem& pb, pff_mg& mg, int transpose, const double
     // restart from the true preconditioned residual
     RET(A(x, W.tmp));
     RET(axpby(n3, W.tmp, b, 1.0, W.tmp, -1.0, s));
-    RET(precond(mg, W.tmp, W.w, s));
-    RET(gather(nc, W.map, W.w, W.wc, s));
-    RET(norm2(pb, nc, W.wc, &beta, s));
+    RET(start(W.tmp, beta));
     res.estimate = beta;
     if (beta <= target) { res.converged = true; return cudaSuccess; }
   }

@@ -125,6 +125,8 @@ struct SolverWS {
   double *partial = nullptr, *h = nullptr, *scal = nullptr;
   double* hh = nullptr;   // one Arnoldi step on the device: both Gram-Schmidt passes and |w|^2 (2 (restart + 1) + 1)
   int* bad = nullptr;
+  unsigned* count = nullptr;   // finished blocks of a Gram-Schmidt stage (0 between launches)
+  double* host = nullptr;      // pinned: coefficients of an Arnoldi step, of the solution, norms (3 (restart + 1) + 8)
   float *x32 = nullptr, *y32 = nullptr;   // FP32 operator applies inside GMRES (3 blocks each)
 };
 
@@ -190,7 +192,8 @@ struct pff_problem {
   double* adj_cell = nullptr;     // n_leaf_cells: per-step modulus gradient of the multi-step adjoint
   double* adj_phit = nullptr;     // n_slots: extrapolated phi_tilde of the step the multi-step adjoint is at
   double* adj_pend = nullptr;     // n_slots: phi share of step k's adjoint that reaches step k - 2
-  cudaEvent_t gm_ev[4] = {};      // GMRES phase timing (created on first use)
+  cudaEvent_t gm_ev[8] = {};      // GMRES phase timing, two steps in turn (created on first use)
+  cudaEvent_t gm_read = nullptr;  // an Arnoldi step's coefficients are on the host
   int sweep_sh = 0;               // Q1 cell-loop strip half-height (pff_set_cell_loop), 0 = by mesh size
 };
 
@@ -300,6 +303,7 @@ cudaError_t launch_leaf_cmask(int64_t n, const uint8_t* slot_flags, const uint8_
 cudaError_t leaf_op(pff_problem& pb, int kop, int mode, const double* lin, const uint8_t* cmask, const double* xu,
                     const double* xp, double* yu, double* yp, cudaStream_t s);
 std::string ensure_workspace(pff_problem& pb, int restart);
+void release_workspace(SolverWS& W);
 cudaError_t gmres_solve(pff_problem& pb, pff_mg& mg, int transpose, const double* b, double* x, double rtol,
                         int restart, int maxiter, GmresResult& res, cudaStream_t s, int matvec = PFF_F64);
 cudaError_t leaf_residual(pff_problem& pb, const double* u, const double* phi, const double* phit, double* R,
