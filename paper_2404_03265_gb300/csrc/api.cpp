@@ -295,6 +295,7 @@ extern "C" pff_status pff_mg_create(pff_problem* pb, int32_t precision, pff_mg**
     std::string e = mg_alloc(*mg);
     if (!e.empty()) {
       mg->mem.release();
+      if (mg->host) cudaFreeHost(mg->host);
       delete mg;
       return fail(PFF_ERR_OOM, e);
     }
@@ -341,6 +342,7 @@ extern "C" void pff_mg_destroy(pff_mg* mg) {
   mg_release_setup_graph(*mg);
   if (mg->su_side) cudaStreamDestroy(mg->su_side);
   if (mg->su_chains) cudaEventDestroy(mg->su_chains);
+  if (mg->host) cudaFreeHost(mg->host);
   if (mg->cap_stream) cudaStreamDestroy(mg->cap_stream);
   if (mg->cap_stream2) cudaStreamDestroy(mg->cap_stream2);
   if (mg->ev_fork) cudaEventDestroy(mg->ev_fork);

@@ -872,6 +872,80 @@ cudaError_t launch_apply(const ApplyArgs& a, int op, cudaStream_t s) {
   }
 }
 
+namespace {
+// Element matrices of a level block on level 0: thread (cell, column) evaluates the cell
+// on a unit vector.  Ke: per cell [row][column], dof = node * ncomp + component.
+template <int OP, int K>
+__global__ void __launch_bounds__(64) coarse_element_kernel(const __grid_constant__ ApplyArgs a, int ncx, int ncells,
+                                                            const int32_t* __restrict__ node_slot,
+                                                            double* __restrict__ Ke) {
+  constexpr int NC = OP == OP_UU ? 2 : 1, NN = (K + 1) * (K + 1), ND = NN * NC;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, cell = t / ND, col = t % ND;
+  if (cell >= ncells) return;
+  const int ci = cell % ncx, cj = cell / ncx, nx = K * ncx + 1;
+  const double* lin = reinterpret_cast<const double*>(a.lin);
+  const int64_t n = a.n_slots;
+  const int N = col / NC, c = col % NC;   // the unit vector
+  int slot[NN];
+#pragma unroll
+  for (int e = 0; e < NN; ++e) slot[e] = node_slot[ci * K + e % (K + 1) + nx * (cj * K + e / (K + 1))];
+  const double ec = a.ecell != nullptr ? reinterpret_cast<const double*>(a.ecell)[slot[0]] : 1.0;
+  double r[ND];
+  if constexpr (K == 1) {
+    NodePair<double> v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      v[e] = NodePair<double>{};
+      if (e == N) {
+        if (OP == OP_UU) (c ? v[e].x1 : v[e].x0) = 1.0; else v[e].xp = 1.0;
+      }
+      v[e].lx = lin[slot[e]];
+      v[e].ly = lin[n + slot[e]];
+      v[e].lw = lin[3 * n + slot[e]];
+    }
+    auto minus = [](const NodePair<double>& p, const NodePair<double>& q) {
+      return NodePair<double>{p.x0 - q.x0, p.x1 - q.x1, p.xp - q.xp, p.lx - q.lx, p.ly - q.ly, p.lz - q.lz, p.lw - q.lw};
+    };
+    double out[12];
+    q1_cell<double, OP>(v[0], minus(v[1], v[0]), v[2], minus(v[3], v[2]), a.md, a.gd[0], ec, out);
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+      for (int q = 0; q < NC; ++q) r[e * NC + q] = out[3 * e + (OP == OP_UU ? q : 2)];
+  } else {
+    auto ld = [&](int k, int i, int j) -> double2 {
+      const int e = i + 3 * j;
+      const double one = e == N ? 1.0 : 0.0;
+      if (k == 0) return make_double2(c == 0 ? one : 0.0, c == 1 ? one : 0.0);
+      if (k == 1) return make_double2(lin[slot[e]], lin[n + slot[e]]);
+      if (k == 2) return make_double2(one, 0.0);
+      return make_double2(lin[3 * n + slot[e]], 0.0);
+    };
+    double2 ru[9];
+    double rp[9], cv[3];
+    q2_cell<double, OP>(ld, a.md, a.gd[0], a.q2d, ec, ru, rp, cv);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      if constexpr (OP == OP_UU) { r[2 * e] = ru[e].x; r[2 * e + 1] = ru[e].y; } else { r[e] = rp[e]; }
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < ND; ++e) Ke[(int64_t(cell) * ND + e) * ND + col] = r[e];
+}
+}  // namespace
+
+cudaError_t launch_coarse_elements(const ApplyArgs& a, int op, int ncx, int ncells, const int32_t* node_slot,
+                                   double* Ke, cudaStream_t s) {
+  const int nd = (a.fe_degree + 1) * (a.fe_degree + 1) * (op == OP_UU ? 2 : 1);
+  const unsigned grid = unsigned((int64_t(ncells) * nd + 63) / 64);
+  if (a.fe_degree == 1 && op == OP_UU) coarse_element_kernel<OP_UU, 1><<<grid, 64, 0, s>>>(a, ncx, ncells, node_slot, Ke);
+  else if (a.fe_degree == 1 && op == OP_PP) coarse_element_kernel<OP_PP, 1><<<grid, 64, 0, s>>>(a, ncx, ncells, node_slot, Ke);
+  else if (a.fe_degree == 2 && op == OP_UU) coarse_element_kernel<OP_UU, 2><<<grid, 64, 0, s>>>(a, ncx, ncells, node_slot, Ke);
+  else if (a.fe_degree == 2 && op == OP_PP) coarse_element_kernel<OP_PP, 2><<<grid, 64, 0, s>>>(a, ncx, ncells, node_slot, Ke);
+  else return cudaErrorInvalidValue;
+  return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t launch_fixup(const FixupArgs& a, cudaStream_t s) {
   if (a.n <= 0) return cudaSuccess;

@@ -202,11 +202,10 @@ __device__ __forceinline__ void q2_point(const Q2Point<T>& q, const MatConst<T>&
   (void)se;
 }
 
-// One Q2 cell, its node (a, b) (a along x, b along y) read by ld.  Contributions to node A = a + 3 b: ru[A] (components u_x,
-// u_y) and rp[A] (phi).  cell[]: per-cell values (OP_VJP).
-template <typename T, int OP>
-__device__ __forceinline__ void q2_cell(const Q2Node<T, OP>& ld, const MatConst<T>& m,
-                                        const LevGeom<T>& g, const Q2Tab<T>& tb, T ec, typename VT<T>::T2 ru[9],
+// One Q2 cell, its node (a, b) (a along x, b along y) read by ld.  Contributions to node
+// A = a + 3 b: ru[A] (components u_x, u_y) and rp[A] (phi).  cell[]: per-cell values (OP_VJP).
+template <typename T, int OP, class Load>
+__device__ __forceinline__ void q2_cell(const Load& ld, const MatConst<T>& m, const LevGeom<T>& g, const Q2Tab<T>& tb, T ec, typename VT<T>::T2 ru[9],
                                         T rp[9], T cell[3]) {
   using N = Needs<OP>;
   using P = typename VT<T>::T2;

@@ -213,6 +213,10 @@ cudaError_t launch_leaf_cells<float>(const ApplyArgs& a, const FixupArgs& f, int
 // The same for Q2 in FP64 (leaf_cells_q2.cu): OP_FULL, OP_FULL_T, OP_RESID.
 cudaError_t launch_leaf_cells_q2(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);
 
+// Element matrices of a level block (OP_UU, OP_PP) on level 0, FP64: see CoarseBlock::Ke.
+cudaError_t launch_coarse_elements(const ApplyArgs& a, int op, int ncx, int ncells, const int32_t* node_slot,
+                                   double* Ke, cudaStream_t s);
+
 // state conversion: lin64/lin32 blocks (u_x, u_y, phi, phi_t), hanging entries from parents;
 // u is the displacement in block layout (u_x block, u_y block)
 // hlin64/hlin32: the hanging nodes' linearisation again, 4 blocks of nhang (read by the Q1 sweep)

@@ -235,156 +235,6 @@ __global__ void k_cheb_step_add(int64_t n, T* xadd, const T* __restrict__ x, con
   }
 }
 
-// Blocked Gauss-Jordan inversion in place, panels of GJB pivots.  With P the
-// panel's rows/columns and R the others, eliminating the pivots of P gives
-//   A_PP <- X = A_PP^-1,  A_PR <- X A_PR,  A_RP <- -A_RP X,  A_RR <- A_RR - A_RP X A_PR
-// (old A_RP, A_PR on the right), the same as GJB scalar Gauss-Jordan steps.  A_PP
-// is then a Schur complement of an SPD matrix, so no pivoting is needed; its
-// inversion (one block, scalar steps in shared memory) flags a non-positive pivot.
-// Two launches per panel: k_gj_panel inverts A_PP and copies the old A_RP and
-// A_PR to scratch; k_gj_update then owns every entry it writes, so no block reads
-// an entry another block of the same launch writes.
-// Scratch layout (double): X (GJB x GJB, zero beyond b), then Cp ((n - b) x GJB:
-// old A_RP by compact row index, zero beyond b), then Rp (GJB x n: old A_PR, zero
-// in the panel's columns and beyond b).
-constexpr int GJB = 32;
-constexpr int GJ_ROWS = 128;   // rows of a k_gj_update tile (its columns: GJB)
-
-__device__ __forceinline__ int gj_row(int ii, int k0, int b) { return ii < k0 ? ii : ii + b; }
-
-// block 0: X = A_PP^-1 (padded with the identity to GJB x GJB); the others copy
-// the old pivot columns and rows
-__global__ void __launch_bounds__(TPB) k_gj_panel(int32_t n, int32_t k0, int32_t b, double* A, double* scr,
-                                                  int32_t* bad) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (blockIdx.x == 0) {
-    // one reciprocal per step: the thread that writes the next pivot inverts it
-    __shared__ double T[GJB][GJB + 1];
-    __shared__ double ipiv[2];
-#pragma unroll
-    for (int r = 0; r < GJB / 8; ++r) {
-      const int i = w + 8 * r;
-      T[i][lane] = (i < b && lane < b) ? A[int64_t(k0 + i) * n + k0 + lane] : (i == lane ? 1.0 : 0.0);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      if (!(T[0][0] > 0.0)) *bad = 1;
-      ipiv[0] = 1.0 / T[0][0];
-    }
-    __syncthreads();
-    for (int k = 0; k < GJB; ++k) {
-      const double ip = ipiv[k & 1];
-      const double sk = T[k][lane] * ip;   // row k scaled by the pivot's reciprocal
-      double v[GJB / 8];
-#pragma unroll
-      for (int r = 0; r < GJB / 8; ++r) {
-        const int i = w + 8 * r;
-        const double pc = T[i][k];
-        if (i == k) v[r] = lane == k ? ip : sk;
-        else if (lane == k) v[r] = -pc * ip;
-        else v[r] = fma(-pc, sk, T[i][lane]);
-      }
-      __syncthreads();
-#pragma unroll
-      for (int r = 0; r < GJB / 8; ++r) {
-        const int i = w + 8 * r;
-        T[i][lane] = v[r];
-        if (i == k + 1 && lane == k + 1) {
-          if (!(v[r] > 0.0)) *bad = 1;
-          ipiv[(k + 1) & 1] = 1.0 / v[r];
-        }
-      }
-      __syncthreads();
-    }
-#pragma unroll
-    for (int r = 0; r < GJB / 8; ++r) {
-      const int i = w + 8 * r;
-      const bool in = i < b && lane < b;
-      scr[i * GJB + lane] = in ? T[i][lane] : 0.0;
-      if (in) A[int64_t(k0 + i) * n + k0 + lane] = T[i][lane];
-    }
-    return;
-  }
-  double* Cp = scr + GJB * GJB;
-  double* Rp = Cp + int64_t(n - b) * GJB;
-  const int64_t nc = int64_t(n - b) * GJB, nr = int64_t(GJB) * n;
-  const int64_t stride = int64_t(gridDim.x - 1) * blockDim.x;
-  for (int64_t e = int64_t(blockIdx.x - 1) * blockDim.x + threadIdx.x; e < nc + nr; e += stride) {
-    if (e < nc) {
-      const int ii = int(e / GJB), k = int(e % GJB);
-      Cp[e] = k < b ? A[int64_t(gj_row(ii, k0, b)) * n + k0 + k] : 0.0;
-    } else {
-      const int64_t f = e - nc;
-      const int k = int(f / n), j = int(f % n);
-      Rp[f] = (k < b && (j < k0 || j >= k0 + b)) ? A[int64_t(k0 + k) * n + j] : 0.0;
-    }
-  }
-}
-
-// tile (GJ_ROWS rows outside P) x (GJB columns): the panel's columns get
-// -A_RP X; any other column tile forms X A_PR for its columns (written back by
-// the first row tile) and subtracts A_RP (X A_PR) from its rows
-__global__ void __launch_bounds__(TPB) k_gj_update(int32_t n, int32_t k0, int32_t b, double* A,
-                                                   const double* scr) {
-  __shared__ double Xs[GJB][GJB];
-  __shared__ double Ps[GJB][GJB];       // old A_PR tile, then X A_PR
-  __shared__ double Cs[GJ_ROWS][GJB];   // old A_RP rows of the tile
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const double* Cp = scr + GJB * GJB;
-  const double* Rp = Cp + int64_t(n - b) * GJB;
-  const int ii0 = int(blockIdx.y) * GJ_ROWS;
-  const int nrow = min(GJ_ROWS, n - b - ii0);
-  const int j0 = int(blockIdx.x) * GJB;
-  const int j = j0 + lane;
-  const bool panel = j0 == k0;
-#pragma unroll
-  for (int r = 0; r < GJB / 8; ++r) Xs[w + 8 * r][lane] = scr[(w + 8 * r) * GJB + lane];
-  for (int r = w; r < GJ_ROWS; r += TPB / 32) Cs[r][lane] = r < nrow ? Cp[int64_t(ii0 + r) * GJB + lane] : 0.0;
-  if (!panel) {
-#pragma unroll
-    for (int r = 0; r < GJB / 8; ++r) Ps[w + 8 * r][lane] = j < n ? Rp[int64_t(w + 8 * r) * n + j] : 0.0;
-  }
-  __syncthreads();
-  if (panel) {
-    // A_RP <- -A_RP X
-    for (int r = w; r < nrow; r += TPB / 32) {
-      double acc = 0.0;
-#pragma unroll
-      for (int k = 0; k < GJB; ++k) acc = fma(Cs[r][k], Xs[k][lane], acc);
-      if (lane < b) A[int64_t(gj_row(ii0 + r, k0, b)) * n + j] = -acc;
-    }
-    return;
-  }
-  double pr[GJB / 8];
-#pragma unroll
-  for (int r = 0; r < GJB / 8; ++r) {
-    const int k = w + 8 * r;
-    double acc = 0.0;
-#pragma unroll
-    for (int m = 0; m < GJB; ++m) acc = fma(Xs[k][m], Ps[m][lane], acc);
-    pr[r] = acc;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < GJB / 8; ++r) {
-    const int k = w + 8 * r;
-    Ps[k][lane] = pr[r];
-    if (blockIdx.y == 0 && k < b && j < n) A[int64_t(k0 + k) * n + j] = pr[r];
-  }
-  __syncthreads();
-  if (j >= n) return;
-  double pc[GJB];
-#pragma unroll
-  for (int k = 0; k < GJB; ++k) pc[k] = Ps[k][lane];
-  for (int r = w; r < nrow; r += TPB / 32) {
-    double acc = 0.0;
-#pragma unroll
-    for (int k = 0; k < GJB; ++k) acc = fma(Cs[r][k], pc[k], acc);
-    double* a = A + int64_t(gj_row(ii0 + r, k0, b)) * n + j;
-    *a = *a - acc;
-  }
-}
-
 // Dense FP64 coarse solve x[idx] = Ainv d[idx], d taken to FP64: one warp per row,
 // lanes stride the columns, fixed-order warp reduction.  The first CP columns of a
 // lane (all of them on a 16 x 16 coarse mesh) and their indices are read before the wait.
@@ -418,14 +268,20 @@ __global__ void k_coarse_matvec(int32_t n, const int32_t* __restrict__ idx, cons
   if (lane == 0) x[out] = T(acc);
 }
 
-__global__ void k_inject_lin(int32_t nsl, const int32_t* __restrict__ sl, const double* __restrict__ lin,
-                             int64_t nsleaf, double* l64, float* l32) {
-  GRID_STRIDE(s, nsl) {
-    const int ls = sl[s];
+// level linearisations from the leaf's, one block per level brick of all levels
+__global__ void __launch_bounds__(TPB) k_inject_lin(const LevBrick* __restrict__ bricks,
+                                                    const int32_t* __restrict__ lev_leaf,
+                                                    const double* __restrict__ lin, int64_t nsleaf, double* l64,
+                                                    float* l32) {
+  const LevBrick b = bricks[blockIdx.x];
+  for (int i = threadIdx.x; i < LD_SLOTS; i += TPB) {
+    const int ls = lev_leaf[b.off + b.base + i];
+#pragma unroll
     for (int f = 0; f < 4; ++f) {
       const double v = ls >= 0 ? lin[f * nsleaf + ls] : 0.0;
-      l64[f * int64_t(nsl) + s] = v;
-      l32[f * int64_t(nsl) + s] = float(v);
+      const int64_t o = 4 * int64_t(b.off) + f * int64_t(b.n) + b.base + i;
+      l64[o] = v;
+      l32[o] = float(v);
     }
   }
 }
@@ -474,21 +330,6 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {
   return z ^ (z >> 31);
 }
 
-__global__ void k_start_vector(int32_t nsl, int ncomp, const int32_t* __restrict__ gx, const int32_t* __restrict__ gy,
-                               const double* __restrict__ dinv, double* r) {
-  GRID_STRIDE(s, nsl) {
-    double v = 0.0;
-    if (gx[s] >= 0) {
-      const uint64_t h = splitmix64((uint64_t(uint32_t(gx[s])) << 32) | uint64_t(uint32_t(gy[s])));
-      v = 1.0 + 0.01 * double(h % 1000ull) / 1000.0;
-    }
-    for (int c = 0; c < ncomp; ++c) {
-      const int64_t i = c * int64_t(nsl) + s;
-      r[i] = dinv[i] != 0.0 ? v : 0.0;
-    }
-  }
-}
-
 constexpr int DOT_BLOCKS = 512;
 
 __global__ void k_dot_partial(int64_t n, const double* __restrict__ a, const double* __restrict__ b, double* part) {
@@ -517,73 +358,106 @@ __global__ void k_dot_final(int nb, const double* __restrict__ part, double* out
   if (threadIdx.x == 0) out[0] = sh[0];
 }
 
-// sc: 0 rz, 1 pq, 2 rz_new, 3 alpha, 4 beta, 5 ok (1 while the iteration is healthy)
-__global__ void k_cg_init(double* sc) {
-  if (threadIdx.x < 8) sc[threadIdx.x] = threadIdx.x == 5 ? 1.0 : 0.0;
-}
-
-// r -= alpha q, z = D^-1 r and the block partial sums of r.z (the grid and the
-// summation order of k_dot_partial, so the dot is the same as a separate one)
-__global__ void k_cg_r_dot(int64_t n, double* r, double* z, const double* __restrict__ q,
-                           const double* __restrict__ dinv, const double* __restrict__ sc, double* part) {
+// Jacobi-preconditioned CG of a set-up chain: three launches a step beside the operator
+// apply (dot p.q; r, z and dot r.z; p).  A dot's last block to finish adds the blocks'
+// partial sums in a fixed order and forms the scalars
+//   sc: 0 rz, 1 pq, 2 rz_new, 3 alpha, 4 beta, 5 ok (1 while the iteration is healthy).
+// Each step's coefficients go to hist (alpha_j, beta_j; alpha_j = 0 marks a stop).
+// Q: precision of q = A p.
+enum CgStage : int { CG_START = 0, CG_PQ = 1, CG_RZ = 2 };
+template <int STAGE, typename Q>
+__global__ void __launch_bounds__(TPB) k_cg(int64_t n, int32_t nsl, const int32_t* __restrict__ gx,
+                                            const int32_t* __restrict__ gy, const double* __restrict__ dinv, double* r,
+                                            double* z, double* p, Q* pq, const Q* q, double* sc, double* hist, int step,
+                                            double* partial, unsigned* count) {
   __shared__ double sh[TPB];
-  const double alpha = sc[3];
+  __shared__ bool last;
+  pdl_wait();
+  pdl_trigger();
+  const int tid = threadIdx.x;
+  const double alpha = STAGE == CG_RZ ? sc[3] : 0.0;
   double acc = 0.0;
   GRID_STRIDE(i, n) {
-    const double ri = r[i] - alpha * q[i];
-    const double zi = dinv[i] * ri;
-    r[i] = ri;
-    z[i] = zi;
-    acc += ri * zi;
+    if (STAGE == CG_START) {
+      // r: 1 + 0.01 (splitmix64((gx << 32) | gy) mod 1000) / 1000 on interior entries; p = z = D^-1 r
+      const int32_t s = int32_t(i % nsl);
+      double v = 0.0;
+      const double di = dinv[i];
+      if (gx[s] >= 0 && di != 0.0) {
+        const uint64_t h = splitmix64((uint64_t(uint32_t(gx[s])) << 32) | uint64_t(uint32_t(gy[s])));
+        v = 1.0 + 0.01 * double(h % 1000ull) / 1000.0;
+      }
+      const double zi = di * v;
+      r[i] = v;
+      z[i] = zi;
+      p[i] = zi;
+      if (sizeof(Q) == 4) pq[i] = Q(zi);
+      acc += v * zi;
+    } else if (STAGE == CG_PQ) {
+      acc += p[i] * double(q[i]);
+    } else {
+      const double ri = r[i] - alpha * double(q[i]);
+      const double zi = dinv[i] * ri;
+      r[i] = ri;
+      z[i] = zi;
+      acc += ri * zi;
+    }
   }
-  sh[threadIdx.x] = acc;
+  sh[tid] = acc;
   __syncthreads();
   for (int o = TPB / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+    if (tid < o) sh[tid] += sh[tid + o];
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
-}
-
-// sc[slot] = sum of the partials (the order of k_dot_final), then slot 1: alpha =
-// rz / pq; slot 2: beta = rz_new / rz, the coefficient history (alpha_j, beta_j;
-// alpha_j = 0 marks a stop) and rz = rz_new.  sc[5] drops to 0 on a breakdown.
-__global__ void k_dot_final_cg(int nb, const double* __restrict__ part, double* sc, int slot, double* hist,
-                               int step) {
-  __shared__ double sh[TPB];
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < nb; i += TPB) acc += part[i];
-  sh[threadIdx.x] = acc;
+  if (tid == 0) {
+    partial[blockIdx.x] = sh[0];
+    __threadfence();
+    last = atomicAdd(count, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  acc = 0.0;
+  for (unsigned b = tid; b < gridDim.x; b += TPB) acc += __ldcg(partial + b);
+  sh[tid] = acc;
   __syncthreads();
   for (int o = TPB / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+    if (tid < o) sh[tid] += sh[tid + o];
     __syncthreads();
   }
-  if (threadIdx.x != 0) return;
-  sc[slot] = sh[0];
-  if (slot == 1) {
-    const double pq = sc[1];
-    const bool ok = sc[5] > 0.5 && pq > 0.0 && sc[0] > 0.0;
-    sc[3] = ok ? sc[0] / pq : 0.0;
+  if (tid != 0) return;
+  *count = 0u;   // for the next launch
+  if (STAGE == CG_START) {
+    sc[0] = sh[0];
+    sc[5] = 1.0;
+  } else if (STAGE == CG_PQ) {
+    sc[1] = sh[0];
+    const bool ok = sc[5] > 0.5 && sh[0] > 0.0 && sc[0] > 0.0;
+    sc[3] = ok ? sc[0] / sh[0] : 0.0;
     if (!ok) sc[5] = 0.0;
-  } else if (slot == 2) {
+  } else {
+    sc[2] = sh[0];
     const bool ok = sc[5] > 0.5;
-    const double beta = ok ? sc[2] / sc[0] : 0.0;
+    const double beta = ok ? sh[0] / sc[0] : 0.0;
     sc[4] = beta;
     hist[2 * step + 0] = ok ? sc[3] : 0.0;
     hist[2 * step + 1] = beta;
-    if (!(ok && sc[2] > 1e-300)) sc[5] = 0.0;
-    sc[0] = sc[2];
+    if (!(ok && sh[0] > 1e-300)) sc[5] = 0.0;
+    sc[0] = sh[0];
   }
 }
 
-__global__ void k_cg_p(int64_t n, double* p, const double* __restrict__ z, const double* __restrict__ sc) {
+template <typename Q>
+__global__ void k_cg_p(int64_t n, double* p, Q* pq, const double* __restrict__ z, const double* __restrict__ sc) {
+  pdl_wait();
+  pdl_trigger();
   const double beta = sc[4];
-  GRID_STRIDE(i, n) p[i] = z[i] + beta * p[i];
+  GRID_STRIDE(i, n) {
+    const double v = z[i] + beta * p[i];
+    p[i] = v;
+    if (sizeof(Q) == 4) pq[i] = Q(v);
+  }
 }
-
-__global__ void k_fill64(int64_t n, double* x, double v) { GRID_STRIDE(i, n) x[i] = v; }
-__global__ void k_copy64(int64_t n, double* d, const double* s) { GRID_STRIDE(i, n) d[i] = s[i]; }
 
 }  // namespace
 
@@ -653,24 +527,6 @@ cudaError_t mg_chebyshev_step_add(int64_t n, T* xadd, const T* x, const T* xprev
     return launch_ex(pdl, &k_cheb_step_add<T>, blocks_for(n), TPB, 0, s, n, xadd, x, xprev, dinv, d, ax, a, b);
   return cudaGetLastError();
 }
-int64_t mg_spd_scratch(int32_t cap) { return int64_t(GJB) * GJB + 2 * int64_t(GJB) * cap; }
-
-cudaError_t mg_spd_invert(int32_t n, double* A, double* scr, int32_t* bad, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int32_t), s);
-  if (e != cudaSuccess || n <= 0) return e;
-  for (int32_t k0 = 0; k0 < n; k0 += GJB) {
-    const int32_t b = n - k0 < GJB ? n - k0 : GJB;
-    const int64_t copies = int64_t(n - b) * GJB + int64_t(GJB) * n;
-    const unsigned cb = n > b ? unsigned(std::min<int64_t>((copies + TPB - 1) / TPB, 64)) : 0u;
-    k_gj_panel<<<1 + cb, TPB, 0, s>>>(n, k0, b, A, scr, bad);
-    if (n > b) {
-      const dim3 grid(unsigned((n + GJB - 1) / GJB), unsigned((n - b + GJ_ROWS - 1) / GJ_ROWS));
-      k_gj_update<<<grid, TPB, 0, s>>>(n, k0, b, A, scr);
-    }
-  }
-  return cudaGetLastError();
-}
-
 template <typename T>
 cudaError_t mg_coarse(int32_t n, const int32_t* idx, const double* Ainv, const T* d, T* x, cudaStream_t s, bool pdl) {
   if (n <= 0) return cudaSuccess;
@@ -679,9 +535,9 @@ cudaError_t mg_coarse(int32_t n, const int32_t* idx, const double* Ainv, const T
                    Ainv, d, x);
 }
 
-cudaError_t mg_inject_lin(int32_t ns_l, const int32_t* slot_leaf, const double* lin64, int64_t ns_leaf,
-                          double* lev64, float* lev32, cudaStream_t s) {
-  if (ns_l > 0) k_inject_lin<<<blocks_for(ns_l), TPB, 0, s>>>(ns_l, slot_leaf, lin64, ns_leaf, lev64, lev32);
+cudaError_t mg_inject_lin(int32_t nbricks, const LevBrick* bricks, const int32_t* lev_leaf, const double* lin64,
+                          int64_t ns_leaf, double* lev64, float* lev32, cudaStream_t s) {
+  if (nbricks > 0) k_inject_lin<<<unsigned(nbricks), TPB, 0, s>>>(bricks, lev_leaf, lin64, ns_leaf, lev64, lev32);
   return cudaGetLastError();
 }
 cudaError_t mg_level_cmask(int32_t ns_l, const uint8_t* flags, const int32_t* slot_leaf, const uint8_t* leaf_cmask,
@@ -697,47 +553,36 @@ cudaError_t mg_invert_diag(int32_t ns_l, int ncomp, const double* diag, const ui
                                                                 dinv32);
   return cudaGetLastError();
 }
-cudaError_t mg_start_vector(int32_t ns_l, int ncomp, const int32_t* gx, const int32_t* gy, const double* dinv,
-                            double* r, cudaStream_t s) {
-  if (ns_l > 0) k_start_vector<<<blocks_for(ns_l), TPB, 0, s>>>(ns_l, ncomp, gx, gy, dinv, r);
-  return cudaGetLastError();
-}
 cudaError_t dot64(int64_t n, const double* a, const double* b, double* partial, double* out, cudaStream_t s) {
   k_dot_partial<<<DOT_BLOCKS, TPB, 0, s>>>(n, a, b, partial);
   k_dot_final<<<1, TPB, 0, s>>>(DOT_BLOCKS, partial, out);
   return cudaGetLastError();
 }
-cudaError_t cg_update_p(int64_t n, double* p, const double* z, const double* sc, cudaStream_t s) {
-  if (n > 0) k_cg_p<<<blocks_for(n), TPB, 0, s>>>(n, p, z, sc);
-  return cudaGetLastError();
+template <typename Q>
+cudaError_t cg_start(int64_t n, int32_t ns_l, const int32_t* gx, const int32_t* gy, const CgChain<Q>& c, cudaStream_t s) {
+  const unsigned grid = unsigned(std::min<int64_t>(DOT_BLOCKS, std::max<int64_t>(1, (n + TPB - 1) / TPB)));
+  return launch_ex(true, &k_cg<CG_START, Q>, grid, unsigned(TPB), 0, s, n, ns_l, gx, gy, c.dinv, c.r, c.z, c.p, c.pq,
+                   static_cast<const Q*>(c.q), c.sc, c.hist, 0, c.partial, c.count);
 }
-cudaError_t dot_partial64(int64_t n, const double* a, const double* b, double* partial, cudaStream_t s) {
-  k_dot_partial<<<DOT_BLOCKS, TPB, 0, s>>>(n, a, b, partial);
-  return cudaGetLastError();
+template <typename Q>
+cudaError_t cg_step(int64_t n, const CgChain<Q>& c, int step, cudaStream_t s) {
+  const unsigned grid = unsigned(std::min<int64_t>(DOT_BLOCKS, std::max<int64_t>(1, (n + TPB - 1) / TPB)));
+  const int32_t* none = nullptr;
+  cudaError_t e = launch_ex(true, &k_cg<CG_PQ, Q>, grid, unsigned(TPB), 0, s, n, 1, none, none, c.dinv, c.r, c.z, c.p,
+                            c.pq, static_cast<const Q*>(c.q), c.sc, c.hist, step, c.partial, c.count);
+  if (e == cudaSuccess)
+    e = launch_ex(true, &k_cg<CG_RZ, Q>, grid, unsigned(TPB), 0, s, n, 1, none, none, c.dinv, c.r, c.z, c.p, c.pq,
+                  static_cast<const Q*>(c.q), c.sc, c.hist, step, c.partial, c.count);
+  if (e == cudaSuccess)
+    e = launch_ex(true, &k_cg_p<Q>, blocks_for(n), unsigned(TPB), 0, s, n, c.p, c.pq,
+                  static_cast<const double*>(c.z), static_cast<const double*>(c.sc));
+  return e;
 }
-cudaError_t cg_dot_final(const double* partial, double* sc, int slot, double* hist, int step, cudaStream_t s) {
-  k_dot_final_cg<<<1, TPB, 0, s>>>(DOT_BLOCKS, partial, sc, slot, hist, step);
-  return cudaGetLastError();
-}
-cudaError_t cg_update_r_dot(int64_t n, double* r, double* z, const double* q, const double* dinv, const double* sc,
-                            double* partial, cudaStream_t s) {
-  k_cg_r_dot<<<DOT_BLOCKS, TPB, 0, s>>>(n, r, z, q, dinv, sc, partial);
-  return cudaGetLastError();
-}
-cudaError_t cg_init_scalars(double* sc, cudaStream_t s) {
-  k_cg_init<<<1, 32, 0, s>>>(sc);
-  return cudaGetLastError();
-}
+template cudaError_t cg_start<float>(int64_t, int32_t, const int32_t*, const int32_t*, const CgChain<float>&, cudaStream_t);
+template cudaError_t cg_start<double>(int64_t, int32_t, const int32_t*, const int32_t*, const CgChain<double>&, cudaStream_t);
+template cudaError_t cg_step<float>(int64_t, const CgChain<float>&, int, cudaStream_t);
+template cudaError_t cg_step<double>(int64_t, const CgChain<double>&, int, cudaStream_t);
 int mg_dot_partials() { return DOT_BLOCKS; }
-cudaError_t fill64(int64_t n, double* x, double v, cudaStream_t s) {
-  if (n > 0) k_fill64<<<blocks_for(n), TPB, 0, s>>>(n, x, v);
-  return cudaGetLastError();
-}
-cudaError_t copy64(int64_t n, double* dst, const double* src, cudaStream_t s) {
-  if (n > 0) k_copy64<<<blocks_for(n), TPB, 0, s>>>(n, dst, src);
-  return cudaGetLastError();
-}
-
 #define INST(T)                                                                                                \
   template cudaError_t mg_chebyshev_first<T>(int64_t, T*, T*, const T*, const T*, T, cudaStream_t, bool);     \
   template cudaError_t mg_chebyshev_step<T>(int64_t, T*, const T*, const T*, const T*, const T*, const T*, T,  \

@@ -91,24 +91,16 @@ cudaError_t mg_chebyshev_first_res(int64_t n, T* x, T* xprev, T* r, const T* din
 template <typename T>
 cudaError_t mg_chebyshev_step_add(int64_t n, T* xadd, const T* x, const T* xprev, const T* dinv, const T* d,
                                   const T* ax, T a, T b, cudaStream_t s, bool pdl = false);
-// In-place inverse of a dense SPD matrix (n x n, row-major, FP64) by blocked
-// Gauss-Jordan elimination without pivoting (panels of 32 pivots, two launches
-// each): the pivots are the diagonals of successive Schur complements, positive
-// for an SPD matrix.  scr: device scratch of mg_spd_scratch(cap) doubles for any
-// n <= cap.  *bad is set to 1 when a pivot is not positive (the matrix is then
-// not SPD and A holds no inverse); it is cleared first.
-int64_t mg_spd_scratch(int32_t cap);
-cudaError_t mg_spd_invert(int32_t n, double* A, double* scr, int32_t* bad, cudaStream_t s);
-
 // coarse solve x[idx] = Ainv (d[idx]) (dense FP64 inverse over the interior entries)
 template <typename T>
 cudaError_t mg_coarse(int32_t n, const int32_t* idx, const double* Ainv, const T* d, T* x, cudaStream_t s,
                       bool pdl = false);
 
 // ---- set-up kernels
-// level lin (4 blocks of ns_l, double and float) from leaf lin64 (4 blocks of ns_leaf)
-cudaError_t mg_inject_lin(int32_t ns_l, const int32_t* slot_leaf, const double* lin64, int64_t ns_leaf,
-                          double* lev64, float* lev32, cudaStream_t s);
+// every level's lin (4 blocks of its slots at 4 off, double and float) from leaf lin64
+// (4 blocks of ns_leaf); lev_leaf: per level slot (concatenated) its leaf slot or -1
+cudaError_t mg_inject_lin(int32_t nbricks, const LevBrick* bricks, const int32_t* lev_leaf, const double* lin64,
+                          int64_t ns_leaf, double* lev64, float* lev32, cudaStream_t s);
 // level cmask: bits 0,1 Dirichlet, bit 2 active (leaf active at the position, or, below the
 // home level, an active child on the next finer level)
 cudaError_t mg_level_cmask(int32_t ns_l, const uint8_t* flags, const int32_t* slot_leaf, const uint8_t* leaf_cmask,
@@ -117,27 +109,27 @@ cudaError_t mg_level_cmask(int32_t ns_l, const uint8_t* flags, const int32_t* sl
 // dinv = 1 / diag on interior entries (node, not fixed, not edge), else 0; both precisions
 cudaError_t mg_invert_diag(int32_t ns_l, int ncomp, const double* diag, const uint8_t* flags,
                            const uint8_t* cmask, int fixbits0, double* dinv64, float* dinv32, cudaStream_t s);
-// Lanczos start vector on interior entries: 1 + 0.01 * (splitmix64((gx << 32) | gy) mod 1000) / 1000
-cudaError_t mg_start_vector(int32_t ns_l, int ncomp, const int32_t* gx, const int32_t* gy, const double* dinv,
-                            double* r, cudaStream_t s);
 // deterministic dot product: partial sums per block, then one ordered sum -> out[0]
 cudaError_t dot64(int64_t n, const double* a, const double* b, double* partial, double* out, cudaStream_t s);
-// Jacobi-preconditioned CG on device scalars sc[] = {rz, pq, rz_new, alpha, beta, ok}.
-// dot_partial64: the block partial sums of a.b (the grid and order of dot64);
-// cg_dot_final: sc[slot] = their sum, then slot 1 sets alpha, slot 2 beta and
-// hist[2 step], hist[2 step + 1]; cg_update_r_dot: r -= alpha q, z = D^-1 r with
-// the partial sums of r.z; cg_update_p: p = z + beta p.  partial holds
-// mg_dot_partials() doubles.
-cudaError_t cg_update_p(int64_t n, double* p, const double* z, const double* sc, cudaStream_t s);
-cudaError_t dot_partial64(int64_t n, const double* a, const double* b, double* partial, cudaStream_t s);
-cudaError_t cg_dot_final(const double* partial, double* sc, int slot, double* hist, int step, cudaStream_t s);
-cudaError_t cg_update_r_dot(int64_t n, double* r, double* z, const double* q, const double* dinv, const double* sc,
-                            double* partial, cudaStream_t s);
-// CG scalars {rz, pq, rz_new, alpha, beta, ok, -, -} = {0, 0, 0, 0, 0, 1, 0, 0}
-cudaError_t cg_init_scalars(double* sc, cudaStream_t s);
+// Jacobi-preconditioned CG of one set-up chain: FP64 vectors and scalars, the apply q = A p
+// in precision Q on pq (p rounded; p itself in FP64).  hist: per step (alpha_j, beta_j).
+// partial: mg_dot_partials() doubles; count: one unsigned that is 0 between launches.
+template <typename Q>
+struct CgChain {
+  const double* dinv;
+  double *r, *z, *p;
+  Q *pq, *q;
+  double *sc, *hist, *partial;
+  unsigned* count;
+};
+// r = the start vector 1 + 0.01 (splitmix64((gx << 32) | gy) mod 1000) / 1000 on interior
+// entries, p = z = D^-1 r
+template <typename Q>
+cudaError_t cg_start(int64_t n, int32_t ns_l, const int32_t* gx, const int32_t* gy, const CgChain<Q>& c, cudaStream_t s);
+// after q = A pq: alpha, r, z, beta, p
+template <typename Q>
+cudaError_t cg_step(int64_t n, const CgChain<Q>& c, int step, cudaStream_t s);
 // number of per-block partial sums dot64 writes (its partial buffer holds this many doubles)
 int mg_dot_partials();
-cudaError_t fill64(int64_t n, double* x, double v, cudaStream_t s);
-cudaError_t copy64(int64_t n, double* dst, const double* src, cudaStream_t s);
 
 }  // namespace pff

@@ -16,7 +16,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <unordered_map>
 
 #include "solve.cuh"
 #include "state.h"
@@ -102,10 +101,9 @@ int chebyshev_degree(double a, double b, double tol = 1e-3, int cap = 64) {
 
 }  // namespace
 
-// pdl: launched dependent on the preceding kernel of the stream (the V-cycle chain)
+// arguments of a level operator in precision T, but for its vectors
 template <typename T>
-cudaError_t level_apply(pff_mg& mg, int level, int op, const T* x, T* y, cudaStream_t s, bool pdl,
-                        const ChebEpi* ch) {
+static ApplyArgs level_args(pff_mg& mg, int level) {
   pff_problem& pb = *mg.pb;
   const Mesh& M = pb.mesh->m;
   const DevMesh::Level& L = pb.mesh->dev.levels[level];
@@ -116,8 +114,6 @@ cudaError_t level_apply(pff_mg& mg, int level, int op, const T* x, T* y, cudaStr
   a.cmask = mg.cmask + L.lv.off;
   const int64_t n = L.lv.n_slots;
   if (sizeof(T) == 8) a.lin = mg.lin64 + 4 * L.lv.off; else a.lin = mg.lin32 + 4 * L.lv.off;
-  a.xu = x; a.xp = x; a.yu = y; a.yp = y;
-  a.ibuf = nullptr;
   a.n_slots = n;
   for (int l = 0; l <= M.Lf && l < kMaxLevels; ++l) { a.hx[l] = M.tree.hx(l); a.hy[l] = M.tree.hy(l); }
   fill_material(pb.prm, a, pb.has_ecell);
@@ -127,8 +123,17 @@ cudaError_t level_apply(pff_mg& mg, int level, int op, const T* x, T* y, cudaStr
   fill_cell_constants(a, M.Lf + 1);
   a.fe_degree = M.k;
   a.sweep_sh = pb.sweep_sh;
-  a.pdl_in = pdl ? 1 : 0;
   a.mode = MODE_MASK_INPUT;
+  return a;
+}
+
+// pdl: launched dependent on the preceding kernel of the stream (the V-cycle chain)
+template <typename T>
+cudaError_t level_apply(pff_mg& mg, int level, int op, const T* x, T* y, cudaStream_t s, bool pdl,
+                        const ChebEpi* ch) {
+  ApplyArgs a = level_args<T>(mg, level);
+  a.xu = x; a.xp = x; a.yu = y; a.yp = y;
+  a.pdl_in = pdl ? 1 : 0;
   if (ch) a.ch = *ch;
   return launch_apply<T>(a, op, s);
 }
@@ -158,14 +163,79 @@ std::string mg_alloc(pff_mg& mg) {
   mg.su_partial = mg.mem.alloc<double>(int64_t(nchain) * mg_dot_partials());
   mg.su_sc = mg.mem.alloc<double>(8 * nchain);
   mg.su_hist = mg.mem.alloc<double>(2 * kMaxLanczos * nchain);
-  const int Mc = 2 * mg.pb->mesh->m.k + 1;
-  const int64_t n0 = D.levels.empty() ? 0 : D.levels[0].lv.n_slots;
-  mg.probe_len = (2 * 2 + 1 * 1) * Mc * Mc * n0;   // sum over blocks of ncomp^2 Mc^2 n_0
-  mg.probe_in = mg.mem.alloc<double>(std::max<int64_t>(mg.probe_len, 1));
-  mg.probe_out = mg.mem.alloc<double>(std::max<int64_t>(mg.probe_len, 1));
+  mg.su_count = mg.mem.alloc<unsigned>(nchain);
   mg.spd_bad = mg.mem.alloc<int32_t>(2);
   if (!mg.mem.err.empty()) return mg.mem.err;
+  mg.host_len = size_t(2) * kMaxLanczos * nchain;
+  if (cudaMallocHost(reinterpret_cast<void**>(&mg.host), mg.host_len * sizeof(double) + 2 * sizeof(int32_t)) != cudaSuccess) {
+    mg.host = nullptr;
+    return "cudaMallocHost failed";
+  }
+  if (cudaMemset(mg.su_count, 0, nchain * sizeof(unsigned)) != cudaSuccess ||
+      cudaMemset(mg.spd_bad, 0, 2 * sizeof(int32_t)) != cudaSuccess)
+    return "cudaMemset failed";
   return "";
+}
+
+// Tables and buffers of the direct coarse solve, made by the first set-up that needs them:
+// the entries of each block (every component of every level-0 node but Dirichlet ones),
+// the grid's node slots, element matrices, the dense blocks and the inversion's scratch.
+static std::string coarse_alloc(pff_mg& mg) {
+  const Mesh& M = mg.pb->mesh->m;
+  const DevMesh& D = mg.pb->mesh->dev;
+  const LevelMesh& lm = M.levels[0];
+  const int32_t n0 = D.levels[0].lv.n_slots;
+  const int k = M.k, ncx = M.tree.ncx, ncy = M.tree.ncy, nx = k * ncx + 1;
+  std::vector<int32_t> node_slot(size_t(nx) * (k * ncy + 1), 0);
+  for (int32_t s = 0; s < n0; ++s)
+    if (lm.slot_X[s] >= 0) node_slot[size_t(lm.slot_X[s] >> M.Lf) + size_t(nx) * (lm.slot_Y[s] >> M.Lf)] = s;
+  CoarseArgs& a = mg.coarse;
+  std::memset(&a, 0, sizeof(a));
+  for (int b = 0; b < 2; ++b) {
+    MGBlock& B = mg.blk[b];
+    std::vector<int32_t> idx, ent(size_t(B.ncomp) * n0, -1);
+    for (int32_t s = 0; s < n0; ++s)
+      for (int c = 0; c < B.ncomp; ++c)
+        if (lm.slot_X[s] >= 0 && !(b == 0 && (lm.slot_flags[s] & 2))) {
+          ent[size_t(c) * n0 + s] = int32_t(idx.size());
+          idx.push_back(c * n0 + s);
+        }
+    const int nd = (k + 1) * (k + 1) * B.ncomp;
+    CoarseBlock& q = a.b[b];
+    q.n = int32_t(idx.size());
+    q.nc = B.ncomp;
+    q.fix0 = b == 0 ? 1 : 4;
+    B.coarse_idx = mg.mem.alloc<int32_t>(idx.size());
+    q.all = mg.mem.upload(idx);
+    q.idx = B.coarse_idx;
+    q.ent = mg.mem.upload(ent);
+    q.Ke = mg.mem.alloc<double>(size_t(ncx) * ncy * nd * nd);
+    B.coarse_inv = mg.mem.alloc<double>(size_t(q.n) * q.n);
+    q.A = B.coarse_inv;
+    q.scr = mg.mem.alloc<double>(size_t(coarse_scratch(q.n)));
+    B.n_coarse = q.n;
+  }
+  a.k = k; a.ncx = ncx; a.ncy = ncy;
+  a.n0 = n0;
+  a.node_slot = mg.mem.upload(node_slot);
+  a.gx = D.levels[0].gx;
+  a.gy = D.levels[0].gy;
+  a.cmask = mg.cmask;   // level 0 comes first
+  a.bad = mg.spd_bad;
+  mg.coarse_ready = mg.mem.err.empty();
+  return mg.mem.err;
+}
+
+// The direct coarse solve's blocks on stream t: element matrices, assembly, inversion
+static cudaError_t launch_coarse_setup(pff_mg& mg, cudaStream_t t) {
+  const CoarseArgs& a = mg.coarse;
+  const ApplyArgs k = level_args<double>(mg, 0);
+  cudaError_t e = cudaSuccess;
+  for (int b = 0; b < 2 && e == cudaSuccess; ++b)
+    if (a.b[b].n > 0) e = launch_coarse_elements(k, block_op(b), a.ncx, a.ncx * a.ncy, a.node_slot, a.b[b].Ke, t);
+  if (e == cudaSuccess) e = coarse_fill(a, t);
+  if (e == cudaSuccess) e = coarse_invert(a, t);
+  return e;
 }
 
 // Per Newton step: level linearisation, level constraint masks, inverse
@@ -183,61 +253,48 @@ void mg_release_setup_graph(pff_mg& mg) {
 }
 
 // The CG run of one (block, level) chain on stream t.  Its vectors, dot products
-// and coefficients are FP64; the level apply q = A p runs in the V-cycle's
-// precision.  In FP32, p is rounded into and q converted out of two FP32
-// vectors that take the chain's diagonal slot (free once the inverse diagonal is
-// formed): the apply's rounding is relative to its operands, so the small
-// residuals of a converging run keep their accuracy.
-static cudaError_t setup_cg(pff_mg& mg, int b, int l, bool f32, cudaStream_t t) {
+// and coefficients are FP64; the level apply q = A p runs in precision Q.  In FP32, p is
+// rounded into and q read from two FP32 vectors that take the chain's diagonal slot (free
+// once the inverse diagonal is formed): the apply's rounding is relative to its operands,
+// so the small residuals of a converging run keep their accuracy.
+template <typename Q>
+static cudaError_t setup_cg(pff_mg& mg, int b, int l, cudaStream_t t) {
   const DevMesh& D = mg.pb->mesh->dev;
   const int nl = int(D.levels.size());
   const int64_t N = D.lev_total;
   MGBlock& B = mg.blk[b];
   const DevLevel& lv = D.levels[l].lv;
   const int64_t nn = B.ncomp * int64_t(lv.n_slots), o = B.ncomp * lv.off, vs = B.ncomp * N;
-  double* r = mg.su_vec[b] + vs + o;
-  double* z = mg.su_vec[b] + 2 * vs + o;
-  double* p = mg.su_vec[b] + 3 * vs + o;
-  double* q = mg.su_vec[b] + 4 * vs + o;
-  float* p32 = reinterpret_cast<float*>(mg.su_vec[b] + o);
-  float* q32 = p32 + nn;
   const int c = b * nl + l;
-  double* part = mg.su_partial + int64_t(c) * mg_dot_partials();
-  double* sc = mg.su_sc + 8 * c;
-  double* hist = mg.su_hist + 2 * kMaxLanczos * c;
-  const double* dinv = B.dinv64 + o;
-  cudaError_t e = cudaSuccess;
-#define SC(call) do { e = (call); if (e != cudaSuccess) return e; } while (0)
-  SC(mg_start_vector(lv.n_slots, B.ncomp, D.levels[l].gx, D.levels[l].gy, dinv, r, t));
-  SC(fill64(nn, q, 0.0, t));
-  // z = D^-1 r, rz = r.z, p = z
-  SC(cg_init_scalars(sc, t));
-  SC(cg_update_r_dot(nn, r, z, q, dinv, sc, part, t));
-  SC(cg_dot_final(part, sc, 0, hist, 0, t));
-  SC(copy64(nn, p, z, t));
-  for (int j = 0; j < mg.lanczos_steps; ++j) {
-    // q = A p; pq, alpha; r -= alpha q, z = D^-1 r, rz_new, beta; p = z + beta p
-    if (f32) {
-      SC(f64_to_f32(nn, p, p32, t));
-      SC(level_apply<float>(mg, l, block_op(b), p32, q32, t));
-      SC(f32_to_f64(nn, q32, q, t));
-    } else {
-      SC(level_apply<double>(mg, l, block_op(b), p, q, t));
-    }
-    SC(dot_partial64(nn, p, q, part, t));
-    SC(cg_dot_final(part, sc, 1, hist, j, t));
-    SC(cg_update_r_dot(nn, r, z, q, dinv, sc, part, t));
-    SC(cg_dot_final(part, sc, 2, hist, j, t));
-    SC(cg_update_p(nn, p, z, sc, t));
+  CgChain<Q> g;
+  g.dinv = B.dinv64 + o;
+  g.r = mg.su_vec[b] + vs + o;
+  g.z = mg.su_vec[b] + 2 * vs + o;
+  g.p = mg.su_vec[b] + 3 * vs + o;
+  if constexpr (sizeof(Q) == 4) {
+    g.pq = reinterpret_cast<Q*>(mg.su_vec[b] + o);
+    g.q = g.pq + nn;
+  } else {
+    g.pq = g.p;
+    g.q = mg.su_vec[b] + 4 * vs + o;
   }
-#undef SC
+  g.sc = mg.su_sc + 8 * c;
+  g.hist = mg.su_hist + 2 * kMaxLanczos * c;
+  g.partial = mg.su_partial + int64_t(c) * mg_dot_partials();
+  g.count = mg.su_count + c;
+  cudaError_t e = cg_start<Q>(nn, lv.n_slots, D.levels[l].gx, D.levels[l].gy, g, t);
+  const bool q1 = mg.pb->mesh->m.k == 1;   // (the Q2 kernel does not wait for its predecessor)
+  for (int j = 0; j < mg.lanczos_steps && e == cudaSuccess; ++j) {
+    e = level_apply<Q>(mg, l, block_op(b), g.pq, g.q, t, q1);
+    if (e == cudaSuccess) e = cg_step<Q>(nn, g, j, t);
+  }
   return e;
 }
 
-// Launches of the set-up chains (section 1 of mg_setup) on the first K pool
-// streams: one chain per (block, level), finest levels first: the inverse
-// diagonal (FP64, cast to both precisions), then the CG run (its applies in the
-// V-cycle's precision; level 0: FP64).
+// Launches of the set-up chains on the first K pool streams: one chain per (block,
+// level), finest levels first: the inverse diagonal (FP64, cast to both precisions), then
+// the CG run (its applies in the V-cycle's precision; level 0: FP64).  The direct coarse
+// solve's blocks on the extra stream beside them.
 static cudaError_t launch_setup_chains(pff_mg& mg) {
   pff_problem& pb = *mg.pb;
   const DevMesh& D = pb.mesh->dev;
@@ -259,9 +316,10 @@ static cudaError_t launch_setup_chains(pff_mg& mg) {
       if (e != cudaSuccess) return e;
       if (l == 0 && mg.coarse_mode == 0) continue;
       // level 0 (the Chebyshev coarse solver's interval and degree) applies in FP64
-      e = setup_cg(mg, b, l, mg.precision == PFF_F32 && l > 0, t);
+      e = mg.precision == PFF_F32 && l > 0 ? setup_cg<float>(mg, b, l, t) : setup_cg<double>(mg, b, l, t);
       if (e != cudaSuccess) return e;
     }
+  if (mg.coarse_mode == 0) e = launch_coarse_setup(mg, mg.su_stream[K]);
   return e;
 }
 
@@ -291,9 +349,9 @@ static bool capture_setup_chains(pff_mg& mg) {
   if (!mg.cap_stream && cudaStreamCreateWithFlags(&mg.cap_stream, cudaStreamNonBlocking) != cudaSuccess) return false;
   if (cudaStreamBeginCapture(mg.cap_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return false;
   cudaError_t e = cudaEventRecord(mg.su_start, mg.cap_stream);
-  for (int i = 0; i < K && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(mg.su_stream[i], mg.su_start, 0);
+  for (int i = 0; i <= K && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(mg.su_stream[i], mg.su_start, 0);
   if (e == cudaSuccess) e = launch_setup_chains(mg);
-  for (int i = 0; i < K && e == cudaSuccess; ++i) {
+  for (int i = 0; i <= K && e == cudaSuccess; ++i) {
     e = cudaEventRecord(mg.su_done[i], mg.su_stream[i]);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(mg.cap_stream, mg.su_done[i], 0);
   }
@@ -341,23 +399,19 @@ std::string mg_setup(pff_mg& mg, cudaStream_t s) {
   const int64_t nsleaf = M.lay.n_slots;
   const int64_t N = D.lev_total;
   if (mg.lanczos_steps > kMaxLanczos) return "too many Lanczos steps";
-  for (int l = 0; l < nl; ++l) {
-    const DevLevel& lv = D.levels[l].lv;
-    CK(mg_inject_lin(lv.n_slots, lv.slot_leaf, pb.lin64, nsleaf, mg.lin64 + 4 * lv.off, mg.lin32 + 4 * lv.off, s));
-  }
+  CK(mg_inject_lin(D.n_lev_bricks, D.lev_bricks, D.lev_leaf, pb.lin64, nsleaf, mg.lin64, mg.lin32, s));
   for (int l = nl - 1; l >= 0; --l) {
     const DevLevel& lv = D.levels[l].lv;
     const DevLevel* fine = (l + 1 < nl) ? &D.levels[l + 1].lv : nullptr;
     CK(mg_level_cmask(lv.n_slots, lv.flags, lv.slot_leaf, pb.cmask, fine ? fine->R_ptr : nullptr,
                       fine ? fine->R_col : nullptr, fine ? mg.cmask + fine->off : nullptr, mg.cmask + lv.off, s));
   }
-  // 1. One chain per (block, level), finest levels first, spread over the stream
-  //    pool: inverse diagonal, then the Jacobi-preconditioned CG run whose
-  //    coefficients give lambda_max of D^-1 A on the interior (level 0: only for
-  //    the Chebyshev coarse solver).  The chains share no buffer.  From the
-  //    second set-up on they replay as one graph on su_side (re-captured when
-  //    their arguments change); the extra pool stream K takes the second coarse
-  //    inversion below either way.
+  // One chain per (block, level), finest levels first, spread over the stream pool:
+  // inverse diagonal, then the Jacobi-preconditioned CG run whose coefficients give
+  // lambda_max of D^-1 A on the interior (level 0: only for the Chebyshev coarse solver);
+  // on the extra pool stream K the direct coarse solve's blocks.  The chains share no
+  // buffer.  From the second set-up on they replay as one graph on su_side (re-captured
+  // when their arguments change).
   constexpr int K = pff_mg::kSetupStreams;
   if (!mg.su_start) CK(cudaEventCreateWithFlags(&mg.su_start, cudaEventDisableTiming));
   if (!mg.su_chains) CK(cudaEventCreateWithFlags(&mg.su_chains, cudaEventDisableTiming));
@@ -372,6 +426,10 @@ std::string mg_setup(pff_mg& mg, cudaStream_t s) {
     B.c0_a = B.c0_b = 0.0;
     B.c0_deg = 0;
   }
+  if (mg.coarse_mode == 0 && !mg.coarse_ready) {
+    const std::string e = coarse_alloc(mg);
+    if (!e.empty()) return e;
+  }
   bool replay = false;
   if (mg.su_graph_ok && mg.su_setups > 0) {
     std::vector<unsigned char> key = setup_key(mg);
@@ -384,139 +442,31 @@ std::string mg_setup(pff_mg& mg, cudaStream_t s) {
   }
   ++mg.su_setups;
   CK(cudaEventRecord(mg.su_start, s));
-  CK(cudaStreamWaitEvent(mg.su_stream[K], mg.su_start, 0));
   if (replay) {
     CK(cudaStreamWaitEvent(mg.su_side, mg.su_start, 0));
     CK(cudaGraphLaunch(mg.su_exec, mg.su_side));
     CK(cudaEventRecord(mg.su_chains, mg.su_side));
-  } else {
-    for (int i = 0; i < K; ++i) CK(cudaStreamWaitEvent(mg.su_stream[i], mg.su_start, 0));
-    CK(launch_setup_chains(mg));
-  }
-  // 2. Direct coarse solve: the dense level-0 block of each block by probing with
-  //    (2k+1)^2 colours per component (all probes applied in one batch on s, beside
-  //    the chains), assembled on the host and inverted on the device.
-  if (mg.coarse_mode == 0) {
-    const DevMesh::Level& L0 = D.levels[0];
-    const LevelMesh& lm0 = M.levels[0];
-    const int n0 = L0.lv.n_slots;
-    std::vector<uint8_t> cm0(n0);
-    CK(cudaMemcpyAsync(cm0.data(), mg.cmask + L0.lv.off, n0, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    const int k = M.k, Mc = 2 * k + 1;
-    std::unordered_map<int64_t, int32_t> pos;  // (gx, gy) -> slot
-    std::vector<int32_t> gx(n0, -1), gy(n0, -1);
-    for (int q = 0; q < n0; ++q)
-      if (lm0.slot_X[q] >= 0) {
-        gx[q] = lm0.slot_X[q] >> M.Lf;
-        gy[q] = lm0.slot_Y[q] >> M.Lf;
-        pos[(int64_t(gx[q]) << 32) | gy[q]] = q;
-      }
-    // probe (b, c, cy, cx) at probe_base[b] + ((c * Mc + cy) * Mc + cx) * ncomp_b * n0
-    int64_t probe_base[2];
-    probe_base[0] = 0;
-    probe_base[1] = int64_t(mg.blk[0].ncomp) * mg.blk[0].ncomp * Mc * Mc * n0;
-    if (probe_base[1] + int64_t(mg.blk[1].ncomp) * mg.blk[1].ncomp * Mc * Mc * n0 > mg.probe_len)
-      return "coarse probe buffer too small";
-    std::vector<double> probes(size_t(mg.probe_len), 0.0), resp(size_t(mg.probe_len));
-    for (int b = 0; b < 2; ++b) {
-      const int nc = mg.blk[b].ncomp;
-      for (int c = 0; c < nc; ++c)
-        for (int cy = 0; cy < Mc; ++cy)
-          for (int cx = 0; cx < Mc; ++cx) {
-            double* pr = probes.data() + probe_base[b] + ((c * Mc + cy) * Mc + cx) * int64_t(nc) * n0;
-            for (int q = 0; q < n0; ++q)
-              if (gx[q] >= 0 && gx[q] % Mc == cx && gy[q] % Mc == cy) pr[size_t(c) * n0 + q] = 1.0;
-          }
-    }
-    CK(cudaMemcpyAsync(mg.probe_in, probes.data(), probes.size() * sizeof(double), cudaMemcpyHostToDevice, s));
-    for (int b = 0; b < 2; ++b) {
-      const int nc = mg.blk[b].ncomp;
-      for (int pi = 0; pi < nc * Mc * Mc; ++pi) {
-        const int64_t off = probe_base[b] + pi * int64_t(nc) * n0;
-        CK(level_apply<double>(mg, 0, block_op(b), mg.probe_in + off, mg.probe_out + off, s));
-      }
-    }
-    CK(cudaMemcpyAsync(resp.data(), mg.probe_out, resp.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    std::vector<double> A[2];
-    std::vector<int32_t> eidx[2];
-    for (int b = 0; b < 2; ++b) {
-      MGBlock& B = mg.blk[b];
-      const int nc = B.ncomp;
-      std::vector<int32_t> ent_of(size_t(nc) * n0, -1);   // interior entries (comp * n0 + slot)
-      for (int q = 0; q < n0; ++q)
-        for (int c = 0; c < nc; ++c) {
-          const int bit = B.fixbits == 4 ? 4 : (1 << c);
-          if (gx[q] >= 0 && !(cm0[q] & bit)) {
-            ent_of[size_t(c) * n0 + q] = int32_t(eidx[b].size());
-            eidx[b].push_back(c * n0 + q);
-          }
-        }
-      const int nI = int(eidx[b].size());
-      A[b].assign(size_t(nI) * nI, 0.0);
-      for (int c = 0; c < nc; ++c)
-        for (int cy = 0; cy < Mc; ++cy)
-          for (int cx = 0; cx < Mc; ++cx) {
-            const double* yv = resp.data() + probe_base[b] + ((c * Mc + cy) * Mc + cx) * int64_t(nc) * n0;
-            for (int q = 0; q < n0; ++q) {
-              if (gx[q] < 0) continue;
-              // the probed node within distance k of q in each direction
-              const int jx = gx[q] - k + ((cx - (gx[q] - k)) % Mc + Mc) % Mc;
-              const int jy = gy[q] - k + ((cy - (gy[q] - k)) % Mc + Mc) % Mc;
-              auto it = pos.find((int64_t(jx) << 32) | jy);
-              if (it == pos.end()) continue;
-              const int32_t col = ent_of[size_t(c) * n0 + it->second];
-              if (col < 0) continue;
-              for (int cr = 0; cr < nc; ++cr) {
-                const int32_t row = ent_of[size_t(cr) * n0 + q];
-                if (row < 0) continue;
-                A[b][size_t(row) * nI + col] = yv[size_t(cr) * n0 + q];
-              }
-            }
-          }
-      if (!B.coarse_idx || nI > B.coarse_cap) {
-        const int32_t cap = std::max(nI, 1);
-        B.coarse_idx = mg.mem.alloc<int32_t>(cap);
-        B.coarse_inv = mg.mem.alloc<double>(int64_t(cap) * cap);
-        B.coarse_rc = mg.mem.alloc<double>(mg_spd_scratch(cap));
-        if (!mg.mem.err.empty()) return mg.mem.err;
-        B.coarse_cap = cap;
-      }
-      B.n_coarse = nI;
-    }
-    // the two inversions run side by side (block 1 on the extra pool stream)
-    for (int b = 0; b < 2; ++b) {
-      MGBlock& B = mg.blk[b];
-      cudaStream_t t = b == 0 ? s : mg.su_stream[K];
-      CK(cudaMemsetAsync(mg.spd_bad + b, 0, sizeof(int32_t), t));
-      if (B.n_coarse == 0) continue;
-      CK(cudaMemcpyAsync(B.coarse_idx, eidx[b].data(), B.n_coarse * sizeof(int32_t), cudaMemcpyHostToDevice, t));
-      CK(cudaMemcpyAsync(B.coarse_inv, A[b].data(), A[b].size() * sizeof(double), cudaMemcpyHostToDevice, t));
-      CK(mg_spd_invert(B.n_coarse, B.coarse_inv, B.coarse_rc, mg.spd_bad + b, t));
-    }
-  }
-  // 3. join the chains and the pool, read the CG coefficients (and coarse status) once
-  if (replay) {
     CK(cudaStreamWaitEvent(s, mg.su_chains, 0));
-    CK(cudaEventRecord(mg.su_done[K], mg.su_stream[K]));
-    CK(cudaStreamWaitEvent(s, mg.su_done[K], 0));
   } else {
+    for (int i = 0; i <= K; ++i) CK(cudaStreamWaitEvent(mg.su_stream[i], mg.su_start, 0));
+    CK(launch_setup_chains(mg));
     for (int i = 0; i <= K; ++i) {
       CK(cudaEventRecord(mg.su_done[i], mg.su_stream[i]));
       CK(cudaStreamWaitEvent(s, mg.su_done[i], 0));
     }
   }
-  std::vector<double> hist(size_t(2) * nl * 2 * kMaxLanczos);
-  int32_t bad[2] = {0, 0};
-  CK(cudaMemcpyAsync(hist.data(), mg.su_hist, hist.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
-  if (mg.coarse_mode == 0) CK(cudaMemcpyAsync(bad, mg.spd_bad, sizeof(bad), cudaMemcpyDeviceToHost, s));
+  // the CG coefficients and the coarse status in one host read (pinned)
+  double* hist = mg.host;
+  int32_t* bad = reinterpret_cast<int32_t*>(mg.host + mg.host_len);
+  bad[0] = bad[1] = 0;
+  CK(cudaMemcpyAsync(hist, mg.su_hist, mg.host_len * sizeof(double), cudaMemcpyDeviceToHost, s));
+  if (mg.coarse_mode == 0) CK(cudaMemcpyAsync(bad, mg.spd_bad, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   if (bad[0] || bad[1]) return "coarse level block is not positive definite";
   for (int b = 0; b < 2; ++b)
     for (int l = 0; l < nl; ++l) {
       if (l == 0 && mg.coarse_mode == 0) continue;
-      eigen_from_cg(mg, mg.blk[b], l, hist.data() + size_t(b * nl + l) * 2 * kMaxLanczos);
+      eigen_from_cg(mg, mg.blk[b], l, hist + size_t(b * nl + l) * 2 * kMaxLanczos);
     }
   mg.ready = true;
   return "";

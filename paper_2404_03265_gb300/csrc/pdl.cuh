@@ -21,10 +21,10 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // Launch of kernel `fn` on stream s, programmatically dependent on the launch
 // before it in the stream when pdl is set.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_ex(bool pdl, void (*fn)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
-                      Args&&... args) {
+cudaError_t launch_grid(bool pdl, void (*fn)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,
+                        Args&&... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -34,6 +34,16 @@ cudaError_t launch_ex(bool pdl, void (*fn)(KArgs...), unsigned grid, unsigned bl
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, fn, std::forward<Args>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_ex2(bool pdl, void (*fn)(KArgs...), dim3 grid, unsigned block, cudaStream_t s, Args&&... args) {
+  return launch_grid(pdl, fn, grid, block, 0, s, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_ex(bool pdl, void (*fn)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                      Args&&... args) {
+  return launch_grid(pdl, fn, dim3(grid), block, smem, s, std::forward<Args>(args)...);
 }
 
 }  // namespace pff

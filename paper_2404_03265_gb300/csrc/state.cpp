@@ -212,7 +212,6 @@ std::string upload_mesh(pff_mesh& pm) {
       L.lv.ntiles = int32_t(tiles.size());
     }
     L.lv.flags = D.mem.upload(lm.slot_flags);
-    L.lv.slot_leaf = D.mem.upload(lm.slot_leaf);
     std::vector<float> pv(lm.P_val.begin(), lm.P_val.end()), rv(lm.R_val.begin(), lm.R_val.end());
     if (l > 0) {
       L.lv.P_ptr = D.mem.upload(lm.P_ptr);
@@ -235,19 +234,23 @@ std::string upload_mesh(pff_mesh& pm) {
     L.cell_child = D.mem.upload(lm.cell_child);
   }
   D.lev_total = off;
-  if (M.k == 1) {
+  {
     std::vector<LevBrick> lb;
-    std::vector<int32_t> home(size_t(off), -1);
+    std::vector<int32_t> home(size_t(off), -1), leaf;
+    leaf.reserve(size_t(off));
     for (size_t l = 0; l < M.levels.size(); ++l) {
       const LevelMesh& lm = M.levels[l];
       const DevLevel& lv = D.levels[l].lv;
       for (size_t b = 0; b < lm.lay.bricks.size(); ++b)
         lb.push_back({int32_t(lv.off), lv.n_slots, int32_t(b) * lm.lay.NB * lm.lay.NB});
+      leaf.insert(leaf.end(), lm.slot_leaf.begin(), lm.slot_leaf.end());
       for (size_t i = 0; i < lm.copy_leaf.size(); ++i) home[size_t(lv.off) + lm.copy_level[i]] = lm.copy_leaf[i];
     }
     D.lev_bricks = D.mem.upload(lb);
     D.n_lev_bricks = int32_t(lb.size());
     D.home_leaf = D.mem.upload(home);
+    D.lev_leaf = D.mem.upload(leaf);
+    for (auto& L : D.levels) L.lv.slot_leaf = D.lev_leaf ? D.lev_leaf + L.lv.off : nullptr;
   }
   {
     // each free leaf node is on the copy list of exactly one level (its home)

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/pff.h"
+#include "coarse.cuh"
 #include "kernels.cuh"
 #include "mesh.h"
 #include "mg.cuh"
@@ -94,10 +95,11 @@ struct DevMesh {
   };
   std::vector<Level> levels;
   int64_t lev_total = 0;     // sum of level slot counts
-  // Q1: the bricks of all levels in storage order, and per level slot its leaf slot
-  // when this is the node's home level (else -1)
+  // the bricks of all levels in storage order; per level slot (concatenated) the leaf slot
+  // at its position (-1: hole), and the same where this is the node's home level (else -1)
   LevBrick* lev_bricks = nullptr;
   int32_t n_lev_bricks = 0;
+  int32_t* lev_leaf = nullptr;
   int32_t* home_leaf = nullptr;
   DevHome home;              // per leaf slot: its home level (copy in and out of the V-cycle)
   void release() {
@@ -213,10 +215,9 @@ struct MGBlock {
   std::vector<double> lam;         // lambda_max estimate per level (level 0: only with the Chebyshev coarse solver)
   double c0_a = 0.0, c0_b = 0.0;   // Chebyshev coarse solver: interval [0.9 lambda_min, 1.2 lambda_max] on level 0
   int c0_deg = 0;                  // and its degree
-  int32_t n_coarse = 0, coarse_cap = 0;
-  int32_t* coarse_idx = nullptr;   // level-0 entries (comp * n_0 + slot) of the coarse interior
+  int32_t n_coarse = 0;
+  int32_t* coarse_idx = nullptr;   // level-0 entries (comp * n_0 + slot) of the coarse block
   double* coarse_inv = nullptr;    // dense FP64 inverse, n_coarse^2
-  double* coarse_rc = nullptr;     // scratch of the inversion: panel inverse, old pivot columns and rows
 };
 
 }  // namespace pff
@@ -238,7 +239,7 @@ struct pff_mg {
   // form an independent chain; the chains run on a pool of streams.  FP64 scratch:
   // per block 5 level vectors (diag, r, z, p, q) of ncomp * lev_total, per chain
   // the dot partials, 8 CG scalars and 2 * 64 CG coefficients.
-  static constexpr int kSetupStreams = 8;   // the extra stream inverts the second coarse block
+  static constexpr int kSetupStreams = 16;  // the extra stream takes the coarse blocks
   cudaStream_t su_stream[kSetupStreams + 1] = {};
   cudaEvent_t su_done[kSetupStreams + 1] = {};
   cudaEvent_t su_start = nullptr;
@@ -253,9 +254,12 @@ struct pff_mg {
   bool su_graph_ok = true;
   double* su_vec[2] = {nullptr, nullptr};
   double *su_partial = nullptr, *su_sc = nullptr, *su_hist = nullptr;
-  // coarse probing: all colours of both blocks at once (in and out, probe_len doubles each)
-  double *probe_in = nullptr, *probe_out = nullptr;
-  int64_t probe_len = 0;
+  unsigned* su_count = nullptr;    // per chain: finished blocks of a dot (0 between launches)
+  // the direct coarse solve's blocks (made by the first set-up that needs them)
+  bool coarse_ready = false;
+  pff::CoarseArgs coarse = {};
+  double* host = nullptr;          // pinned: CG coefficients (host_len doubles), then the coarse status
+  size_t host_len = 0;
   bool ready = false;
   // V-cycles replayed as CUDA graphs, captured after each set-up: graph 0 and 1 one
   // block each, graph 2 both (the phi block on a forked branch beside the u block).
