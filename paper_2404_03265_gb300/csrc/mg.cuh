@@ -26,12 +26,6 @@ struct DevLevel {
   int32_t ntiles = 0, tile = 0;       // their number and nodes per side
 };
 
-// A brick of the concatenated level storage (900 slots): its level's slot offset
-// and slot count, and the brick's first slot on its level.
-struct LevBrick {
-  int32_t off, n, base;
-};
-
 // Home level of each leaf slot: a free leaf node's defect enters, and its
 // correction leaves, the coarsest level among its leaf cells.  Per leaf slot:
 // that level's slot offset in the concatenated level storage, its slot on that

@@ -164,6 +164,7 @@ std::string mg_alloc(pff_mg& mg) {
   mg.su_sc = mg.mem.alloc<double>(8 * nchain);
   mg.su_hist = mg.mem.alloc<double>(2 * kMaxLanczos * nchain);
   mg.su_count = mg.mem.alloc<unsigned>(nchain);
+  for (int b = 0; b < 2; ++b) mg.su_part[b] = mg.mem.alloc<double>(512 * D.levels.size());
   mg.spd_bad = mg.mem.alloc<int32_t>(2);
   if (!mg.mem.err.empty()) return mg.mem.err;
   mg.host_len = size_t(2) * kMaxLanczos * nchain;
@@ -171,6 +172,12 @@ std::string mg_alloc(pff_mg& mg) {
     mg.host = nullptr;
     return "cudaMallocHost failed";
   }
+  for (int b = 0; b < 2; ++b)   // slots without a node keep a zero inverse diagonal, CG vectors zero there
+    if (cudaMemset(mg.su_vec[b], 0, 5 * mg.blk[b].ncomp * N * sizeof(double)) != cudaSuccess) return "cudaMemset failed";
+  for (int b = 0; b < 2; ++b)
+    if (cudaMemset(mg.blk[b].dinv64, 0, mg.blk[b].ncomp * N * sizeof(double)) != cudaSuccess ||
+        cudaMemset(mg.blk[b].dinv32, 0, mg.blk[b].ncomp * N * sizeof(float)) != cudaSuccess)
+      return "cudaMemset failed";
   if (cudaMemset(mg.su_count, 0, nchain * sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(mg.spd_bad, 0, 2 * sizeof(int32_t)) != cudaSuccess)
     return "cudaMemset failed";
@@ -291,35 +298,88 @@ static cudaError_t setup_cg(pff_mg& mg, int b, int l, cudaStream_t t) {
   return e;
 }
 
-// Launches of the set-up chains on the first K pool streams: one chain per (block,
-// level), finest levels first: the inverse diagonal (FP64, cast to both precisions), then
-// the CG run (its applies in the V-cycle's precision; level 0: FP64).  The direct coarse
-// solve's blocks on the extra stream beside them.
+// Arguments of the tiled set-up of block b (setup.cu)
+static SetupArgs setup_args(pff_mg& mg, int b) {
+  pff_problem& pb = *mg.pb;
+  const Mesh& M = pb.mesh->m;
+  const DevMesh& D = pb.mesh->dev;
+  const int nl = int(D.levels.size());
+  const MGBlock& B = mg.blk[b];
+  const int64_t vs = B.ncomp * D.lev_total;
+  ApplyArgs k;
+  std::memset(&k, 0, sizeof(k));
+  for (int l = 0; l <= M.Lf && l < kMaxLevels; ++l) { k.hx[l] = M.tree.hx(l); k.hy[l] = M.tree.hy(l); }
+  fill_material(pb.prm, k, pb.has_ecell);
+  fill_cell_constants(k, M.Lf + 1);
+  SetupArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.tiles = D.setup_tiles; a.ntiles = D.n_setup_tiles;
+  a.flags = D.lev_flags; a.cmask = mg.cmask;
+  a.lin64 = mg.lin64; a.lin32 = mg.lin32;
+  a.ecell64 = pb.has_ecell ? pb.lev_ecell64 : nullptr;
+  a.ecell32 = pb.has_ecell ? pb.lev_ecell32 : nullptr;
+  a.gx = D.lev_gx; a.gy = D.lev_gy;
+  a.dinv64 = B.dinv64; a.dinv32 = B.dinv32;
+  a.q = reinterpret_cast<float*>(mg.su_vec[b]);
+  a.r = mg.su_vec[b] + vs;
+  a.z = mg.su_vec[b] + 2 * vs;
+  a.p[0] = mg.su_vec[b] + 3 * vs;
+  a.p[1] = mg.su_vec[b] + 4 * vs;
+  a.sc = mg.su_sc + 8 * b * nl;
+  a.hist = mg.su_hist + 2 * kMaxLanczos * b * nl;
+  a.hist_stride = 2 * kMaxLanczos;
+  a.partial = mg.su_part[b];
+  a.count = mg.su_count + b * nl;
+  a.tile1 = nl > 1 ? D.levels[1].tile0 : a.ntiles;
+  for (int l = 0; l < nl; ++l) {
+    a.off[l] = int32_t(D.levels[l].lv.off);
+    a.n[l] = D.levels[l].lv.n_slots;
+    a.dot0[l + 1] = a.dot0[l] + (l == 0 ? 0 : setup_dot_blocks(B.ncomp * int64_t(a.n[l])));
+  }
+  for (int l = nl; l < kMaxLevels; ++l) a.dot0[l + 1] = a.dot0[nl];
+  a.mf = k.mf; a.md = k.md;
+  for (int l = 0; l < kMaxLevels; ++l) { a.gf[l] = k.gf[l]; a.gd[l] = k.gd[l]; }
+  return a;
+}
+
+// Launches of the set-up chains on the pool streams: inverse diagonals (FP64, cast to both
+// precisions) and CG runs (applies in the V-cycle's precision; level 0, for the Chebyshev
+// coarse solver: FP64); on the extra stream K the direct coarse solve's blocks.
+//  - FP32, Q1, default cell loop: all levels of a block in shared launches (setup.cu).
+//  - else one chain per (block, level), finest levels first, spread over the pool.
 static cudaError_t launch_setup_chains(pff_mg& mg) {
   pff_problem& pb = *mg.pb;
   const DevMesh& D = pb.mesh->dev;
   const int nl = int(D.levels.size());
   constexpr int K = pff_mg::kSetupStreams;
   cudaError_t e = cudaSuccess;
-  int chain = 0;
-  for (int l = nl - 1; l >= 0; --l)
-    for (int b = 0; b < 2; ++b, ++chain) {
-      cudaStream_t t = mg.su_stream[chain % K];
-      MGBlock& B = mg.blk[b];
-      const DevLevel& lv = D.levels[l].lv;
-      const int64_t o = B.ncomp * lv.off;
-      double* diag = mg.su_vec[b] + o;
-      e = level_apply<double>(mg, l, block_diag_op(b), diag, diag, t);
-      if (e == cudaSuccess)
-        e = mg_invert_diag(lv.n_slots, B.ncomp, diag, lv.flags, mg.cmask + lv.off, B.fixbits, B.dinv64 + o,
-                           B.dinv32 + o, t);
-      if (e != cudaSuccess) return e;
-      if (l == 0 && mg.coarse_mode == 0) continue;
-      // level 0 (the Chebyshev coarse solver's interval and degree) applies in FP64
-      e = mg.precision == PFF_F32 && l > 0 ? setup_cg<float>(mg, b, l, t) : setup_cg<double>(mg, b, l, t);
-      if (e != cudaSuccess) return e;
+  if (mg.precision == PFF_F32 && pb.mesh->m.k == 1 && pb.sweep_sh == 0) {
+    for (int b = 0; b < 2 && e == cudaSuccess; ++b) {
+      const SetupArgs a = setup_args(mg, b);
+      e = launch_setup_diag(a, block_op(b), mg.su_stream[b]);
+      if (e == cudaSuccess) e = launch_setup_cg(a, block_op(b), mg.lanczos_steps, mg.su_stream[b]);
+      if (e == cudaSuccess && mg.coarse_mode != 0) e = setup_cg<double>(mg, b, 0, mg.su_stream[b]);
     }
-  if (mg.coarse_mode == 0) e = launch_coarse_setup(mg, mg.su_stream[K]);
+  } else {
+    int chain = 0;
+    for (int l = nl - 1; l >= 0; --l)
+      for (int b = 0; b < 2; ++b, ++chain) {
+        cudaStream_t t = mg.su_stream[chain % K];
+        MGBlock& B = mg.blk[b];
+        const DevLevel& lv = D.levels[l].lv;
+        const int64_t o = B.ncomp * lv.off;
+        double* diag = mg.su_vec[b] + o;
+        e = level_apply<double>(mg, l, block_diag_op(b), diag, diag, t);
+        if (e == cudaSuccess)
+          e = mg_invert_diag(lv.n_slots, B.ncomp, diag, lv.flags, mg.cmask + lv.off, B.fixbits, B.dinv64 + o,
+                             B.dinv32 + o, t);
+        if (e != cudaSuccess) return e;
+        if (l == 0 && mg.coarse_mode == 0) continue;
+        e = mg.precision == PFF_F32 && l > 0 ? setup_cg<float>(mg, b, l, t) : setup_cg<double>(mg, b, l, t);
+        if (e != cudaSuccess) return e;
+      }
+  }
+  if (e == cudaSuccess && mg.coarse_mode == 0) e = launch_coarse_setup(mg, mg.su_stream[K]);
   return e;
 }
 
@@ -406,8 +466,7 @@ std::string mg_setup(pff_mg& mg, cudaStream_t s) {
     CK(mg_level_cmask(lv.n_slots, lv.flags, lv.slot_leaf, pb.cmask, fine ? fine->R_ptr : nullptr,
                       fine ? fine->R_col : nullptr, fine ? mg.cmask + fine->off : nullptr, mg.cmask + lv.off, s));
   }
-  // One chain per (block, level), finest levels first, spread over the stream pool:
-  // inverse diagonal, then the Jacobi-preconditioned CG run whose coefficients give
+  // Inverse diagonals, then the Jacobi-preconditioned CG runs whose coefficients give
   // lambda_max of D^-1 A on the interior (level 0: only for the Chebyshev coarse solver);
   // on the extra pool stream K the direct coarse solve's blocks.  The chains share no
   // buffer.  From the second set-up on they replay as one graph on su_side (re-captured

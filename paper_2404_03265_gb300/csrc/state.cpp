@@ -211,7 +211,6 @@ std::string upload_mesh(pff_mesh& pm) {
       L.lv.tiles = D.mem.upload(tiles);
       L.lv.ntiles = int32_t(tiles.size());
     }
-    L.lv.flags = D.mem.upload(lm.slot_flags);
     std::vector<float> pv(lm.P_val.begin(), lm.P_val.end()), rv(lm.R_val.begin(), lm.R_val.end());
     if (l > 0) {
       L.lv.P_ptr = D.mem.upload(lm.P_ptr);
@@ -221,13 +220,6 @@ std::string upload_mesh(pff_mesh& pm) {
       L.lv.R_col = D.mem.upload(lm.R_col);
       L.lv.R_val = D.mem.upload(rv);
     }
-    std::vector<int32_t> gx(lm.slot_X.size()), gy(lm.slot_Y.size());
-    for (size_t q = 0; q < gx.size(); ++q) {
-      gx[q] = lm.slot_X[q] < 0 ? -1 : (lm.slot_X[q] >> (M.Lf - int(l)));
-      gy[q] = lm.slot_Y[q] < 0 ? -1 : (lm.slot_Y[q] >> (M.Lf - int(l)));
-    }
-    L.gx = D.mem.upload(gx);
-    L.gy = D.mem.upload(gy);
     L.n_cells = int32_t(lm.cell_dst.size());
     L.cell_dst = D.mem.upload(lm.cell_dst);
     L.cell_src = D.mem.upload(lm.cell_src);
@@ -236,21 +228,46 @@ std::string upload_mesh(pff_mesh& pm) {
   D.lev_total = off;
   {
     std::vector<LevBrick> lb;
-    std::vector<int32_t> home(size_t(off), -1), leaf;
-    leaf.reserve(size_t(off));
+    std::vector<int32_t> home(size_t(off), -1), leaf, gx, gy;
+    std::vector<uint8_t> flags;
+    std::vector<SmoothTile> tiles;
+    leaf.reserve(size_t(off)); gx.reserve(size_t(off)); gy.reserve(size_t(off)); flags.reserve(size_t(off));
     for (size_t l = 0; l < M.levels.size(); ++l) {
       const LevelMesh& lm = M.levels[l];
       const DevLevel& lv = D.levels[l].lv;
       for (size_t b = 0; b < lm.lay.bricks.size(); ++b)
         lb.push_back({int32_t(lv.off), lv.n_slots, int32_t(b) * lm.lay.NB * lm.lay.NB});
       leaf.insert(leaf.end(), lm.slot_leaf.begin(), lm.slot_leaf.end());
+      flags.insert(flags.end(), lm.slot_flags.begin(), lm.slot_flags.end());
+      for (size_t q = 0; q < lm.slot_X.size(); ++q) {
+        gx.push_back(lm.slot_X[q] < 0 ? -1 : (lm.slot_X[q] >> (M.Lf - int(l))));
+        gy.push_back(lm.slot_Y[q] < 0 ? -1 : (lm.slot_Y[q] >> (M.Lf - int(l))));
+      }
+      if (M.k == 1) {
+        D.levels[l].tile0 = int32_t(tiles.size());
+        for (SmoothTile t : smooth_tiles(lm, lm, kSetupTile)) {
+          t.pad = int32_t(l);
+          tiles.push_back(t);
+        }
+      }
       for (size_t i = 0; i < lm.copy_leaf.size(); ++i) home[size_t(lv.off) + lm.copy_level[i]] = lm.copy_leaf[i];
     }
     D.lev_bricks = D.mem.upload(lb);
     D.n_lev_bricks = int32_t(lb.size());
     D.home_leaf = D.mem.upload(home);
     D.lev_leaf = D.mem.upload(leaf);
-    for (auto& L : D.levels) L.lv.slot_leaf = D.lev_leaf ? D.lev_leaf + L.lv.off : nullptr;
+    D.lev_flags = D.mem.upload(flags);
+    D.lev_gx = D.mem.upload(gx);
+    D.lev_gy = D.mem.upload(gy);
+    if (M.k == 1) D.setup_tiles = D.mem.upload(tiles);
+    D.n_setup_tiles = int32_t(tiles.size());
+    if (D.mem.err.empty())
+      for (auto& L : D.levels) {
+        L.lv.slot_leaf = D.lev_leaf + L.lv.off;
+        L.lv.flags = D.lev_flags + L.lv.off;
+        L.gx = D.lev_gx + L.lv.off;
+        L.gy = D.lev_gy + L.lv.off;
+      }
   }
   {
     // each free leaf node is on the copy list of exactly one level (its home)

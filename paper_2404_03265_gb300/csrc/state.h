@@ -88,6 +88,7 @@ struct DevMesh {
     DevLevel lv;
     int32_t* gx = nullptr;   // level-grid coordinates (units h_l / k), -1 for holes
     int32_t* gy = nullptr;
+    int32_t tile0 = 0;       // first of the level's set-up tiles
     int32_t n_cells = 0;     // cells of this level and their per-cell value sources
     int32_t* cell_dst = nullptr;
     int32_t* cell_src = nullptr;
@@ -100,6 +101,10 @@ struct DevMesh {
   LevBrick* lev_bricks = nullptr;
   int32_t n_lev_bricks = 0;
   int32_t* lev_leaf = nullptr;
+  uint8_t* lev_flags = nullptr;    // and every level's flags and grid coordinates
+  int32_t *lev_gx = nullptr, *lev_gy = nullptr;
+  SmoothTile* setup_tiles = nullptr;   // Q1: tiles of all levels (setup.cu), level l from levels[l].tile0
+  int32_t n_setup_tiles = 0;
   int32_t* home_leaf = nullptr;
   DevHome home;              // per leaf slot: its home level (copy in and out of the V-cycle)
   void release() {
@@ -254,6 +259,7 @@ struct pff_mg {
   bool su_graph_ok = true;
   double* su_vec[2] = {nullptr, nullptr};
   double *su_partial = nullptr, *su_sc = nullptr, *su_hist = nullptr;
+  double* su_part[2] = {nullptr, nullptr};   // tiled set-up: per block the dots' parts
   unsigned* su_count = nullptr;    // per chain: finished blocks of a dot (0 between launches)
   // the direct coarse solve's blocks (made by the first set-up that needs them)
   bool coarse_ready = false;
