@@ -43,10 +43,13 @@ __device__ __forceinline__ void q1_cell(const NodePair<P>& b, const NodePair<P>&
   P rux[4] = {zero, zero, zero, zero}, ruy[4] = {zero, zero, zero, zero}, rp[4] = {zero, zero, zero, zero};
   const P ihx = bc<P>(g.ihx), ihy = bc<P>(g.ihy);
   const P c2ml = pmul(bc<P>(m.c2ml), ec), cl = pmul(bc<P>(m.cl), ec), cm = pmul(bc<P>(m.cm), ec), omk = bc<P>(m.omk);
-  // du_x/dy + du_y/dx at a Gauss point: FP64 forms the first product inside the sum
-  // (its rate is the limit), FP32 rounds it (the level operators' V-cycles)
+  // du_x/dy + du_y/dx at a Gauss point.  FP64's rate is the limit: here, and in the
+  // sums of two products below, the first product is formed inside the sum (always
+  // this one, so that every path over the cells gives the same bits).  FP32 rounds
+  // both, as the level operators' V-cycles do.
+  constexpr bool f64 = sizeof(T) == 8;
   auto shear = [&](const PField<P>& f, int q1, const P* xy, P yx) {
-    return sizeof(T) == 8 ? pfma(f.deta[q1], ihy, yx) : padd(xy[q1], yx);
+    return f64 ? pfma(f.deta[q1], ihy, yx) : padd(xy[q1], yx);
   };
   // ---- linearisation
   PField<P> fux, fuy, fphi, fphit;
@@ -86,7 +89,7 @@ __device__ __forceinline__ void q1_cell(const NodePair<P>& b, const NodePair<P>&
     //   A_phi(psi) = ((1-kappa) phi sigma(u):e(u) + 2 p phi div u - G_c/l (1 - phi), psi)
     //                + G_c l (grad phi, grad psi)
     // MASS: (1, psi);  TCV: (u . grad phi, psi)
-    P S11[2][2], S12[2][2], S22[2][2], fv[2][2];
+    P S11[2][2], S12[2][2], S22[2][2], fv[2][2], G[2][2], U12[2][2];
     P uxq[2][2], uyq[2][2];
     if (OP == OP_TCV) { fux.values(b.lx, uxq); fuy.values(b.ly, uyq); }
 #pragma unroll
@@ -109,6 +112,7 @@ __device__ __forceinline__ void q1_cell(const NodePair<P>& b, const NodePair<P>&
         S11[q1][q2] = pfma(gq, s11, pt2);
         S22[q1][q2] = pfma(gq, s22, pt2);
         S12[q1][q2] = pmul(gq, s12);
+        G[q1][q2] = gq; U12[q1][q2] = s12;
         const P se = pfma(s11, e11[q2], pfma(s22, e22[q1], pmul(s12, ge12)));
         const P ph = phiq[q1][q2];
         // (1-kappa) phi se + 2 p phi div u - G_c/l (1 - phi)
@@ -117,9 +121,12 @@ __device__ __forceinline__ void q1_cell(const NodePair<P>& b, const NodePair<P>&
       }
     const P wx = bc<P>(g.wx), wy = bc<P>(g.wy), nwx = bc<P>(-g.wx), nwy = bc<P>(-g.wy);
     if (OP == OP_RESID) {
-      ptest_grad(padd(S11[0][0], S11[1][0]), padd(S11[0][1], S11[1][1]),
-                 padd(S12[0][0], S12[0][1]), padd(S12[1][0], S12[1][1]), wx, wy, nwx, nwy, rux);
-      ptest_grad(padd(S12[0][0], S12[1][0]), padd(S12[0][1], S12[1][1]),
+      auto sum = [&](int a, int b, int c, int d) {
+        return f64 ? pfma(G[a][b], U12[a][b], S12[c][d]) : padd(S12[a][b], S12[c][d]);
+      };
+      ptest_grad(padd(S11[0][0], S11[1][0]), padd(S11[0][1], S11[1][1]), sum(0, 0, 0, 1), sum(1, 1, 1, 0), wx, wy, nwx,
+                 nwy, rux);
+      ptest_grad(sum(0, 0, 1, 0), sum(0, 1, 1, 1),
                  padd(S22[0][0], S22[0][1]), padd(S22[1][0], S22[1][1]), wx, wy, nwx, nwy, ruy);
       ptest_grad(fphi.dxi[0], fphi.dxi[1], fphi.deta[0], fphi.deta[1], bc<P>(g.wpx), bc<P>(g.wpy), bc<P>(-g.wpx),
                  bc<P>(-g.wpy), rp);
@@ -236,12 +243,13 @@ __device__ __forceinline__ void q1_cell(const NodePair<P>& b, const NodePair<P>&
 #pragma unroll
           for (int A = 0; A < 4; ++A) {
             const T dx = dxs[A] * g.ihx, dyy = dys[A] * g.ihy;
-            rp[A] = padd(rp[A], pmul(bc<P>(g.jxw), pfma(mq, bc<P>(Ns[A] * Ns[A]), bc<P>(m.gcL * (dx * dx + dyy * dyy)))));
+            const P w = pfma(mq, bc<P>(Ns[A] * Ns[A]), bc<P>(m.gcL * (dx * dx + dyy * dyy)));
+            rp[A] = f64 ? pfma(bc<P>(g.jxw), w, rp[A]) : padd(rp[A], pmul(bc<P>(g.jxw), w));
           }
         }
       }
   } else {
-    P S11[2][2], S12[2][2], S22[2][2], fv[2][2];
+    P S11[2][2], S12[2][2], S22[2][2], fv[2][2], G[2][2], U11[2][2], U12[2][2], U22[2][2];
     // q = (1-kappa) sigma(u) + p I, so that the phi rows' coefficients are
     //   (1-kappa) sigma(u):e(u) + 2 p div u + G_c/l = q : e(u) + p div u + G_c/l,
     //   2 phi ((1-kappa) sigma(u) + p I) = 2 phi q
@@ -269,9 +277,11 @@ __device__ __forceinline__ void q1_cell(const NodePair<P>& b, const NodePair<P>&
         }
         if (N::xu) {
           const P gxy = shear(fxu, q1, bxy, cyx[q2]);
-          P s11 = pmul(gq, pfma(c2ml, ax[q2], pmul(cl, dy[q1])));
-          P s22 = pmul(gq, pfma(cl, ax[q2], pmul(c2ml, dy[q1])));
-          P s12 = pmul(gq, pmul(cm, gxy));
+          const P t11 = pfma(c2ml, ax[q2], pmul(cl, dy[q1])), t22 = pfma(cl, ax[q2], pmul(c2ml, dy[q1])), t12 = pmul(cm, gxy);
+          P s11 = pmul(gq, t11);
+          P s22 = pmul(gq, t22);
+          P s12 = pmul(gq, t12);
+          G[q1][q2] = gq; U11[q1][q2] = t11; U22[q1][q2] = t22; U12[q1][q2] = t12;
           if (OP == OP_FULL_T) {
             s11 = pfma(xpq[q1][q2], T11, s11);
             s22 = pfma(xpq[q1][q2], T22, s22);
@@ -283,7 +293,15 @@ __device__ __forceinline__ void q1_cell(const NodePair<P>& b, const NodePair<P>&
         if (N::xp && OP != OP_FULL) fv[q1][q2] = pmul(mq, xpq[q1][q2]);
       }
     const P wx = bc<P>(g.wx), wy = bc<P>(g.wy), nwx = bc<P>(-g.wx), nwy = bc<P>(-g.wy);
-    if (N::xu) {
+    if (f64 && OP == OP_FULL) {
+      auto sum = [&](const P (*U)[2], const P (*S)[2], int a, int b, int c, int d) {
+        return pfma(G[a][b], U[a][b], S[c][d]);
+      };
+      ptest_grad(sum(U11, S11, 0, 0, 1, 0), sum(U11, S11, 0, 1, 1, 1), sum(U12, S12, 0, 0, 0, 1),
+                 sum(U12, S12, 1, 1, 1, 0), wx, wy, nwx, nwy, rux);
+      ptest_grad(sum(U12, S12, 0, 0, 1, 0), sum(U12, S12, 0, 1, 1, 1), sum(U22, S22, 0, 0, 0, 1),
+                 sum(U22, S22, 1, 0, 1, 1), wx, wy, nwx, nwy, ruy);
+    } else if (N::xu) {
       // u_x test: (S11, S12) . grad psi;  u_y test: (S12, S22) . grad psi
       ptest_grad(padd(S11[0][0], S11[1][0]), padd(S11[0][1], S11[1][1]),
                  padd(S12[0][0], S12[0][1]), padd(S12[1][0], S12[1][1]), wx, wy, nwx, nwy, rux);

@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(TPB) k_gram_schmidt(int64_t n, int k, const do
     if (tid < jn) partial[int64_t(j0 + tid) * gridDim.x + blockIdx.x] = sh[tid][0];
     __syncthreads();
   }
-  // the last block adds the blocks' partials: a warp per vector, fixed order
+  // the last block adds the blocks' partials: a warp per vector, fixed order,
   __threadfence();
   if (tid == 0) last = atomicAdd(count, 1u) == gridDim.x - 1;
   __syncthreads();
@@ -332,8 +332,21 @@ __global__ void __launch_bounds__(TPB) k_gram_schmidt(int64_t n, int k, const do
   if (tid == 0) *count = 0u;   // for the next launch
   const int lane = tid & 31;
   for (int j = tid >> 5; j < nj; j += TPB / 32) {
-    double acc = 0.0;
-    for (unsigned b = lane; b < gridDim.x; b += 32) acc += __ldcg(partial + int64_t(j) * gridDim.x + b);
+    // as a tree over TPB sums of two blocks each, lane + 32 i of them in this lane
+    static_assert(TPB == 256 && RED_BLOCKS <= 2 * TPB, "");
+    const double* p = partial + int64_t(j) * gridDim.x;
+    double a[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const unsigned b = lane + 32 * i;
+      a[i] = b < gridDim.x ? __ldcg(p + b) : 0.0;
+      if (b + TPB < gridDim.x) a[i] += __ldcg(p + b + TPB);
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+      for (int i = 0; i < o; ++i) a[i] += a[i + o];
+    double acc = a[0];
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     if (lane == 0) out[j] = acc;
   }
