@@ -157,9 +157,10 @@ pff_status pff_extrapolate_phi(pff_problem* pb, const double* phi_prev, const do
  * sweeps a strip of 2 * strip_half_rows node rows of a 30 x 30 brick, its lower
  * and upper halves side by side.  strip_half_rows: 15 (one strip per brick), 5
  * or 1 (3 or 15 shorter strips: more warps for small level meshes of the
- * V-cycle), or 0 (default: chosen per call from the number of bricks).  It acts
- * on the Jacobian (pff_apply) and the multigrid level block operators; the other
- * Q1 operators always use 15; Q2 meshes ignore it.  V-cycles captured by an
+ * V-cycle), or 0 (default: chosen per call; the FP64 and the smaller FP32 Jacobians
+ * then go cell by cell in two passes, and FP32 V-cycles and set-ups take tiles of the
+ * levels in place of strips).  It acts on the Jacobian (pff_apply) and the multigrid
+ * level block operators; the other Q1 operators and Q2 meshes ignore it.  V-cycles captured by an
  * earlier pff_mg_setup keep their shape until the next one.
  * Errors: PFF_ERR_INVALID_ARG for other values.                               */
 pff_status pff_set_cell_loop(pff_problem* pb, int32_t strip_half_rows);
@@ -175,12 +176,10 @@ pff_status pff_set_cell_loop(pff_problem* pb, int32_t strip_half_rows);
  * arithmetic (PFF_F32: applies, smoothing and transfers in FP32).
  * pff_mg_setup uses the problem's current state and active set (call it after
  * pff_set_state / pff_set_active); it synchronises the stream.  Its per-level
- * work (inverse diagonals, eigenvalue estimates) runs on an internal pool of
- * streams that is joined back into `stream` before it returns (from the second
- * set-up on, replayed as one captured graph while the material, the modulus, the
- * cell-loop shape and the coarse mode are unchanged); the level-0 blocks are
- * assembled by probing and inverted on the device (blocked Gauss-Jordan, two
- * launches per 32 pivots).
+ * work (inverse diagonals, eigenvalue estimates, the level-0 blocks' assembly and
+ * inversion) runs on an internal pool of streams that is joined back into `stream`
+ * before it returns (from the second set-up on, replayed as one captured graph while
+ * the material, the modulus, the cell-loop shape and the coarse mode are unchanged).
  * pff_vcycle: z = MG(r) for one block; fixed leaf DoFs (Dirichlet u, active phi)
  * get z = r, hanging entries and holes 0.  r and z are device vectors.          */
 pff_status pff_mg_create(pff_problem* pb, int32_t precision, pff_mg** out);

@@ -145,39 +145,17 @@ __device__ __forceinline__ void q2_point(const Q2Point<T>& q, const MatConst<T>&
     se = s11 * q.uxx + s22 * q.uyy + s12 * ge12;
     mq = m.omk * se + m.p2 * (q.uxx + q.uyy) + m.gcl;
   }
-  if constexpr (OP == OP_FULL || OP == OP_FULL_T || OP == OP_UU) {
+  if constexpr (OP == OP_UU) {
     const T bc = q.bxy + q.cyx;
-    T S11 = gq * (c2ml * q.ax + cl * q.dy);
-    T S22 = gq * (cl * q.ax + c2ml * q.dy);
-    T S12 = gq * (cm * bc);
-    if constexpr (OP == OP_FULL || OP == OP_FULL_T) {
-      const T tp = q.phi + q.phi;
-      const T T11 = tp * (m.omk * s11 + m.p), T22 = tp * (m.omk * s22 + m.p), T12 = tp * (m.omk * s12);
-      if constexpr (OP == OP_FULL) {
-        c.f0[2] = T11 * q.ax + T22 * q.dy + T12 * bc + mq * q.xp;
-      } else {
-        S11 += q.xp * T11;
-        S22 += q.xp * T22;
-        S12 += q.xp * T12;
-        c.f0[2] = mq * q.xp;
-      }
-      c.fx[2] = m.gcL * q.xpx;
-      c.fy[2] = m.gcL * q.xpy;
-    }
+    const T S11 = gq * (c2ml * q.ax + cl * q.dy);
+    const T S22 = gq * (cl * q.ax + c2ml * q.dy);
+    const T S12 = gq * (cm * bc);
     c.fx[0] = S11; c.fy[0] = S12;
     c.fx[1] = S12; c.fy[1] = S22;
   } else if constexpr (OP == OP_PP) {
     c.f0[2] = mq * q.xp;
     c.fx[2] = m.gcL * q.xpx;
     c.fy[2] = m.gcL * q.xpy;
-  } else if constexpr (OP == OP_RESID) {
-    // R = -A(U)(psi), Problem 2 (sigma^+ read as sigma); the sign is applied by the caller
-    const T pt2 = m.p * q.phit * q.phit;
-    c.fx[0] = gq * s11 + pt2; c.fy[0] = gq * s12;
-    c.fx[1] = gq * s12;       c.fy[1] = gq * s22 + pt2;
-    c.f0[2] = m.omk * q.phi * se + m.p2 * q.phi * (q.uxx + q.uyy) + m.gcl * (q.phi - T(1));
-    c.fx[2] = m.gcL * q.phix;
-    c.fy[2] = m.gcL * q.phiy;
   } else if constexpr (OP == OP_MASS) {
     c.f0[2] = T(1);
   } else if constexpr (OP == OP_TCV) {
@@ -328,10 +306,6 @@ __device__ __forceinline__ void q2_cell(const Load& ld, const MatConst<T>& m, co
           rp[A] += tb.L[b][q2] * Rvp[a] + tb.D[b][q2] * Rep[a];
         }
     }
-  }
-  if constexpr (OP == OP_RESID) {
-#pragma unroll
-    for (int k = 0; k < 9; ++k) { ru[k] = pmul(pbc(T(-1)), ru[k]); rp[k] = -rp[k]; }
   }
   if constexpr (OP == OP_VJP) {
     cell[0] = -cell[0]; cell[1] = -cell[1]; cell[2] = -cell[2];
@@ -520,7 +494,7 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
     P ru[9];
     T rp[9], cell[3];
     if (act) {
-      if constexpr (OP == OP_FULL || OP == OP_FULL_T || OP == OP_RESID)
+      if constexpr (OP == OP_FULL || OP == OP_FULL_T)
         if (a.ecell == nullptr) q2_jac<T, OP, false>(node, q2mat<T>(a), Q2Own<T>(mc, geom<T>(a, level), T(1)), ru, rp);
         else q2_jac<T, OP, true>(node, q2mat<T>(a), Q2Own<T>(mc, geom<T>(a, level), ec), ru, rp);
       else
@@ -631,27 +605,27 @@ cudaError_t launch_apply_q2(const ApplyArgs& a, int op, cudaStream_t s) {
     const int full = resident_blocks(fn, Q2T, smem);
     return unsigned(a.lay.nbricks < full ? a.lay.nbricks : full);
   };
-  switch (op) {
-#define PFF_LAUNCH2(OPV)                                                                       \
-    case OPV: {                                                                                \
-      const void* fn = reinterpret_cast<const void*>(&apply_q2_kernel<T, OPV>);               \
-      apply_q2_kernel<T, OPV><<<grid_of(fn), Q2T, smem, s>>>(a);                               \
-      break;                                                                                   \
+  auto go = [&](auto fn) {
+    fn<<<grid_of(reinterpret_cast<const void*>(fn)), Q2T, smem, s>>>(a);
+    return cudaGetLastError();
+  };
+  if constexpr (sizeof(T) == 8) {   // formed in FP64 only
+    switch (op) {
+      case OP_UU_DIAG: return go(&apply_q2_kernel<T, OP_UU_DIAG>);
+      case OP_PP_DIAG: return go(&apply_q2_kernel<T, OP_PP_DIAG>);
+      case OP_MASS: return go(&apply_q2_kernel<T, OP_MASS>);
+      case OP_TCV: return go(&apply_q2_kernel<T, OP_TCV>);
+      case OP_TCV_GRAD: return go(&apply_q2_kernel<T, OP_TCV_GRAD>);
+      case OP_VJP: return go(&apply_q2_kernel<T, OP_VJP>);
+      case OP_PHIT_VJP: return go(&apply_q2_kernel<T, OP_PHIT_VJP>);
+      default: break;
     }
-    PFF_LAUNCH2(OP_FULL)
-    PFF_LAUNCH2(OP_FULL_T)
-    PFF_LAUNCH2(OP_UU)
-    PFF_LAUNCH2(OP_PP)
-    PFF_LAUNCH2(OP_UU_DIAG)
-    PFF_LAUNCH2(OP_PP_DIAG)
-    PFF_LAUNCH2(OP_RESID)
-    PFF_LAUNCH2(OP_MASS)
-    PFF_LAUNCH2(OP_TCV)
-    PFF_LAUNCH2(OP_TCV_GRAD)
-    PFF_LAUNCH2(OP_VJP)
-    PFF_LAUNCH2(OP_PHIT_VJP)
-#undef PFF_LAUNCH2
+  }
+  switch (op) {
+    case OP_FULL: return go(&apply_q2_kernel<T, OP_FULL>);
+    case OP_FULL_T: return go(&apply_q2_kernel<T, OP_FULL_T>);
+    case OP_UU: return go(&apply_q2_kernel<T, OP_UU>);
+    case OP_PP: return go(&apply_q2_kernel<T, OP_PP>);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }

@@ -12,7 +12,7 @@
 // cell rows, with most of the chip idle.  One tile per block needs one round trip
 // per level and direction, and the halo's extra cells (1.8x down, 1.5x up) cost
 // idle issue slots.  Measured (u block, 1.04M-DoF crack mesh, 13 levels): 101 launches
-// and 482 us before, 29 launches and 172 us with the tiles.
+// and 482 us before; 29 launches and 135 us with the tiles.
 //
 // Arithmetic: every cell, nodal sum, smoother step and transfer row is the
 // expression and order of sweep_q1_kernel, k_restrict and k_prolong (the transfer
