@@ -71,10 +71,6 @@ struct LeafCells {
   const int4* node = nullptr;
   const int4* part = nullptr;       // the same per partial sum of the fix-up list
   const uint8_t* part_pos = nullptr;   // Q2: parity of the partial's brick position, column | row << 1
-  // Q1: the regular bricks; the others; and the cell pairs that the others' nodes sum
-  const BrickDesc* reg = nullptr;
-  const int32_t *irr = nullptr, *pair = nullptr;
-  int32_t nreg = 0, nirr = 0, npairs = 0;
   void* out = nullptr;              // 12 (Q2: 27) blocks of ncells: the contributions (3 * node + component)
 };
 
@@ -213,11 +209,6 @@ template <>
 cudaError_t launch_leaf_cells<double>(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);
 template <>
 cudaError_t launch_leaf_cells<float>(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);
-
-// OP_FULL and OP_FULL_T in FP32 on large meshes: the regular bricks in tiles (leaf_tiles.cu), the
-// others' nodes in two passes.  launch_leaf_tiles: that first part, between the two passes.
-cudaError_t launch_leaf_mixed(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);
-cudaError_t launch_leaf_tiles(const ApplyArgs& a, int op, bool after, cudaStream_t s);
 
 // The same for Q2 in FP64 (leaf_cells_q2.cu): OP_FULL, OP_FULL_T, OP_RESID.
 cudaError_t launch_leaf_cells_q2(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);

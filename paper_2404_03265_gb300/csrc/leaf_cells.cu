@@ -28,7 +28,6 @@ namespace {
 
 constexpr int CELL_TPB = 128;
 constexpr int NODE_TPB = 256;
-constexpr int SLOTS = 900;   // of a brick
 
 // Kernel arguments, in the precision T of the pass (small ones: they are copied per launch).
 template <typename T>
@@ -48,8 +47,6 @@ struct CellArgs {
 template <typename T>
 struct NodeArgs {
   int32_t nc;
-  const int32_t* irr;   // bricks to take, or all slots
-  int32_t nirr;
   int mode;
   int64_t n;
   const T* out;
@@ -142,9 +139,7 @@ __global__ void __launch_bounds__(CELL_TPB) leaf_cell_kernel(const __grid_consta
   constexpr int M = sizeof(T) == 4 ? 2 : 1;
   using P = typename std::conditional<M == 2, float2, T>::type;
   const int32_t nc = a.lc.ncells;
-  int32_t c = blockIdx.x * CELL_TPB + threadIdx.x;
-  if (a.lc.pair != nullptr) c = c < a.lc.npairs ? __ldg(a.lc.pair + c) : nc;   // some of the pairs
-  c *= M;
+  const int32_t c = M * (blockIdx.x * CELL_TPB + threadIdx.x);
   int4 k[M];
   int lev, cs[M];
 #pragma unroll
@@ -199,11 +194,7 @@ template <typename T, int OP>
 __global__ void __launch_bounds__(NODE_TPB) leaf_node_kernel(const __grid_constant__ NodeArgs<T> a) {
   constexpr int C0 = Out<OP>::c0;
   pdl_trigger();
-  int64_t s = int64_t(blockIdx.x) * NODE_TPB + threadIdx.x;
-  if (a.irr != nullptr) {   // the slots of some bricks
-    const int32_t b = int32_t(s) / SLOTS;
-    s = b < a.nirr ? int64_t(__ldg(a.irr + b)) * SLOTS + int32_t(s) % SLOTS : a.n;
-  }
+  const int64_t s = int64_t(blockIdx.x) * NODE_TPB + threadIdx.x;
   // everything but the contributions was there before pass 1 let this launch start
   int4 k = make_int4(-1, -1, -1, -1);
   uint32_t cm = 0;
@@ -245,11 +236,10 @@ __global__ void __launch_bounds__(NODE_TPB) leaf_node_kernel(const __grid_consta
 }
 
 template <typename T, int OP>
-cudaError_t launch_op(const ApplyArgs& a, const FixupArgs& f, cudaStream_t s, bool mixed = false) {
+cudaError_t launch_op(const ApplyArgs& a, const FixupArgs& f, cudaStream_t s) {
   if (a.lc.ncells <= 0 || a.n_slots <= 0) return cudaSuccess;
   CellArgs<T> c;
   c.lc = a.lc;
-  if (!mixed) c.lc.pair = nullptr;
   c.hang = a.hang;
   c.cmask = a.cmask;
   c.lin = static_cast<const T*>(a.lin);
@@ -261,8 +251,6 @@ cudaError_t launch_op(const ApplyArgs& a, const FixupArgs& f, cudaStream_t s, bo
   constants<T>(c, a);
   NodeArgs<T> n;
   n.nc = a.lc.ncells;
-  n.irr = mixed ? a.lc.irr : nullptr;
-  n.nirr = a.lc.nirr;
   n.mode = a.mode;
   n.n = a.n_slots;
   n.out = static_cast<const T*>(a.lc.out);
@@ -277,15 +265,9 @@ cudaError_t launch_op(const ApplyArgs& a, const FixupArgs& f, cudaStream_t s, bo
   // it reads or writes a vector); under a capture that may not be a kernel
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   const bool pdl = cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
-  cudaError_t e = cudaSuccess;
-  const unsigned tpb = CELL_TPB;
-  if (mixed && a.lc.nirr <= 0) return launch_leaf_tiles(a, OP, false, s);
-  e = launch_ex(pdl, &leaf_cell_kernel<T, OP>, unsigned(((mixed ? a.lc.npairs : nt) + tpb - 1) / tpb), tpb, 0, s, c);
-  if (e == cudaSuccess && mixed) e = launch_leaf_tiles(a, OP, true, s);
+  const cudaError_t e = launch_ex(pdl, &leaf_cell_kernel<T, OP>, unsigned((nt + CELL_TPB - 1) / CELL_TPB),
+                                  unsigned(CELL_TPB), 0, s, c);
   if (e != cudaSuccess) return e;
-  if (mixed)
-    return launch_ex(true, &leaf_node_kernel<T, OP>, unsigned((a.lc.nirr * SLOTS + NODE_TPB - 1) / NODE_TPB),
-                     unsigned(NODE_TPB), 0, s, n);
   return launch_ex(true, &leaf_node_kernel<T, OP>, unsigned((a.n_slots + NODE_TPB - 1) / NODE_TPB), unsigned(NODE_TPB),
                    0, s, n);
 }
@@ -313,12 +295,6 @@ cudaError_t launch_leaf_cells<float>(const ApplyArgs& a, const FixupArgs& f, int
     case OP_FULL_T: return launch_op<float, OP_FULL_T>(a, f, s);
     default: return cudaErrorInvalidValue;
   }
-}
-
-cudaError_t launch_leaf_mixed(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s) {
-  if (op == OP_FULL) return launch_op<float, OP_FULL>(a, f, s, true);
-  if (op == OP_FULL_T) return launch_op<float, OP_FULL_T>(a, f, s, true);
-  return cudaErrorInvalidValue;
 }
 
 }  // namespace pff

@@ -126,46 +126,18 @@ static LeafCells upload_leaf_cells(DevAllocs& mem, const Mesh& M) {
   L.slot = mem.upload(slot);
   L.node = mem.upload(node);
   L.part = mem.upload(part);
-  if (k == 1) {
-    std::vector<BrickDesc> reg;
-    std::vector<int32_t> irr, pair;
-    std::vector<uint8_t> need(nc / 2, 0);
-    auto take = [&](int4 q) {
-      for (int32_t c : {q.x, q.y, q.z, q.w})
-        if (c >= 0) need[c / 2] = 1;
-    };
-    for (size_t b = 0; b < M.lay.bricks.size(); ++b) {
-      if (M.lay.bricks[b].irr < 0) { reg.push_back(M.lay.bricks[b]); continue; }
-      irr.push_back(int32_t(b));
-      for (size_t s = b * size_t(NB) * NB; s < (b + 1) * size_t(NB) * NB; ++s) {
-        if (node[s].x >= -1) { take(node[s]); continue; }
-        const size_t i = size_t(-2 - node[s].x);
-        for (int32_t e = M.fix_ptr[i]; e < M.fix_ptr[i + 1]; ++e) take(part[M.fix_part[e]]);
-      }
-    }
-    for (size_t p = 0; p < need.size(); ++p)
-      if (need[p]) pair.push_back(int32_t(p));
-    L.reg = mem.upload(reg);
-    L.irr = mem.upload(irr);
-    L.pair = mem.upload(pair);
-    L.nreg = int32_t(reg.size());
-    L.nirr = int32_t(irr.size());
-    L.npairs = int32_t(pair.size());
-  }
   return L;
 }
 
 // A leaf operator and its fix-up: Q1 in two passes over the cell and node lists where
 // that is the faster path (leaf_cells.cu), else the cell loop and the fix-up kernel.
 //  - FP64: always two passes (bound by the FP64 rate, and they evaluate only cells that
-//    exist): Jacobian 992 -> 741 us on 4.1M DoFs, 633 -> 199 us on the 1.04M-DoF crack
+//    exist): Jacobian 992 -> 741 us on 4.1M DoFs, 633 -> 204 us on the 1.04M-DoF crack
 //    mesh, 45 -> 22 us on 4.3k DoFs.  A forced strip height asks for the sweep's Jacobian.
 //  - FP32: two passes up to kTwoPassCells, while the 48 bytes of contributions per cell
 //    stay small beside L2: 13.1 -> 11.1 us on 65k DoFs, 30.7 -> 19.6 us on the crack mesh,
 //    26.6 -> 22.0 us at 0.53M cells, but 31.1 -> 34.0 us at 0.77M and 37.9 -> 61 us at
-//    1.36M (the sweep writes no contributions to memory).  Larger meshes take their regular
-//    bricks in tiles and only the others in two passes (leaf_tiles.cu): 24.5 us at 0.73M
-//    cells, 38.9 -> 36.2 us at 1.36M.
+//    1.36M (the sweep writes no contributions to memory).
 constexpr int32_t kTwoPassCells = 650000;
 static bool use_two_passes(const ApplyArgs& a, int op, bool f64) {
   if (op == OP_VJP || a.lc.out == nullptr) return false;
@@ -179,9 +151,6 @@ template <typename T>
 cudaError_t launch_leaf(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s) {
   if (use_two_passes(a, op, sizeof(T) == 8))
     return a.fe_degree == 1 ? launch_leaf_cells<T>(a, f, op, s) : launch_leaf_cells_q2(a, f, op, s);
-  if constexpr (sizeof(T) == 4)
-    if (a.fe_degree == 1 && a.sweep_sh == 0 && a.lc.out != nullptr && a.lc.nreg > 0 && (op == OP_FULL || op == OP_FULL_T))
-      return launch_leaf_mixed(a, f, op, s);
   const cudaError_t e = launch_apply<T>(a, op, s);
   if (e != cudaSuccess || op == OP_VJP) return e;   // OP_VJP: per-cell outputs only
   return launch_fixup<T>(f, s);
