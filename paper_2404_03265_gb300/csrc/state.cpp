@@ -132,7 +132,7 @@ static LeafCells upload_leaf_cells(DevAllocs& mem, const Mesh& M) {
 // A leaf operator and its fix-up: Q1 in two passes over the cell and node lists where
 // that is the faster path (leaf_cells.cu), else the cell loop and the fix-up kernel.
 //  - FP64: always two passes (bound by the FP64 rate, and they evaluate only cells that
-//    exist): Jacobian 992 -> 741 us on 4.1M DoFs, 633 -> 204 us on the 1.04M-DoF crack
+//    exist): Jacobian 992 -> 741 us on 4.1M DoFs, 633 -> 199 us on the 1.04M-DoF crack
 //    mesh, 45 -> 22 us on 4.3k DoFs.  A forced strip height asks for the sweep's Jacobian.
 //  - FP32: two passes up to kTwoPassCells, while the 48 bytes of contributions per cell
 //    stay small beside L2: 13.1 -> 11.1 us on 65k DoFs, 30.7 -> 19.6 us on the crack mesh,
