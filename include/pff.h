@@ -137,7 +137,12 @@ pff_status pff_set_active(pff_problem* pb, const uint8_t* active, void* stream);
  * free (not Dirichlet, not active, not hanging) DoFs; I_fixed: identity on
  * Dirichlet u and active phi DoFs.  precision PFF_F64: double vectors, PFF_F32:
  * float vectors (state cast to float).  xu/yu: 2*n_slots, xp/yp: n_slots.
- * x and y must not overlap.                                                    */
+ * x and y must not overlap.
+ * Concurrency: on a mesh without refinement edges (n_hanging = 0) an apply writes
+ * nothing but y, so applies of one problem may run at the same time on several
+ * streams and from several threads.  On other meshes the applies of one precision
+ * (FP64: and the solver calls) share scratch of the problem and must be ordered; an
+ * FP32 and an FP64 apply may still run at the same time.                         */
 pff_status pff_apply(pff_problem* pb, int32_t precision, int32_t op, const void* xu, const void* xp,
                      void* yu, void* yp, void* stream);
 
@@ -157,9 +162,9 @@ pff_status pff_extrapolate_phi(pff_problem* pb, const double* phi_prev, const do
  * sweeps a strip of 2 * strip_half_rows node rows of a 30 x 30 brick, its lower
  * and upper halves side by side.  strip_half_rows: 15 (one strip per brick), 5
  * or 1 (3 or 15 shorter strips: more warps for small level meshes of the
- * V-cycle), or 0 (default: chosen per call; the FP64 and the smaller FP32 Jacobians
- * then go cell by cell in two passes, and FP32 V-cycles and set-ups take tiles of the
- * levels in place of strips).  It acts on the Jacobian (pff_apply) and the multigrid
+ * V-cycle), or 0 (default: chosen per call; on meshes with refinement edges the FP64
+ * and the smaller FP32 Jacobians then go cell by cell in two passes, and FP32 V-cycles
+ * and set-ups take tiles of the levels in place of strips).  It acts on the Jacobian (pff_apply) and the multigrid
  * level block operators; the other Q1 operators and Q2 meshes ignore it.  V-cycles captured by an
  * earlier pff_mg_setup keep their shape until the next one.
  * Errors: PFF_ERR_INVALID_ARG for other values.                               */

@@ -244,6 +244,7 @@ extern "C" void pff_problem_destroy(pff_problem* pb) {
   if (pb->gm_read) cudaEventDestroy(pb->gm_read);
   release_workspace(pb->ws);
   pb->bufs.release();
+  if (pb->cells64_late) cudaFree(pb->cells64_late);
   delete pb;
 }
 

@@ -34,7 +34,7 @@ cudaError_t leaf_op(pff_problem& pb, int kop, int mode, const double* lin, const
   std::memset(&a, 0, sizeof(a));
   a.lay = D.leaf;
   a.lc = D.cells;
-  a.lc.out = pb.cell_buf;
+  if (kop != OP_VJP) a.lc.out = leaf_contributions64(pb);
   a.hang = D.hang;
   a.cmask = cmask;
   a.lin = lin;
@@ -106,6 +106,7 @@ std::string ensure_workspace(pff_problem& pb, int restart) {
   W.x32 = W.mem.alloc<float>(n3);
   W.y32 = W.mem.alloc<float>(n3);
   if (!W.mem.err.empty()) return W.mem.err;
+  if (!leaf_contributions64(pb)) return "workspace: out of device memory for the cells' contributions";
   if (cudaMallocHost(reinterpret_cast<void**>(&W.host), (3 * size_t(restart + 1) + 8) * sizeof(double)) != cudaSuccess) {
     W.host = nullptr;
     return "workspace: cudaMallocHost failed";

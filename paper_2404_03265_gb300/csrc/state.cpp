@@ -138,7 +138,41 @@ static LeafCells upload_leaf_cells(DevAllocs& mem, const Mesh& M) {
 //    stay small beside L2: 13.1 -> 11.1 us on 65k DoFs, 30.7 -> 19.6 us on the crack mesh,
 //    26.6 -> 22.0 us at 0.53M cells, but 31.1 -> 34.0 us at 0.77M and 37.9 -> 61 us at
 //    1.36M (the sweep writes no contributions to memory).
+// Without a buffer of contributions (see below) the Jacobian takes the cell loop.
 constexpr int32_t kTwoPassCells = 650000;
+
+// Who may use the contributions.  An apply of the caller (pff_apply) on a mesh without
+// refinement edges keeps to the cell loop, which writes nothing but the result: such
+// applies of one problem may run at the same time on several streams and from several
+// threads.  On other meshes applies of one precision share partial sums and hanging inputs
+// anyway, and the contributions have a buffer per precision as those have.  The operators
+// inside a solver call share the solver's workspace and may always use the FP64 buffer.
+static bool refinement_edges(const DevMesh& D) { return D.nhang > 0 || D.nfix > 0; }
+
+// Contributions of the FP64 operators: with the problem while they are small, larger ones
+// (FP32 applies never read them: 131 MB on 4.1M Q1 DoFs) on first use.
+constexpr size_t kCellsWithProblem = size_t(64) << 20;
+static size_t cell_values(const pff_problem& pb) {
+  return (pb.mesh->m.k == 1 ? 12 : 27) * size_t(pb.mesh->dev.cells.ncells);
+}
+
+double* leaf_contributions64(pff_problem& pb) {
+  std::lock_guard<std::mutex> lk(pb.cells_mu);
+  if (pb.cells64) return pb.cells64;
+  // a stream of the caller may be capturing, and this memory is no part of its graph
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  void* p = nullptr;
+  const cudaError_t e = cudaMalloc(&p, std::max<size_t>(cell_values(pb), 1) * sizeof(double));
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;   // the Jacobian then takes the cell loop
+  }
+  pb.cells64 = pb.cells64_late = static_cast<double*>(p);
+  return pb.cells64;
+}
+
 static bool use_two_passes(const ApplyArgs& a, int op, bool f64) {
   if (op == OP_VJP || a.lc.out == nullptr) return false;
   const bool jacobian = op == OP_FULL || op == OP_FULL_T;
@@ -314,7 +348,10 @@ std::string alloc_problem(pff_problem& pb) {
   pb.bufs.reserve(pb.hlin32, 4 * nh);
   pb.bufs.reserve(pb.hx64, 3 * nh);
   pb.bufs.reserve(pb.hx32, 3 * nh);
-  pb.bufs.reserve(pb.cell_buf, (M.k == 1 ? 12 : 27) * size_t(pb.mesh->dev.cells.ncells));
+  const DevMesh& D = pb.mesh->dev;
+  const size_t nv = cell_values(pb);
+  if (nv * sizeof(double) <= kCellsWithProblem) pb.bufs.reserve(pb.cells64, nv);
+  if (M.k == 1 && refinement_edges(D) && D.cells.ncells <= kTwoPassCells) pb.bufs.reserve(pb.cells32, nv);
   pb.bufs.commit();
   if (!pb.bufs.err.empty()) {
     std::string err = pb.bufs.err;
@@ -356,7 +393,8 @@ cudaError_t leaf_apply(pff_problem& pb, int precision, int op, const void* xu, c
   std::memset(&a, 0, sizeof(a));
   a.lay = D.leaf;
   a.lc = D.cells;
-  a.lc.out = pb.cell_buf;
+  if (refinement_edges(D))
+    a.lc.out = precision == PFF_F64 ? static_cast<void*>(leaf_contributions64(pb)) : static_cast<void*>(pb.cells32);
   a.hang = D.hang;
   a.cmask = pb.cmask;
   a.lin = precision == PFF_F64 ? static_cast<const void*>(pb.lin64) : static_cast<const void*>(pb.lin32);

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -187,7 +188,13 @@ struct pff_problem {
   float* hlin32 = nullptr;
   double* hx64 = nullptr;    // per hanging node: the input resolved from its parents, 3 blocks of n_hang
   float* hx32 = nullptr;
-  double* cell_buf = nullptr;  // 12 (Q2: 27) doubles per leaf cell, the contributions of the two-pass operators
+  // Contributions of the two-pass operators, 12 (Q2: 27) values per leaf cell, one buffer
+  // per precision as for the other scratch; nullptr where no operator uses it or, FP64,
+  // not yet (leaf_contributions in state.cpp)
+  float* cells32 = nullptr;
+  double* cells64 = nullptr;
+  double* cells64_late = nullptr;  // cells64 when it has an allocation of its own
+  std::mutex cells_mu;             // guards cells64 and cells64_late
   bool has_state = false;
   // per-cell modulus E_K (cell-slot layout; levels concatenated like level vectors)
   bool has_ecell = false;
@@ -302,6 +309,8 @@ void fill_material(const pff_params& prm, ApplyArgs& a, bool unit_E = false);
 // the current device (noalloc.cu).
 cudaError_t noalloc_prepare();
 void leaf_modulus(const pff_problem& pb, int precision, ApplyArgs& a);
+// scratch of the FP64 two-pass operators, made on first use; nullptr when memory is out
+double* leaf_contributions64(pff_problem& pb);
 // a leaf operator with its fix-up, by the faster path (state.cpp)
 template <typename T>
 cudaError_t launch_leaf(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);
