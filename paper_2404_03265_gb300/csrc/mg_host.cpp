@@ -179,7 +179,7 @@ std::string mg_alloc(pff_mg& mg) {
         cudaMemset(mg.blk[b].dinv32, 0, mg.blk[b].ncomp * N * sizeof(float)) != cudaSuccess)
       return "cudaMemset failed";
   if (cudaMemset(mg.su_count, 0, nchain * sizeof(unsigned)) != cudaSuccess ||
-      cudaMemset(mg.spd_bad, 0, 2 * sizeof(int32_t)) != cudaSuccess)
+      cudaMemset(mg.spd_bad, 0, 2 * sizeof(int32_t)) != cudaSuccess || wait_for_clears() != cudaSuccess)
     return "cudaMemset failed";
   return "";
 }
@@ -229,6 +229,7 @@ static std::string coarse_alloc(pff_mg& mg) {
   a.gy = D.levels[0].gy;
   a.cmask = mg.cmask;   // level 0 comes first
   a.bad = mg.spd_bad;
+  if (mg.mem.err.empty() && wait_for_clears() != cudaSuccess) return "coarse tables: upload failed";
   mg.coarse_ready = mg.mem.err.empty();
   return mg.mem.err;
 }

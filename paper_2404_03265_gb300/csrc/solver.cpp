@@ -112,7 +112,7 @@ std::string ensure_workspace(pff_problem& pb, int restart) {
     return "workspace: cudaMallocHost failed";
   }
   if (cudaMemset(W.vc, 0, n3 * sizeof(double)) != cudaSuccess ||
-      cudaMemset(W.count, 0, sizeof(unsigned)) != cudaSuccess)
+      cudaMemset(W.count, 0, sizeof(unsigned)) != cudaSuccess || wait_for_clears() != cudaSuccess)
     return "workspace: cudaMemset failed";
   W.ready = true;
   return "";

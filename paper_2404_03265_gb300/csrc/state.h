@@ -16,6 +16,11 @@
 
 namespace pff {
 
+// Waits for clears (cudaMemset) and uploads of fresh buffers.  Both run on the legacy
+// default stream and may still be on their way when the call returns, and neither the
+// set-up's pool streams nor a caller's non-blocking stream waits for that stream.
+inline cudaError_t wait_for_clears() { return cudaStreamSynchronize(cudaStreamLegacy); }
+
 // Owns a list of cudaMalloc'ed blocks.
 struct DevAllocs {
   std::vector<void*> ptrs;

@@ -2,7 +2,10 @@
 calls one after the other.  On a mesh without refinement edges an apply has no scratch,
 so any two may overlap; on other meshes an FP32 apply may overlap an FP64 operator.
 
-The calls of both streams queue up behind a delay, so that they run side by side."""
+The calls of both streams queue up behind a delay, so that they run side by side.
+
+Fresh buffers are ready before a stream of the caller uses them: a multigrid, its set-up
+and a solve made on a side stream while the default stream is busy."""
 import numpy as np
 import pytest
 
@@ -78,3 +81,30 @@ def test_two_streams_match_one(name, k, calls):
     for w in (0, 1):
         for r in range(n):
             assert torch.equal(got[w][r], want[w][r % 2]), (calls[w], r)
+
+
+@pytest.mark.parametrize("coarse", ["direct", "chebyshev"])
+@pytest.mark.parametrize("k", [1, 2])
+def test_fresh_solver_on_a_side_stream(k, coarse):
+    import torch
+    from paper_2404_03265_gb300 import MG, PFF_F32, gmres
+
+    def solve(stream, busy):
+        m, pb, state, xs = problem("box4_2_2", k)
+        b = xs[0]
+        z, x = torch.zeros_like(b[:2]), torch.zeros_like(b)
+        torch.cuda.synchronize()
+        if busy:
+            torch.cuda._sleep(400_000_000)   # about 0.2 s on the default stream
+        mg = MG(pb, PFF_F32, coarse=coarse)
+        mg.setup(stream=stream)
+        r = gmres(pb, mg, b, x, rtol=1e-6, stream=stream)
+        torch.cuda.synchronize()             # whatever the default stream still held back
+        mg.vcycle(0, b[:2], z, stream=stream)
+        torch.cuda.synchronize()
+        return [mg.lam(0), mg.lam(1), z.cpu().numpy(), x.cpu().numpy(), r["iterations"]]
+
+    want = solve(torch.cuda.current_stream(), False)
+    got = solve(torch.cuda.Stream(), True)
+    for a, b in zip(want, got):
+        assert np.all(np.isfinite(a)) and np.array_equal(a, b)
