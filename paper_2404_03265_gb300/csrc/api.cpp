@@ -353,6 +353,7 @@ extern "C" void pff_mg_destroy(pff_mg* mg) {
     if (mg->su_done[i]) cudaEventDestroy(mg->su_done[i]);
   }
   if (mg->su_start) cudaEventDestroy(mg->su_start);
+  mg->coarse_mem.release();
   mg->mem.release();
   delete mg;
 }

@@ -189,6 +189,8 @@ std::string mg_alloc(pff_mg& mg) {
 // the grid's node slots, element matrices, the dense blocks and the inversion's scratch.
 static std::string coarse_alloc(pff_mg& mg) {
   const Mesh& M = mg.pb->mesh->m;
+  DevAllocs& mem = mg.coarse_mem;
+  mem.release();   // (what an attempt cut short by an exception left)
   const DevMesh& D = mg.pb->mesh->dev;
   const LevelMesh& lm = M.levels[0];
   const int32_t n0 = D.levels[0].lv.n_slots;
@@ -212,26 +214,36 @@ static std::string coarse_alloc(pff_mg& mg) {
     q.n = int32_t(idx.size());
     q.nc = B.ncomp;
     q.fix0 = b == 0 ? 1 : 4;
-    B.coarse_idx = mg.mem.alloc<int32_t>(idx.size());
-    q.all = mg.mem.upload(idx);
+    B.coarse_idx = mem.alloc<int32_t>(idx.size());
+    q.all = mem.upload(idx);
     q.idx = B.coarse_idx;
-    q.ent = mg.mem.upload(ent);
-    q.Ke = mg.mem.alloc<double>(size_t(ncx) * ncy * nd * nd);
-    B.coarse_inv = mg.mem.alloc<double>(size_t(q.n) * q.n);
+    q.ent = mem.upload(ent);
+    q.Ke = mem.alloc<double>(size_t(ncx) * ncy * nd * nd);
+    B.coarse_inv = mem.alloc<double>(size_t(q.n) * q.n);
     q.A = B.coarse_inv;
-    q.scr = mg.mem.alloc<double>(size_t(coarse_scratch(q.n)));
+    q.scr = mem.alloc<double>(size_t(coarse_scratch(q.n)));
     B.n_coarse = q.n;
   }
   a.k = k; a.ncx = ncx; a.ncy = ncy;
   a.n0 = n0;
-  a.node_slot = mg.mem.upload(node_slot);
+  a.node_slot = mem.upload(node_slot);
   a.gx = D.levels[0].gx;
   a.gy = D.levels[0].gy;
   a.cmask = mg.cmask;   // level 0 comes first
   a.bad = mg.spd_bad;
-  if (mg.mem.err.empty() && wait_for_clears() != cudaSuccess) return "coarse tables: upload failed";
-  mg.coarse_ready = mg.mem.err.empty();
-  return mg.mem.err;
+  std::string err = mem.err;
+  if (err.empty() && wait_for_clears() != cudaSuccess) err = "coarse tables: upload failed";
+  if (!err.empty()) {   // give everything back: a later set-up starts afresh
+    mem.release();
+    std::memset(&a, 0, sizeof(a));
+    for (MGBlock& B : mg.blk) {
+      B.coarse_idx = nullptr;
+      B.coarse_inv = nullptr;
+      B.n_coarse = 0;
+    }
+  }
+  mg.coarse_ready = err.empty();
+  return err;
 }
 
 // The direct coarse solve's blocks on stream t: element matrices, assembly, inversion

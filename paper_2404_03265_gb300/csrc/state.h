@@ -31,6 +31,7 @@ struct DevAllocs {
     void* p = nullptr;
     const cudaError_t e = cudaMalloc(&p, n * sizeof(T));
     if (e != cudaSuccess) {
+      cudaGetLastError();   // reported here: no later launch finds it
       if (err.empty()) err = std::string("cudaMalloc: ") + cudaGetErrorString(e);
       return nullptr;
     }
@@ -69,6 +70,7 @@ struct DevAllocs {
   void release() {
     for (void* p : ptrs) cudaFree(p);
     ptrs.clear();
+    err.clear();
   }
 };
 
@@ -274,6 +276,7 @@ struct pff_mg {
   double* su_part[2] = {nullptr, nullptr};   // tiled set-up: per block the dots' parts
   unsigned* su_count = nullptr;    // per chain: finished blocks of a dot (0 between launches)
   // the direct coarse solve's blocks (made by the first set-up that needs them)
+  pff::DevAllocs coarse_mem;
   bool coarse_ready = false;
   pff::CoarseArgs coarse = {};
   double* host = nullptr;          // pinned: CG coefficients (host_len doubles), then the coarse status

@@ -119,3 +119,32 @@ def test_invalid_arguments_are_reported():
     assert L.pff_mg_set_fused_smoother(mg._h, 2) == INVALID_ARG
     assert L.pff_mg_set_coarse(mg._h, 5) == INVALID_ARG
     assert L.pff_mg_set_fused_smoother(mg._h, 0) == 0
+
+
+def test_coarse_memory_failure_leaves_nothing_behind():
+    """A coarse grid whose dense level-0 blocks no device holds (522,242 entries: 2.2 TB):
+    the set-up reports it, gives back what it had allocated, fails the same way again
+    without holding more, and the Chebyshev coarse solver then works on the same object."""
+    import torch
+    from paper_2404_03265_gb300 import MG, PFF_F32, Mesh, PffError, Problem, _lib
+    m = Mesh(-10.0, 10.0, -10.0, 10.0, 512, 512).finalize(1)
+    ns = m.info["n_slots"]
+    pb = Problem(m, E=1.0, nu=0.2, Gc=1.0, eps=0.1, kappa=1e-3, p=0.0)
+    one = torch.ones(ns, dtype=torch.float64, device="cuda")
+    pb.set_state(torch.zeros((2, ns), dtype=torch.float64, device="cuda"), one, one)
+    mg = MG(pb, PFF_F32)
+    free = []
+    for _ in range(3):
+        with pytest.raises(PffError, match="out of memory"):
+            mg.setup()
+        torch.cuda.synchronize()
+        free.append(torch.cuda.mem_get_info()[0])
+    assert free[1] >= free[0] and free[2] >= free[0]
+    assert _lib.lib().pff_mg_set_coarse(mg._h, 1) == 0
+    mg.setup()
+    r = torch.zeros_like(one)
+    r[torch.tensor((m.slots()[2] & 1) == 1, device="cuda")] = 1.0
+    z = torch.full_like(r, float("nan"))
+    mg.vcycle(1, r, z)
+    torch.cuda.synchronize()
+    assert torch.isfinite(z).all() and z.abs().max() > 0
