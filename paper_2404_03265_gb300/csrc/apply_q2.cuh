@@ -20,7 +20,8 @@
 //   3. the cells write their contributions to shared memory, one column per cell, and a
 //      thread sums them for the four owned nodes (2i, 2j) .. (2i + 1, 2j + 1): the cells
 //      around a node in the order (even column, even row), (odd, even), (even, odd),
-//      (odd, odd), so every nodal sum has a fixed order;
+//      (odd, odd), so every nodal sum has a fixed order (the FP64 Jacobian: below,
+//      below-left, left, own);
 //   4. the owned nodes are written (constraint rows, partial sums, holes; pairs of
 //      unconstrained nodes of regular bricks as one 8-byte store in FP32), or for the
 //      level block operators the fused Chebyshev step of ChebEpi.
@@ -536,6 +537,14 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
             const int cx0 = px || !ox ? 0 : -1, ax0 = px ? 1 : (ox ? 2 : 0), cx1 = ox ? 0 : -1, ax1 = ox ? 0 : 2;
             const int cy0 = py || !oy ? 0 : -Q2C, ay0 = py ? 1 : (oy ? 2 : 0), cy1 = oy ? 0 : -Q2C, ay1 = oy ? 0 : 2;
             auto sum = [&](auto (*con)[Q2T]) {
+              if constexpr (sizeof(T) == 8 && (OP == OP_FULL || OP == OP_FULL_T)) {
+                // the order of the two passes (leaf_cells_q2.cu), which give the same bits
+                using V = typename std::remove_reference<decltype(con[0][0])>::type;
+                const V none{};
+                const V below = py ? none : con[px + 6][own - Q2C], corner = px || py ? none : con[8][own - Q2C - 1],
+                        left = px ? none : con[2 + 3 * py][own - 1];
+                return padd(padd(padd(below, corner), left), con[px + 3 * py][own]);
+              }
               auto v = con[ax0 + 3 * ay0][own + cx0 + cy0];
               if (!px) v = padd(v, con[ax1 + 3 * ay0][own + cx1 + cy0]);
               if (!py) {

@@ -289,8 +289,31 @@ __device__ __forceinline__ void q2_jac(const Load& ld, const Q2Mat<T>& k, const 
     ru[i] = P{T(0), T(0)};
     rp[i] = T(0);
   }
+  if constexpr (sizeof(T) == 8) {
+    // FP64: each row from zero, then (row 0 + row 1) + row 2, the bits of the kernel that
+    // gives a row to a warp (leaf_cells_q2.cu)
+    q2_jac_row<T, OP, MOD>(RowAt<T, 0>(), ld, k, o, ru, rp);
+    P u[9];
+    T p[9];
+    auto add = [&](const auto& row) {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        u[i] = P{T(0), T(0)};
+        p[i] = T(0);
+      }
+      q2_jac_row<T, OP, MOD>(row, ld, k, o, u, p);
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        ru[i] = padd(ru[i], u[i]);
+        rp[i] = padd(rp[i], p[i]);
+      }
+    };
+    add(RowAt<T, 1>());
+    add(RowAt<T, 2>());
+  } else {
 #pragma unroll 1
-  for (int q = 0; q < 3; ++q) q2_jac_row<T, OP, MOD>(RowVar<T>(q), ld, k, o, ru, rp);
+    for (int q = 0; q < 3; ++q) q2_jac_row<T, OP, MOD>(RowVar<T>(q), ld, k, o, ru, rp);
+  }
 }
 
 }  // namespace pff
