@@ -138,9 +138,10 @@ pff_status pff_set_active(pff_problem* pb, const uint8_t* active, void* stream);
  * Dirichlet u and active phi DoFs.  precision PFF_F64: double vectors, PFF_F32:
  * float vectors (state cast to float).  xu/yu: 2*n_slots, xp/yp: n_slots.
  * x and y must not overlap.
- * Concurrency: on a mesh without refinement edges (n_hanging = 0) an apply writes
- * nothing but y, so applies of one problem may run at the same time on several
- * streams and from several threads.  On other meshes the applies of one precision
+ * Concurrency: on a mesh without refinement edges (n_hanging = 0) applies of one
+ * problem may run at the same time on several streams and from several threads
+ * (FP64: scratch per stream, made by its first apply; from the fifth stream on and
+ * in a stream capture without scratch, more slowly, the same bits).  On other meshes the applies of one precision
  * (FP64: and the solver calls) share scratch of the problem and must be ordered; an
  * FP32 and an FP64 apply may still run at the same time.                         */
 pff_status pff_apply(pff_problem* pb, int32_t precision, int32_t op, const void* xu, const void* xp,

@@ -245,6 +245,8 @@ extern "C" void pff_problem_destroy(pff_problem* pb) {
   release_workspace(pb->ws);
   pb->bufs.release();
   if (pb->cells64_late) cudaFree(pb->cells64_late);
+  for (auto& c : pb->stream_cells)
+    if (c.values) cudaFree(c.values);
   delete pb;
 }
 

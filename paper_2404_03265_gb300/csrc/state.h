@@ -201,7 +201,13 @@ struct pff_problem {
   float* cells32 = nullptr;
   double* cells64 = nullptr;
   double* cells64_late = nullptr;  // cells64 when it has an allocation of its own
-  std::mutex cells_mu;             // guards cells64 and cells64_late
+  // FP64 applies on a mesh without refinement edges: a buffer per stream
+  static constexpr int kStreamCells = 4;
+  struct StreamCells {
+    unsigned long long stream = 0;   // cudaStreamGetId: never given to another stream
+    double* values = nullptr;
+  } stream_cells[kStreamCells];
+  std::mutex cells_mu;             // guards cells64, cells64_late and stream_cells
   bool has_state = false;
   // per-cell modulus E_K (cell-slot layout; levels concatenated like level vectors)
   bool has_ecell = false;

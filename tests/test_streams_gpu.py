@@ -1,8 +1,8 @@
-"""Operators of one problem on two streams at once: the results are the bits of the same
+"""Operators of one problem on several streams at once: the results are the bits of the same
 calls one after the other.  On a mesh without refinement edges an apply has no scratch,
 so any two may overlap; on other meshes an FP32 apply may overlap an FP64 operator.
 
-The calls of both streams queue up behind a delay, so that they run side by side.
+The calls of the streams queue up behind a delay, so that they run side by side.
 
 Fresh buffers are ready before a stream of the caller uses them: a multigrid, its set-up
 and a solve made on a side stream while the default stream is busy."""
@@ -39,15 +39,18 @@ def problem(name, k):
 
 @pytest.mark.parametrize("name,k,calls", [
     ("box16_3_0", 1, (F64, F64)), ("box16_3_0", 1, (F32, F32)), ("box16_2_0", 2, (F64, F64)),
+    ("box16_3_0", 1, (F64,) * 6), ("box8_3_0", 2, (F64, "residual", F64)),
     ("box9_4_2", 1, (F32, F64)), ("box9_4_2", 1, (F32, "residual")), ("box9_3_2", 2, (F32, F64)),
 ], ids=str)
-def test_two_streams_match_one(name, k, calls):
+def test_streams_match_one(name, k, calls):
     import torch
     from paper_2404_03265_gb300 import PFF_OP_JACOBIAN, PFF_OP_TRANSPOSE
     m, pb, state, xs = problem(name, k)
     assert (m.info["n_hanging"] == 0) == name.endswith("_0")
-    n = 100
-    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    n = 200 // len(calls)
+    every = range(len(calls))
+    streams = [torch.cuda.Stream() for _ in calls]
+    xs = [xs[w % 2] * (1 + w) for w in every]
     xs = [x if c == "residual" else x.to(getattr(torch, c)) for x, c in zip(xs, calls)]
 
     def call(which, rep, y, stream):
@@ -61,10 +64,10 @@ def test_two_streams_match_one(name, k, calls):
 
     def outputs():
         dt = [torch.float64 if c == "residual" else getattr(torch, c) for c in calls]
-        return [[torch.full(xs[0].shape, float("nan"), dtype=dt[w], device="cuda") for _ in range(n)] for w in (0, 1)]
+        return [[torch.full(xs[0].shape, float("nan"), dtype=dt[w], device="cuda") for _ in range(n)] for w in every]
 
     want, got = outputs(), outputs()
-    for w in (0, 1):
+    for w in every:
         for r in range(2):
             call(w, r, want[w][r], torch.cuda.current_stream())
     torch.cuda.synchronize()
@@ -75,10 +78,10 @@ def test_two_streams_match_one(name, k, calls):
     for s in streams:
         s.wait_event(go)
     for r in range(n):
-        for w in (0, 1):
+        for w in every:
             call(w, r, got[w][r], streams[w])
     torch.cuda.synchronize()
-    for w in (0, 1):
+    for w in every:
         for r in range(n):
             assert torch.equal(got[w][r], want[w][r % 2]), (calls[w], r)
 
