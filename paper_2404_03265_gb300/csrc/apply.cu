@@ -54,12 +54,23 @@ __device__ __forceinline__ dbl4 ldg4(const dbl4* p) {
 }
 __device__ __forceinline__ float4 ldg4(const float4* p) { return __ldg(p); }
 
-template <typename T> __device__ __forceinline__ const MatConst<T>& matc(const ApplyArgs& a);
-template <> __device__ __forceinline__ const MatConst<float>& matc<float>(const ApplyArgs& a) { return a.mf; }
-template <> __device__ __forceinline__ const MatConst<double>& matc<double>(const ApplyArgs& a) { return a.md; }
-template <typename T> __device__ __forceinline__ LevGeom<T> geom(const ApplyArgs& a, int level);
-template <> __device__ __forceinline__ LevGeom<float> geom<float>(const ApplyArgs& a, int level) { return a.gf[level]; }
-template <> __device__ __forceinline__ LevGeom<double> geom<double>(const ApplyArgs& a, int level) { return a.gd[level]; }
+// Argument blocks of the kernels from those of a launch.
+template <typename T>
+SweepArgs<T> sweep_args(const ApplyArgs& a) {
+  SweepArgs<T> k;
+  static_cast<LoopArgs&>(k) = a;
+  if constexpr (sizeof(T) == 4) k.m = a.mf; else k.m = a.md;
+  for (int l = 0; l < kMaxLevels; ++l)
+    if constexpr (sizeof(T) == 4) k.g[l] = a.gf[l]; else k.g[l] = a.gd[l];
+  return k;
+}
+template <typename T>
+BrickArgs<T> brick_args(const ApplyArgs& a) {
+  BrickArgs<T> k;
+  static_cast<SweepArgs<T>&>(k) = sweep_args<T>(a);
+  if constexpr (sizeof(T) == 4) { k.q2 = a.q2f; k.q2m = a.q2mf; } else { k.q2 = a.q2d; k.q2m = a.q2md; }
+  return k;
+}
 
 // Node fields of the cell loops.
 enum Field : int { F_XU = 0, F_XV = 1, F_XP = 2, F_LU = 3, F_LV = 4, F_LP = 5, F_LT = 6, NF = 7 };
@@ -72,7 +83,7 @@ __device__ __forceinline__ constexpr bool field_used(int f) {
 }
 
 template <typename T>
-__device__ __forceinline__ const T* field_ptr(const ApplyArgs& a, int f) {
+__device__ __forceinline__ const T* field_ptr(const LoopArgs& a, int f) {
   const T* xu = reinterpret_cast<const T*>(a.xu);
   const T* lin = reinterpret_cast<const T*>(a.lin);
   switch (f) {
@@ -183,7 +194,7 @@ __device__ __forceinline__ uint32_t& half_of_u(uint2& p, int h) { return h ? p.y
 // from the node's own slot (resolved there by set_lin).  Absent nodes are zero.
 // Hanging and absent nodes carry no constraint of their own.
 template <typename T, int OP>
-__device__ __forceinline__ void issue_node(const ApplyArgs& a, int32_t code, SweepStage<T>& st, int h, int lane) {
+__device__ __forceinline__ void issue_node(const LoopArgs& a, int32_t code, SweepStage<T>& st, int h, int lane) {
   using N = Needs<OP>;
   if (code >= 0) {
 #pragma unroll
@@ -271,7 +282,7 @@ __device__ __forceinline__ void load_row(const SweepStage<T>& st, int lane, Node
 // original x of the node, read back from the input vectors).  Predicated rather
 // than branched: the lanes of a row take different actions.
 template <typename T, int OP>
-__device__ __forceinline__ void store_owned(const ApplyArgs& a, int slot, int act_s, int part, uint8_t cm, T y0, T y1,
+__device__ __forceinline__ void store_owned(const LoopArgs& a, int slot, int act_s, int part, uint8_t cm, T y0, T y1,
                                             T y2) {
   constexpr bool outU = (OP != OP_PP && OP != OP_PP_DIAG);
   constexpr bool outP = (OP != OP_UU && OP != OP_UU_DIAG);
@@ -307,7 +318,7 @@ struct ChebOps {
 };
 
 template <typename T, int OP>
-__device__ __forceinline__ void cheb_load(const ApplyArgs& a, int slot, ChebOps<T, OP>& o) {
+__device__ __forceinline__ void cheb_load(const LoopArgs& a, int slot, ChebOps<T, OP>& o) {
   const ChebEpi& ch = a.ch;
   const T* x = reinterpret_cast<const T*>(OP == OP_UU ? a.xu : a.xp);
 #pragma unroll
@@ -324,7 +335,7 @@ __device__ __forceinline__ void cheb_load(const ApplyArgs& a, int slot, ChebOps<
 }
 
 template <typename T, int OP>
-__device__ __forceinline__ void cheb_store(const ApplyArgs& a, int slot, int act_s, uint8_t cm, T y0, T y1, T y2,
+__device__ __forceinline__ void cheb_store(const LoopArgs& a, int slot, int act_s, uint8_t cm, T y0, T y1, T y2,
                                            const ChebOps<T, OP>& o) {
   const ChebEpi& ch = a.ch;
   const T ca = sizeof(T) == 4 ? T(ch.af) : T(ch.ad);
@@ -350,7 +361,7 @@ __device__ __forceinline__ void cheb_store(const ApplyArgs& a, int slot, int act
 
 template <typename T, int OP>
 __global__ void __launch_bounds__(32 * SW_WARPS, (sw_min_blocks<T, OP>()))
-sweep_q1_kernel(const __grid_constant__ ApplyArgs a, const int32_t* __restrict__ units, int32_t nunits) {
+sweep_q1_kernel(const __grid_constant__ SweepArgs<T> a, const int32_t* __restrict__ units, int32_t nunits) {
   static_assert(SW_DEPTH >= 3, "the ring holds the lower row, the upper row and at least one row in flight");
   using P = typename VT<T>::T2;
   constexpr bool outU = (OP != OP_PP && OP != OP_PP_DIAG);
@@ -370,8 +381,8 @@ sweep_q1_kernel(const __grid_constant__ ApplyArgs a, const int32_t* __restrict__
   const int NROW = SH + 2;                             // node rows per half
   const BrickDesc* bd = a.lay.bricks + bi;
   const int irr = __ldg(&bd->irr);
-  const LevGeom<T> g = geom<T>(a, __ldg(&bd->level));
-  const MatConst<T>& mc = matc<T>(a);
+  const LevGeom<T> g = a.g[__ldg(&bd->level)];
+  const MatConst<T>& mc = a.m;
   const bool mask = (a.mode & MODE_MASK_INPUT) != 0;
   const int n = lane - 1;                              // window node column -1..30
   const int dx = n < 0 ? -1 : (n >= NB ? 1 : 0);
@@ -837,7 +848,8 @@ cudaError_t launch_sweep(const ApplyArgs& a, cudaStream_t s) {
   const size_t smem = sizeof(SweepStage<T>) * SW_DEPTH * SW_WARPS;
   const auto fn = &sweep_q1_kernel<T, OP>;
   resident_blocks(reinterpret_cast<const void*>(fn), int(blk), smem);   // sets the shared-memory limit once
-  return launch_ex(pdl, fn, unsigned((nunits + SW_WARPS - 1) / SW_WARPS), blk, smem, s, a, units, nunits);
+  return launch_ex(pdl, fn, unsigned((nunits + SW_WARPS - 1) / SW_WARPS), blk, smem, s,
+                   sweep_args<T>(a), units, nunits);
 }
 
 // The other leaf operators (residual, mass, crack volume and its derivatives) go through
@@ -875,7 +887,7 @@ namespace {
 // Element matrices of a level block on level 0: thread (cell, column) evaluates the cell
 // on a unit vector.  Ke: per cell [row][column], dof = node * ncomp + component.
 template <int OP, int K>
-__global__ void __launch_bounds__(64) coarse_element_kernel(const __grid_constant__ ApplyArgs a, int ncx, int ncells,
+__global__ void __launch_bounds__(64) coarse_element_kernel(const __grid_constant__ BrickArgs<double> a, int ncx, int ncells,
                                                             const int32_t* __restrict__ node_slot,
                                                             double* __restrict__ Ke) {
   constexpr int NC = OP == OP_UU ? 2 : 1, NN = (K + 1) * (K + 1), ND = NN * NC;
@@ -906,7 +918,7 @@ __global__ void __launch_bounds__(64) coarse_element_kernel(const __grid_constan
       return NodePair<double>{p.x0 - q.x0, p.x1 - q.x1, p.xp - q.xp, p.lx - q.lx, p.ly - q.ly, p.lz - q.lz, p.lw - q.lw};
     };
     double out[12];
-    q1_cell<double, OP>(v[0], minus(v[1], v[0]), v[2], minus(v[3], v[2]), a.md, a.gd[0], ec, out);
+    q1_cell<double, OP>(v[0], minus(v[1], v[0]), v[2], minus(v[3], v[2]), a.m, a.g[0], ec, out);
 #pragma unroll
     for (int e = 0; e < 4; ++e)
 #pragma unroll
@@ -922,7 +934,7 @@ __global__ void __launch_bounds__(64) coarse_element_kernel(const __grid_constan
     };
     double2 ru[9];
     double rp[9], cv[3];
-    q2_cell<double, OP>(ld, a.md, a.gd[0], a.q2d, ec, ru, rp, cv);
+    q2_cell<double, OP>(ld, a.m, a.g[0], a.q2, ec, ru, rp, cv);
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
       if constexpr (OP == OP_UU) { r[2 * e] = ru[e].x; r[2 * e + 1] = ru[e].y; } else { r[e] = rp[e]; }
@@ -937,10 +949,11 @@ cudaError_t launch_coarse_elements(const ApplyArgs& a, int op, int ncx, int ncel
                                    double* Ke, cudaStream_t s) {
   const int nd = (a.fe_degree + 1) * (a.fe_degree + 1) * (op == OP_UU ? 2 : 1);
   const unsigned grid = unsigned((int64_t(ncells) * nd + 63) / 64);
-  if (a.fe_degree == 1 && op == OP_UU) coarse_element_kernel<OP_UU, 1><<<grid, 64, 0, s>>>(a, ncx, ncells, node_slot, Ke);
-  else if (a.fe_degree == 1 && op == OP_PP) coarse_element_kernel<OP_PP, 1><<<grid, 64, 0, s>>>(a, ncx, ncells, node_slot, Ke);
-  else if (a.fe_degree == 2 && op == OP_UU) coarse_element_kernel<OP_UU, 2><<<grid, 64, 0, s>>>(a, ncx, ncells, node_slot, Ke);
-  else if (a.fe_degree == 2 && op == OP_PP) coarse_element_kernel<OP_PP, 2><<<grid, 64, 0, s>>>(a, ncx, ncells, node_slot, Ke);
+  const BrickArgs<double> k = brick_args<double>(a);
+  if (a.fe_degree == 1 && op == OP_UU) coarse_element_kernel<OP_UU, 1><<<grid, 64, 0, s>>>(k, ncx, ncells, node_slot, Ke);
+  else if (a.fe_degree == 1 && op == OP_PP) coarse_element_kernel<OP_PP, 1><<<grid, 64, 0, s>>>(k, ncx, ncells, node_slot, Ke);
+  else if (a.fe_degree == 2 && op == OP_UU) coarse_element_kernel<OP_UU, 2><<<grid, 64, 0, s>>>(k, ncx, ncells, node_slot, Ke);
+  else if (a.fe_degree == 2 && op == OP_PP) coarse_element_kernel<OP_PP, 2><<<grid, 64, 0, s>>>(k, ncx, ncells, node_slot, Ke);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }

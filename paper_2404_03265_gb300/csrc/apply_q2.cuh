@@ -313,16 +313,8 @@ __device__ __forceinline__ void q2_cell(const Load& ld, const MatConst<T>& m, co
   }
 }
 
-template <typename T> __device__ __forceinline__ const Q2Tab<T>& q2tab(const ApplyArgs& a);
-template <> __device__ __forceinline__ const Q2Tab<float>& q2tab<float>(const ApplyArgs& a) { return a.q2f; }
-template <> __device__ __forceinline__ const Q2Tab<double>& q2tab<double>(const ApplyArgs& a) { return a.q2d; }
-
-template <typename T> __device__ __forceinline__ const Q2Mat<T>& q2mat(const ApplyArgs& a);
-template <> __device__ __forceinline__ const Q2Mat<float>& q2mat<float>(const ApplyArgs& a) { return a.q2mf; }
-template <> __device__ __forceinline__ const Q2Mat<double>& q2mat<double>(const ApplyArgs& a) { return a.q2md; }
-
 template <typename T, int OP>
-__global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(const __grid_constant__ ApplyArgs a) {
+__global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(const __grid_constant__ BrickArgs<T> a) {
   using P = typename VT<T>::T2;
   constexpr bool isVjp = (OP == OP_VJP);
   constexpr int NBUF = Q2Smem<T>::NBUF;
@@ -330,8 +322,8 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
   Q2Smem<T>& sm = *reinterpret_cast<Q2Smem<T>*>(smem_raw);
   const int tid = threadIdx.x;
   const bool mask = (a.mode & MODE_MASK_INPUT) != 0;
-  const MatConst<T>& mc = matc<T>(a);
-  const Q2Tab<T>& tb = q2tab<T>(a);
+  const MatConst<T>& mc = a.m;
+  const Q2Tab<T>& tb = a.q2;
   const int ci = tid % Q2C, cj = tid / Q2C;          // window cell (cell ci - 1, cj - 1)
   Q2Node<T, OP> node;
   node.at(ci, cj);
@@ -496,10 +488,10 @@ __global__ void __launch_bounds__(Q2T, sizeof(T) == 4 ? 2 : 1) apply_q2_kernel(c
     T rp[9], cell[3];
     if (act) {
       if constexpr (OP == OP_FULL || OP == OP_FULL_T)
-        if (a.ecell == nullptr) q2_jac<T, OP, false>(node, q2mat<T>(a), Q2Own<T>(mc, geom<T>(a, level), T(1)), ru, rp);
-        else q2_jac<T, OP, true>(node, q2mat<T>(a), Q2Own<T>(mc, geom<T>(a, level), ec), ru, rp);
+        if (a.ecell == nullptr) q2_jac<T, OP, false>(node, a.q2m, Q2Own<T>(mc, a.g[level], T(1)), ru, rp);
+        else q2_jac<T, OP, true>(node, a.q2m, Q2Own<T>(mc, a.g[level], ec), ru, rp);
       else
-        q2_cell<T, OP>(node, mc, geom<T>(a, level), tb, ec, ru, rp, cell);
+        q2_cell<T, OP>(node, mc, a.g[level], tb, ec, ru, rp, cell);
     }
     if constexpr (isVjp) {
       // the brick owns the cells whose lower-left node it owns (cells 0..14)
@@ -614,8 +606,9 @@ cudaError_t launch_apply_q2(const ApplyArgs& a, int op, cudaStream_t s) {
     const int full = resident_blocks(fn, Q2T, smem);
     return unsigned(a.lay.nbricks < full ? a.lay.nbricks : full);
   };
+  const BrickArgs<T> k = brick_args<T>(a);
   auto go = [&](auto fn) {
-    fn<<<grid_of(reinterpret_cast<const void*>(fn)), Q2T, smem, s>>>(a);
+    fn<<<grid_of(reinterpret_cast<const void*>(fn)), Q2T, smem, s>>>(k);
     return cudaGetLastError();
   };
   if constexpr (sizeof(T) == 8) {   // formed in FP64 only

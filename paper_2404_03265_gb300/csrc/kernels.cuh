@@ -131,9 +131,9 @@ struct ChebEpi {
   double ad, bd;
 };
 
-struct ApplyArgs {
+// What a cell-loop kernel reads in either precision.
+struct LoopArgs {
   DevLayout lay;
-  LeafCells lc;           // leaf operators
   const DevHanging* hang;
   const uint8_t* cmask;   // per slot: bit0/bit1 u_x/u_y fixed, bit2 phi fixed
   const void* lin;        // 4 blocks of n_slots T: u_x, u_y, phi, phi_tilde (hanging entries resolved)
@@ -148,6 +148,30 @@ struct ApplyArgs {
   const void* ecell;      // per-cell modulus E_K (T, cell-slot layout) or nullptr: constants carry E
   void* cell_out;         // OP_VJP: 3 blocks of n_slots T (E_K, p, G_c) at cell slots
   int64_t n_slots;
+  int mode;
+  int pair_store;         // Q2: the output vectors allow stores of two neighbouring slots (set by launch_apply)
+  int wide;               // Q2: the input vectors allow 16-byte copies of whole bricks (set by launch_apply)
+  int pdl_in;             // Q1: launched dependent on the preceding kernel, which wrote x (pdl.cuh)
+  ChebEpi ch;             // level applies: fused Chebyshev store (mode CHEB_OFF: plain y = A x)
+};
+
+// The kernels' own argument blocks: one precision, and Q2 constants only where they are
+// read (arguments are copied per launch; with everything in one block, 4,312 bytes, the
+// FP32 Jacobian of 4.1M DoFs took 34.95 us instead of 34.87).
+template <typename T>
+struct SweepArgs : LoopArgs {
+  MatConst<T> m;
+  LevGeom<T> g[kMaxLevels];
+};
+template <typename T>
+struct BrickArgs : SweepArgs<T> {
+  Q2Tab<T> q2;
+  Q2Mat<T> q2m;
+};
+
+// A launch of an operator, on the host.
+struct ApplyArgs : LoopArgs {
+  LeafCells lc;           // leaf operators
   double hx[kMaxLevels], hy[kMaxLevels];
   double mu, lam;         // Lame constants (E applied, or unit E when ecell is set)
   double ell;             // length scale l
@@ -160,13 +184,8 @@ struct ApplyArgs {
   Q2Tab<double> q2d;
   Q2Mat<float> q2mf;
   Q2Mat<double> q2md;
-  int mode;
   int fe_degree;
   int sweep_sh;           // Q1 strip half-height: 0 = by mesh size, else 15, 5 or 1 (schedules of DevLayout::units)
-  int pair_store;         // Q2: the output vectors allow stores of two neighbouring slots (set by launch_apply)
-  int wide;               // Q2: the input vectors allow 16-byte copies of whole bricks (set by launch_apply)
-  int pdl_in;             // Q1: launched dependent on the preceding kernel, which wrote x (pdl.cuh)
-  ChebEpi ch;             // level applies: fused Chebyshev store (mode CHEB_OFF: plain y = A x)
 };
 
 struct FixupArgs {
