@@ -134,12 +134,22 @@ static LeafCells upload_leaf_cells(DevAllocs& mem, const Mesh& M) {
 //  - FP64: always two passes (bound by the FP64 rate, and they evaluate only cells that
 //    exist): Jacobian 992 -> 741 us on 4.1M DoFs, 633 -> 199 us on the 1.04M-DoF crack
 //    mesh, 45 -> 22 us on 4.3k DoFs.  A forced strip height asks for the sweep's Jacobian.
-//  - FP32: two passes up to kTwoPassCells, while the 48 bytes of contributions per cell
-//    stay small beside L2: 13.1 -> 11.1 us on 65k DoFs, 30.7 -> 19.6 us on the crack mesh,
-//    26.6 -> 22.0 us at 0.53M cells, but 31.1 -> 34.0 us at 0.77M and 37.9 -> 61 us at
-//    1.36M (the sweep writes no contributions to memory).
+//  - FP32: two passes while the contributions (48 bytes per cell, written and read again)
+//    cost less than the sweep's cells that do not exist and its few long units.  Both loops
+//    (us; input vectors in L2, and rotating through more than L2), sweep against passes:
+//      86k cells, 0.76 of the slots   12.1 / 12.3 against 12.3 / 13.9
+//      340k, 0.46 (crack mesh)        28.5 / 29.3 against 19.6 / 24.6
+//      401k, 0.77                     22.5 / 23.2 against 18.9 / 23.6
+//      433k, 0.85                     21.2 / 22.5 against 18.8 / 24.6
+//      507k, 0.54                     37.0 / 38.9 against 26.8 / 31.0
+//      534k, 0.89                     22.1 / 22.5 against 23.0 / 27.5
+//      619k, 0.82                     27.6 / 28.9 against 31.9 / 36.1
+//      648k, 0.72                     29.9 / 30.7 against 35.6 / 38.0
+//    So up to 450k cells, and up to 550k where bricks are less than 0.6 full.
 // Without a buffer of contributions (see below) the Jacobian takes the cell loop.
-constexpr int32_t kTwoPassCells = 650000;
+static bool two_passes_f32(int64_t cells, int64_t slots) {
+  return cells <= 450000 || (cells <= 550000 && 10 * cells < 6 * slots);
+}
 
 // Who may use the contributions.  On a mesh without refinement edges the cell loop writes
 // nothing but the result, and applies of one problem (pff_apply) may run at the same time
@@ -203,7 +213,7 @@ static bool use_two_passes(const ApplyArgs& a, int op, bool f64) {
   const bool jacobian = op == OP_FULL || op == OP_FULL_T;
   if (a.fe_degree == 2) return f64 && (jacobian || op == OP_RESID);
   if (a.sweep_sh != 0 && jacobian) return false;
-  return f64 || (jacobian && a.lc.ncells <= kTwoPassCells);
+  return f64 || (jacobian && two_passes_f32(a.lc.ncells, a.n_slots));
 }
 
 template <typename T>
@@ -376,7 +386,7 @@ std::string alloc_problem(pff_problem& pb) {
   const DevMesh& D = pb.mesh->dev;
   const size_t nv = cell_values(pb);
   if (refinement_edges(D) && nv * sizeof(double) <= kCellsWithProblem) pb.bufs.reserve(pb.cells64, nv);
-  if (M.k == 1 && refinement_edges(D) && D.cells.ncells <= kTwoPassCells) pb.bufs.reserve(pb.cells32, nv);
+  if (M.k == 1 && refinement_edges(D) && two_passes_f32(D.cells.ncells, ns)) pb.bufs.reserve(pb.cells32, nv);
   pb.bufs.commit();
   if (!pb.bufs.err.empty()) {
     std::string err = pb.bufs.err;
