@@ -4,7 +4,9 @@
 // A full vector has three blocks of n_slots doubles: u_x, u_y, phi.
 // Leaf slot flags: bit0 node, bit1 boundary (Dirichlet u), bit2 hanging.
 // All reductions are deterministic (fixed partition, fixed summation order).
+#include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "kernels.cuh"
 #include "pdl.cuh"
@@ -195,16 +197,33 @@ __device__ __forceinline__ int64_t basis_row(int64_t i, int64_t ldb) {
 //   GS_GATHER  w[i] = z[map[i]]
 //   GS_AXPY    w[i] -= sum_j h[j] V_j[i] (the sum in the order j = 0, 1, ...)
 // then out[j] = V_j . w, j < k, or with NORM out[0] = w . w.  A block's partial sums of a
-// vector come from one shared-memory tree over its threads; the last block to finish adds
-// the blocks' partials in a fixed order, so the sums do not depend on which block that is.
+// vector are a tree over its threads, a warp per vector; the last block to finish adds the
+// blocks' partials in a fixed order, so the sums do not depend on which block that is.
 // The basis vectors go in chunks of MD_J (the last one in its own instantiation, so no
 // multiply is spent on padding).
-// Measured: 65k DoFs, 8 Arnoldi steps with their V-cycles 1323 -> 1150 us; 4.3k DoFs, the
-// orthogonalisation of a step 49 -> 26 us.  On a million rows the FP64 rate bounds it.
+// What bounds it: the FP64 rate (1.04M rows: 179 us of multiply-adds a step at 25 vectors)
+// and the phases between chunks.  So every SM gets as many blocks, no FP64 operation goes to
+// a visit without rows, and a chunk's trees take two barriers (the same tree over shared
+// memory took ten, with one warp at work in half of them).  Measured, 50 Arnoldi steps of
+// one cycle, us a step: eight launches; three with 512 blocks and padded visits; now
+//     65k rows  126 / 115 / 55      260k  164 / 185 / 144
+//   1.04M rows  299 / 327 / 290     4.1M  918 / 1084 / 866
 constexpr int MD_J = 8;
 constexpr int MD_R = 4;
 constexpr int MAX_BASIS = 512;
 enum GsStage : int { GS_GATHER = 0, GS_AXPY = 1 };
+
+// The block's visits in groups of MD_R and a rest: f(R, i0) takes rows i0 + e S, e < R, of
+// this thread (rows beyond n only in the last visit of the last blocks).
+template <class F>
+__device__ __forceinline__ void gs_visits(int64_t n, const F& f) {
+  const int64_t S = int64_t(gridDim.x) * TPB;
+  int64_t b0 = int64_t(blockIdx.x) * TPB;   // the block's first row of the visit
+  for (; b0 + (MD_R - 1) * S < n; b0 += MD_R * S) f(std::integral_constant<int, MD_R>(), b0 + threadIdx.x);
+  if (b0 + 2 * S < n) f(std::integral_constant<int, 3>(), b0 + threadIdx.x);
+  else if (b0 + S < n) f(std::integral_constant<int, 2>(), b0 + threadIdx.x);
+  else if (b0 < n) f(std::integral_constant<int, 1>(), b0 + threadIdx.x);
+}
 
 // w is written by the same thread earlier in the kernel: plain loads
 template <int JN>
@@ -214,10 +233,11 @@ __device__ __forceinline__ void md_chunk(int64_t n, const double* __restrict__ V
   double acc[JN];
 #pragma unroll
   for (int q = 0; q < JN; ++q) acc[q] = 0.0;
-  for (int64_t i0 = int64_t(blockIdx.x) * TPB + threadIdx.x; i0 < n; i0 += MD_R * S) {
-    double wv[MD_R], vv[JN][MD_R];
+  gs_visits(n, [&](auto group, int64_t i0) {
+    constexpr int R = decltype(group)::value;
+    double wv[R], vv[JN][R];
 #pragma unroll
-    for (int e = 0; e < MD_R; ++e) {
+    for (int e = 0; e < R; ++e) {
       const int64_t i = i0 + e * S;
       const int64_t bi = basis_row(i, ldb);
       wv[e] = i < n ? w[i] : 0.0;
@@ -225,15 +245,31 @@ __device__ __forceinline__ void md_chunk(int64_t n, const double* __restrict__ V
       for (int q = 0; q < JN; ++q) vv[q][e] = i < n ? Vc[bi + q * kBasisBlock] : 0.0;
     }
 #pragma unroll
-    for (int e = 0; e < MD_R; ++e) {
+    for (int e = 0; e < R; ++e) {
       if (i0 + e * S < n) {
 #pragma unroll
         for (int q = 0; q < JN; ++q) acc[q] += vv[q][e] * wv[e];
       }
     }
-  }
+  });
 #pragma unroll
   for (int q = 0; q < JN; ++q) sh[q][threadIdx.x] = acc[q];
+}
+
+// Sum of f(0) .. f(TPB - 1) by one warp, as the tree t += t + TPB / 2, .. , t += t + 1 adds
+// them; complete in lane 0
+template <class F>
+__device__ __forceinline__ double warp_tree(const F& f) {
+  static_assert(TPB == 256, "eight values a lane");
+  double a[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) a[i] = f((threadIdx.x & 31) + 32 * i);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < o; ++i) a[i] += a[i + o];
+  for (int o = 16; o > 0; o >>= 1) a[0] += __shfl_down_sync(0xffffffffu, a[0], o);
+  return a[0];
 }
 
 template <int STAGE, bool NORM>
@@ -253,49 +289,50 @@ __global__ void __launch_bounds__(TPB) k_gram_schmidt(int64_t n, int k, const do
     for (int j = tid; j < k; j += TPB) hs[j] = h[j];
     __syncthreads();
   }
-  for (int64_t i0 = int64_t(blockIdx.x) * TPB + tid; i0 < n; i0 += MD_R * S) {
-    double v[MD_R];
+  gs_visits(n, [&](auto group, int64_t i0) {
+    constexpr int R = decltype(group)::value;
+    double v[R];
     if (STAGE == GS_GATHER) {
-      int32_t at[MD_R];
+      int32_t at[R];
 #pragma unroll
-      for (int e = 0; e < MD_R; ++e) at[e] = i0 + e * S < n ? map[i0 + e * S] : 0;
+      for (int e = 0; e < R; ++e) at[e] = i0 + e * S < n ? map[i0 + e * S] : 0;
 #pragma unroll
-      for (int e = 0; e < MD_R; ++e) v[e] = z[at[e]];
+      for (int e = 0; e < R; ++e) v[e] = z[at[e]];
     } else {
-      double acc[MD_R];
-      int64_t bi[MD_R];
+      double acc[R];
+      int64_t bi[R];
 #pragma unroll
-      for (int e = 0; e < MD_R; ++e) {
-        const int64_t i = i0 + e * S < n ? i0 + e * S : i0;
+      for (int e = 0; e < R; ++e) {
+        const int64_t i = i0 + e * S;
         acc[e] = 0.0;
-        v[e] = w[i];
-        bi[e] = basis_row(i, ldb);
+        v[e] = i < n ? w[i] : 0.0;
+        bi[e] = basis_row(i < n ? i : n - 1, ldb);
       }
       int j = 0;
       for (; j + 4 <= k; j += 4) {
-        double x[4][MD_R];
+        double x[4][R];
 #pragma unroll
         for (int q = 0; q < 4; ++q)
 #pragma unroll
-          for (int e = 0; e < MD_R; ++e) x[q][e] = V[bi[e] + (j + q) * kBasisBlock];
+          for (int e = 0; e < R; ++e) x[q][e] = V[bi[e] + (j + q) * kBasisBlock];
 #pragma unroll
         for (int q = 0; q < 4; ++q)
 #pragma unroll
-          for (int e = 0; e < MD_R; ++e) acc[e] += hs[j + q] * x[q][e];
+          for (int e = 0; e < R; ++e) acc[e] += hs[j + q] * x[q][e];
       }
       for (; j < k; ++j)
 #pragma unroll
-        for (int e = 0; e < MD_R; ++e) acc[e] += hs[j] * V[bi[e] + j * kBasisBlock];
+        for (int e = 0; e < R; ++e) acc[e] += hs[j] * V[bi[e] + j * kBasisBlock];
 #pragma unroll
-      for (int e = 0; e < MD_R; ++e) v[e] -= acc[e];
+      for (int e = 0; e < R; ++e) v[e] -= acc[e];
     }
 #pragma unroll
-    for (int e = 0; e < MD_R; ++e)
+    for (int e = 0; e < R; ++e)
       if (i0 + e * S < n) {
         w[i0 + e * S] = v[e];
         if (NORM) nrm += v[e] * v[e];
       }
-  }
+  });
   // block partials: partial[j * gridDim.x + block]
   const int nj = NORM ? 1 : k;
   for (int j0 = 0; j0 < nj; j0 += MD_J) {
@@ -316,16 +353,14 @@ __global__ void __launch_bounds__(TPB) k_gram_schmidt(int64_t n, int k, const do
       }
     }
     __syncthreads();
-    for (int o = TPB / 2; o > 0; o >>= 1) {
-      if (tid < o) {
-        for (int q = 0; q < jn; ++q) sh[q][tid] += sh[q][tid + o];
-      }
-      __syncthreads();
+    static_assert(MD_J <= TPB / 32, "a warp per vector of the chunk");
+    if (const int q = tid >> 5; q < jn) {
+      const double acc = warp_tree([&](int i) { return sh[q][i]; });
+      if ((tid & 31) == 0) partial[int64_t(j0 + q) * gridDim.x + blockIdx.x] = acc;
     }
-    if (tid < jn) partial[int64_t(j0 + tid) * gridDim.x + blockIdx.x] = sh[tid][0];
     __syncthreads();
   }
-  // the last block adds the blocks' partials: a warp per vector, fixed order,
+  // the last block adds the blocks' partials: a warp per vector, fixed order
   __threadfence();
   if (tid == 0) last = atomicAdd(count, 1u) == gridDim.x - 1;
   __syncthreads();
@@ -334,22 +369,12 @@ __global__ void __launch_bounds__(TPB) k_gram_schmidt(int64_t n, int k, const do
   if (tid == 0) *count = 0u;   // for the next launch
   const int lane = tid & 31;
   for (int j = tid >> 5; j < nj; j += TPB / 32) {
-    // as a tree over TPB sums of two blocks each, lane + 32 i of them in this lane
-    static_assert(TPB == 256 && RED_BLOCKS <= 2 * TPB, "");
     const double* p = partial + int64_t(j) * gridDim.x;
-    double a[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const unsigned b = lane + 32 * i;
-      a[i] = b < gridDim.x ? __ldcg(p + b) : 0.0;
-      if (b + TPB < gridDim.x) a[i] += __ldcg(p + b + TPB);
-    }
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1)
-#pragma unroll
-      for (int i = 0; i < o; ++i) a[i] += a[i + o];
-    double acc = a[0];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    const double acc = warp_tree([&](unsigned b) {   // every TPB-th block
+      double v = b < gridDim.x ? __ldcg(p + b) : 0.0;
+      for (unsigned c = b + TPB; c < gridDim.x; c += TPB) v += __ldcg(p + c);
+      return v;
+    });
     if (lane == 0) out[j] = acc;
   }
 }
@@ -494,13 +519,16 @@ cudaError_t axpby(int64_t n, double* out, const double* x, double a, const doubl
 }
 
 
-int reduction_partials() { return RED_BLOCKS; }
-
-// blocks of a Gram-Schmidt stage: a fixed function of the rows (so are its sums)
+// Blocks of a Gram-Schmidt stage: one wave of as many blocks on every SM (four: 64 registers a
+// thread; 512 left 96 of 152 SMs with three), a fixed function of the rows and the device, and
+// so are the sums.
+static int64_t gs_most_blocks() { return int64_t(4) * sm_count(); }
 static unsigned gs_blocks(int64_t n) {
-  const int64_t b = (n + TPB - 1) / TPB;
-  return unsigned(b < 1 ? 1 : b < RED_BLOCKS ? b : RED_BLOCKS);
+  const int64_t b = (n + TPB - 1) / TPB, most = gs_most_blocks();
+  return unsigned(b < 1 ? 1 : b < most ? b : most);
 }
+
+int reduction_partials() { return int(std::max<int64_t>(RED_BLOCKS, gs_most_blocks())); }
 
 cudaError_t gs_gather_dot(int64_t n, int k, const double* V, int64_t ldb, const double* z, const int32_t* map,
                           double* w, double* partial, unsigned* count, double* out, cudaStream_t s) {
