@@ -884,11 +884,12 @@ static cudaError_t vcycle_replay(pff_mg& mg, int g, const double* r, double* z, 
   const int64_t n = mg.pb->mesh->m.lay.n_slots;
   const int b0 = g == 2 ? 0 : g, b1 = g == 2 ? 1 : g;
   const int64_t off = b0 == 0 ? 0 : 2 * n, len = (b0 == 0 ? 2 * n : 0) + (b1 == 1 ? n : 0);
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  const bool capturing = cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
+  // the last kernel reads r on fixed rows while it writes z: vectors that share memory go
+  // through the staging vectors
+  const uintptr_t ra = reinterpret_cast<uintptr_t>(r), za = reinterpret_cast<uintptr_t>(z);
+  const uintptr_t span = uintptr_t(len) * sizeof(double);
   cudaError_t e = cudaSuccess;
-  if (capturing) {
-    cudaGetLastError();
+  if (ra < za + span && za < ra + span) {
     const size_t bytes = size_t(len) * sizeof(double);
     for (int b = b0; b <= b1 && e == cudaSuccess; ++b)
       e = vcycle_bind(mg, g, b, mg.vc_in + (b == 0 ? 0 : 2 * n), mg.vc_out + (b == 0 ? 0 : 2 * n));

@@ -291,9 +291,9 @@ struct pff_mg {
   // V-cycles replayed as CUDA graphs, captured after each set-up: graph 0 and 1 one
   // block each, graph 2 both (the phi block on a forked branch beside the u block).
   // The kernels that read r and write z get the call's pointers before each launch
-  // (VcIo: those two nodes per block and their arguments); under a caller's stream
-  // capture, and while a graph is made, the vectors pass through the staging vectors
-  // vc_in and vc_out (3 * n_slots doubles).
+  // (VcIo: those two nodes per block and their arguments).  Vectors that share memory,
+  // and those of a graph being made, are the staging vectors vc_in and vc_out
+  // (3 * n_slots doubles).  A graph cannot be launched into a stream that captures.
   bool graphs_ok = true;
   cudaGraph_t vc_graph[3] = {};
   cudaGraphExec_t vc_exec[3] = {};

@@ -131,3 +131,34 @@ def test_newton_already_solved_state():
     torch.cuda.synchronize()
     assert info["converged"] and info["newton"] == 0, info
     assert bool((u == 0).all()) and bool((phi == phi_old).all()) and int(act.sum()) == 0
+
+
+@pytest.mark.parametrize("k", [1, 2])
+def test_vcycle_vectors_that_share_memory(k):
+    """r and z of a V-cycle in one buffer, shifted against each other (equal ones are
+    refused): z is what separate vectors give."""
+    import torch
+    from paper_2404_03265_gb300 import MG, PFF_F32, Problem
+    P = Pair("small", k)
+    pb = Problem(P.lm, **P.material(kappa=1e-3, p=0.05))
+    u, phi, phit = random_linearisation(P, seed=3, u_std=1e-2)
+
+    def dev(a):
+        return torch.tensor(np.ascontiguousarray(a), device="cuda")
+
+    pb.set_state(dev(P.to_slots(u).T), dev(P.to_slots(phi)), dev(P.to_slots(phit)))
+    mg = MG(pb, PFF_F32)
+    mg.setup()
+    n = P.n_slots
+    for block, size in ((0, 2 * n), (1, n)):
+        r = torch.randn(size, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(7))
+        want = torch.empty_like(r)
+        mg.vcycle(block, r, want)
+        for shift in (2, 900, n // 2, -2, -n // 2):
+            buf = torch.zeros(2 * size, dtype=torch.float64, device="cuda")
+            at = size // 2
+            buf[at:at + size] = r
+            z = buf[at + shift:at + shift + size]
+            mg.vcycle(block, buf[at:at + size], z)
+            torch.cuda.synchronize()
+            assert torch.equal(z, want), (block, shift)
