@@ -2,6 +2,9 @@
 against the sweeps that a forced strip height selects: the same bits, since both
 evaluate every cell, nodal sum, Chebyshev step and transfer row in the same order.
 
+The tile side (6, 10 or 15 nodes) goes by the tiles of a level; the larger meshes reach all
+three on whole levels and on levels with refinement edges.
+
 Meshes with one brick and with many, odd coarse grids (brick edges at every position
 of the refinement edges), hanging levels, active sets, with and without a cell modulus."""
 import numpy as np
@@ -52,3 +55,34 @@ def test_tiles_match_sweeps_bitwise(name, modulus, coarse):
     for b in (0, 1):
         assert np.all(np.isfinite(out[b][0])) and np.abs(out[b][0]).max() > 0
         assert np.array_equal(out[b][0], out[b][1]), (b, np.abs(out[b][0] - out[b][1]).max())
+
+
+def tile_sides(m):
+    """The tile side of every level >= 1: the smallest of 6, 10, 15 whose tiles that hold a
+    node are at most 2, 4, any number per streaming multiprocessor."""
+    import torch
+    from paper_2404_03265_gb300 import MG, PFF_F32, Problem
+    pb = Problem(m)
+    one = torch.ones(m.info["n_slots"], dtype=torch.float64, device="cuda")
+    pb.set_state(torch.zeros((2, m.info["n_slots"]), dtype=torch.float64, device="cuda"), one, one)
+    mg = MG(pb, PFF_F32)
+    mg.setup()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    sides = []
+    for l in range(1, mg.n_levels):
+        node = (mg.inverse_diagonal(l, 1)[1] >= 0).reshape(-1, 30, 30)
+        for t, most in ((6, 2), (10, 4), (15, None)):
+            n = node.reshape(-1, 30 // t, t, 30 // t, t).any(axis=(2, 4)).sum()
+            if most is None or n <= most * sms:
+                break
+        sides.append(t)
+    return sides
+
+
+@pytest.mark.parametrize("name", ["box9_5_1", "box9_4_4"])
+@pytest.mark.parametrize("modulus", [False, True])
+@pytest.mark.parametrize("coarse", ["direct", "chebyshev"])
+def test_every_tile_side_matches_sweeps_bitwise(name, modulus, coarse):
+    from paper_2404_03265_gb300 import Mesh
+    assert set(tile_sides(Mesh.from_recipe(synth.recipe(name)).finalize(1))) == {6, 10, 15}
+    test_tiles_match_sweeps_bitwise(name, modulus, coarse)
