@@ -293,7 +293,7 @@ __device__ __forceinline__ void q1_cell(const NodePair<P>& b, const NodePair<P>&
         if (N::xp && OP != OP_FULL) fv[q1][q2] = pmul(mq, xpq[q1][q2]);
       }
     const P wx = bc<P>(g.wx), wy = bc<P>(g.wy), nwx = bc<P>(-g.wx), nwy = bc<P>(-g.wy);
-    if (f64 && OP == OP_FULL) {
+    if (f64 && (OP == OP_FULL || OP == OP_UU)) {
       auto sum = [&](const P (*U)[2], const P (*S)[2], int a, int b, int c, int d) {
         return pfma(G[a][b], U[a][b], S[c][d]);
       };
