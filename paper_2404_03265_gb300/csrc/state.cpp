@@ -59,53 +59,68 @@ static std::vector<SmoothTile> smooth_tiles(const LevelMesh& lm, const LevelMesh
 
 // Tables of the two-pass leaf operators
 static LeafCells upload_leaf_cells(DevAllocs& mem, const Mesh& M) {
-  const int NB = M.lay.NB;
-  const size_t ns = size_t(M.lay.n_slots);
+  constexpr int NB = 30;
+  constexpr size_t SLOTS = size_t(NB) * NB;
+  const size_t ns = size_t(M.lay.n_slots), nb = M.lay.bricks.size();
+  const int k = M.k, W = M.lay.W;
   // cells in the order of their slots (brick by brick, and so level by level), each
   // level filled up to an even number with a repeated cell that no node refers to
-  std::vector<int32_t> cells(M.cell_slot), at(ns, -1), slot;
-  std::sort(cells.begin(), cells.end());
-  auto level_of = [&](int32_t s) { return M.lay.bricks[size_t(s) / (size_t(NB) * NB)].level; };
-  for (size_t q = 0; q < cells.size(); ++q) {
-    at[cells[q]] = int32_t(slot.size());
-    slot.push_back(cells[q]);
-    if ((q + 1 == cells.size() || level_of(cells[q + 1]) != level_of(cells[q])) && slot.size() % 2)
-      slot.push_back(cells[q]);
+  std::vector<int32_t> at(ns, -1), in_brick(nb, 0);
+  for (int32_t s : M.cell_slot) {
+    at[s] = 0;
+    ++in_brick[size_t(s) / SLOTS];
   }
-  const size_t nc = slot.size();
-  const int k = M.k, W = M.lay.W;
+  size_t nc = 0;
+  for (size_t b = 0; b < nb; ++b) {
+    nc += size_t(in_brick[b]);
+    if (b + 1 == nb || M.lay.bricks[b + 1].level != M.lay.bricks[b].level) nc += nc % 2;
+  }
   std::vector<int4> corner(k == 1 ? nc : 0), node(ns, make_int4(-1, -1, -1, -1)), part(size_t(M.n_partials));
-  std::vector<int32_t> nodes9(k == 2 ? 9 * nc : 0);
+  std::vector<int32_t> nodes9(k == 2 ? 9 * nc : 0), slot(nc);
   std::vector<uint8_t> level(nc), part_pos(size_t(M.n_partials), 0);
-  for (size_t q = 0; q < nc; ++q) {
-    const int32_t s = slot[q];
-    const BrickDesc& d = M.lay.bricks[size_t(s) / (size_t(NB) * NB)];
-    const int n = s % (NB * NB) % NB, r = s % (NB * NB) / NB;
-    int32_t code[9];
-    for (int b = 0; b <= k; ++b)
-      for (int a = 0; a <= k; ++a) {
-        const int i = n + a, j = r + b;   // brick position, 0..NB
-        code[a + (k + 1) * b] = d.irr >= 0 ? M.lay.win[size_t(d.irr) * W * W + (i + k) + size_t(W) * (j + k)]
-                                           : d.nbr_base[(j < NB ? 3 : 6) + (i < NB ? 1 : 2)] + i % NB + NB * (j % NB);
+  size_t q = 0;
+  for (size_t b = 0; b < nb; ++b) {
+    const BrickDesc& d = M.lay.bricks[b];
+    const int32_t* win = d.irr >= 0 ? M.lay.win.data() + size_t(d.irr) * W * W : nullptr;
+    // node at brick position (i, j), 0..NB
+    auto code = [&](int i, int j) -> int32_t {
+      if (win) return win[(i + k) + size_t(W) * (j + k)];
+      return d.nbr_base[(j < NB ? 3 : 6) + (i < NB ? 1 : 2)] + (i < NB ? i : i - NB) + NB * (j < NB ? j : j - NB);
+    };
+    for (int r = 0; in_brick[b] && r < NB; ++r)
+      for (int n = 0; n < NB; ++n) {
+        const size_t s = b * SLOTS + size_t(n + NB * r);
+        if (at[s] < 0) continue;
+        at[s] = int32_t(q);
+        slot[q] = int32_t(s);
+        level[q] = uint8_t(d.level);
+        if (k == 1) corner[q] = make_int4(code(n, r), code(n + 1, r), code(n, r + 1), code(n + 1, r + 1));
+        else
+          for (int e = 0; e < 9; ++e) nodes9[size_t(e) * nc + q] = code(n + e % 3, r + e / 3);
+        ++q;
       }
-    if (k == 1) corner[q] = make_int4(code[0], code[1], code[2], code[3]);
-    else
-      for (int e = 0; e < 9; ++e) nodes9[size_t(e) * nc + q] = code[e];
-    level[q] = uint8_t(d.level);
+    if (q % 2 && (b + 1 == nb || M.lay.bricks[b + 1].level != d.level)) {
+      slot[q] = slot[q - 1];
+      level[q] = level[q - 1];
+      if (k == 1) corner[q] = corner[q - 1];
+      else
+        for (int e = 0; e < 9; ++e) nodes9[size_t(e) * nc + q] = nodes9[size_t(e) * nc + q - 1];
+      ++q;
+    }
   }
-  for (size_t b = 0; b < M.lay.bricks.size(); ++b) {
+  for (size_t b = 0; b < nb; ++b) {
     const BrickDesc& d = M.lay.bricks[b];
     auto cell_at = [&](int n, int r) -> int32_t {   // the leaf cell of this level with lower-left node (n, r) >= -k
       const int32_t base = d.nbr_base[(r < 0 ? 0 : 3) + (n < 0 ? 0 : 1)];
-      return base < 0 ? -1 : at[size_t(base) + (n < 0 ? n + NB : n) + size_t(NB) * (r < 0 ? r + NB : r)];
+      return base < 0 ? -1 : at[size_t(base) + size_t((n < 0 ? n + NB : n) + NB * (r < 0 ? r + NB : r))];
     };
     for (int r = 0; r < NB; ++r)
       for (int n = 0; n < NB; ++n) {
-        const size_t o = size_t(n) + size_t(NB) * r, s = b * size_t(NB) * NB + o;
-        const int px = n % k, py = r % k, n0 = n - px, r0 = r - py;   // inside a Q2 cell: no left (lower) neighbour
+        const size_t o = size_t(n + NB * r), s = b * SLOTS + o;
+        const int px = n & (k - 1), py = r & (k - 1), n0 = n - px, r0 = r - py;   // inside a Q2 cell: no left (lower) neighbour
         const int4 q = make_int4(cell_at(n0, r0), px ? -1 : cell_at(n0 - k, r0), py ? -1 : cell_at(n0, r0 - k),
                                  px || py ? -1 : cell_at(n0 - k, r0 - k));
-        const int32_t p = d.irr >= 0 ? M.lay.own_part[size_t(d.irr) * NB * NB + o] : -1;
+        const int32_t p = d.irr >= 0 ? M.lay.own_part[size_t(d.irr) * SLOTS + o] : -1;
         if (p >= 0) {
           part[p] = q;
           part_pos[p] = uint8_t(px | py << 1);
@@ -273,9 +288,11 @@ std::string upload_mesh(pff_mesh& pm) {
       // 6 against 15 on a 5-level mesh of 4.3k DoFs 43.2 against 47.3 us per u-block
       // V-cycle; 10 beyond 8 tiles per SM costs 8% on the 1.04M-DoF mesh
       for (int tn : {6, 10, 15}) {
+        const int64_t most = int64_t(tn == 6 ? 2 : 4) * sm_count();
+        if (tn < 15 && lm.n_nodes > most * tn * tn) continue;   // more tiles than that
         tiles = smooth_tiles(lm, M.levels[l - 1], tn);
         L.lv.tile = tn;
-        if (int64_t(tiles.size()) <= int64_t(tn == 6 ? 2 : 4) * sm_count()) break;
+        if (int64_t(tiles.size()) <= most) break;
       }
       L.lv.tiles = D.mem.upload(tiles);
       L.lv.ntiles = int32_t(tiles.size());
@@ -297,20 +314,21 @@ std::string upload_mesh(pff_mesh& pm) {
   D.lev_total = off;
   {
     std::vector<LevBrick> lb;
-    std::vector<int32_t> home(size_t(off), -1), leaf, gx, gy;
-    std::vector<uint8_t> flags;
+    std::vector<int32_t> home(size_t(off), -1), leaf(static_cast<size_t>(off)), gx(static_cast<size_t>(off)),
+        gy(static_cast<size_t>(off));
+    std::vector<uint8_t> flags(static_cast<size_t>(off));
     std::vector<SmoothTile> tiles;
-    leaf.reserve(size_t(off)); gx.reserve(size_t(off)); gy.reserve(size_t(off)); flags.reserve(size_t(off));
     for (size_t l = 0; l < M.levels.size(); ++l) {
       const LevelMesh& lm = M.levels[l];
       const DevLevel& lv = D.levels[l].lv;
       for (size_t b = 0; b < lm.lay.bricks.size(); ++b)
         lb.push_back({int32_t(lv.off), lv.n_slots, int32_t(b) * lm.lay.NB * lm.lay.NB});
-      leaf.insert(leaf.end(), lm.slot_leaf.begin(), lm.slot_leaf.end());
-      flags.insert(flags.end(), lm.slot_flags.begin(), lm.slot_flags.end());
-      for (size_t q = 0; q < lm.slot_X.size(); ++q) {
-        gx.push_back(lm.slot_X[q] < 0 ? -1 : (lm.slot_X[q] >> (M.Lf - int(l))));
-        gy.push_back(lm.slot_Y[q] < 0 ? -1 : (lm.slot_Y[q] >> (M.Lf - int(l))));
+      std::copy(lm.slot_leaf.begin(), lm.slot_leaf.end(), leaf.begin() + lv.off);
+      std::copy(lm.slot_flags.begin(), lm.slot_flags.end(), flags.begin() + lv.off);
+      const int shift = M.Lf - int(l);
+      for (size_t q = 0; q < lm.slot_X.size(); ++q) {   // (a hole's -1 stays -1)
+        gx[size_t(lv.off) + q] = lm.slot_X[q] >> shift;
+        gy[size_t(lv.off) + q] = lm.slot_Y[q] >> shift;
       }
       if (M.k == 1) {
         D.levels[l].tile0 = int32_t(tiles.size());
