@@ -141,47 +141,43 @@ cudaError_t level_apply(pff_mg& mg, int level, int op, const T* x, T* y, cudaStr
 std::string mg_alloc(pff_mg& mg) {
   const DevMesh& D = mg.pb->mesh->dev;
   const int64_t N = D.lev_total;
-  mg.vc_in = mg.mem.alloc<double>(3 * mg.pb->mesh->m.lay.n_slots);
-  mg.vc_out = mg.mem.alloc<double>(3 * mg.pb->mesh->m.lay.n_slots);
-  mg.lin64 = mg.mem.alloc<double>(4 * N);
-  mg.lin32 = mg.mem.alloc<float>(4 * N);
-  mg.cmask = mg.mem.alloc<uint8_t>(N);
-  const size_t esz = mg.precision == PFF_F64 ? sizeof(double) : sizeof(float);
+  const int64_t ns = mg.pb->mesh->m.lay.n_slots;
+  const int nchain = 2 * int(D.levels.size());
+  // Cleared: slots without a node keep a zero inverse diagonal and zero CG vectors, and the
+  // counters are 0 between launches.
   for (int b = 0; b < 2; ++b) {
     MGBlock& B = mg.blk[b];
     B.ncomp = b == 0 ? 2 : 1;
     B.fixbits = b == 0 ? 3 : 4;
-    const int64_t n = B.ncomp * N;
-    B.dinv64 = mg.mem.alloc<double>(n);
-    B.dinv32 = mg.mem.alloc<float>(n);
-    void** bufs[6] = {&B.d, &B.x, &B.r, &B.y, &B.yp, &B.t};
-    for (auto* p : bufs) *p = mg.mem.alloc<unsigned char>(n * esz);
+    mg.mem.reserve(B.dinv64, B.ncomp * N);
+    mg.mem.reserve(B.dinv32, B.ncomp * N);
+    mg.mem.reserve(mg.su_vec[b], 5 * B.ncomp * N);
     B.lam.assign(D.levels.size(), 0.0);
   }
-  const int nchain = 2 * int(D.levels.size());
-  for (int b = 0; b < 2; ++b) mg.su_vec[b] = mg.mem.alloc<double>(5 * mg.blk[b].ncomp * N);
-  mg.su_partial = mg.mem.alloc<double>(int64_t(nchain) * mg_dot_partials());
-  mg.su_sc = mg.mem.alloc<double>(8 * nchain);
-  mg.su_hist = mg.mem.alloc<double>(2 * kMaxLanczos * nchain);
-  mg.su_count = mg.mem.alloc<unsigned>(nchain);
-  for (int b = 0; b < 2; ++b) mg.su_part[b] = mg.mem.alloc<double>(512 * D.levels.size());
-  mg.spd_bad = mg.mem.alloc<int32_t>(2);
+  mg.mem.reserve(mg.su_count, nchain);
+  mg.mem.reserve(mg.spd_bad, 2);
+  mg.mem.commit(true);
+  mg.mem.reserve(mg.vc_in, 3 * ns);
+  mg.mem.reserve(mg.vc_out, 3 * ns);
+  mg.mem.reserve(mg.lin64, 4 * N);
+  mg.mem.reserve(mg.lin32, 4 * N);
+  mg.mem.reserve(mg.cmask, N);
+  for (MGBlock& B : mg.blk)
+    for (void** p : {&B.d, &B.x, &B.r, &B.y, &B.yp, &B.t})
+      mg.mem.reserve(reinterpret_cast<unsigned char*&>(*p),
+                     size_t(B.ncomp) * N * (mg.precision == PFF_F64 ? sizeof(double) : sizeof(float)));
+  mg.mem.reserve(mg.su_partial, int64_t(nchain) * mg_dot_partials());
+  mg.mem.reserve(mg.su_sc, 8 * nchain);
+  mg.mem.reserve(mg.su_hist, 2 * kMaxLanczos * nchain);
+  for (int b = 0; b < 2; ++b) mg.mem.reserve(mg.su_part[b], 512 * D.levels.size());
+  mg.mem.commit();
   if (!mg.mem.err.empty()) return mg.mem.err;
   mg.host_len = size_t(2) * kMaxLanczos * nchain;
   if (cudaMallocHost(reinterpret_cast<void**>(&mg.host), mg.host_len * sizeof(double) + 2 * sizeof(int32_t)) != cudaSuccess) {
     mg.host = nullptr;
     return "cudaMallocHost failed";
   }
-  for (int b = 0; b < 2; ++b)   // slots without a node keep a zero inverse diagonal, CG vectors zero there
-    if (cudaMemset(mg.su_vec[b], 0, 5 * mg.blk[b].ncomp * N * sizeof(double)) != cudaSuccess) return "cudaMemset failed";
-  for (int b = 0; b < 2; ++b)
-    if (cudaMemset(mg.blk[b].dinv64, 0, mg.blk[b].ncomp * N * sizeof(double)) != cudaSuccess ||
-        cudaMemset(mg.blk[b].dinv32, 0, mg.blk[b].ncomp * N * sizeof(float)) != cudaSuccess)
-      return "cudaMemset failed";
-  if (cudaMemset(mg.su_count, 0, nchain * sizeof(unsigned)) != cudaSuccess ||
-      cudaMemset(mg.spd_bad, 0, 2 * sizeof(int32_t)) != cudaSuccess || wait_for_clears() != cudaSuccess)
-    return "cudaMemset failed";
-  return "";
+  return wait_for_clears() == cudaSuccess ? "" : "cudaMemset failed";
 }
 
 // Tables and buffers of the direct coarse solve, made by the first set-up that needs them:

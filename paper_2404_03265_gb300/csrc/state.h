@@ -38,7 +38,8 @@ struct DevAllocs {
     ptrs.push_back(p);
     return static_cast<T*>(p);
   }
-  // Several blocks out of one allocation: reserve(n) each pointer, then commit() once.
+  // Several blocks out of one allocation: reserve(n) each pointer, then commit() once
+  // (clear: all bytes zero, see wait_for_clears).
   struct Part {
     void** p;
     size_t off;
@@ -51,8 +52,12 @@ struct DevAllocs {
     parts.push_back({reinterpret_cast<void**>(&p), part_bytes});
     part_bytes += (std::max<size_t>(n, 1) * sizeof(T) + 255) / 256 * 256;
   }
-  void commit() {
+  void commit(bool clear = false) {
     unsigned char* base = parts.empty() ? nullptr : alloc<unsigned char>(part_bytes);
+    if (base && clear) {
+      const cudaError_t e = cudaMemset(base, 0, part_bytes);
+      if (e != cudaSuccess && err.empty()) err = std::string("cudaMemset: ") + cudaGetErrorString(e);
+    }
     for (const Part& q : parts)
       if (base) *q.p = base + q.off;
     parts.clear();
