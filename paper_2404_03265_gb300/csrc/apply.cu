@@ -284,7 +284,7 @@ __device__ __forceinline__ void load_row(const SweepStage<T>& st, int lane, Node
 template <typename T, int OP>
 __device__ __forceinline__ void store_owned(const LoopArgs& a, int slot, int act_s, int part, uint8_t cm, T y0, T y1,
                                             T y2) {
-  constexpr bool outU = (OP != OP_PP && OP != OP_PP_DIAG);
+  constexpr bool outU = (OP != OP_PP && OP != OP_PP_DIAG && OP != OP_MASS);
   constexpr bool outP = (OP != OP_UU && OP != OP_UU_DIAG);
   constexpr bool isDiag = (OP == OP_UU_DIAG || OP == OP_PP_DIAG);
   if (part >= 0) {
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(32 * SW_WARPS, (sw_min_blocks<T, OP>()))
 sweep_q1_kernel(const __grid_constant__ SweepArgs<T> a, const int32_t* __restrict__ units, int32_t nunits) {
   static_assert(SW_DEPTH >= 3, "the ring holds the lower row, the upper row and at least one row in flight");
   using P = typename VT<T>::T2;
-  constexpr bool outU = (OP != OP_PP && OP != OP_PP_DIAG);
+  constexpr bool outU = (OP != OP_PP && OP != OP_PP_DIAG && OP != OP_MASS);
   constexpr bool outP = (OP != OP_UU && OP != OP_UU_DIAG);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const unsigned FULL = 0xffffffffu;
@@ -852,8 +852,8 @@ cudaError_t launch_sweep(const ApplyArgs& a, cudaStream_t s) {
                    sweep_args<T>(a), units, nunits);
 }
 
-// The other leaf operators (residual, mass, crack volume and its derivatives) go through
-// the two passes of leaf_cells.cu.
+// The other leaf operators (residual, crack volume and its derivatives; the mass on meshes
+// with refinement edges) go through the two passes of leaf_cells.cu.
 template <typename T>
 cudaError_t launch_apply(const ApplyArgs& a, int op, cudaStream_t s) {
   if (a.lay.nbricks <= 0) return cudaSuccess;
@@ -873,6 +873,7 @@ cudaError_t launch_apply(const ApplyArgs& a, int op, cudaStream_t s) {
     if (op == OP_UU_DIAG) return launch_sweep<T, OP_UU_DIAG>(a, s);
     if (op == OP_PP_DIAG) return launch_sweep<T, OP_PP_DIAG>(a, s);
     if (op == OP_VJP) return launch_sweep<T, OP_VJP>(a, s);
+    if (op == OP_MASS) return launch_sweep<T, OP_MASS>(a, s);
   }
   switch (op) {
     case OP_FULL: return launch_sweep<T, OP_FULL>(a, s);
