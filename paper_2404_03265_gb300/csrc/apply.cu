@@ -852,8 +852,8 @@ cudaError_t launch_sweep(const ApplyArgs& a, cudaStream_t s) {
                    sweep_args<T>(a), units, nunits);
 }
 
-// The other leaf operators (residual, crack volume and its derivatives; the mass on meshes
-// with refinement edges) go through the two passes of leaf_cells.cu.
+// The other leaf operators (residual, crack volume and its derivatives) go through the two
+// passes of leaf_cells.cu.
 template <typename T>
 cudaError_t launch_apply(const ApplyArgs& a, int op, cudaStream_t s) {
   if (a.lay.nbricks <= 0) return cudaSuccess;

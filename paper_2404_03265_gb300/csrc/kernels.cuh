@@ -221,7 +221,7 @@ template <typename T>
 cudaError_t launch_fixup(const FixupArgs& a, cudaStream_t s);
 
 // A Q1 leaf operator with its fix-up in two passes over a.lc (leaf_cells.cu): any but
-// OP_VJP in FP64, OP_FULL and OP_FULL_T in FP32; no level operators.
+// OP_VJP and OP_MASS in FP64, OP_FULL and OP_FULL_T in FP32; no level operators.
 template <typename T>
 cudaError_t launch_leaf_cells(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s);
 template <>

@@ -123,7 +123,7 @@ __device__ __forceinline__ NodePair<P> diff(const NodePair<P>& r, const NodePair
 
 // Components an operator writes.
 template <int OP> struct Out {
-  static constexpr bool u = (OP != OP_MASS && OP != OP_TCV && OP != OP_PHIT_VJP);
+  static constexpr bool u = (OP != OP_TCV && OP != OP_PHIT_VJP);
   static constexpr int c0 = u ? 0 : 2;
 };
 
@@ -280,7 +280,6 @@ cudaError_t launch_leaf_cells<double>(const ApplyArgs& a, const FixupArgs& f, in
     case OP_FULL: return launch_op<double, OP_FULL>(a, f, s);
     case OP_FULL_T: return launch_op<double, OP_FULL_T>(a, f, s);
     case OP_RESID: return launch_op<double, OP_RESID>(a, f, s);
-    case OP_MASS: return launch_op<double, OP_MASS>(a, f, s);
     case OP_TCV: return launch_op<double, OP_TCV>(a, f, s);
     case OP_TCV_GRAD: return launch_op<double, OP_TCV_GRAD>(a, f, s);
     case OP_PHIT_VJP: return launch_op<double, OP_PHIT_VJP>(a, f, s);

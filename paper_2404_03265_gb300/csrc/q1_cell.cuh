@@ -83,12 +83,17 @@ __device__ __forceinline__ void q1_cell(const NodePair<P>& b, const NodePair<P>&
     }
   }
   if (N::xp) { fxp.init(b.xp, hb.xp, t.xp, ht.xp); fxp.values(b.xp, xpq); }
-  if (OP == OP_RESID || OP == OP_MASS || OP == OP_TCV) {
+  if (OP == OP_MASS) {
+    // (1, psi): the test below of f = 1 gives every node jxw, exactly
+    static_assert(GA + GB == 1.0, "");
+#pragma unroll
+    for (int A = 0; A < 4; ++A) rp[A] = bc<P>(g.jxw);
+  } else if (OP == OP_RESID || OP == OP_TCV) {
     // R = -A(U)(psi), Problem 2 with sigma^+ read as sigma:
     //   A_u(psi)   = (g(phi~) sigma(u), e(psi)) + (phi~^2 p, div psi)
     //   A_phi(psi) = ((1-kappa) phi sigma(u):e(u) + 2 p phi div u - G_c/l (1 - phi), psi)
     //                + G_c l (grad phi, grad psi)
-    // MASS: (1, psi);  TCV: (u . grad phi, psi)
+    // TCV: (u . grad phi, psi)
     P S11[2][2], S12[2][2], S22[2][2], fv[2][2], G[2][2], U12[2][2];
     P uxq[2][2], uyq[2][2];
     if (OP == OP_TCV) { fux.values(b.lx, uxq); fuy.values(b.ly, uyq); }
@@ -96,7 +101,6 @@ __device__ __forceinline__ void q1_cell(const NodePair<P>& b, const NodePair<P>&
     for (int q1 = 0; q1 < 2; ++q1)
 #pragma unroll
       for (int q2 = 0; q2 < 2; ++q2) {
-        if (OP == OP_MASS) { fv[q1][q2] = bc<P>(T(1)); continue; }
         if (OP == OP_TCV) {
           // u . grad phi, grad phi from the reference derivatives of phi
           const P gpx = pmul(fphi.dxi[q2], ihx), gpy = pmul(fphi.deta[q1], ihy);

@@ -149,8 +149,8 @@ static LeafCells upload_leaf_cells(DevAllocs& mem, const Mesh& M) {
 //  - FP64: always two passes (bound by the FP64 rate, and they evaluate only cells that
 //    exist): Jacobian 992 -> 741 us on 4.1M DoFs, 633 -> 199 us on the 1.04M-DoF crack
 //    mesh, 45 -> 22 us on 4.3k DoFs.  A forced strip height asks for the sweep's Jacobian.
-//    But the mass, which reads nothing and is bound by its launches, stays with the sweep
-//    where no edge needs a fix-up: 9.9 against 14.7 us on a uniform 0.79M-DoF mesh.
+//    The mass, which reads nothing and does next to no arithmetic, stays with the sweep:
+//    28 against 57 us on 4.1M DoFs, 22.6 against 20.6 on the crack mesh, 9.3 against 9.1 on 4.3k.
 //  - FP32: two passes while the contributions (48 bytes per cell, written and read again)
 //    cost less than the sweep's cells that do not exist and its few long units.  Both loops
 //    (us; input vectors in L2, and rotating through more than L2), sweep against passes:
@@ -225,9 +225,8 @@ static double* stream_contributions(pff_problem& pb, cudaStream_t s) {
   return nullptr;
 }
 
-static bool use_two_passes(const ApplyArgs& a, const FixupArgs& f, int op, bool f64) {
-  if (op == OP_VJP || a.lc.out == nullptr) return false;
-  if (op == OP_MASS && f.n == 0) return false;
+static bool use_two_passes(const ApplyArgs& a, int op, bool f64) {
+  if (op == OP_VJP || op == OP_MASS || a.lc.out == nullptr) return false;
   const bool jacobian = op == OP_FULL || op == OP_FULL_T;
   if (a.fe_degree == 2) return f64 && (jacobian || op == OP_RESID);
   if (a.sweep_sh != 0 && jacobian) return false;
@@ -236,7 +235,7 @@ static bool use_two_passes(const ApplyArgs& a, const FixupArgs& f, int op, bool 
 
 template <typename T>
 cudaError_t launch_leaf(const ApplyArgs& a, const FixupArgs& f, int op, cudaStream_t s) {
-  if (use_two_passes(a, f, op, sizeof(T) == 8))
+  if (use_two_passes(a, op, sizeof(T) == 8))
     return a.fe_degree == 1 ? launch_leaf_cells<T>(a, f, op, s) : launch_leaf_cells_q2(a, f, op, s);
   const cudaError_t e = launch_apply<T>(a, op, s);
   if (e != cudaSuccess || op == OP_VJP) return e;   // OP_VJP: per-cell outputs only
