@@ -393,11 +393,10 @@ __global__ void k_vector_final(int nb, const double* __restrict__ partial, doubl
   if (threadIdx.x == 0) out[0] = sh[0];
 }
 
-// w[map(i)] += sign * sum_j h_j V_j[i] (the sum in the order j = 0, 1, ...; loads
-// of four basis entries are issued together; h staged in shared memory; map(i) = i
-// without a map)
+// w[map[i]] += sum_j h_j V_j[i] (the sum in the order j = 0, 1, ...; loads of four basis
+// entries are issued together; h staged in shared memory)
 __global__ void k_multi_axpy(int64_t n, int k, const double* __restrict__ V, int64_t ldb, const double* __restrict__ h,
-                             double sign, double* w, const int32_t* __restrict__ map) {
+                             double* w, const int32_t* __restrict__ map) {
   __shared__ double hs[MAX_BASIS];
   for (int j = threadIdx.x; j < k; j += blockDim.x) hs[j] = h[j];
   __syncthreads();
@@ -414,8 +413,7 @@ __global__ void k_multi_axpy(int64_t n, int k, const double* __restrict__ V, int
       acc += hs[j + 3] * v3;
     }
     for (; j < k; ++j) acc += hs[j] * Vi[j * kBasisBlock];
-    const int64_t o = map ? int64_t(map[i]) : i;
-    w[o] += sign * acc;
+    w[map[i]] += acc;
   }
 }
 
@@ -552,10 +550,10 @@ cudaError_t gs_axpy_dot(int64_t n, int k, const double* V, int64_t ldb, const do
                    h, w, partial, count, out);
 }
 
-cudaError_t multi_axpy(int64_t n, int k, const double* V, int64_t ldb, const double* h, double sign, double* w,
-                       cudaStream_t s, const int32_t* map) {
+cudaError_t multi_axpy(int64_t n, int k, const double* V, int64_t ldb, const double* h, double* w, const int32_t* map,
+                       cudaStream_t s) {
   if (k > MAX_BASIS) return cudaErrorInvalidValue;
-  if (n > 0 && k > 0) k_multi_axpy<<<blocks_for(n), TPB, 0, s>>>(n, k, V, ldb, h, sign, w, map);
+  if (n > 0 && k > 0) k_multi_axpy<<<blocks_for(n), TPB, 0, s>>>(n, k, V, ldb, h, w, map);
   return cudaGetLastError();
 }
 

@@ -53,9 +53,9 @@ cudaError_t gs_gather_dot(int64_t n, int k, const double* V, int64_t ldb, const 
                           double* w, double* partial, unsigned* count, double* out, cudaStream_t s);
 cudaError_t gs_axpy_dot(int64_t n, int k, const double* V, int64_t ldb, const double* h, double* w, bool norm,
                         double* partial, unsigned* count, double* out, cudaStream_t s);
-// w[map[i]] += sign * sum_j h[j] V_j[i]  (h on the device; map[i] = i when map is null)
-cudaError_t multi_axpy(int64_t n, int k, const double* V, int64_t ldb, const double* h, double sign, double* w,
-                       cudaStream_t s, const int32_t* map = nullptr);
+// w[map[i]] += sum_j h[j] V_j[i]  (h on the device)
+cudaError_t multi_axpy(int64_t n, int k, const double* V, int64_t ldb, const double* h, double* w, const int32_t* map,
+                       cudaStream_t s);
 // V_j = a x, and vc[map[i]] = a x[i]; with nn (device) a = 1 / sqrt(nn[0]) instead
 cudaError_t store_basis(int64_t n, double* V, int64_t ldb, int j, const double* x, double a, const double* nn,
                         double* vc, const int32_t* map, cudaStream_t s);

@@ -259,7 +259,7 @@ cudaError_t gmres_solve(pff_problem& pb, pff_mg& mg, int transpose, const double
     }
     if (jd > 0) {
       RET(cudaMemcpyAsync(W.h, yh, jd * sizeof(double), cudaMemcpyHostToDevice, s));
-      RET(multi_axpy(nc, jd, W.V, ldb, W.h, 1.0, x, s, W.map));
+      RET(multi_axpy(nc, jd, W.V, ldb, W.h, x, W.map, s));
     }
     res.iterations = it;
     res.estimate = std::fabs(g[jd]);
