@@ -81,39 +81,39 @@ std::string ensure_workspace(pff_problem& pb, int restart) {
     W.nc = int64_t(map.size());
     W.map = W.mem.upload(map);
   }
-  W.V = W.mem.alloc<double>(size_t(basis_blocks(W.nc)) * size_t(restart + 1) * kBasisBlock);
-  W.wc = W.mem.alloc<double>(W.nc);
-  W.vc = W.mem.alloc<double>(n3);
-  W.w = W.mem.alloc<double>(n3);
-  W.tmp = W.mem.alloc<double>(n3);
-  W.rhs = W.mem.alloc<double>(n3);
-  W.R = W.mem.alloc<double>(n3);
-  W.res = W.mem.alloc<double>(n3);
-  W.dU = W.mem.alloc<double>(n3);
-  W.du0 = W.mem.alloc<double>(n3);
-  W.st = W.mem.alloc<double>(4 * n);
-  W.ut = W.mem.alloc<double>(3 * n);
-  W.B = W.mem.alloc<double>(n3);
-  W.act = W.mem.alloc<uint8_t>(n);
-  W.act_prev = W.mem.alloc<uint8_t>(n);
-  W.stats = W.mem.alloc<unsigned long long>(4);
-  W.partial = W.mem.alloc<double>(size_t(reduction_partials()) * (restart + 2));
-  W.h = W.mem.alloc<double>(restart + 2);
-  W.hh = W.mem.alloc<double>(2 * (restart + 1) + 1);
-  W.scal = W.mem.alloc<double>(8);
-  W.bad = W.mem.alloc<int>(1);
-  W.count = W.mem.alloc<unsigned>(1);
-  W.x32 = W.mem.alloc<float>(n3);
-  W.y32 = W.mem.alloc<float>(n3);
+  W.mem.reserve(W.vc, n3);
+  W.mem.reserve(W.count, 1);
+  W.mem.commit(true);
+  W.mem.reserve(W.V, size_t(basis_blocks(W.nc)) * size_t(restart + 1) * kBasisBlock);
+  W.mem.reserve(W.wc, W.nc);
+  W.mem.reserve(W.w, n3);
+  W.mem.reserve(W.tmp, n3);
+  W.mem.reserve(W.rhs, n3);
+  W.mem.reserve(W.R, n3);
+  W.mem.reserve(W.res, n3);
+  W.mem.reserve(W.dU, n3);
+  W.mem.reserve(W.du0, n3);
+  W.mem.reserve(W.st, 4 * n);
+  W.mem.reserve(W.ut, 3 * n);
+  W.mem.reserve(W.B, n3);
+  W.mem.reserve(W.act, n);
+  W.mem.reserve(W.act_prev, n);
+  W.mem.reserve(W.stats, 4);
+  W.mem.reserve(W.partial, size_t(reduction_partials()) * (restart + 2));
+  W.mem.reserve(W.h, restart + 2);
+  W.mem.reserve(W.hh, 2 * (restart + 1) + 1);
+  W.mem.reserve(W.scal, 8);
+  W.mem.reserve(W.bad, 1);
+  W.mem.reserve(W.x32, n3);
+  W.mem.reserve(W.y32, n3);
+  W.mem.commit();
   if (!W.mem.err.empty()) return W.mem.err;
   if (!leaf_contributions64(pb)) return "workspace: out of device memory for the cells' contributions";
   if (cudaMallocHost(reinterpret_cast<void**>(&W.host), (3 * size_t(restart + 1) + 8) * sizeof(double)) != cudaSuccess) {
     W.host = nullptr;
     return "workspace: cudaMallocHost failed";
   }
-  if (cudaMemset(W.vc, 0, n3 * sizeof(double)) != cudaSuccess ||
-      cudaMemset(W.count, 0, sizeof(unsigned)) != cudaSuccess || wait_for_clears() != cudaSuccess)
-    return "workspace: cudaMemset failed";
+  if (wait_for_clears() != cudaSuccess) return "workspace: cudaMemset failed";
   W.ready = true;
   return "";
 }
