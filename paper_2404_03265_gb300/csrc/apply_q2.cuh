@@ -26,8 +26,9 @@
 //      unconstrained nodes of regular bricks as one 8-byte store in FP32), or for the
 //      level block operators the fused Chebyshev step of ChebEpi.
 
-// Measured (Jacobian FP32, 16.4M DoFs): 212 us with single-value copies, colour phases and
-// plain contractions; 176 us in this form, with half the error against 64 bits.  16 warps
+// Measured (Jacobian FP32, 16.4M DoFs, the same vectors every call): 212 us with single-value
+// copies, colour phases and plain contractions; 176 us in this form (rotating vectors: 204 and
+// 158), with half the error against 64 bits.  16 warps
 // an SM wait in turn for the window, the barriers and the stores of irregular bricks
 // (issue slots 36% busy); the vectors and the linearisation take 32 us at the copy rate.
 

@@ -14,7 +14,8 @@
 // cells evaluated.  The sweep evaluates every position of its bricks in lock step: on a
 // crack mesh (1.04M DoFs, 348k nodes in 743k slots) 2.4 times the cells that exist, in
 // 826 one-warp strips for 152 SMs.  The contributions cost 96 bytes per cell written and
-// read again, from L2 at these sizes.
+// read again, from L2 at these sizes.  Jacobian 647 -> 200 us there, 971 -> 724 us on 4.1M
+// DoFs.
 #include "cheb.cuh"
 #include "kernels.cuh"
 #include "pdl.cuh"

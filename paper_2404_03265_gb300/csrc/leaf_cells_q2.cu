@@ -60,8 +60,8 @@ struct NodeArgs {
 // A block takes 32 cells: warp w evaluates their Gauss row w, so a cell's work is spread
 // over three warps (a third of the serial chain of a thread per cell, and units fine
 // enough to balance over the SMs); the rows' contributions meet in shared memory.
-// Measured on the 267k-DoF band mesh (22k cells), operator apply: brick kernel 141 us, one
-// thread per cell 97 us, this split 72 us (85 us when the compiler aims at 80 registers
+// Measured on the 267k-DoF band mesh (22k cells), operator apply: brick kernel 141 us (92 us
+// with the cells of q2_jac.cuh), one thread per cell 97 us, this split 72 us (85 us when the compiler aims at 80 registers
 // and more resident blocks: the FP64 pipe wants independent instructions, not warps).
 template <int OP, bool MOD>
 __global__ void __launch_bounds__(96, 5) q2_cell_kernel(const __grid_constant__ CellArgs a) {

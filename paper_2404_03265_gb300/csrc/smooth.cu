@@ -4,15 +4,18 @@
 // Down: Chebyshev degree 3 from zero on A x = d, the residual d - A x and its
 // restriction into the coarser level.  Up: prolongation of the coarse correction and
 // Chebyshev degree 3 on the new residual.  Each does three level applies; a block
-// takes a tile of 15 x 15 nodes and evaluates the cells around it that the three
-// applies need (halo 4 down, 3 up), so nothing is exchanged between blocks.
+// takes a tile of 6, 10 or 15 nodes a side (by the size of the level) and evaluates the
+// cells around it that the three applies need (halo 4 down, 3 up), so nothing is
+// exchanged between blocks.
 //
 // Why: level meshes of a crack mesh hold 10^2..10^5 nodes; a launch per apply is a
 // chain of ~100 dependent launches of 4-6 us, each a few serial L2 round trips and
 // cell rows, with most of the chip idle.  One tile per block needs one round trip
-// per level and direction, and the halo's extra cells (1.8x down, 1.5x up) cost
-// idle issue slots.  Measured (u block, 1.04M-DoF crack mesh, 13 levels): 101 launches
-// and 482 us before; 29 launches and 135 us with the tiles.
+// per level and direction, and the halo's extra cells cost idle issue slots (cells
+// evaluated per cell of the tile, down and up: side 15 1.8 and 1.5, side 10 2.3 and 1.7,
+// side 6 3.4 and 2.3).  Measured (u block, 1.04M-DoF crack mesh, 13 levels): 101 launches
+// and 482 us before; 27 launches (12 down, 12 up, defects, coarse solve, copy out) and
+// 135 us with the tiles.
 //
 // Arithmetic: every cell, nodal sum, smoother step and transfer row is the
 // expression and order of sweep_q1_kernel, k_restrict and k_prolong (the transfer

@@ -146,11 +146,12 @@ static LeafCells upload_leaf_cells(DevAllocs& mem, const Mesh& M) {
 
 // A leaf operator and its fix-up: Q1 in two passes over the cell and node lists where
 // that is the faster path (leaf_cells.cu), else the cell loop and the fix-up kernel.
-//  - FP64: always two passes (bound by the FP64 rate, and they evaluate only cells that
-//    exist): Jacobian 992 -> 741 us on 4.1M DoFs, 633 -> 199 us on the 1.04M-DoF crack
-//    mesh, 45 -> 22 us on 4.3k DoFs.  A forced strip height asks for the sweep's Jacobian.
+//  - FP64: two passes (bound by the FP64 rate, and they evaluate only cells that exist):
+//    Jacobian 971 -> 724 us on 4.1M DoFs, 647 -> 200 us on the 1.04M-DoF crack mesh, 44 ->
+//    20 us on 4.3k DoFs.  A forced strip height asks for the sweep's Jacobian.
 //    The mass, which reads nothing and does next to no arithmetic, stays with the sweep:
-//    28 against 57 us on 4.1M DoFs, 22.6 against 20.6 on the crack mesh, 9.3 against 9.1 on 4.3k.
+//    28 against 56 us on 4.1M DoFs, 22.6 against 20.6 on the crack mesh, 9.4 against 9.1 on
+//    4.3k.
 //  - FP32: two passes while the contributions (48 bytes per cell, written and read again)
 //    cost less than the sweep's cells that do not exist and its few long units.  Both loops
 //    (us; input vectors in L2, and rotating through more than L2), sweep against passes:
@@ -285,10 +286,12 @@ std::string upload_mesh(pff_mesh& pm) {
     off += lm.lay.n_slots;
     if (M.k == 1 && l > 0) {
       std::vector<SmoothTile> tiles;
-      // small levels take small tiles (a shorter chain per block) as long as the tiles
-      // are few per SM, large ones the tile with the least repeated work.  Measured:
-      // 6 against 15 on a 5-level mesh of 4.3k DoFs 43.2 against 47.3 us per u-block
-      // V-cycle; 10 beyond 8 tiles per SM costs 8% on the 1.04M-DoF mesh
+      // Small levels take small tiles (a shorter chain per block) as long as the tiles are
+      // few per SM: up to 2 of side 6, 4 of side 10; large ones side 15, which repeats the
+      // least work.  u-block V-cycles (us) on 4.3k, 65k, 0.26M-DoF box and 1.04M-DoF crack
+      // meshes: 32.8, 46.5, 69.6, 129.0; with 1 and 2 per SM 32.8, 46.7, 67.7, 128.1; with 4
+      // and 8 32.8, 45.1, 69.6, 129.6 (a 1M-DoF box 94.3, 94.3, 98.2); side 15 alone 36.9,
+      // 51.2, 69.9, 130.7.
       for (int tn : {6, 10, 15}) {
         const int64_t most = int64_t(tn == 6 ? 2 : 4) * sm_count();
         if (tn < 15 && lm.n_nodes > most * tn * tn) continue;   // more tiles than that
@@ -393,6 +396,10 @@ std::string alloc_problem(pff_problem& pb) {
   const Mesh& M = pb.mesh->m;
   const int64_t ns = M.lay.n_slots;
   const int64_t nh = int64_t(M.hang.size());
+  const DevMesh& D = pb.mesh->dev;
+  const size_t nv = cell_values(pb);
+  if (M.k == 1 && refinement_edges(D) && two_passes_f32(D.cells.ncells, ns)) pb.bufs.reserve(pb.cells32, nv);
+  if (refinement_edges(D) && nv * sizeof(double) <= kCellsWithProblem) pb.bufs.reserve(pb.cells64, nv);
   pb.bufs.reserve(pb.lin64, 4 * ns);
   pb.bufs.reserve(pb.lin32, 4 * ns);
   pb.bufs.reserve(pb.cmask, ns);
@@ -403,10 +410,6 @@ std::string alloc_problem(pff_problem& pb) {
   pb.bufs.reserve(pb.hlin32, 4 * nh);
   pb.bufs.reserve(pb.hx64, 3 * nh);
   pb.bufs.reserve(pb.hx32, 3 * nh);
-  const DevMesh& D = pb.mesh->dev;
-  const size_t nv = cell_values(pb);
-  if (refinement_edges(D) && nv * sizeof(double) <= kCellsWithProblem) pb.bufs.reserve(pb.cells64, nv);
-  if (M.k == 1 && refinement_edges(D) && two_passes_f32(D.cells.ncells, ns)) pb.bufs.reserve(pb.cells32, nv);
   pb.bufs.commit();
   if (!pb.bufs.err.empty()) {
     std::string err = pb.bufs.err;
