@@ -584,7 +584,7 @@ def kernel_source_hash():
     which the committed ncu summaries record their counters)."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("apply.cu", "apply_q2.cuh", "kernels.cuh"):
+    for name in ("apply.cu", "apply_q2.cuh", "kernels.cuh", "q1_cell.cuh", "q1_pair.cuh", "q2_jac.cuh", "leaf_cells.cu"):
         with open(os.path.join(ROOT, "paper_2404_03265_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -690,8 +690,8 @@ def main():
     t64 = time_applies(sets64, k64, 3, 1)
     g64 = dofs * k64 / t64 / 1e9
     del sets64
-    # its arithmetic roof: FP64 flops of the cell-loop kernel per launch (ncu DFMA, DADD,
-    # DMUL counts of the committed capture) against the measured FP64 FMA rate
+    # its arithmetic roof: FP64 flops of an apply's kernels (ncu DFMA, DADD, DMUL counts of
+    # the committed capture) against the measured FP64 FMA rate
     f64_flops = profiled("apply_q1_f64_apply_workload_flops.md", "fp64_flops_per_launch")
     f64 = {"value": g64, "unit": "GDoF/s", "steps": k64, "us_per_apply": 1e6 * t64 / k64,
            "hbm_frac": info["n_nodes"] * 80 / (t64 / k64) / 1e9 / load_peaks()[0],
