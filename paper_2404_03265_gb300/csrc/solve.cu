@@ -196,7 +196,7 @@ __device__ __forceinline__ int64_t basis_row(int64_t i, int64_t ldb) {
 // ... (S = the grid's thread count), the loads of MD_R visits issued together.
 //   GS_GATHER  w[i] = z[map[i]]
 //   GS_AXPY    w[i] -= sum_j h[j] V_j[i] (the sum in the order j = 0, 1, ...)
-// then out[j] = V_j . w, j < k, or with NORM out[0] = w . w.  A block's partial sums of a
+// then out[j] = V_j . w, j < k, or with NORM out[0] = w . w, out[1] = 1 / |w|.  A block's partial sums of a
 // vector are a tree over its threads, a warp per vector; the last block to finish adds the
 // blocks' partials in a fixed order, so the sums do not depend on which block that is.
 // The basis vectors go in chunks of MD_J (the last one in its own instantiation, so no
@@ -375,7 +375,10 @@ __global__ void __launch_bounds__(TPB) k_gram_schmidt(int64_t n, int k, const do
       for (unsigned c = b + TPB; c < gridDim.x; c += TPB) v += __ldcg(p + c);
       return v;
     });
-    if (lane == 0) out[j] = acc;
+    if (lane == 0) {
+      out[j] = acc;
+      if (NORM) out[1] = __ddiv_rn(1.0, __dsqrt_rn(acc));
+    }
   }
 }
 
@@ -417,10 +420,11 @@ __global__ void k_multi_axpy(int64_t n, int k, const double* __restrict__ V, int
   }
 }
 
-// basis vector j = a x, also written to vc[map[i]]; a = 1 / sqrt(nn[0]) when nn is given
+// basis vector j = a x, also written to vc[map[i]]; a = inv[0] when inv is given (formed once
+// by the norm's last block: a square root and a division per row here cost 22 us on 1.04M rows)
 __global__ void k_store_basis(int64_t n, double* V, int64_t ldb, int j, const double* __restrict__ x, double a,
-                              const double* nn, double* vc, const int32_t* __restrict__ map) {
-  if (nn) a = __ddiv_rn(1.0, __dsqrt_rn(nn[0]));
+                              const double* inv, double* vc, const int32_t* __restrict__ map) {
+  if (inv) a = inv[0];
   GRID_STRIDE(i, n) {
     const double v = a * x[i];
     V[basis_row(i, ldb) + int64_t(j) * kBasisBlock] = v;
@@ -557,9 +561,9 @@ cudaError_t multi_axpy(int64_t n, int k, const double* V, int64_t ldb, const dou
   return cudaGetLastError();
 }
 
-cudaError_t store_basis(int64_t n, double* V, int64_t ldb, int j, const double* x, double a, const double* nn,
+cudaError_t store_basis(int64_t n, double* V, int64_t ldb, int j, const double* x, double a, const double* inv,
                         double* vc, const int32_t* map, cudaStream_t s) {
-  if (n > 0) k_store_basis<<<blocks_for(n), TPB, 0, s>>>(n, V, ldb, j, x, a, nn, vc, map);
+  if (n > 0) k_store_basis<<<blocks_for(n), TPB, 0, s>>>(n, V, ldb, j, x, a, inv, vc, map);
   return cudaGetLastError();
 }
 

@@ -47,8 +47,8 @@ constexpr int64_t kBasisBlock = 2048;
 inline int64_t basis_blocks(int64_t n) { return (n + kBasisBlock - 1) / kBasisBlock; }
 // Gram-Schmidt stages, one launch each (partial: reduction_partials() doubles per vector,
 // count: one unsigned that is 0 between launches):
-//   gs_gather_dot: w[i] = z[map[i]], out[j] = V_j . w, j < k (k = 0: out[0] = w . w)
-//   gs_axpy_dot: w -= sum_j h[j] V_j, out[j] = V_j . w, j < k (norm: out[0] = w . w)
+//   gs_gather_dot: w[i] = z[map[i]], out[j] = V_j . w, j < k (k = 0: out[0] = w . w, out[1] = 1 / |w|)
+//   gs_axpy_dot: w -= sum_j h[j] V_j, out[j] = V_j . w, j < k (norm: out[0], out[1] as above)
 cudaError_t gs_gather_dot(int64_t n, int k, const double* V, int64_t ldb, const double* z, const int32_t* map,
                           double* w, double* partial, unsigned* count, double* out, cudaStream_t s);
 cudaError_t gs_axpy_dot(int64_t n, int k, const double* V, int64_t ldb, const double* h, double* w, bool norm,
@@ -56,8 +56,8 @@ cudaError_t gs_axpy_dot(int64_t n, int k, const double* V, int64_t ldb, const do
 // w[map[i]] += sum_j h[j] V_j[i]  (h on the device)
 cudaError_t multi_axpy(int64_t n, int k, const double* V, int64_t ldb, const double* h, double* w, const int32_t* map,
                        cudaStream_t s);
-// V_j = a x, and vc[map[i]] = a x[i]; with nn (device) a = 1 / sqrt(nn[0]) instead
-cudaError_t store_basis(int64_t n, double* V, int64_t ldb, int j, const double* x, double a, const double* nn,
+// V_j = a x, and vc[map[i]] = a x[i]; with inv (device) a = inv[0] instead
+cudaError_t store_basis(int64_t n, double* V, int64_t ldb, int j, const double* x, double a, const double* inv,
                         double* vc, const int32_t* map, cudaStream_t s);
 cudaError_t vsum(int64_t n, const double* a, double* partial, double* out, cudaStream_t s);
 // phi_tilde = clip(2 phi^(n-1) - phi^(n-2), 0, 1) per slot

@@ -101,7 +101,7 @@ std::string ensure_workspace(pff_problem& pb, int restart) {
   W.mem.reserve(W.stats, 4);
   W.mem.reserve(W.partial, size_t(reduction_partials()) * (restart + 2));
   W.mem.reserve(W.h, restart + 2);
-  W.mem.reserve(W.hh, 2 * (restart + 1) + 1);
+  W.mem.reserve(W.hh, 2 * (restart + 1) + 2);
   W.mem.reserve(W.scal, 8);
   W.mem.reserve(W.bad, 1);
   W.mem.reserve(W.x32, n3);
@@ -181,12 +181,12 @@ cudaError_t gmres_solve(pff_problem& pb, pff_mg& mg, int transpose, const double
   std::vector<double> H(size_t(restart + 1) * restart), cs(restart), sn(restart), g(restart + 1);
   double* h1d = W.hh;                     // first pass coefficients
   double* h2d = W.hh + (restart + 1);     // second pass
-  double* nwd = W.hh + 2 * (restart + 1); // |w|^2
-  // basis vector j (from W.wc, scaled by a or by 1 / sqrt(|w|^2) on the device) and A V_j
-  // into W.tmp; events of step j in set j % 2
-  auto next = [&](int j, double a, const double* nn) -> cudaError_t {
+  double* nwd = W.hh + 2 * (restart + 1); // |w|^2, 1 / |w|
+  // basis vector j (from W.wc, scaled by a or by inv[0] on the device) and A V_j into W.tmp;
+  // events of step j in set j % 2
+  auto next = [&](int j, double a, const double* inv) -> cudaError_t {
     cudaEvent_t* ev = pb.gm_ev + 4 * (j % 2);
-    RET(store_basis(nc, W.V, ldb, j, W.wc, a, nn, W.vc, W.map, s));
+    RET(store_basis(nc, W.V, ldb, j, W.wc, a, inv, W.vc, W.map, s));
     RET(cudaEventRecord(ev[0], s));
     RET(A(W.vc, W.tmp));
     return cudaEventRecord(ev[1], s);
@@ -217,7 +217,7 @@ cudaError_t gmres_solve(pff_problem& pb, pff_mg& mg, int transpose, const double
       // all the same leaves one apply unused (no result depends on it).
       const double red = j > 0 ? std::fabs(g[j]) / std::fabs(g[j - 1]) : 1.0;
       const bool ahead = j + 1 < restart && it + 1 < maxiter && !(std::fabs(g[j]) * red <= target);
-      if (ahead) RET(next(j + 1, 0.0, nwd));
+      if (ahead) RET(next(j + 1, 0.0, nwd + 1));
       RET(cudaEventSynchronize(pb.gm_read));
       const double* h = hh;
       const double* h2 = hh + (restart + 1);

@@ -143,7 +143,7 @@ struct SolverWS {
   uint8_t *act = nullptr, *act_prev = nullptr;
   unsigned long long* stats = nullptr;
   double *partial = nullptr, *h = nullptr, *scal = nullptr;
-  double* hh = nullptr;   // one Arnoldi step on the device: both Gram-Schmidt passes and |w|^2 (2 (restart + 1) + 1)
+  double* hh = nullptr;   // one Arnoldi step on the device: both Gram-Schmidt passes, |w|^2 and 1 / |w| (2 (restart + 1) + 2)
   int* bad = nullptr;
   unsigned* count = nullptr;   // finished blocks of a Gram-Schmidt stage (0 between launches)
   double* host = nullptr;      // pinned: coefficients of an Arnoldi step, of the solution, norms (3 (restart + 1) + 8)
