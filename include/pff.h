@@ -264,13 +264,16 @@ typedef struct pff_newton_opts {
 } pff_newton_opts;
 
 /* ---- allocation-free variant of pff_apply (no counterpart in the paper) ----
- * Same operators, arguments, layout and results as pff_apply.  The difference is
- * where the apply keeps its scratch: the interface partial sums (one triple per
- * interface node of an irregular brick, condensed by a second kernel) and, on Q1
- * meshes, the input resolved on each hanging node (one triple each).  pff_apply
- * uses buffers made by pff_problem_create; this call uses one fixed device array
- * of PFF_NOALLOC_MAX_PARTIALS triples (1.5 MiB) that is part of the library
- * image.  No device or pinned memory is allocated by the call, directly or
+ * Same operators, arguments, layout and results (the same bits) as pff_apply.  The
+ * difference is where the apply keeps its scratch.  This call goes by the cell
+ * loop, whose scratch is the interface partial sums (one triple per interface
+ * node of an irregular brick, condensed by a second kernel) and, on Q1 meshes, the
+ * input resolved on each hanging node (one triple each).  It uses one fixed device
+ * array of PFF_NOALLOC_MAX_PARTIALS triples (1.5 MiB) that is part of the library
+ * image.  pff_apply uses buffers of the problem; in FP64, and for smaller FP32 Q1
+ * applies, it goes cell by cell in two passes that also need a buffer for every
+ * cell's contributions and are faster (FP64 on a crack mesh: 3.2 times; the FP64
+ * buffer of large or uniform meshes is made by the first such apply).  No device or pinned memory is allocated by the call, directly or
  * through a library.  It serves callers that must not allocate while they run: a
  * host whose caching allocator has reserved nearly all device memory (a library
  * cudaMalloc could fail at any time there), or a latency-bound loop that cannot
