@@ -273,11 +273,12 @@ typedef struct pff_newton_opts {
  * image.  pff_apply uses buffers of the problem; in FP64, and for smaller FP32 Q1
  * applies, it goes cell by cell in two passes that also need a buffer for every
  * cell's contributions and are faster (FP64 on a crack mesh: 3.2 times; the FP64
- * buffer of large or uniform meshes is made by the first such apply).  No device or pinned memory is allocated by the call, directly or
- * through a library.  It serves callers that must not allocate while they run: a
- * host whose caching allocator has reserved nearly all device memory (a library
- * cudaMalloc could fail at any time there), or a latency-bound loop that cannot
- * afford cudaFree's implicit device synchronisation.
+ * buffer of large or uniform meshes is made by the first such apply).
+ * This call allocates no device or pinned memory, directly or through a library.
+ * It serves callers that must not allocate while they run: a host whose caching
+ * allocator has reserved nearly all device memory (a library cudaMalloc could fail
+ * at any time there), or a latency-bound loop that cannot afford cudaFree's
+ * implicit device synchronisation.
  * Set-up: pff_problem_create loads the module holding the array on the current
  * device and caches the array's address (cudaGetSymbolAddress), so that loading
  * the module, which reserves the array, does not happen inside this call.  On a
