@@ -5,7 +5,9 @@ so any two may overlap; on other meshes an FP32 apply may overlap an FP64 operat
 The calls of the streams queue up behind a delay, so that they run side by side.
 
 Fresh buffers are ready before a stream of the caller uses them: a multigrid, its set-up
-and a solve made on a side stream while the default stream is busy."""
+and a solve made on a side stream while the default stream is busy.
+
+An apply captured into a graph gives the bits of an eager one."""
 import numpy as np
 import pytest
 
@@ -111,3 +113,27 @@ def test_fresh_solver_on_a_side_stream(k, coarse):
     got = solve(torch.cuda.Stream(), True)
     for a, b in zip(want, got):
         assert np.all(np.isfinite(a)) and np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("name,k,dtype", [
+    ("box9_4_2", 1, F64), ("box9_4_2", 1, F32), ("box9_3_2", 2, F64), ("box9_3_2", 2, F32),
+    ("box16_3_0", 1, F64), ("box8_3_0", 2, F64),   # no refinement edges: the cell loop under capture
+    ("box16_6_1", 1, F64),                         # contributions made by the first apply, here under capture
+], ids=str)
+def test_captured_apply_matches_eager(name, k, dtype):
+    import torch
+    from paper_2404_03265_gb300 import PFF_OP_TRANSPOSE
+    m, pb, state, xs = problem(name, k)
+    xs = [x.to(getattr(torch, dtype)) for x in xs]
+    x, y = xs[0].clone(), torch.full_like(xs[0], float("nan"))
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        pb.apply(x[:2], x[2], y[:2], y[2], op=PFF_OP_TRANSPOSE)
+    for v in xs:
+        want = torch.full_like(v, float("nan"))
+        pb.apply(v[:2], v[2], want[:2], want[2], op=PFF_OP_TRANSPOSE)
+        x.copy_(v)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.isfinite(want).all() and torch.equal(y, want)
