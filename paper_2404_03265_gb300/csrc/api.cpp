@@ -392,7 +392,7 @@ extern "C" pff_status pff_residual(pff_problem* pb, const double* u, const doubl
                                    double* R, void* stream) {
   PFF_TRY({
     if (!pb || !u || !phi || !phi_tilde || !R) return fail(PFF_ERR_INVALID_ARG, "NULL argument");
-    std::string e = ensure_workspace(*pb, 50);
+    std::string e = ensure_workspace(*pb, 50, cudaStream_t(stream));
     if (!e.empty()) return fail(PFF_ERR_OOM, e);
     PFF_CUDA(leaf_residual(*pb, u, phi, phi_tilde, R, cudaStream_t(stream)));
     return PFF_OK;
@@ -402,7 +402,7 @@ extern "C" pff_status pff_residual(pff_problem* pb, const double* u, const doubl
 extern "C" pff_status pff_lumped_mass(pff_problem* pb, double* B, void* stream) {
   PFF_TRY({
     if (!pb || !B) return fail(PFF_ERR_INVALID_ARG, "NULL argument");
-    std::string e = ensure_workspace(*pb, 50);
+    std::string e = ensure_workspace(*pb, 50, cudaStream_t(stream));
     if (!e.empty()) return fail(PFF_ERR_OOM, e);
     PFF_CUDA(lumped_mass(*pb, B, cudaStream_t(stream)));
     return PFF_OK;
@@ -412,7 +412,7 @@ extern "C" pff_status pff_lumped_mass(pff_problem* pb, double* B, void* stream) 
 extern "C" pff_status pff_tcv(pff_problem* pb, const double* u, const double* phi, double* out_host, void* stream) {
   PFF_TRY({
     if (!pb || !u || !phi || !out_host) return fail(PFF_ERR_INVALID_ARG, "NULL argument");
-    std::string e = ensure_workspace(*pb, 50);
+    std::string e = ensure_workspace(*pb, 50, cudaStream_t(stream));
     if (!e.empty()) return fail(PFF_ERR_OOM, e);
     PFF_CUDA(total_crack_volume(*pb, u, phi, out_host, cudaStream_t(stream)));
     return PFF_OK;
@@ -451,7 +451,7 @@ extern "C" pff_status pff_gmres_solve(pff_problem* pb, pff_mg* mg, int32_t trans
     if (!pb || !mg || !rhs || !x) return fail(PFF_ERR_INVALID_ARG, "NULL argument");
     if (restart < 1 || restart > 500 || maxiter < 1 || !(rtol > 0)) return fail(PFF_ERR_INVALID_ARG, "bad options");
     if (!mg->ready) return fail(PFF_ERR_STATE, "pff_mg_setup has not been called");
-    std::string e = ensure_workspace(*pb, restart);
+    std::string e = ensure_workspace(*pb, restart, cudaStream_t(stream));
     if (!e.empty()) return fail(PFF_ERR_OOM, e);
     GmresResult gr;
     PFF_CUDA(gmres_solve(*pb, *mg, transpose, rhs, x, rtol, restart, maxiter, gr, cudaStream_t(stream)));
@@ -489,7 +489,7 @@ extern "C" pff_status pff_newton_pdas_step(pff_problem* pb, pff_mg* mg, double* 
     if (o.matvec != PFF_F64 && o.matvec != PFF_F32) return fail(PFF_ERR_INVALID_ARG, "bad matvec precision");
     if (o.restart < 1 || o.restart > 500 || o.max_newton < 0 || o.ls_max < 1 || !(o.omega > 0 && o.omega <= 1))
       return fail(PFF_ERR_INVALID_ARG, "bad Newton options");
-    std::string e = ensure_workspace(*pb, o.restart);
+    std::string e = ensure_workspace(*pb, o.restart, cudaStream_t(stream));
     if (!e.empty()) return fail(PFF_ERR_OOM, e);
     NewtonInfo ni;
     cudaError_t ce = newton_pdas_step(*pb, *mg, u, phi, phi_old, active, o, ni, cudaStream_t(stream));
@@ -527,7 +527,7 @@ extern "C" pff_status pff_tcv_gradient(pff_problem* pb, const double* u, const d
                                        void* stream) {
   PFF_TRY({
     if (!pb || !u || !phi || !g) return fail(PFF_ERR_INVALID_ARG, "NULL argument");
-    std::string e = ensure_workspace(*pb, 50);
+    std::string e = ensure_workspace(*pb, 50, cudaStream_t(stream));
     if (!e.empty()) return fail(PFF_ERR_OOM, e);
     PFF_CUDA(tcv_gradient(*pb, u, phi, g, cudaStream_t(stream)));
     return PFF_OK;
@@ -539,7 +539,7 @@ extern "C" pff_status pff_param_vjp(pff_problem* pb, const double* w, double* gE
   PFF_TRY({
     if (!pb || !w || !g_host) return fail(PFF_ERR_INVALID_ARG, "NULL argument");
     if (!pb->has_state) return fail(PFF_ERR_STATE, "pff_set_state has not been called");
-    std::string e = ensure_workspace(*pb, 50);
+    std::string e = ensure_workspace(*pb, 50, cudaStream_t(stream));
     if (!e.empty()) return fail(PFF_ERR_OOM, e);
     PFF_CUDA(param_vjp(*pb, w, gE_cells, g_host, cudaStream_t(stream)));
     return PFF_OK;
@@ -554,7 +554,7 @@ extern "C" pff_status pff_tcv_adjoint(pff_problem* pb, pff_mg* mg, const double*
     if (!pb || !mg || !u || !phi || !phi_old || !active || !g_host) return fail(PFF_ERR_INVALID_ARG, "NULL argument");
     if (mg->pb != pb) return fail(PFF_ERR_INVALID_ARG, "multigrid object of another problem");
     if (restart < 1 || restart > 500 || maxiter < 1 || !(rtol > 0)) return fail(PFF_ERR_INVALID_ARG, "bad options");
-    std::string e = ensure_workspace(*pb, restart);
+    std::string e = ensure_workspace(*pb, restart, cudaStream_t(stream));
     if (!e.empty()) return fail(PFF_ERR_OOM, e);
     GmresResult gr;
     std::string err;
@@ -594,7 +594,7 @@ extern "C" pff_status pff_tcv_adjoint_steps(pff_problem* pb, pff_mg* mg, int32_t
     if (restart < 1 || restart > 500 || maxiter < 1 || !(rtol > 0)) return fail(PFF_ERR_INVALID_ARG, "bad options");
     if (phi_tilde_mode != PFF_PHIT_PREVIOUS && phi_tilde_mode != PFF_PHIT_EXTRAPOLATED)
       return fail(PFF_ERR_INVALID_ARG, "phi_tilde_mode must be PFF_PHIT_PREVIOUS or PFF_PHIT_EXTRAPOLATED");
-    std::string e = ensure_workspace(*pb, restart);
+    std::string e = ensure_workspace(*pb, restart, cudaStream_t(stream));
     if (!e.empty()) return fail(PFF_ERR_OOM, e);
     AdjointStats st;
     std::string err;
@@ -625,7 +625,7 @@ extern "C" pff_status pff_active_set(pff_problem* pb, const double* R, const dou
                                      void* stream) {
   PFF_TRY({
     if (!pb || !R || !phi || !phi_old || !active) return fail(PFF_ERR_INVALID_ARG, "NULL argument");
-    std::string e = ensure_workspace(*pb, 50);
+    std::string e = ensure_workspace(*pb, 50, cudaStream_t(stream));
     if (!e.empty()) return fail(PFF_ERR_OOM, e);
     const cudaStream_t s = cudaStream_t(stream);
     SolverWS& W = pb->ws;
@@ -704,7 +704,7 @@ extern "C" pff_status pff_cod(pff_problem* pb, const double* u, const double* ph
   PFF_TRY({
     if (!pb || !u || !phi || (n_x > 0 && (!x_host || !cod_host))) return fail(PFF_ERR_INVALID_ARG, "NULL argument");
     if (n_x < 0) return fail(PFF_ERR_INVALID_ARG, "n_x < 0");
-    std::string e = ensure_workspace(*pb, 50);
+    std::string e = ensure_workspace(*pb, 50, cudaStream_t(stream));
     if (!e.empty()) return fail(PFF_ERR_OOM, e);
     e = cod_profile(*pb, u, phi, x_host, n_x, cod_host, cudaStream_t(stream));
     if (!e.empty()) return fail(PFF_ERR_CUDA, "pff_cod: " + e);

@@ -177,7 +177,7 @@ std::string mg_alloc(pff_mg& mg) {
     mg.host = nullptr;
     return "cudaMallocHost failed";
   }
-  return wait_for_clears() == cudaSuccess ? "" : "cudaMemset failed";
+  return "";
 }
 
 // Tables and buffers of the direct coarse solve, made by the first set-up that needs them:
@@ -228,7 +228,6 @@ static std::string coarse_alloc(pff_mg& mg) {
   a.cmask = mg.cmask;   // level 0 comes first
   a.bad = mg.spd_bad;
   std::string err = mem.err;
-  if (err.empty() && wait_for_clears() != cudaSuccess) err = "coarse tables: upload failed";
   if (!err.empty()) {   // give everything back: a later set-up starts afresh
     mem.release();
     std::memset(&a, 0, sizeof(a));
@@ -495,9 +494,11 @@ std::string mg_setup(pff_mg& mg, cudaStream_t s) {
     B.c0_deg = 0;
   }
   if (mg.coarse_mode == 0 && !mg.coarse_ready) {
+    mg.settled = false;
     const std::string e = coarse_alloc(mg);
     if (!e.empty()) return e;
   }
+  if (!mg.settled) CK(after_clears(s));
   bool replay = false;
   if (mg.su_graph_ok && mg.su_setups > 0) {
     std::vector<unsigned char> key = setup_key(mg);
@@ -530,6 +531,7 @@ std::string mg_setup(pff_mg& mg, cudaStream_t s) {
   CK(cudaMemcpyAsync(hist, mg.su_hist, mg.host_len * sizeof(double), cudaMemcpyDeviceToHost, s));
   if (mg.coarse_mode == 0) CK(cudaMemcpyAsync(bad, mg.spd_bad, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
+  mg.settled = true;
   if (bad[0] || bad[1]) return "coarse level block is not positive definite";
   for (int b = 0; b < 2; ++b)
     for (int l = 0; l < nl; ++l) {

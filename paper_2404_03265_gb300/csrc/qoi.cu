@@ -139,7 +139,7 @@ std::string cod_profile(pff_problem& pb, const double* u, const double* phi, con
   auto ck = [&](cudaError_t e) {
     if (e != cudaSuccess && err.empty()) err = cudaGetErrorString(e);
   };
-  if (err.empty()) ck(wait_for_clears());   // the uploads, before s reads them
+  if (err.empty()) ck(after_clears(s));   // the uploads
   if (err.empty()) ck(make_state(n, u, phi, phi, D.slot_flags, D.hang, D.nhang, k, W.st, s));
   if (err.empty() && nx > 0) {
     k_cod<<<nx, COD_T, 0, s>>>(k, dptr, dent, W.st, n, deta, dw, dout);

@@ -64,7 +64,7 @@ void release_workspace(SolverWS& W) {
   W = SolverWS();
 }
 
-std::string ensure_workspace(pff_problem& pb, int restart) {
+std::string ensure_workspace(pff_problem& pb, int restart, cudaStream_t s) {
   SolverWS& W = pb.ws;
   const int64_t n = pb.mesh->m.lay.n_slots;
   if (W.ready && W.restart >= restart) return "";
@@ -113,7 +113,7 @@ std::string ensure_workspace(pff_problem& pb, int restart) {
     W.host = nullptr;
     return "workspace: cudaMallocHost failed";
   }
-  if (wait_for_clears() != cudaSuccess) return "workspace: cudaMemset failed";
+  if (after_clears(s) != cudaSuccess) return "workspace: ordering after the clears failed";
   W.ready = true;
   return "";
 }

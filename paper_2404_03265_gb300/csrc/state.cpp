@@ -24,6 +24,16 @@ static DevLayout upload_layout(DevAllocs& mem, const Layout& L) {
   return d;
 }
 
+cudaError_t after_clears(cudaStream_t s) {
+  if (s == nullptr || s == cudaStreamLegacy) return cudaSuccess;
+  cudaEvent_t ev = nullptr;
+  cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventRecord(ev, cudaStreamLegacy);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev, 0);
+  if (ev) cudaEventDestroy(ev);   // released when it has completed
+  return e;
+}
+
 // Tiles of the fused smoothers: every tn x tn part of a brick of level mesh lm that
 // holds a node, with the storage bases around the brick and around its parent brick (bx / 2,
 // by / 2) of the next coarser level.

@@ -16,10 +16,11 @@
 
 namespace pff {
 
-// Waits for clears (cudaMemset) and uploads of fresh buffers.  Both run on the legacy
-// default stream and may still be on their way when the call returns, and neither the
-// set-up's pool streams nor a caller's non-blocking stream waits for that stream.
-inline cudaError_t wait_for_clears() { return cudaStreamSynchronize(cudaStreamLegacy); }
+// Orders stream s after the clears (cudaMemset) and uploads of fresh buffers made so far.
+// Both run on the legacy default stream and may still be on their way when the call
+// returns, and neither the set-up's pool streams nor a caller's non-blocking stream waits
+// for that stream by itself.
+cudaError_t after_clears(cudaStream_t s);
 
 // Owns a list of cudaMalloc'ed blocks.
 struct DevAllocs {
@@ -39,7 +40,7 @@ struct DevAllocs {
     return static_cast<T*>(p);
   }
   // Several blocks out of one allocation: reserve(n) each pointer, then commit() once
-  // (clear: all bytes zero, see wait_for_clears).
+  // (clear: all bytes zero, see after_clears).
   struct Part {
     void** p;
     size_t off;
@@ -289,6 +290,7 @@ struct pff_mg {
   // the direct coarse solve's blocks (made by the first set-up that needs them)
   pff::DevAllocs coarse_mem;
   bool coarse_ready = false;
+  bool settled = false;            // a set-up has waited for the clears and uploads of all buffers
   pff::CoarseArgs coarse = {};
   double* host = nullptr;          // pinned: CG coefficients (host_len doubles), then the coarse status
   size_t host_len = 0;
@@ -340,7 +342,7 @@ cudaError_t launch_leaf_cmask(int64_t n, const uint8_t* slot_flags, const uint8_
 // solvers (solver.cpp)
 cudaError_t leaf_op(pff_problem& pb, int kop, int mode, const double* lin, const uint8_t* cmask, const double* xu,
                     const double* xp, double* yu, double* yp, cudaStream_t s);
-std::string ensure_workspace(pff_problem& pb, int restart);
+std::string ensure_workspace(pff_problem& pb, int restart, cudaStream_t s);
 void release_workspace(SolverWS& W);
 cudaError_t gmres_solve(pff_problem& pb, pff_mg& mg, int transpose, const double* b, double* x, double rtol,
                         int restart, int maxiter, GmresResult& res, cudaStream_t s, int matvec = PFF_F64);
